@@ -213,7 +213,7 @@ template <int W, int BLOCK>
 __global__ void __launch_bounds__(BLOCK, (BLOCK <= 256 ? 4 : 2))
 k_b_pmerge(BatchBufs<W> S, int step, double delta) {
     using A = PassArgs<W>;
-    constexpr uint32_t C = Stage<W>::C, SL = Stage<W>::S;
+    constexpr uint32_t C = Stage<W>::C;
     __shared__ __align__(8) uint64_t s_bar;
     __shared__ unsigned long long s_base;
     __shared__ uint32_t s_n;
@@ -227,18 +227,18 @@ k_b_pmerge(BatchBufs<W> S, int step, double delta) {
         g_range[0] = g_range[1] = 0ULL;
         mbar_init(&s_bar, 1);
     }
-    for (uint32_t k = threadIdx.x; k < SL; k += BLOCK) A::tab()[k] = 0u;
+    pass_init<W, BLOCK>();
     __syncthreads();
     const unsigned long long dbits = (unsigned long long)__double_as_longlong(delta);
     const unsigned long long total = S.tile_prefix[S.B];
     const CandRegions cd{};
     Pending<W> pd;
     pd.on = false;
-    pd.all_ties = false;
+    pd.all_ties = true;
     pd.T = 0;
 #pragma unroll
     for (int w = 0; w < W; ++w) { pd.tk.x[w] = 0; pd.tk.z[w] = 0; }
-    uint32_t tag = 0, parity = 0;
+    uint32_t pass = 0, parity = 0;
     for (unsigned long long t = blockIdx.x; t < total; t += gridDim.x) {
         const int b = owner(S.tile_prefix, S.B, t);
         const uint32_t p = (uint32_t)(t - S.tile_prefix[b]);
@@ -253,6 +253,7 @@ k_b_pmerge(BatchBufs<W> S, int step, double delta) {
         const GateArg<W>& g = s_g;
         const double rnorm = s_rnorm;
         const uint64_t R = S.part_cap / ctl->part_P;
+        const uint32_t p_id = identity_part<W>(ctl->part_P);
         unsigned int* cur_p = S.cursor + (uint64_t)b * S.part_max + p;
         uint64_t np = *cur_p;
         if (np > R) np = R;
@@ -301,12 +302,13 @@ k_b_pmerge(BatchBufs<W> S, int step, double delta) {
             }
             // every thread has read the cursor: leave it zero for the next step
             if (threadIdx.x == 0) *cur_p = 0u;
-            tag = next_tag<W, BLOCK>(tag, A::tab());
-            stage_pass<W, BLOCK>((uint32_t)np, shift, g, pd, rnorm, dbits, ctl, nxt, tag, kout,
-                                 cout, st, cd, room);
+            ++pass;
+            stage_pass<W, BLOCK, PassRoom::kExact>((uint32_t)np, shift, g, pd, rnorm, dbits,
+                                                   p == p_id, ctl, nxt, pass, kout, cout, st, cd,
+                                                   room);
         } else {
-            merge_long<W, BLOCK>(kp, cp, np, g, pd, rnorm, dbits, ctl, nxt, &tag, kout, cout, st,
-                                 cd, ~0ULL, room, cur_p, &s_n);
+            merge_long<W, BLOCK>(kp, cp, np, g, pd, rnorm, dbits, p == p_id, ctl, nxt, &pass, kout,
+                                 cout, st, cd, ~0ULL, room, cur_p, &s_n);
         }
         // the largest written pattern (overflow check of post_one)
 #pragma unroll

@@ -241,6 +241,16 @@ __device__ __forceinline__ bool key_is_zero_xor(const PKey<W>& k, const GateArg<
     return a == 0;
 }
 
+// Whether a == k * Q.
+template <int W>
+__device__ __forceinline__ bool key_is_partner(const PKey<W>& a, const PKey<W>& k,
+                                                    const GateArg<W>& g) {
+    uint64_t d = 0;
+#pragma unroll
+    for (int w = 0; w < W; ++w) d |= (a.x[w] ^ k.x[w] ^ g.qx[w]) | (a.z[w] ^ k.z[w] ^ g.qz[w]);
+    return d == 0;
+}
+
 template <int W>
 __device__ __forceinline__ bool key_eq(const PKey<W>& a, const PKey<W>& b) {
     uint64_t d = 0;

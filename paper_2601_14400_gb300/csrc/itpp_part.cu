@@ -215,7 +215,7 @@ k_gate_part(const PKey<W>* __restrict__ pk, const double* __restrict__ pc,
             ChunkDesc* chunks1, uint32_t max_chunks, int retry_pass) {
     using G = Stage<W>;
     using A = PassArgs<W>;
-    constexpr uint32_t C = G::C, S = G::S;
+    constexpr uint32_t C = G::C;
     __shared__ __align__(8) uint64_t s_bar;
     __shared__ unsigned long long s_chunk, s_chsz, s_nout;
     __shared__ uint32_t s_long, s_n;
@@ -255,7 +255,7 @@ k_gate_part(const PKey<W>* __restrict__ pk, const double* __restrict__ pc,
         s_thr = thr;
         if (blockIdx.x == 0 && !ctl->status && !retry_pass) ctl->drop_on = thr != dbits;
     }
-    for (uint32_t k = threadIdx.x; k < S; k += BLOCK) A::tab()[k] = 0u;
+    pass_init<W, BLOCK>();
     __syncthreads();
     if (s_stop) return;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -271,7 +271,8 @@ k_gate_part(const PKey<W>* __restrict__ pk, const double* __restrict__ pc,
     // this CTA's output chunk: [ch_start, ch_pos) written, [ch_pos, ch_end)
     // free (the same on every thread)
     unsigned long long ch_start = 0, ch_pos = 0, ch_end = 0;
-    uint32_t tag = 0, parity = 0;
+    uint32_t pass = 0, parity = 0;
+    const uint32_t p_id = identity_part<W>(P);
     ChunkDesc* __restrict__ chunks_out = cur ? chunks0 : chunks1;
     // record the written run of a chunk for the readers of the whole state
     auto record_chunk = [&](unsigned long long start, unsigned long long end) {
@@ -366,14 +367,16 @@ k_gate_part(const PKey<W>* __restrict__ pk, const double* __restrict__ pc,
                 }
                 parity ^= 1u;
             }
-            tag = next_tag<W, BLOCK>(tag, A::tab());
-            // room for the pass's kept children, claimed once their number
-            // is known: the rest of the current chunk, else a fresh one (the
-            // rest of the old one is left as a hole)
+            ++pass;
+            // room for the most children the pass can have, claimed once the
+            // pairs are known: the rest of the current chunk, else a fresh one
+            // (the rest of the old one is left as a hole); the next partition
+            // starts right behind the kept ones
             unsigned long long at = 0;
             bool failed = false;
-            const uint32_t tot = stage_pass<W, BLOCK>(
-                (uint32_t)np, shift, g, pd, rnorm, s_thr, ctl, nxt, tag, kout, cout, st, cd,
+            const uint32_t tot = stage_pass<W, BLOCK, PassRoom::kBound>(
+                (uint32_t)np, shift, g, pd, rnorm, s_thr, p == p_id, ctl, nxt, pass, kout, cout,
+                st, cd,
                 [&](uint32_t t) -> unsigned long long {
                     if (ch_end - ch_pos < t && !claim(t)) {
                         failed = true;
@@ -404,7 +407,8 @@ k_gate_part(const PKey<W>* __restrict__ pk, const double* __restrict__ pc,
             unsigned long long at = pre;
             bool failed = false;
             const uint32_t done = merge_long<W, BLOCK>(
-                kp, cp, np, g, pd, rnorm, s_thr, ctl, nxt, &tag, kout, cout, st, cd, pre,
+                kp, cp, np, g, pd, rnorm, s_thr, p == p_id, ctl, nxt, &pass, kout, cout, st, cd,
+                pre,
                 [&](uint32_t t) -> unsigned long long {
                     if (ch_end - ch_pos < t && !claim(t)) {
                         failed = true;

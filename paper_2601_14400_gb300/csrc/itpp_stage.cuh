@@ -97,8 +97,9 @@ template <int W>
 __device__ __forceinline__ Pending<W> pending_of(const DevCtl* ctl) {
     Pending<W> q;
     q.on = ctl->pend != 0;
-    q.all_ties = ctl->pend_all_ties != 0;
-    q.T = ctl->pend_T;
+    // without a pending select every pattern passes: none lies below zero
+    q.all_ties = !q.on || ctl->pend_all_ties != 0;
+    q.T = q.on ? ctl->pend_T : 0ULL;
 #pragma unroll
     for (int w = 0; w < W; ++w) { q.tk.x[w] = ctl->pend_tie_key[w]; q.tk.z[w] = ctl->pend_tie_key[W + w]; }
     return q;
@@ -221,84 +222,110 @@ template <> struct StageGeom<1> { static constexpr int kItems = 1024, kSlots = 2
 template <> struct StageGeom<2> { static constexpr int kItems = 512, kSlots = 1024; };
 
 // Dynamic shared memory of the merge: the staged keys, their values (raw
-// coefficient in, normalised coefficient after phase A, merged children
-// after phase B; two spare slots let a copy start at the 16-byte boundary
-// below an odd element), the pair table and per-item flags.
+// coefficient in, normalised coefficient after the join; two spare slots let
+// a copy start at the 16-byte boundary below an odd element), the pair table
+// and the pass's work list.
 template <int W>
 struct Stage {
     static constexpr int C = StageGeom<W>::kItems, S = StageGeom<W>::kSlots;
     static constexpr size_t kKeys = 0;
     static constexpr size_t kVals = kKeys + sizeof(PKey<W>) * C;
     static constexpr size_t kTab = kVals + sizeof(double) * (C + 2);
-    static constexpr size_t kFlags = kTab + sizeof(uint32_t) * S;
-    static constexpr size_t kBytes = (kFlags + sizeof(uint16_t) * C + 15) / 16 * 16;
+    static constexpr size_t kList = kTab + sizeof(uint32_t) * S;
+    static constexpr size_t kBytes = (kList + sizeof(uint16_t) * C + 15) / 16 * 16;
     static_assert(kVals % 16 == 0 && kTab % 16 == 0, "alignment");
-    static_assert(C <= 1024 && S <= 2048, "slot and index fields");
+    static_assert(C <= 1024 && S <= 65536, "slot and index fields");
 };
 
 // The merge's dynamic shared memory (Stage<W> layout) and its small shared
 // counters, at file scope so that every access is a constant offset from the
 // CTA's shared window rather than a pointer held in registers.
 extern __shared__ __align__(16) unsigned char g_stage[];
-__shared__ uint32_t g_warp[32];  // the block scan's warp totals
 __shared__ uint32_t g_cn;        // this CTA's candidates
 __shared__ unsigned long long g_range[2];   // candidate range [lo, hi] (hi == 0: none)
+// per pass (indexed by its parity): the work list's lengths (pairs in the low
+// half, pass-through strings in the high half) and the children kept so far
+__shared__ uint32_t g_lists[2], g_kept[2];
 
 // Waits on a staging copy's barrier before the CTA gives up: each wait
 // sleeps up to a millisecond, and a copy of a few tens of kilobytes completes
 // within microseconds; this bound is seconds.
 constexpr uint32_t kWaitPolls = 4096u;
 
-// Pair table of one pass.  A commuting string K and its partner Q.K agree
-// outside the gate's bits, so both hash the key with those bits cleared and
-// walk the same probe sequence.  A slot holds (tag << 20) | (late << 10) |
-// early: the first string of a pair to arrive claims a free slot as `early`
-// (late = early while it is alone); its partner, arriving later, finds it on
-// the way (the first free slot of the sequence is claimed by exactly one of
-// them, and the other sees the claim) and records itself as `late`.  After
-// the pass's barrier a string reads its partner from its own slot, with no
-// second walk.  Tags grow with every pass of the CTA, so a slot of an
-// earlier pass is free and the table needs no clearing.  Returns the slot,
-// or kNoSlot when the table is full.
-constexpr uint32_t kNoSlot = 0xffffffffu;
-constexpr uint32_t kTagMax = 0xfffu;
-
+// Commutation and the sign of Q P = s R in one pass over the masks.  Site by
+// site Q and P anticommute where bit (x qz ^ z qx) is set, and there their
+// product is +i or -i times a letter: minus for (Q, P) = (X, Z), (Z, Y),
+// (Y, X), that is where (x qx) ^ (z qz ~qx) ^ (qx ~qz) is set.  With a
+// anticommuting sites, m of them minus, the phase is i^(a - 2m): P and Q
+// commute when a is even, and then s = -1 when a/2 - m is odd.  Only a
+// modulo 4 and the parity of m are needed, so the second count is one popc of
+// the xor of the halves (popc runs at a quarter of the integer rate).
 template <int W>
-__device__ __forceinline__ uint32_t pair_join(const PKey<W>& K, const GateArg<W>& g, uint32_t i,
-                                              const PKey<W>* keys_s, uint32_t* tab,
-                                              uint32_t tag) {
+__device__ __forceinline__ bool commute_sign(const PKey<W>& k, const GateArg<W>& g, bool* neg) {
+    int a = 0;
+    uint32_t mw = 0;
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+        const uint64_t an = (k.x[w] & g.qz[w]) ^ (k.z[w] & g.qx[w]);
+        const uint64_t mi = an & ((k.x[w] & g.qx[w]) ^ (k.z[w] & (g.qz[w] & ~g.qx[w])) ^
+                                  (g.qx[w] & ~g.qz[w]));
+        a += __popcll(an);
+        mw ^= (uint32_t)mi ^ (uint32_t)(mi >> 32);
+    }
+    *neg = (((a >> 1) ^ __popc(mw)) & 1) != 0;
+    return (a & 1) == 0;
+}
+
+// Slot of a commuting string in the pair table: a multilinear hash of the key
+// with the gate's bits cleared, on which K and Q.K agree (32-bit multiplies:
+// the 64-bit ones cost four times as many issue slots).
+template <int W>
+__device__ __forceinline__ uint32_t pair_slot(const PKey<W>& K, const GateArg<W>& g) {
     constexpr uint32_t S = StageGeom<W>::kSlots;
     constexpr int kBits = S == 2048 ? 11 : 10;
     static_assert(S == (1u << kBits), "slots");
-    // multiplicative hash of the key with the gate's bits cleared (K and Q.K
-    // agree on it)
-    uint64_t hm = 0;
+    uint32_t h = 0;
 #pragma unroll
     for (int w = 0; w < W; ++w) {
-        hm = (hm ^ (K.x[w] & ~g.qx[w])) * 0x9E3779B97F4A7C15ULL;
-        hm = (hm ^ (K.z[w] & ~g.qz[w])) * 0xC2B2AE3D27D4EB4FULL;
+        const uint64_t mx = K.x[w] & ~g.qx[w], mz = K.z[w] & ~g.qz[w];
+        h = h * 0x2c1b3c6du + (uint32_t)mx * 0x9e3779b1u + (uint32_t)(mx >> 32) * 0x85ebca77u +
+            (uint32_t)mz * 0xc2b2ae3du + (uint32_t)(mz >> 32) * 0x27d4eb2fu;
     }
-    uint32_t h = (uint32_t)(hm >> (64 - kBits));
-    const PKey<W> P = key_xor(K, g);
+    return h >> (32 - kBits);
+}
+
+// Pair table of one pass.  A commuting string K and its partner Q.K agree
+// outside the gate's bits, so both hash to the same slot and walk the same
+// probe sequence.  An occupied slot holds the index of the first string of a
+// pair to arrive and the sign, and, once its partner has come by, the
+// partner's index; 0 is a free slot.  The first free slot of the sequence is
+// claimed by exactly one of the two (compare-and-swap), and the other finds
+// the claim on its way; only it changes a claimed slot, with a plain store.
+// The phase that consumes the table leaves every slot free again.
+constexpr uint32_t kSlotUsed = 0x80000000u, kSlotNeg = 0x00200000u, kSlotPair = 0x00100000u;
+
+// Enter string i into its pair; true when it claimed the pair's slot (*slot).
+template <int W>
+__device__ __forceinline__ bool pair_enter(const PKey<W>& K, const GateArg<W>& g, uint32_t i,
+                                           bool neg, const PKey<W>* keys_s, uint32_t* tab,
+                                           DevCtl* ctl, uint32_t* slot) {
+    constexpr uint32_t S = StageGeom<W>::kSlots;
+    const uint32_t claim = kSlotUsed | (neg ? kSlotNeg : 0u) | i;
+    uint32_t h = pair_slot(K, g);
     for (uint32_t q = 0; q < S; ++q) {
-        uint32_t v = tab[h];
-        for (;;) {
-            if ((v >> 20) != tag) {                                // free: claim it
-                const uint32_t o = atomicCAS(tab + h, v, (tag << 20) | (i << 10) | i);
-                if (o == v) return h;
-                v = o;
-                continue;
-            }
-            const uint32_t e = v & 0x3ffu;
-            if (((v >> 10) & 0x3ffu) != e || !key_eq(keys_s[e], P)) break;   // not mine
-            // my partner, alone: only I write this slot now (a claimed slot is
-            // changed by the partner of its string alone), no atomic needed
-            tab[h] = (v & ~(0x3ffu << 10)) | (i << 10);
-            return h;
+        const uint32_t v = atomicCAS(tab + h, 0u, claim);
+        if (v == 0u) {
+            *slot = h;
+            return true;
+        }
+        if (!(v & kSlotPair) && key_is_partner(keys_s[v & 0x3ffu], K, g)) {
+            tab[h] = v | kSlotPair | (i << 10);
+            return false;
         }
         h = (h + 1) & (S - 1);
     }
-    return kNoSlot;
+    set_status(ctl, ST_CAPACITY, 41);   // not reached: the table is at most half full
+    return false;
 }
 
 // Statistics of the kept children for the top-M select: the largest
@@ -307,34 +334,6 @@ struct SelStats {
     unsigned long long out_max;
     uint32_t above;
 };
-
-// Write one staged item's kept children at pos (and pos + 1) and fold them
-// into the statistics.  Every lane of the warp calls it.
-template <int W>
-__device__ __forceinline__ void stage_emit(const PKey<W>& K, double va, double b, uint32_t o,
-                                           const GateArg<W>& g, PKey<W>* kout, double* cout,
-                                           uint64_t pos, SelStats& st, const CandRegions& cd) {
-    if (o & 1u) {
-        store_key_stream(kout + pos, K);
-        __stcs(cout + pos, va);
-    }
-    const uint64_t pb = pos + (o & 1u);
-    if (o & 2u) {
-        store_key_stream(kout + pb, key_xor(K, g));
-        __stcs(cout + pb, b);
-    }
-    const unsigned long long a = (o & 1u) ? abs_pattern(va) : 0ULL;
-    const unsigned long long bb = (o & 2u) ? abs_pattern(b) : 0ULL;
-    st.out_max = max(st.out_max, max(a, bb));
-    const unsigned long long hi = g_range[1];
-    if (hi) {   // uniform
-        const unsigned long long lo = g_range[0], w = hi - lo;
-        st.above += (a > hi ? 1u : 0u) + (bb > hi ? 1u : 0u);
-        // a - lo <= w on unsigned values: lo <= a <= hi (a kept child has a > 0)
-        cand_push((o & 1u) && a - lo <= w, a - lo, pos, cd, &g_cn);
-        cand_push((o & 2u) && bb - lo <= w, bb - lo, pb, cd, &g_cn);
-    }
-}
 
 template <int W>
 struct PassArgs {
@@ -347,187 +346,244 @@ struct PassArgs {
     __device__ __forceinline__ static uint32_t* tab() {
         return reinterpret_cast<uint32_t*>(g_stage + Stage<W>::kTab);
     }
-    __device__ __forceinline__ static uint16_t* flags() {   // phase A: slot | live | comm
-        return reinterpret_cast<uint16_t*>(g_stage + Stage<W>::kFlags);
+    __device__ __forceinline__ static uint16_t* list() {
+        return reinterpret_cast<uint16_t*>(g_stage + Stage<W>::kList);
     }
 };
 
-// Exclusive block scan with one barrier: every warp writes its total, then
-// every warp scans the warp totals with shuffles (g_warp may be rewritten
-// only after the caller's next barrier).
-template <int BLOCK>
-__device__ __forceinline__ uint32_t block_scan_1bar(uint32_t v, uint32_t* total) {
-    constexpr int NW = BLOCK / 32;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t x = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
+// The shared state of the passes before a CTA's first one (a barrier must
+// follow): every slot free, both parities' counters zero.
+template <int W, int BLOCK>
+__device__ __forceinline__ void pass_init() {
+    uint32_t* tab = PassArgs<W>::tab();
+    for (uint32_t k = threadIdx.x; k < (uint32_t)StageGeom<W>::kSlots; k += BLOCK) tab[k] = 0u;
+    if (threadIdx.x < 2) {
+        g_lists[threadIdx.x] = 0u;
+        g_kept[threadIdx.x] = 0u;
     }
-    if (lane == 31) g_warp[warp] = x;
-    __syncthreads();
-    uint32_t t = lane < NW ? g_warp[lane] : 0u;
-#pragma unroll
-    for (int o = 1; o < NW; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, t, o);
-        if (lane >= o) t += y;
-    }
-    const uint32_t before = __shfl_sync(0xffffffffu, t, warp > 0 ? warp - 1 : 0);
-    *total = __shfl_sync(0xffffffffu, t, NW - 1);
-    return (warp > 0 ? before : 0u) + x - v;
 }
 
-// One pass of the gate over n staged strings.  Phase A: the deferred
-// select's kept set, commutation, sign, the normalised coefficient c, and
-// each commuting string joins its pair in the table.  Phase B: the later
-// string of each pair present computes both merged children,
-//   K:   c_K cosh(theta) + c_QK (-sinh(theta)) s,
-//   QK:  c_QK cosh(theta) + c_K (-sinh(theta)) s
-// (the sign s of Q.K = s QK is also that of Q.QK = s K, Sec. II.B), and
-// owns both for writing; a string without its partner owns itself and its
-// child QK; an anticommuting string passes through; threshold and weight
-// cutoff per child, the identity's merged coefficient as the next
-// normaliser.  Then a block scan of the owned children, room(total) for the
-// position of the pass's segment (the same on every thread; ~0 when there is
-// none: nothing is written) and the write pass.  Three barriers (and any the
-// room call takes); the staging arrays are free again when it returns.
-// Returns the kept children counted (the same on every thread).
-template <int W, int BLOCK, class Room>
-__device__ __forceinline__ uint32_t stage_pass(uint32_t n, uint32_t shift, const GateArg<W>& g,
-                                               const Pending<W>& pd, double rnorm,
-                                               unsigned long long dbits, DevCtl* ctl, int nxt,
-                                               uint32_t tag, PKey<W>* kout, double* cout,
-                                               SelStats& st, const CandRegions& cd, Room&& room) {
-    using A = PassArgs<W>;
-    double* vals = A::vals() + shift;
-    // phase A; flags: slot (11 bits) | neg << 13 | live << 14 | comm << 15
-    for (uint32_t i = threadIdx.x; i < n; i += BLOCK) {
-        const PKey<W> K = A::keys()[i];
-        const double raw = vals[i];
-        const bool live = !pd.on || cap_keep(K, raw, pd.T, pd.all_ties, pd.tk);
-        const bool id = key_is_zero(K);
-        if (!live && id) set_status(ctl, ST_TRACE_ZERO, 43);
-        const bool comm = live && commutes(K, g);
-        const bool neg = comm && product_negative(K, g);
-        // the identity's normalised value is exactly 1
-        vals[i] = id ? 1.0 : __dmul_rn(raw, rnorm);
-        uint32_t slot = 0;
-        if (comm) {
-            slot = pair_join(K, g, i, A::keys(), A::tab(), tag);
-            if (slot == kNoSlot) {
-                set_status(ctl, ST_CAPACITY, 41);
-                slot = 0;
-            }
-        }
-        A::flags()[i] = (uint16_t)(slot | (neg ? 0x2000u : 0u) | (live ? 0x4000u : 0u) |
-                                   (comm ? 0x8000u : 0u));
+// Count (and with kWrite store) a warp's kept children: K with va, and KQ with
+// vb.  One shared atomic per warp gives the run; the order inside a
+// partition's segment is immaterial.  Every lane of the warp calls it.
+template <int W, bool kWrite>
+__device__ __forceinline__ void emit_children(bool ka, bool kb, const PKey<W>& K,
+                                              const GateArg<W>& g, double va, double vb,
+                                              PKey<W>* kout, double* cout, uint64_t base,
+                                              uint32_t* kept, SelStats& st,
+                                              const CandRegions& cd) {
+    const unsigned int ba = __ballot_sync(0xffffffffu, ka), bb = __ballot_sync(0xffffffffu, kb);
+    const uint32_t na = __popc(ba), tot = na + __popc(bb);
+    if (!tot) return;
+    const int lane = threadIdx.x & 31;
+    uint32_t q = 0;
+    if (lane == 0) q = atomicAdd(kept, tot);
+    if (!kWrite) return;
+    q = __shfl_sync(0xffffffffu, q, 0);
+    const unsigned int lt = (1u << lane) - 1u;
+    const uint64_t pa = base + q + __popc(ba & lt), pb = base + q + na + __popc(bb & lt);
+    unsigned long long a = 0, b = 0;
+    if (ka) {
+        store_key_stream(kout + pa, K);
+        __stcs(cout + pa, va);
+        a = abs_pattern(va);
     }
-    __syncthreads();                                                  // (1) table built
-    // phase B; flags: kept children (2 bits) | alone << 2 | neg << 3 |
-    // partner << 4 (10 bits) | late << 14
-    uint32_t cnt = 0;
-    for (uint32_t i = threadIdx.x; i < n; i += BLOCK) {
-        const uint32_t f = A::flags()[i];
-        uint32_t o = 0;
-        if (f & 0x4000u) {
-            const PKey<W> K = A::keys()[i];
-            const double c = vals[i];
-            if (!(f & 0x8000u)) {            // {P,Q} = 0: unchanged
-                bool keep = above(c, dbits) && light(K, g.maxw);
-                if (key_is_zero(K)) {
-                    ctl->norm[nxt] = c;
-                    if (!keep) set_status(ctl, ST_TRACE_ZERO, 1);
-                    keep = true;
-                }
-                o = keep ? 1u : 0u;
-            } else {
-                const uint32_t v = A::tab()[f & 0x7ffu];
-                const uint32_t e = v & 0x3ffu, l = (v >> 10) & 0x3ffu;
-                const bool neg = (f & 0x2000u) != 0;
+    if (kb) {
+        store_key_stream(kout + pb, key_xor(K, g));
+        __stcs(cout + pb, vb);
+        b = abs_pattern(vb);
+    }
+    st.out_max = max(st.out_max, max(a, b));
+    const unsigned long long hi = g_range[1];
+    if (hi) {   // uniform
+        const unsigned long long lo = g_range[0], w = hi - lo;
+        st.above += (a > hi ? 1u : 0u) + (b > hi ? 1u : 0u);
+        // a - lo <= w on unsigned values: lo <= a <= hi (a kept child has a > 0)
+        cand_push(ka && a - lo <= w, a - lo, pa, cd, &g_cn);
+        cand_push(kb && b - lo <= w, b - lo, pb, cd, &g_cn);
+    }
+}
+
+// Phase B of a pass: the work list, pairs first (whole warps), then the
+// strings that pass through.  kWrite: store the kept children from `base` on;
+// kClear: leave the pair table free for the next pass.
+template <int W, int BLOCK, bool kWrite, bool kClear>
+__device__ __forceinline__ void pass_children(uint32_t n_pair, uint32_t n_through, uint32_t shift,
+                                              const GateArg<W>& g, unsigned long long dbits,
+                                              bool has_id, DevCtl* ctl, int nxt, PKey<W>* kout,
+                                              double* cout, uint64_t base, uint32_t* kept,
+                                              SelStats& st, const CandRegions& cd) {
+    using A = PassArgs<W>;
+    const double* vals = A::vals() + shift;
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t pair_end = (n_pair + 31u) & ~31u;
+    for (uint32_t j0 = threadIdx.x & ~31u; j0 < pair_end + n_through; j0 += BLOCK) {
+        PKey<W> K;
+#pragma unroll
+        for (int w = 0; w < W; ++w) { K.x[w] = 0; K.z[w] = 0; }
+        double va = 0.0, vb = 0.0;
+        bool ka = false, kb = false;
+        if (j0 < pair_end) {   // warp-uniform
+            const uint32_t j = j0 + lane;
+            if (j < n_pair) {
+                const uint32_t slot = A::list()[j];
+                const uint32_t v = A::tab()[slot];
+                if (kClear) A::tab()[slot] = 0u;
+                const uint32_t e = v & 0x3ffu;
+                K = A::keys()[e];
+                const double c = vals[e];
+                // a lone string's absent partner contributes a zero addend,
+                // which changes no nonzero sum
+                const double cq = (v & kSlotPair) ? vals[(v >> 10) & 0x3ffu] : 0.0;
                 const double m = __longlong_as_double(
-                    __double_as_longlong(g.msh) ^ (neg ? (long long)0x8000000000000000ULL : 0LL));
-                const PKey<W> KQ = key_xor(K, g);
-                double va, vb;
-                uint32_t own = 0;
-                if (l == e) {                // alone: K and its child QK
-                    va = __dmul_rn(c, g.ch);
-                    vb = __dmul_rn(c, m);
-                    own = 0x4u;
-                } else if (l == i) {         // the pair's later string: both
-                    const double cq = vals[e];
-                    va = __dadd_rn(__dmul_rn(c, g.ch), __dmul_rn(cq, m));
-                    vb = __dadd_rn(__dmul_rn(cq, g.ch), __dmul_rn(c, m));
-                    vals[i] = va;
-                    vals[e] = vb;
-                    own = 0x4000u | (e << 4);
-                }
-                if (own) {
-                    bool ka = above(va, dbits) && light(K, g.maxw);
-                    bool kb = above(vb, dbits) && light(KQ, g.maxw);
+                    __double_as_longlong(g.msh) ^
+                    ((v & kSlotNeg) ? (long long)0x8000000000000000ULL : 0LL));
+                va = __dadd_rn(__dmul_rn(c, g.ch), __dmul_rn(cq, m));
+                vb = __dadd_rn(__dmul_rn(cq, g.ch), __dmul_rn(c, m));
+                ka = above(va, dbits) && light(K, g.maxw);
+                kb = above(vb, dbits) && light(key_xor(K, g), g.maxw);
+                if (has_id) {
                     if (key_is_zero(K)) {
-                        ctl->norm[nxt] = va;
+                        if (kWrite) ctl->norm[nxt] = va;
                         if (!ka) set_status(ctl, ST_TRACE_ZERO, 1);
                         ka = true;
                     }
-                    if (key_is_zero(KQ)) {
-                        ctl->norm[nxt] = vb;
+                    if (key_is_zero_xor(K, g)) {
+                        if (kWrite) ctl->norm[nxt] = vb;
                         if (!kb) set_status(ctl, ST_TRACE_ZERO, 1);
                         kb = true;
                     }
-                    o = (ka ? 1u : 0u) | (kb ? 2u : 0u) | own | (neg ? 0x8u : 0u);
+                }
+            }
+        } else {
+            const uint32_t j = j0 - pair_end + lane;
+            if (j < n_through) {   // {P,Q} = 0: unchanged
+                const uint32_t i = A::list()[Stage<W>::C - 1 - j];
+                K = A::keys()[i];
+                va = vals[i];
+                ka = above(va, dbits) && light(K, g.maxw);
+                if (has_id && key_is_zero(K)) {
+                    if (kWrite) ctl->norm[nxt] = va;
+                    if (!ka) set_status(ctl, ST_TRACE_ZERO, 1);
+                    ka = true;
                 }
             }
         }
-        A::flags()[i] = (uint16_t)o;
-        cnt += __popc(o & 3u);
+        emit_children<W, kWrite>(ka, kb, K, g, va, vb, kout, cout, base, kept, st, cd);
     }
-    uint32_t tot;
-    const uint32_t off = block_scan_1bar<BLOCK>(cnt, &tot);          // (2)
-    const unsigned long long base = room(tot);
-    if (base != ~0ULL) {
-        uint64_t pos = base + off;
-        // write pass: warp-uniform rounds (the candidate list is filled warp-wide)
-        for (uint32_t i0 = 0; i0 < n; i0 += BLOCK) {
-            const uint32_t i = i0 + threadIdx.x;
-            uint32_t o = 0;
-            PKey<W> K;
-#pragma unroll
-            for (int w = 0; w < W; ++w) { K.x[w] = 0; K.z[w] = 0; }
-            double va = 0.0, vb = 0.0;
-            if (i < n) {
-                const uint32_t f = A::flags()[i];
-                o = f & 3u;
-                if (o) {
-                    K = A::keys()[i];
-                    va = vals[i];
-                    if (f & 0x4u) {          // alone: both children from c
-                        const double m = __longlong_as_double(
-                            __double_as_longlong(g.msh) ^
-                            ((f & 0x8u) ? (long long)0x8000000000000000ULL : 0LL));
-                        vb = __dmul_rn(va, m);
-                        va = __dmul_rn(va, g.ch);
-                    } else if (f & 0x4000u) {
-                        vb = vals[(f >> 4) & 0x3ffu];
-                    }
-                }
-            }
-            stage_emit(K, va, vb, o, g, kout, cout, pos, st, cd);
-            pos += __popc(o);
-        }
-    }
-    __syncthreads();                                                  // (3) staging free
-    return tot;
 }
 
-// The tag of the next pass (every thread calls it): slots hold 12-bit tags,
-// so after 4095 passes of one CTA the table is cleared and tags restart.
-template <int W, int BLOCK>
-__device__ __forceinline__ uint32_t next_tag(uint32_t tag, uint32_t* tab) {
-    if (tag < kTagMax) return tag + 1u;
-    for (uint32_t k = threadIdx.x; k < (uint32_t)StageGeom<W>::kSlots; k += BLOCK) tab[k] = 0u;
+// How a pass learns where its children go.  kBound: room(most) is asked for
+// the most children the pass can have (live pass-through strings once,
+// pairs twice: at most twice the live strings, so the claims of a gate never
+// exceed twice its input), before any child is computed; what stays unused
+// behind the kept ones is the caller's.  kExact: the children are counted
+// first and room(kept) gives a run with no holes (the batch's contiguous
+// output).  kCount: they are counted only.
+enum class PassRoom { kBound, kExact, kCount };
+
+// One pass of the gate over n staged strings.
+//
+// Join: the deferred select's kept set, commutation and sign, the normalised
+// coefficient c; each commuting string enters its pair in the table, the
+// claimers go on the work list and so do the strings that pass through.
+// Children: one thread per pair (not per string) computes both merged
+// children,
+//   K:   c_K cosh(theta) + c_QK (-sinh(theta)) s,
+//   QK:  c_QK cosh(theta) + c_K (-sinh(theta)) s
+// (the sign s of Q.K = s QK is also that of Q.QK = s K, Sec. II.B), tests them
+// and stores the kept ones.
+//
+// What bounds it: instruction issue, and the double-precision pipe (about two
+// lanes per clock and SM on GB300, a whole warp's slot for every instruction
+// however few lanes take part).  Hence the work list: over the strings
+// themselves only the quarter or so that owns a pair would be active in the
+// six double-precision instructions.  Against a per-string second phase, a
+// block scan and a third, writing phase this issues about a third of the
+// instructions and waits twice per partition instead of three times.
+// Two barriers (and any the room call takes); returns the kept children
+// (the same on every thread).  `pass` numbers the CTA's passes: counters
+// alternate by its parity.
+template <int W, int BLOCK, PassRoom kRoom, class Room>
+__device__ __forceinline__ uint32_t stage_pass(uint32_t n, uint32_t shift, const GateArg<W>& g,
+                                               const Pending<W>& pd, double rnorm,
+                                               unsigned long long dbits, bool has_id, DevCtl* ctl,
+                                               int nxt, uint32_t pass, PKey<W>* kout, double* cout,
+                                               SelStats& st, const CandRegions& cd, Room&& room) {
+    using A = PassArgs<W>;
+    double* vals = A::vals() + shift;
+    const uint32_t lane = threadIdx.x & 31u, par = pass & 1u;
+    const unsigned int lt = (1u << lane) - 1u;
+    for (uint32_t i0 = threadIdx.x & ~31u; i0 < n; i0 += BLOCK) {   // whole warps
+        const uint32_t i = i0 + lane;
+        uint32_t slot = 0;
+        bool owner = false, through = false;
+        if (i < n) {
+            const PKey<W> K = A::keys()[i];
+            const double raw = vals[i];
+            const unsigned long long b = abs_pattern(raw);
+            bool live = b >= pd.T;   // pd.T == 0 with every tie kept: no select pending
+            if (b == pd.T && !pd.all_ties) live = !key_less(pd.tk, K);
+            double c = __dmul_rn(raw, rnorm);
+            if (has_id && key_is_zero(K)) {
+                c = 1.0;   // the identity's normalised value is exactly 1
+                if (!live) set_status(ctl, ST_TRACE_ZERO, 43);
+            }
+            vals[i] = c;
+            bool neg;
+            const bool comm = commute_sign(K, g, &neg);
+            through = live && !comm;
+            if (live && comm) owner = pair_enter(K, g, i, neg, A::keys(), A::tab(), ctl, &slot);
+        }
+        __syncwarp();
+        const unsigned int bo = __ballot_sync(0xffffffffu, owner);
+        const unsigned int bt = __ballot_sync(0xffffffffu, through);
+        uint32_t q = 0;
+        if (lane == 0) q = atomicAdd(&g_lists[par], (uint32_t)__popc(bo) | (__popc(bt) << 16));
+        q = __shfl_sync(0xffffffffu, q, 0);
+        if (owner) A::list()[(q & 0xffffu) + __popc(bo & lt)] = (uint16_t)slot;
+        if (through) A::list()[Stage<W>::C - 1 - ((q >> 16) + __popc(bt & lt))] = (uint16_t)i;
+    }
+    __syncthreads();                                                  // (1) pairs and list built
+    const uint32_t lists = g_lists[par];
+    const uint32_t n_pair = lists & 0xffffu, n_through = lists >> 16;
+    // the other parity's counters: last read before barrier (1), next used
+    // after barrier (2)
+    if (threadIdx.x == 0) {
+        g_lists[par ^ 1u] = 0u;
+        g_kept[par ^ 1u] = 0u;
+    }
+    uint32_t* kept = &g_kept[par];
+    if (kRoom == PassRoom::kBound) {
+        const unsigned long long base = room(n_through + 2u * n_pair);
+        if (base != ~0ULL)
+            pass_children<W, BLOCK, true, true>(n_pair, n_through, shift, g, dbits, has_id, ctl,
+                                                nxt, kout, cout, base, kept, st, cd);
+        __syncthreads();                                              // (2) staging free
+        return *kept;
+    }
+    if (kRoom == PassRoom::kCount) {
+        pass_children<W, BLOCK, false, true>(n_pair, n_through, shift, g, dbits, has_id, ctl, nxt,
+                                             kout, cout, 0ULL, kept, st, cd);
+        __syncthreads();
+        return *kept;
+    }
+    pass_children<W, BLOCK, false, false>(n_pair, n_through, shift, g, dbits, has_id, ctl, nxt,
+                                          kout, cout, 0ULL, kept, st, cd);
     __syncthreads();
-    return 1u;
+    const uint32_t tot = *kept;
+    const unsigned long long base = room(tot);
+    __syncthreads();   // every thread has read the count: it restarts as the write position
+    if (threadIdx.x == 0) *kept = 0u;
+    __syncthreads();
+    if (base != ~0ULL)
+        pass_children<W, BLOCK, true, true>(n_pair, n_through, shift, g, dbits, has_id, ctl, nxt,
+                                            kout, cout, base, kept, st, cd);
+    else   // no room: the caller goes on with other instances, the table free
+        pass_children<W, BLOCK, false, true>(n_pair, n_through, shift, g, dbits, has_id, ctl, nxt,
+                                             kout, cout, 0ULL, kept, st, cd);
+    __syncthreads();
+    return tot;
 }
 
 // A partition above the staging capacity, in k sub-passes over the hash
@@ -541,8 +597,8 @@ __device__ __forceinline__ uint32_t next_tag(uint32_t tag, uint32_t* tab) {
 template <int W, int BLOCK, class Room>
 __device__ __forceinline__ uint32_t merge_long(const PKey<W>* kp, const double* cp, uint64_t np,
                                             const GateArg<W>& g, const Pending<W>& pd,
-                                            double rnorm, unsigned long long dbits, DevCtl* ctl,
-                                            int nxt, uint32_t* tag,
+                                            double rnorm, unsigned long long dbits, bool has_id,
+                                            DevCtl* ctl, int nxt, uint32_t* pass,
                                             PKey<W>* kout, double* cout, SelStats& st,
                                             const CandRegions& cd, unsigned long long pre,
                                             Room&& room, unsigned int* cursor_p, uint32_t* s_n) {
@@ -563,7 +619,7 @@ __device__ __forceinline__ uint32_t merge_long(const PKey<W>* kp, const double* 
             for (uint64_t i = threadIdx.x; i < np; i += BLOCK) {
                 const PKey<W> K = load_key_stream(kp + i);
                 const double raw = __ldcs(cp + i);
-                const bool live = !pd.on || cap_keep(K, raw, pd.T, pd.all_ties, pd.tk);
+                const bool live = cap_keep(K, raw, pd.T, pd.all_ties, pd.tk);
                 if (!live) {
                     if (key_is_zero(K)) set_status(ctl, ST_TRACE_ZERO, 43);
                     continue;
@@ -582,14 +638,32 @@ __device__ __forceinline__ uint32_t merge_long(const PKey<W>* kp, const double* 
             // every thread has read the cursor: leave it zero for the next scatter
             if (j == 0 && cursor_p && threadIdx.x == 0) *cursor_p = 0u;
             const uint32_t n = *s_n < C ? *s_n : C;
-            *tag = next_tag<W, BLOCK>(*tag, A::tab());
-            const unsigned long long at = write ? base + done : ~0ULL;
-            done += stage_pass<W, BLOCK>(n, 0u, g, pd, rnorm, dbits, ctl, nxt, *tag, kout, cout,
-                                         st, cd, [at](uint32_t) { return at; });
+            *pass += 1u;
+            if (write) {
+                const unsigned long long at = base + done;
+                done += stage_pass<W, BLOCK, PassRoom::kBound>(
+                    n, 0u, g, pd, rnorm, dbits, has_id, ctl, nxt, *pass, kout, cout, st, cd,
+                    [at](uint32_t) { return at; });
+            } else {
+                done += stage_pass<W, BLOCK, PassRoom::kCount>(
+                    n, 0u, g, pd, rnorm, dbits, has_id, ctl, nxt, *pass, kout, cout, st, cd,
+                    [](uint32_t) { return 0ULL; });
+            }
         }
         total = done;
     }
     return total;
+}
+
+// The partition that holds the identity (the all-zero key, in every mode of
+// the partition function): only there the identity and the child that falls
+// on it need looking for.
+template <int W>
+__device__ __forceinline__ uint32_t identity_part(uint32_t P) {
+    PKey<W> k;
+#pragma unroll
+    for (int w = 0; w < W; ++w) { k.x[w] = 0; k.z[w] = 0; }
+    return (uint32_t)((key_hash(k) * (uint64_t)P) >> 32);
 }
 
 template <int W, int BLOCK>
