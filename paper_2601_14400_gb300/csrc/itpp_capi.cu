@@ -14,6 +14,7 @@
 #include "itpp_common.cuh"
 #include "itpp_ctx.h"
 #include "itpp_launch.h"
+#include "itpp_run.cuh"
 
 using namespace itpp;
 
@@ -67,6 +68,8 @@ void free_all(itpp_ctx* h) {
     if (h->psd_mem) cudaFree(h->psd_mem);
     if (h->s.cand.cnt) cudaFree(h->s.cand.cnt);
     if (h->s.sp_drift) cudaFree(h->s.sp_drift);
+    if (h->run_shared) cudaFree(h->run_shared);
+    if (h->run_cnt) cudaFree(h->run_cnt);
     if (h->h_ctl) cudaFreeHost(h->h_ctl);
     for (int k = 0; k < kKinds; ++k)
         for (auto& e : h->ev[k]) { cudaEventDestroy(e.a); cudaEventDestroy(e.b); }
@@ -116,10 +119,106 @@ itpp_status sync_ctl(itpp_ctx* h) {
     return h->sticky;
 }
 
+// Bounds up to this run a layer in one launch (itpp_run.cu).
+constexpr uint64_t kRunMax = 1ULL << 21;
+
+// Gates [k0, k0 + n) n_layers times in one launch (n <= kRunChunk).
+template <int W>
+itpp_status run_launch(itpp_ctx* h, int k0, int n, int n_layers, unsigned long long* log) {
+    DeviceState& s = h->s;
+    RunChunk<W> ch;
+    for (int j = 0; j < n; ++j) {
+        const HostGate& g = h->gates[(size_t)(k0 + j)];
+        RunGate<W>& r = ch.g[j];
+        for (int w = 0; w < W; ++w) {
+            r.qx[w] = g.qx[w];
+            r.qz[w] = g.qz[w];
+            r.win[w] = ~g.keep_x[w];
+        }
+        r.ch = g.ch;
+        r.msh = g.msh;
+        r.pair = g.pair_mode;
+        r.sites = g.win_sites;
+        r.start = g.win_start;
+        r.pad = 0;
+    }
+    RunArgs<W> a{};
+    for (int i = 0; i < 2; ++i) {
+        a.k[i] = static_cast<PKey<W>*>(s.keys[i]);
+        a.c[i] = s.coef[i];
+    }
+    a.kp = static_cast<PKey<W>*>(s.part_keys);
+    a.cp = s.part_coef;
+    a.cnt = h->run_cnt;
+    a.ctl = s.ctl;
+    a.scratch = s.table;
+    a.shared = h->run_shared;
+    a.drift = s.sp_drift;
+    a.log = log;
+    a.buf_cap = s.buf_cap;
+    a.home_cap = s.part_cap < s.buf_cap ? s.part_cap : s.buf_cap;
+    const uint64_t bytes = s.table_slots * slot_bytes(W);
+    a.cand_cap = bytes / (12 + sizeof(PKey<W>)) - 64;
+    if (a.cand_cap > a.home_cap) a.cand_cap = a.home_cap;
+    a.tie_off = (a.cand_cap * 12 + 255) / 256 * 256;
+    a.cap_M = s.cap_M;
+    a.cand_hi = 4096;
+    std::memcpy(&a.delta_bits, &s.delta, sizeof a.delta_bits);
+    a.part_max = h->run_part_max;
+    a.drift_stride = s.layer_gates + 1;
+    a.drift_gates = s.layer_gates;
+    a.B = 1;
+    a.one_gates = n;
+    a.one_n = s.n;
+    a.gate0 = k0;
+    a.n_layers = n_layers;
+    a.target = s.part_target;
+    a.min_part = kRunMinPart;
+    a.cap_policy = s.cap_policy;
+    a.maxw = h->p.max_weight ? h->p.max_weight : (1 << 30);
+    if (!h->contiguous && launch_materialize(s, h->stream) != cudaSuccess) return cuda_fail(h);
+    h->contiguous = true;
+    itpp_detail_touch(h);
+    if (cudaMemsetAsync(h->run_shared, 0, run_shared_head(), h->stream) != cudaSuccess ||
+        launch_run<W>(a, ch, h->run_grid, h->stream) != cudaSuccess)
+        return cuda_fail(h);
+    h->launches += 1;
+    return ITPP_OK;
+}
+
+itpp_status run_gates(itpp_ctx* h, int k0, int n, int n_layers, unsigned long long* log) {
+    return h->s.W == 1 ? run_launch<1>(h, k0, n, n_layers, log)
+                       : run_launch<2>(h, k0, n, n_layers, log);
+}
+
+// n_layers layers of the schedule: as few launches as the gate argument
+// allows, each of at most kRunGates gates (a launch holds the GPU's CTA slots
+// while it runs).
+itpp_status run_layers(itpp_ctx* h, int n_layers, unsigned long long* log) {
+    const int G = (int)h->gates.size();
+    constexpr int kRunGates = 4096;
+    for (int l = 0; l < n_layers && G > 0;) {
+        const int fit = G <= kRunChunk ? std::max(1, kRunGates / G) : 1;
+        const int nl = std::min(fit, n_layers - l);
+        for (int k = 0; k < G; k += kRunChunk) {
+            itpp_status st = run_gates(h, k, std::min(kRunChunk, G - k), nl, log);
+            if (st) return st;
+            if (log) log += (size_t)std::min(kRunChunk, G - k) * nl;
+        }
+        l += nl;
+    }
+    return ITPP_OK;
+}
+
+// The per-kernel timing of itpp_profile_* wants the gate's kernels one by one.
+bool use_run(const itpp_ctx* h) { return h->run_ok && !h->prof; }
+
 itpp_status launch_one_gate(itpp_ctx* h, int k) {
+    if (use_run(h)) return run_gates(h, k, 1, 1, nullptr);
     const HostGate& g = h->gates[(size_t)k];
     cudaError_t e = cudaSuccess;
     if (h->p.merge_path == 0) {
+        h->contiguous = false;
         // a window's first gate (or any gate after the state changed
         // elsewhere) re-partitions; later gates of the window read the
         // previous gate's segments unless a partition outgrew the limit
@@ -217,6 +316,29 @@ itpp_status check_obs_args(itpp_ctx* h, const uint64_t* ox, const uint64_t* oz, 
 
 itpp_status itpp_detail_sync_ctl(itpp_ctx* h) { return sync_ctl(h); }
 itpp_status itpp_detail_launch_gate(itpp_ctx* h, int k) { return launch_one_gate(h, k); }
+
+__global__ static void k_log_count(const DevCtl* ctl, unsigned long long* log) {
+    if (threadIdx.x == 0) *log = ctl->status ? ~0ULL : ctl->count[ctl->cur];
+}
+
+itpp_status itpp_detail_layers(itpp_ctx* h, int n_layers, unsigned long long* log) {
+    if (use_run(h)) return run_layers(h, n_layers, log);
+    for (int l = 0; l < n_layers; ++l)
+        for (int k = 0; k < (int)h->gates.size(); ++k) {
+            itpp_status st = launch_one_gate(h, k);
+            if (st) return st;
+            if (log) k_log_count<<<1, 32, 0, h->stream>>>(h->s.ctl, log++);
+        }
+    return ITPP_OK;
+}
+
+// The state as one contiguous run with no select pending.
+cudaError_t itpp_detail_materialize(itpp_ctx* h) {
+    itpp_detail_touch(h);
+    if (h->contiguous) return cudaSuccess;
+    h->contiguous = true;
+    return launch_materialize(h->s, h->stream);
+}
 
 // ---------------------------------------------------------------------------
 // Canonical order and checkpoints (host side)
@@ -449,6 +571,18 @@ itpp_status itpp_create(int n, const uint64_t* gate_x, const uint64_t* gate_z,
         ok &= ok && cudaMemsetAsync(s.sp_drift, 0, (size_t)(s.layer_gates + 1) * sizeof(long long),
                                     h->stream) == cudaSuccess;
         plan_windows(W, h->gates);
+        // whole layers in one launch, for the default launch shape: as many
+        // CTAs as there can be partitions, at most what fits
+        if (p->cap_M <= kRunMax && (p->block_threads == 0 || p->block_threads == 256)) {
+            const uint64_t parts = p->cap_M / kRunMinPart + 1;
+            h->run_grid = (int)std::min<uint64_t>((uint64_t)sms * run_fit(W), parts);
+            h->run_part_max = (uint32_t)std::max<uint64_t>(p->cap_M / s.part_target + 2,
+                                                           (uint64_t)h->run_grid + 1);
+            ok &= ok && cudaMalloc(&h->run_shared, run_shared_bytes()) == cudaSuccess;
+            ok &= ok && cudaMalloc(reinterpret_cast<void**>(&h->run_cnt),
+                                   (size_t)h->run_part_max * 2 * sizeof(unsigned int)) == cudaSuccess;
+            h->run_ok = ok;
+        }
     }
     if (ok && p->merge_path == 1) {
         h->sort_bytes = sorted_scratch_bytes(W, s.buf_cap);
@@ -493,12 +627,7 @@ itpp_status itpp_apply_gate(itpp_handle h, int k) {
 itpp_status itpp_apply_trotter_layer(itpp_handle h, int n_layers) {
     if (!h || n_layers < 0) return ITPP_ERR_ARG;
     if (h->sticky) return h->sticky;
-    for (int l = 0; l < n_layers; ++l)
-        for (int k = 0; k < (int)h->gates.size(); ++k) {
-            itpp_status st = launch_one_gate(h, k);
-            if (st) return st;
-        }
-    return ITPP_OK;
+    return itpp_detail_layers(h, n_layers, nullptr);
 }
 
 itpp_status itpp_reset(itpp_handle h) {
@@ -506,13 +635,14 @@ itpp_status itpp_reset(itpp_handle h) {
     if (h->sticky == ITPP_ERR_CUDA) return h->sticky;
     h->sticky = ITPP_OK;
     itpp_detail_touch(h);
+    h->contiguous = true;
     return launch_reset_identity(h->s, h->stream) == cudaSuccess ? ITPP_OK : cuda_fail(h);
 }
 
 itpp_status itpp_truncate(itpp_handle h, double delta) {
     if (!h || !(delta >= 0.0) || !std::isfinite(delta)) return ITPP_ERR_ARG;
     if (h->sticky) return h->sticky;
-    if ((itpp_detail_touch(h), launch_materialize(h->s, h->stream)) != cudaSuccess) return cuda_fail(h);
+    if (itpp_detail_materialize(h) != cudaSuccess) return cuda_fail(h);
     return launch_truncate(h->s, delta + 0.0, h->stream) == cudaSuccess ? ITPP_OK : cuda_fail(h);
 }
 
@@ -553,7 +683,7 @@ itpp_status itpp_get_stats(itpp_handle h, itpp_stats* o) {
 itpp_status itpp_get_terms(itpp_handle h, uint64_t* x, uint64_t* z, double* c,
                            uint64_t capacity, uint64_t* count) {
     if (!h || !count) return ITPP_ERR_ARG;
-    if (!h->sticky && (itpp_detail_touch(h), launch_materialize(h->s, h->stream)) != cudaSuccess) return cuda_fail(h);
+    if (!h->sticky && itpp_detail_materialize(h) != cudaSuccess) return cuda_fail(h);
     itpp_status st = sync_ctl(h);
     if (st) return st;
     const uint64_t n = h->h_ctl->count[h->h_ctl->cur];
@@ -664,6 +794,7 @@ itpp_status itpp_set_terms(itpp_handle h, const uint64_t* x, const uint64_t* z, 
         cudaMemcpyAsync(dc, c, (size_t)count * 8, cudaMemcpyHostToDevice, h->stream) != cudaSuccess)
         return cuda_fail(h);
     itpp_detail_touch(h);
+    h->contiguous = true;
     if (launch_import(h->s, dx, dz, dc, count, h->stream) != cudaSuccess) return cuda_fail(h);
     h->sticky = ITPP_OK;
     itpp_status st = sync_ctl(h);
@@ -684,7 +815,7 @@ itpp_status itpp_expect_device(itpp_handle h, const uint64_t* d_ox, const uint64
     itpp_status st = ensure_obs(h, m, h->s.W);
     if (st) return st;
     ObsPtrs o = obs_layout(h, m, h->s.W);
-    if ((itpp_detail_touch(h), launch_materialize(h->s, h->stream)) != cudaSuccess) return cuda_fail(h);
+    if (itpp_detail_materialize(h) != cudaSuccess) return cuda_fail(h);
     EventPair* ev = prof_begin(h, 3);
     cudaError_t e = launch_expect(h->s, d_ox, d_oz, d_ow, m, o.tsize, o.tab, o.first, o.vals,
                                   d_out, h->stream);
@@ -707,7 +838,7 @@ static itpp_status expect_host(itpp_handle h, const uint64_t* ox, const uint64_t
     if (ow && cudaMemcpyAsync(o.ow, ow, (size_t)m * 8, cudaMemcpyHostToDevice, h->stream) !=
                   cudaSuccess)
         return cuda_fail(h);
-    if ((itpp_detail_touch(h), launch_materialize(h->s, h->stream)) != cudaSuccess) return cuda_fail(h);
+    if (itpp_detail_materialize(h) != cudaSuccess) return cuda_fail(h);
     EventPair* ev = prof_begin(h, 3);
     cudaError_t e = launch_expect(h->s, o.ox, o.oz, ow ? o.ow : nullptr, m, o.tsize, o.tab,
                                   o.first, o.vals, o.out, h->stream);
@@ -751,7 +882,7 @@ itpp_status itpp_expect_psd(itpp_handle h, const uint64_t* obs_x, const uint64_t
         cudaMemcpyAsync(o.ow, obs_w, (size_t)m * 8, cudaMemcpyHostToDevice, h->stream) !=
             cudaSuccess)
         return cuda_fail(h);
-    if ((itpp_detail_touch(h), launch_materialize(h->s, h->stream)) != cudaSuccess) return cuda_fail(h);
+    if (itpp_detail_materialize(h) != cudaSuccess) return cuda_fail(h);
     double* d_out = h->psd_mem + 2 * (size_t)n_part;
     EventPair* ev = prof_begin(h, 3);
     cudaError_t e = launch_expect_psd(h->s, o.ox, o.oz, o.ow, m, h->psd_mem, n_part, d_out,

@@ -184,10 +184,11 @@ __device__ __forceinline__ void set_status(DevCtl* ctl, int code, unsigned int i
 // [P, Q] = 0 iff the symplectic product sum_i (xP_i zQ_i + zP_i xQ_i) is even.
 template <int W>
 __device__ __forceinline__ bool commutes(const PKey<W>& k, const GateArg<W>& g) {
-    int s = 0;
+    // only the parity is needed: one popc of all words folded together
+    uint64_t t = 0;
 #pragma unroll
-    for (int w = 0; w < W; ++w) s += __popcll((k.x[w] & g.qz[w]) ^ (k.z[w] & g.qx[w]));
-    return (s & 1) == 0;
+    for (int w = 0; w < W; ++w) t ^= (k.x[w] & g.qz[w]) ^ (k.z[w] & g.qx[w]);
+    return (__popc((uint32_t)t ^ (uint32_t)(t >> 32)) & 1) == 0;
 }
 
 // For a commuting pair, Q P = s R with R = (xQ^xP, zQ^zP) and s = +-1.

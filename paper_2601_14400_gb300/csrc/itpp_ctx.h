@@ -55,6 +55,14 @@ struct itpp_ctx {
     // changes the state bumps state_epoch
     uint64_t state_epoch = 1, part_epoch = 0;
     int part_last = -1;
+    // gates run in one launch (itpp_run.cu): bounds up to run_max terms; the
+    // team's shared block and the partition cursors
+    bool run_ok = false;
+    int run_grid = 0;
+    uint32_t run_part_max = 0;
+    void* run_shared = nullptr;
+    unsigned int* run_cnt = nullptr;
+    bool contiguous = true;   // the state is one run with no select pending
     // profiling
     bool prof = false;
     std::vector<EventPair> ev[kKinds];
@@ -67,5 +75,9 @@ struct itpp_ctx {
 // Helpers of the C ABI used by more than one translation unit.
 itpp_status itpp_detail_sync_ctl(itpp_ctx* h);
 itpp_status itpp_detail_launch_gate(itpp_ctx* h, int k);
+// n_layers whole layers; log (device, or null) receives the term count after
+// every gate.
+itpp_status itpp_detail_layers(itpp_ctx* h, int n_layers, unsigned long long* log);
+cudaError_t itpp_detail_materialize(itpp_ctx* h);
 // The state changed outside a window's merges (partitions must be rebuilt).
 inline void itpp_detail_touch(itpp_ctx* h) { ++h->state_epoch; }

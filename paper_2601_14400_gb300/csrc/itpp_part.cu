@@ -42,63 +42,6 @@ namespace itpp {
 // The state is a contiguous run of terms, or (after a partitioned merge)
 // the segments its descriptors list.
 template <int W>
-__device__ __forceinline__ void scatter_run(const PKey<W>* __restrict__ kin,
-                                            const double* __restrict__ cin, uint64_t n,
-                                            uint64_t first, uint64_t stride, const Pending<W>& pd,
-                                            DevCtl* ctl, PKey<W>* pk, double* pc,
-                                            unsigned int* cursor, const PartPlan& pl,
-                                            const GateArg<W>& g, const PartFn<W>& f) {
-    // whole warps iterate together (the cursor claim below is warp-wide);
-    // U items per thread per round, their loads issued before any claim
-    constexpr int U = 4;
-    const unsigned int lt = (1u << (threadIdx.x & 31)) - 1u;
-    for (uint64_t i0 = first; i0 < n; i0 += U * stride) {
-        PKey<W> K[U];
-        double c[U];
-        bool live[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const uint64_t i = i0 + (uint64_t)u * stride + threadIdx.x;
-            live[u] = i < n;
-            c[u] = 0.0;
-#pragma unroll
-            for (int w = 0; w < W; ++w) { K[u].x[w] = 0; K[u].z[w] = 0; }
-            if (live[u]) {
-                K[u] = load_key_stream(kin + i);
-                c[u] = __ldcs(cin + i);
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            if (live[u] && pd.on && !cap_keep(K[u], c[u], pd.T, pd.all_ties, pd.tk)) {
-                if (key_is_zero(K[u])) set_status(ctl, ST_TRACE_ZERO, 42);
-                live[u] = false;
-            }
-            // one cursor claim per distinct partition in the warp: terms of
-            // one group arrive together and would otherwise serialise on it
-            const uint32_t p = live[u] ? part_of(K[u], g, f, pl.P) : 0xffffffffu;
-            const unsigned int peers = __match_any_sync(0xffffffffu, p);
-            const int leader = __ffs(peers) - 1;
-            unsigned int base = 0;
-            if (live[u] && (threadIdx.x & 31) == leader) base = atomicAdd(cursor + p, __popc(peers));
-            base = __shfl_sync(0xffffffffu, base, leader);
-            if (live[u]) {
-                const unsigned int pos = base + __popc(peers & lt);
-                if (pos < pl.R) {
-                    const uint64_t d = (uint64_t)p * pl.R + pos;
-                    store_key(pk + d, K[u]);
-                    pc[d] = c[u];
-                } else if (!f.pair) {
-                    ctl->scatter_over = 1;   // the gate scatters again by its pair key
-                } else {
-                    set_status(ctl, ST_CAPACITY, 40);
-                }
-            }
-        }
-    }
-}
-
-template <int W>
 __global__ void __launch_bounds__(256, W == 1 ? 6 : 4)
 k_part_scatter(Bufs<W> B, DevCtl* ctl, PKey<W>* pk, double* pc, unsigned int* cursor,
                uint64_t pbuf_cap, uint32_t p_max, GateArg<W> g, PartFn<W> f, int force,
@@ -177,7 +120,7 @@ k_part_scatter(Bufs<W> B, DevCtl* ctl, PKey<W>* pk, double* pc, unsigned int* cu
         const uint64_t first = seg ? 0ULL : (uint64_t)blockIdx.x * blockDim.x;
         const uint64_t stride = seg ? (uint64_t)blockDim.x : (uint64_t)gridDim.x * blockDim.x;
         scatter_run(B.key(cur) + off, B.coef(cur) + off, cnt, first, stride, pd, ctl, pk, pc,
-                    cursor, pl, g, f);
+                    cursor, pl, g, f, &ctl->scatter_over);
     }
 }
 

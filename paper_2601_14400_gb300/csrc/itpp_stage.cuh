@@ -8,6 +8,7 @@
 
 #include "itpp_common.cuh"
 #include "itpp_gate_body.cuh"
+#include "itpp_launch.h"
 
 namespace itpp {
 
@@ -103,6 +104,68 @@ __device__ __forceinline__ Pending<W> pending_of(const DevCtl* ctl) {
 #pragma unroll
     for (int w = 0; w < W; ++w) { q.tk.x[w] = ctl->pend_tie_key[w]; q.tk.z[w] = ctl->pend_tie_key[W + w]; }
     return q;
+}
+
+// Scatter terms [0, n) of a run (this CTA's part of it: from `first` on, every
+// `stride`) into the partitions of a plan: the kept set of a pending select,
+// one cursor claim per distinct partition of a warp.
+template <int W>
+__device__ __forceinline__ void scatter_run(const PKey<W>* __restrict__ kin,
+                                            const double* __restrict__ cin, uint64_t n,
+                                            uint64_t first, uint64_t stride, const Pending<W>& pd,
+                                            DevCtl* ctl, PKey<W>* pk, double* pc,
+                                            unsigned int* cursor, const PartPlan& pl,
+                                            const GateArg<W>& g, const PartFn<W>& f,
+                                            int* over) {
+    // whole warps iterate together (the cursor claim below is warp-wide);
+    // U items per thread per round, their loads issued before any claim
+    constexpr int U = 4;
+    const unsigned int lt = (1u << (threadIdx.x & 31)) - 1u;
+    for (uint64_t i0 = first; i0 < n; i0 += U * stride) {
+        PKey<W> K[U];
+        double c[U];
+        bool live[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const uint64_t i = i0 + (uint64_t)u * stride + threadIdx.x;
+            live[u] = i < n;
+            c[u] = 0.0;
+#pragma unroll
+            for (int w = 0; w < W; ++w) { K[u].x[w] = 0; K[u].z[w] = 0; }
+            if (live[u]) {
+                K[u] = load_key_stream(kin + i);
+                c[u] = __ldcs(cin + i);
+                live[u] = abs_pattern(c[u]) != 0ULL;   // a zero is no term
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (live[u] && pd.on && !cap_keep(K[u], c[u], pd.T, pd.all_ties, pd.tk)) {
+                if (key_is_zero(K[u])) set_status(ctl, ST_TRACE_ZERO, 42);
+                live[u] = false;
+            }
+            // one cursor claim per distinct partition in the warp: terms of
+            // one group arrive together and would otherwise serialise on it
+            const uint32_t p = live[u] ? part_of(K[u], g, f, pl.P) : 0xffffffffu;
+            const unsigned int peers = __match_any_sync(0xffffffffu, p);
+            const int leader = __ffs(peers) - 1;
+            unsigned int base = 0;
+            if (live[u] && (threadIdx.x & 31) == leader) base = atomicAdd(cursor + p, __popc(peers));
+            base = __shfl_sync(0xffffffffu, base, leader);
+            if (live[u]) {
+                const unsigned int pos = base + __popc(peers & lt);
+                if (pos < pl.R) {
+                    const uint64_t d = (uint64_t)p * pl.R + pos;
+                    store_key(pk + d, K[u]);
+                    pc[d] = c[u];
+                } else if (!f.pair) {
+                    *over = 1;   // the gate scatters again by its pair key
+                } else {
+                    set_status(ctl, ST_CAPACITY, 40);
+                }
+            }
+        }
+    }
 }
 
 // Prefetch [p, p + bytes) into L2 with one bulk (TMA) request; the range is
@@ -522,8 +585,9 @@ __device__ __forceinline__ uint32_t stage_pass(uint32_t n, uint32_t shift, const
             const PKey<W> K = A::keys()[i];
             const double raw = vals[i];
             const unsigned long long b = abs_pattern(raw);
-            bool live = b >= pd.T;   // pd.T == 0 with every tie kept: no select pending
-            if (b == pd.T && !pd.all_ties) live = !key_less(pd.tk, K);
+            // pd.T == 0 with every tie kept: no select pending; a zero is no term
+            bool live = b >= pd.T && b != 0ULL;
+            if (b == pd.T && !pd.all_ties) live = live && !key_less(pd.tk, K);
             double c = __dmul_rn(raw, rnorm);
             if (has_id && key_is_zero(K)) {
                 c = 1.0;   // the identity's normalised value is exactly 1
@@ -619,7 +683,8 @@ __device__ __forceinline__ uint32_t merge_long(const PKey<W>* kp, const double* 
             for (uint64_t i = threadIdx.x; i < np; i += BLOCK) {
                 const PKey<W> K = load_key_stream(kp + i);
                 const double raw = __ldcs(cp + i);
-                const bool live = cap_keep(K, raw, pd.T, pd.all_ties, pd.tk);
+                const bool live = abs_pattern(raw) != 0ULL &&
+                                  cap_keep(K, raw, pd.T, pd.all_ties, pd.tk);
                 if (!live) {
                     if (key_is_zero(K)) set_status(ctl, ST_TRACE_ZERO, 43);
                     continue;
