@@ -206,8 +206,9 @@ __global__ void k_import_begin(DevCtl* ctl, uint64_t count) {
         ctl->drop_on = ctl->retry = ctl->scatter_over = 0;
         ctl->sel_k = 0;   // reused below as "identity seen" flag
         ctl->pend = 0;
-        ctl->seg = 0;
-        ctl->sp_lo = ctl->sp_hi = 0;
+        ctl->home = 0;
+        ctl->need_scatter = ctl->part_over = ctl->scattered = ctl->over = 0;
+        ctl->sp_lo = ctl->sp_hi = ctl->sp_thr = 0;
         ctl->sp_shift = 0;
         ctl->sp_tprev = 0;
     }
@@ -340,8 +341,9 @@ __global__ void k_reset_identity(BufsA<W> B, DevCtl* ctl) {
         ctl->sel_tie_n = 0;
         ctl->sel_k = 0;
         ctl->pend = 0;
-        ctl->seg = 0;
-        ctl->sp_lo = ctl->sp_hi = 0;
+        ctl->home = 0;
+        ctl->need_scatter = ctl->part_over = ctl->scattered = ctl->over = 0;
+        ctl->sp_lo = ctl->sp_hi = ctl->sp_thr = 0;
         ctl->sp_shift = 0;
         ctl->sp_tprev = 0;
         ctl->stat_gates = ctl->stat_in = ctl->stat_out = ctl->stat_cap = ctl->stat_probes = 0;

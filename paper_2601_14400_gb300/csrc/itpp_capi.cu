@@ -58,10 +58,6 @@ void free_all(itpp_ctx* h) {
     if (h->s.part_keys) cudaFree(h->s.part_keys);
     if (h->s.part_coef) cudaFree(h->s.part_coef);
     if (h->s.part_cursor) cudaFree(h->s.part_cursor);
-    for (int i = 0; i < 2; ++i) {
-        if (h->s.part_desc[i]) cudaFree(h->s.part_desc[i]);
-        if (h->s.chunks[i]) cudaFree(h->s.chunks[i]);
-    }
     if (h->s.ctl) cudaFree(h->s.ctl);
     if (h->obs_mem) cudaFree(h->obs_mem);
     if (h->sort_mem) cudaFree(h->sort_mem);
@@ -119,6 +115,13 @@ itpp_status sync_ctl(itpp_ctx* h) {
     return h->sticky;
 }
 
+// A gate that ended with a device error may leave partition cursors behind.
+cudaError_t clear_cursors(itpp_ctx* h) {
+    if (!h->s.part_cursor) return cudaSuccess;
+    return cudaMemsetAsync(h->s.part_cursor, 0, (size_t)h->s.part_max * 3 * sizeof(unsigned int),
+                           h->stream);
+}
+
 // Bounds up to this run a layer in one launch (itpp_run.cu).
 constexpr uint64_t kRunMax = 1ULL << 21;
 
@@ -126,22 +129,18 @@ constexpr uint64_t kRunMax = 1ULL << 21;
 template <int W>
 itpp_status run_launch(itpp_ctx* h, int k0, int n, int n_layers, unsigned long long* log) {
     DeviceState& s = h->s;
-    RunChunk<W> ch;
+    RunChunk<W> ch{};
     for (int j = 0; j < n; ++j) {
         const HostGate& g = h->gates[(size_t)(k0 + j)];
         RunGate<W>& r = ch.g[j];
         for (int w = 0; w < W; ++w) {
             r.qx[w] = g.qx[w];
             r.qz[w] = g.qz[w];
-            r.win[w] = ~g.keep_x[w];
         }
         r.ch = g.ch;
         r.msh = g.msh;
-        r.pair = g.pair_mode;
-        r.sites = g.win_sites;
-        r.start = g.win_start;
-        r.pad = 0;
     }
+    plan_run_windows(ch.g, n);
     RunArgs<W> a{};
     for (int i = 0; i < 2; ++i) {
         a.k[i] = static_cast<PKey<W>*>(s.keys[i]);
@@ -162,7 +161,7 @@ itpp_status run_launch(itpp_ctx* h, int k0, int n, int n_layers, unsigned long l
     if (a.cand_cap > a.home_cap) a.cand_cap = a.home_cap;
     a.tie_off = (a.cand_cap * 12 + 255) / 256 * 256;
     a.cap_M = s.cap_M;
-    a.cand_hi = 4096;
+    a.cand_hi = std::max<uint64_t>(1024, s.cap_M / 16);
     std::memcpy(&a.delta_bits, &s.delta, sizeof a.delta_bits);
     a.part_max = h->run_part_max;
     a.drift_stride = s.layer_gates + 1;
@@ -249,9 +248,10 @@ itpp_status launch_one_gate(itpp_ctx* h, int k) {
             prof_end(h, ev1);
         }
     }
-    if (e == cudaSuccess) e = launch_gate_post(h->s, h->stream);
+    if (e == cudaSuccess)
+        e = h->p.merge_path == 0 ? launch_part_post(h->s, h->stream) : launch_gate_post(h->s, h->stream);
     // scatter, merge, post (partitioned: also the scatter's clear and second
-    // launch, the merge's check and second launch, which return at once
+    // launch, the merge's check and the merge in full, which return at once
     // unless the scatter or the merge must be redone)
     h->launches += h->p.merge_path == 0 ? 7 : 3;
     if (e == cudaSuccess && h->s.cap_policy == 1) {
@@ -459,11 +459,10 @@ itpp_status itpp_create(int n, const uint64_t* gate_x, const uint64_t* gate_z,
     s.buf_cap = 2 * p->cap_M;
     s.max_ctas = std::min(8 * sms, 1024);   // the select reads at most 1024 candidate regions
     if (p->merge_path == 0) {
-        // merge CTAs claim output chunks: room for what the chunks leave
-        // unused, and an even count (the L2 bulk prefetch rounds byte ranges
-        // to 16 bytes); candidate positions are 32-bit
-        s.chunk = merge_chunk(p->cap_M, s.max_ctas, W);
-        s.buf_cap += merge_slack(p->cap_M, s.max_ctas, W);
+        // a buffer also serves as a home of partitions (room for what is
+        // appended in a window); an even count (the L2 bulk prefetch rounds
+        // byte ranges to 16 bytes); candidate positions are 32-bit
+        s.buf_cap += p->cap_M / 4 * 3 + 4096;
         s.buf_cap += s.buf_cap & 1ULL;
         if (s.buf_cap >= (1ULL << 32)) {
             delete h;
@@ -537,18 +536,9 @@ itpp_status itpp_create(int n, const uint64_t* gate_x, const uint64_t* gate_z,
         ok &= cudaMalloc(&s.part_keys, s.part_cap * 16 * W) == cudaSuccess;
         ok &= ok && cudaMalloc(reinterpret_cast<void**>(&s.part_coef), s.part_cap * 8) == cudaSuccess;
         ok &= ok && cudaMalloc(reinterpret_cast<void**>(&s.part_cursor),
-                               (size_t)s.part_max * sizeof(unsigned int)) == cudaSuccess;
-        for (int i = 0; i < 2; ++i)
-            ok &= ok && cudaMalloc(reinterpret_cast<void**>(&s.part_desc[i]),
-                                   (size_t)s.part_max * sizeof(PartDesc)) == cudaSuccess;
-        // output chunks: every claim takes at least one chunk of the buffer
-        // or (exact claims) one partition's children, and each CTA leaves
-        // one partly used
-        s.max_chunks = (uint32_t)((s.chunk ? s.buf_cap / s.chunk : 0ULL) + s.part_max +
-                                  2ULL * (uint64_t)s.max_ctas + 64);
-        for (int i = 0; i < 2; ++i)
-            ok &= ok && cudaMalloc(reinterpret_cast<void**>(&s.chunks[i]),
-                                   (size_t)s.max_chunks * sizeof(ChunkDesc)) == cudaSuccess;
+                               (size_t)s.part_max * 3 * sizeof(unsigned int)) == cudaSuccess;
+        ok &= ok && cudaMemsetAsync(s.part_cursor, 0, (size_t)s.part_max * 3 * sizeof(unsigned int),
+                                    h->stream) == cudaSuccess;
         // the merge's candidate regions for the top-M select: about half the
         // bound's worth of entries over the merge's CTAs
         uint64_t region = p->cap_M / (2ULL * (uint64_t)s.max_ctas);
@@ -580,7 +570,7 @@ itpp_status itpp_create(int n, const uint64_t* gate_x, const uint64_t* gate_z,
                                                            (uint64_t)h->run_grid + 1);
             ok &= ok && cudaMalloc(&h->run_shared, run_shared_bytes()) == cudaSuccess;
             ok &= ok && cudaMalloc(reinterpret_cast<void**>(&h->run_cnt),
-                                   (size_t)h->run_part_max * 2 * sizeof(unsigned int)) == cudaSuccess;
+                                   (size_t)h->run_part_max * 3 * kRunPad * sizeof(unsigned int)) == cudaSuccess;
             h->run_ok = ok;
         }
     }
@@ -636,6 +626,7 @@ itpp_status itpp_reset(itpp_handle h) {
     h->sticky = ITPP_OK;
     itpp_detail_touch(h);
     h->contiguous = true;
+    if (clear_cursors(h) != cudaSuccess) return cuda_fail(h);
     return launch_reset_identity(h->s, h->stream) == cudaSuccess ? ITPP_OK : cuda_fail(h);
 }
 
@@ -795,6 +786,7 @@ itpp_status itpp_set_terms(itpp_handle h, const uint64_t* x, const uint64_t* z, 
         return cuda_fail(h);
     itpp_detail_touch(h);
     h->contiguous = true;
+    if (clear_cursors(h) != cudaSuccess) return cuda_fail(h);
     if (launch_import(h->s, dx, dz, dc, count, h->stream) != cudaSuccess) return cuda_fail(h);
     h->sticky = ITPP_OK;
     itpp_status st = sync_ctl(h);

@@ -100,24 +100,26 @@ struct DevCtl {
     unsigned long long pend_T;
     uint64_t pend_tie_key[4];
     uint64_t sel_tie_key[4];         // largest kept tie key (x..., z...)
-    // partitioned merge: where the next merge finds its partitions
+    // partitioned merge: layout of the state.  home 0: a contiguous run in
+    // buffer cur (count[cur] terms, or pend_n with a pending select); home 1:
+    // partitions of stride part_R in a home (itpp_part.cu): key array hb,
+    // coefficient array hx, cursor array hc; ha is the buffer left free for
+    // a contiguous run.  to_*: where this gate's scatter put the state.
+    int home, ha, hb, hx, hc;
     unsigned int part_P;             // partitions of the current state
-    int part_from_scatter;           // 1: in the scatter buffer; 0: segments of the state
+    unsigned long long part_R;
+    int scattered, to_b, to_x, to_c;
+    unsigned int to_P;
+    unsigned long long to_R;
     int part_over;                   // this gate's partitions hold for this gate only
     int need_scatter;                // ... so the next gate re-partitions
-    // segmented state: the merge writes every partition's children as one
-    // segment of a chunk its CTA claimed (alloc[] is the chunk allocator of
-    // each buffer); the buffer then holds seg_P segments, described by the
-    // partition descriptors, with unused room between them
-    int seg;                         // 1: the current buffer is segmented
-    unsigned int seg_P;
-    unsigned long long alloc[2];
-    unsigned int nchunk[2];          // output chunks in use per buffer (contiguous runs)
-    // top-M select folded into the merge: the merge counts its kept
-    // children above sp_hi and lists those in [sp_lo, sp_hi] (a range around
-    // the previous gate's threshold); the select then reads only that list
+    int over;                        // the merge found no room in a partition's stride
+    unsigned long long alloc;        // terms a merge done again, or a gather, has written
+    // top-M select folded into the merge: children at or below sp_thr are
+    // left out, kept ones in [sp_lo = sp_thr + 1, sp_hi] (a range around the
+    // predicted threshold) are listed; the select then reads only that list
+    unsigned long long sp_thr;
     unsigned long long sp_lo, sp_hi; // candidate range (sp_hi == 0: none)
-    unsigned long long sp_above;     // kept children with pattern > sp_hi
     unsigned long long sp_tprev;     // the last select's threshold pattern (0: none)
     int sp_ovf;                      // a CTA's candidate region overflowed
     int sp_shift;                    // log2 of the range's half-width (0: unset)
@@ -128,9 +130,9 @@ struct DevCtl {
     int sel_top;                     // bits of v = pattern - sel_lo still to resolve
     unsigned long long sel_lo;       // offset of the select's values
     unsigned long long stat_sel_full, stat_long;
-    // children below the candidate range left unwritten by this gate's merge
-    // (drop_on); the merge is run again in full when fewer than cap_M were
-    // kept (retry), counted in stat_retry
+    // children at or below sp_thr are left out of this gate's merge (drop_on);
+    // the merge is run again in full when fewer than cap_M were kept (retry),
+    // counted in stat_retry
     int drop_on, retry;
     unsigned long long stat_retry;
     int scatter_over;                // a window's partition stride overflowed: the
@@ -330,6 +332,23 @@ __device__ __forceinline__ PKey<W> load_key_stream(const PKey<W>* p) {
         k.z[0] = a.y;
     } else {
         ulonglong2 a = __ldcs(v), b = __ldcs(v + 1);
+        k.x[0] = a.x; k.x[1] = a.y;
+        k.z[0] = b.x; k.z[1] = b.y;
+    }
+    return k;
+}
+
+// A load that may hit L1 (of memory that this kernel also writes elsewhere).
+template <int W>
+__device__ __forceinline__ PKey<W> load_key_ca(const PKey<W>* p) {
+    PKey<W> k;
+    const ulonglong2* v = reinterpret_cast<const ulonglong2*>(p);
+    if constexpr (W == 1) {
+        const ulonglong2 a = *v;
+        k.x[0] = a.x;
+        k.z[0] = a.y;
+    } else {
+        const ulonglong2 a = v[0], b = v[1];
         k.x[0] = a.x; k.x[1] = a.y;
         k.z[0] = b.x; k.z[1] = b.y;
     }

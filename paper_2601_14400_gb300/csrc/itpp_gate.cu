@@ -19,6 +19,17 @@ static Bufs<W> bufs_of(const DeviceState& s) {
 }
 
 template <int W>
+static Homes<W> homes_of(const DeviceState& s) {
+    Homes<W> h;
+    h.kp = reinterpret_cast<PKey<W>*>(s.part_keys);
+    h.cp = s.part_coef;
+    h.cnt = s.part_cursor;
+    h.part_max = s.part_max;
+    h.cap = s.part_cap < s.buf_cap ? s.part_cap : s.buf_cap;
+    return h;
+}
+
+template <int W>
 static GateArg<W> gate_arg(const HostGate& h) {
     GateArg<W> g;
     for (int w = 0; w < W; ++w) { g.qx[w] = h.qx[w]; g.qz[w] = h.qz[w]; }
@@ -227,80 +238,73 @@ __device__ __forceinline__ PKey<W> pend_tie_key(const DevCtl* ctl) {
 }
 
 // Materialise the state of the partitioned merge for a reader that wants a
-// contiguous run: apply a deferred select (its kept set), and gather the
-// segments of a segmented buffer, into the other buffer (normaliser
-// unchanged), then switch to it.
-__device__ __forceinline__ bool mat_needed(const DevCtl* ctl) { return ctl->pend || ctl->seg; }
+// contiguous run: the stored terms that the pending select keeps (a zero is no
+// term), gathered from the partitions into the buffer they leave free, or
+// compacted into the other buffer.
+__device__ __forceinline__ bool mat_needed(const DevCtl* ctl) { return ctl->pend || ctl->home; }
+__device__ __forceinline__ int mat_buf(const DevCtl* ctl) { return ctl->home ? ctl->ha : ctl->cur ^ 1; }
 
 __global__ void k_mat_begin(DevCtl* ctl) {
     if (threadIdx.x != 0 || !mat_needed(ctl) || ctl->status) return;
-    const int cur = ctl->cur;
-    ctl->count[cur ^ 1] = 0ULL;
-    ctl->norm[cur ^ 1] = ctl->norm[cur];
-    ctl->rnorm[cur ^ 1] = ctl->rnorm[cur];
-}
-
-// One round of up to BLOCK terms [i0, i0 + BLOCK) of a run of n (every
-// thread calls it).
-template <int W, int BLOCK>
-__device__ __forceinline__ void mat_round(const Bufs<W>& B, DevCtl* ctl, int cur, uint64_t off,
-                                          uint64_t n, uint64_t i0, bool pend, unsigned long long T,
-                                          bool all_ties, const PKey<W>& tk, uint32_t* s_scan,
-                                          unsigned long long* s_base) {
-    const uint64_t i = i0 + threadIdx.x;
-    PKey<W> K;
-    double c = 0;
-    bool keep = false;
-    if (i < n) {
-        K = load_key_stream(B.key(cur) + off + i);
-        c = __ldcs(B.coef(cur) + off + i);
-        keep = !pend || cap_keep(K, c, T, all_ties, tk);
-        if (key_is_zero(K) && !keep) set_status(ctl, ST_TRACE_ZERO, 3);
-    }
-    uint32_t tot;
-    const uint32_t o = block_exclusive_scan<BLOCK>(keep ? 1u : 0u, &tot, s_scan);
-    if (threadIdx.x == 0)
-        *s_base = tot ? atomicAdd(&ctl->count[cur ^ 1], (unsigned long long)tot) : 0ULL;
-    __syncthreads();
-    if (keep) {
-        store_key_stream(B.key(cur ^ 1) + *s_base + o, K);
-        __stcs(B.coef(cur ^ 1) + *s_base + o, c);
-    }
+    ctl->alloc = 0ULL;
 }
 
 template <int W, int BLOCK>
 __global__ void __launch_bounds__(BLOCK)
-k_materialize(Bufs<W> B, DevCtl* ctl, const ChunkDesc* chunks0, const ChunkDesc* chunks1) {
+k_materialize(Bufs<W> B, Homes<W> H, DevCtl* ctl) {
     if (!mat_needed(ctl) || ctl->status) return;
     __shared__ uint32_t s_scan[BLOCK / 32];
     __shared__ unsigned long long s_base;
-    const int cur = ctl->cur;
     const bool pend = ctl->pend != 0;
-    const unsigned long long T = ctl->pend_T;
-    const bool all_ties = ctl->pend_all_ties;
+    const unsigned long long T = pend ? ctl->pend_T : 0ULL;
+    const bool all_ties = !pend || ctl->pend_all_ties;
     const PKey<W> tk = pend_tie_key<W>(ctl);
-    if (ctl->seg) {
-        const ChunkDesc* din = cur ? chunks1 : chunks0;
-        const uint32_t P = ctl->nchunk[cur];
-        for (uint32_t p = blockIdx.x; p < P; p += gridDim.x) {
-            const uint64_t off = din[p].off, n = din[p].cnt;
-            for (uint64_t i0 = 0; i0 < n; i0 += BLOCK)
-                mat_round<W, BLOCK>(B, ctl, cur, off, n, i0, pend, T, all_ties, tk, s_scan, &s_base);
+    const StateRuns<W> r = state_runs(ctl, B, H);
+    PKey<W>* ko = B.key(mat_buf(ctl));
+    double* co = B.coef(mat_buf(ctl));
+    // each partition by one CTA, or the run by the whole grid
+    const uint32_t step = r.cnt ? gridDim.x : 1u;
+    for (uint32_t p = r.cnt ? blockIdx.x : 0u; p < r.P; p += step) {
+        const PKey<W>* ki = r.keys + (uint64_t)p * r.R;
+        const double* ci = r.coef + (uint64_t)p * r.R;
+        const uint64_t n = r.cnt ? (r.cnt[p] < r.R ? r.cnt[p] : r.R) : r.n;
+        const uint64_t stride = r.cnt ? (uint64_t)BLOCK : (uint64_t)gridDim.x * BLOCK;
+        for (uint64_t i0 = r.cnt ? 0ULL : (uint64_t)blockIdx.x * BLOCK; i0 < n; i0 += stride) {
+            const uint64_t i = i0 + threadIdx.x;
+            PKey<W> K;
+            double c = 0;
+            bool keep = false;
+            if (i < n) {
+                K = load_key_stream(ki + i);
+                c = __ldcs(ci + i);
+                keep = abs_pattern(c) != 0ULL && cap_keep(K, c, T, all_ties, tk);
+                if (key_is_zero(K) && !keep) set_status(ctl, ST_TRACE_ZERO, 3);
+            }
+            uint32_t tot;
+            const uint32_t o = block_exclusive_scan<BLOCK>(keep ? 1u : 0u, &tot, s_scan);
+            if (threadIdx.x == 0)
+                s_base = tot ? atomicAdd(&ctl->alloc, (unsigned long long)tot) : 0ULL;
+            __syncthreads();
+            if (keep) {
+                store_key_stream(ko + s_base + o, K);
+                __stcs(co + s_base + o, c);
+            }
         }
-    } else {
-        uint64_t n = pend ? ctl->pend_n : ctl->count[cur];
-        if (n > ctl->buf_cap) n = ctl->buf_cap;
-        const uint64_t tiles = (n + BLOCK - 1) / BLOCK;
-        for (uint64_t t = blockIdx.x; t < tiles; t += gridDim.x)
-            mat_round<W, BLOCK>(B, ctl, cur, 0, n, t * BLOCK, pend, T, all_ties, tk, s_scan, &s_base);
     }
 }
 
 __global__ void k_mat_end(DevCtl* ctl) {
     if (threadIdx.x != 0 || !mat_needed(ctl)) return;
-    if (!ctl->status) ctl->cur ^= 1;
+    if (!ctl->status) {
+        const int cur = ctl->cur, d = mat_buf(ctl);
+        const double norm = ctl->norm[cur], rnorm = ctl->rnorm[cur];
+        ctl->norm[d] = norm;
+        ctl->rnorm[d] = rnorm;
+        ctl->count[d] = ctl->alloc;
+        ctl->cur = d;
+    }
     ctl->pend = 0;
-    ctl->seg = 0;
+    ctl->home = 0;
 }
 
 // ---------------------------------------------------------------------------
@@ -408,8 +412,8 @@ int cap_launches(const DeviceState& s) {
 template <int W>
 static cudaError_t materialize_w(const DeviceState& s, cudaStream_t st) {
     k_mat_begin<<<1, 32, 0, st>>>(s.ctl);
-    k_materialize<W, 256><<<stream_grid(s, 256, 8), 256, 0, st>>>(bufs_of<W>(s), s.ctl,
-                                                                  s.chunks[0], s.chunks[1]);
+    k_materialize<W, 256><<<stream_grid(s, 256, 8), 256, 0, st>>>(bufs_of<W>(s), homes_of<W>(s),
+                                                                  s.ctl);
     k_mat_end<<<1, 32, 0, st>>>(s.ctl);
     return cudaGetLastError();
 }

@@ -31,6 +31,66 @@ struct Bufs {
     __device__ __forceinline__ double* coef(int i) const { return i ? c[1] : c[0]; }
 };
 
+// The partitioned merge's homes.  With a = ctl->ha the buffer that held the
+// contiguous run, home 0's keys are kp and home 1's the keys of buffer a ^ 1;
+// the coefficients go to and fro between cp and those of buffer a ^ 1; three
+// cursor arrays take turns (a gate's input, its output, the next scatter's).
+template <int W>
+struct Homes {
+    PKey<W>* kp;
+    double* cp;
+    unsigned int* cnt;       // [3][part_max]
+    uint32_t part_max;
+    uint64_t cap;            // terms a home holds
+    __device__ __forceinline__ PKey<W>* keys(const Bufs<W>& B, int a, int h) const {
+        return h ? B.key(a ^ 1) : kp;
+    }
+    __device__ __forceinline__ double* coef(const Bufs<W>& B, int a, int x) const {
+        return x ? B.coef(a ^ 1) : cp;
+    }
+    __device__ __forceinline__ unsigned int* cursors(int c) const {
+        return cnt + (uint64_t)c * part_max;
+    }
+};
+
+__device__ __forceinline__ int next3(int i) { return i == 2 ? 0 : i + 1; }
+
+// The current state as runs of stored terms: P partitions of stride R with
+// a cursor each, or (cnt null) one run of n.
+template <int W>
+struct StateRuns {
+    const PKey<W>* keys;
+    const double* coef;
+    const unsigned int* cnt;
+    uint32_t P;
+    uint64_t R, n;
+};
+
+template <int W>
+__device__ __forceinline__ StateRuns<W> state_runs(const DevCtl* ctl, const Bufs<W>& B,
+                                                   const Homes<W>& H) {
+    StateRuns<W> r;
+    if (ctl->home) {
+        r.keys = H.keys(B, ctl->ha, ctl->hb);
+        r.coef = H.coef(B, ctl->ha, ctl->hx);
+        r.cnt = H.cursors(ctl->hc);
+        r.P = ctl->part_P;
+        r.R = ctl->part_R;
+        r.n = 0;
+    } else {
+        const int cur = ctl->cur;
+        uint64_t n = ctl->pend ? ctl->pend_n : ctl->count[cur];
+        if (n > ctl->buf_cap) n = ctl->buf_cap;
+        r.keys = B.key(cur);
+        r.coef = B.coef(cur);
+        r.cnt = nullptr;
+        r.P = 1;
+        r.R = 0;
+        r.n = n;
+    }
+    return r;
+}
+
 // ---------------------------------------------------------------------------
 // Merge-table probe
 // ---------------------------------------------------------------------------
@@ -457,6 +517,28 @@ __device__ __forceinline__ void tie_find_range(DevCtl* ctl, const PKey<W>* tie_l
         if (tie_prefix_match<W>(k, pre, p))
             for (int w = 0; w < 2 * W; ++w) ctl->sel_tie_key[w] = key_word(k, w);
     }
+}
+
+// The next gate's candidate range around a predicted threshold pattern C: up
+// to C + 2^sft, down to C - 2 2^sft but no lower than C / 2, where also
+// children are no longer left out.  (The coefficients of these states lie on a
+// ladder of powers of the gate angle: halving the limit takes in 6 % of the
+// strings' children where the threshold itself takes in 2 to 4 %, a tenth of
+// it takes in 20 to 60 %.)
+constexpr int kRangeShiftMax = 51;
+struct SelRange {
+    unsigned long long thr, hi;
+};
+__device__ __forceinline__ SelRange sel_range(unsigned long long C, int sft,
+                                              unsigned long long delta_bits) {
+    const unsigned long long h = 1ULL << sft, half = 1ULL << 52;
+    const unsigned long long down = 2ULL * h < half ? 2ULL * h : half;
+    SelRange r;
+    r.thr = C > down ? C - down : 0ULL;
+    if (r.thr < delta_bits) r.thr = delta_bits;
+    r.hi = C + h;
+    if (r.hi <= r.thr) r.hi = r.thr + 1ULL;
+    return r;
 }
 
 // Does a term survive the top-M select?

@@ -14,11 +14,10 @@
 //
 // What bounds the pass is instruction issue and the double-precision pipe (two
 // lanes per clock and SM; a warp holds it for every instruction however few
-// lanes take part).  Hence: one multiplication for the normalisation and one
+// lanes take part), and the latency of a partition's few dependent steps.  Hence: one multiplication for the normalisation and one
 // for cosh over whole warps, and everything rare (a partner, a child that may
-// pass the threshold) is put on a list per warp and done densely at its end.
-// Whether a child can pass is decided before it is computed, on the exponent
-// fields.  Two barriers per partition.
+// pass the threshold) is put on a list and done densely afterwards.  Whether
+// a child can pass is decided before it is computed, on the exponent fields.
 #pragma once
 
 #include "itpp_common.cuh"
@@ -28,193 +27,251 @@ namespace itpp {
 
 namespace {
 
-// Shared memory of one pass: staged keys and values, the heads of the chains
-// of strings that share a pair slot, the chain links with two state bits, the
-// original index of a gathered string (sub-passes), the warps' lists of rare
-// strings and a bit per string that shares its slot with another.
+// Geometry and shared memory of one pass: up to kItems strings, each read from
+// global memory into registers (nothing is staged: the rare ones are read
+// again, from L1 or L2), the heads of the chains of strings that share a slot,
+// the chain links, the index of a gathered string (sub-passes) and the list of
+// rare strings.
 template <int W>
-struct InStage {
-    static constexpr int C = StageGeom<W>::kItems, S = StageGeom<W>::kSlots;
-    static constexpr size_t kKeys = 0;
-    static constexpr size_t kVals = kKeys + sizeof(PKey<W>) * C;
-    static constexpr size_t kHeads = kVals + sizeof(double) * (C + 2);
+struct InPass {
+    static constexpr int C = StageGeom<W>::kItems, S = 4096, kSlotBits = 12;
+    static constexpr size_t kHeads = 0;
     static constexpr size_t kNext = kHeads + sizeof(uint32_t) * S;
     static constexpr size_t kSrc = kNext + sizeof(uint16_t) * C;
     static constexpr size_t kRare = kSrc + sizeof(uint16_t) * C;
-    static constexpr size_t kDup = kRare + sizeof(uint16_t) * C;
-    static constexpr size_t kBytes = (kDup + sizeof(uint32_t) * (C / 32) + 15) / 16 * 16;
-    static_assert(kVals % 16 == 0 && kHeads % 16 == 0 && kNext % 16 == 0, "alignment");
-    __device__ __forceinline__ static PKey<W>* keys() { return reinterpret_cast<PKey<W>*>(g_stage + kKeys); }
-    __device__ __forceinline__ static double* vals() { return reinterpret_cast<double*>(g_stage + kVals); }
+    static constexpr size_t kBytes = (kRare + sizeof(uint16_t) * C + 15) / 16 * 16;
+    static_assert(S == (1 << kSlotBits), "slots");
     __device__ __forceinline__ static uint32_t* heads() { return reinterpret_cast<uint32_t*>(g_stage + kHeads); }
     __device__ __forceinline__ static uint16_t* next() { return reinterpret_cast<uint16_t*>(g_stage + kNext); }
     __device__ __forceinline__ static uint16_t* src() { return reinterpret_cast<uint16_t*>(g_stage + kSrc); }
     __device__ __forceinline__ static uint16_t* rare() { return reinterpret_cast<uint16_t*>(g_stage + kRare); }
-    __device__ __forceinline__ static uint32_t* dup() { return reinterpret_cast<uint32_t*>(g_stage + kDup); }
+    __device__ __forceinline__ static uint32_t slot(const PKey<W>& K, const GateArg<W>& g) {
+        return pair_hash(K, g) >> (32 - kSlotBits);
+    }
 };
 
 // A chain head holds (tag << 11) | (index + 1): heads of earlier passes carry
 // another tag and read as empty, so nothing is cleared between passes.
 constexpr uint32_t kHeadTagMax = (1u << 21) - 1u;
-constexpr uint32_t kInLive = 0x8000u, kInComm = 0x4000u, kInPrev = 0x7ffu;
+constexpr uint32_t kInPrev = 0x7ffu;
 
 // Where a pass puts things and what it counts.  Every pointer is the
 // partition's own: index 0 is its first string.
 template <int W>
 struct InPlace {
     PKey<W>* keys;        // the home (new strings are appended)
+    const double* cin;    // its coefficients
     double* cout;         // the other coefficient array, same indices
     uint64_t first;       // index of the partition's first string in the home
     uint32_t n;           // strings stored before the gate
     uint32_t room;        // the partition's stride
-    uint32_t* s_app;      // strings appended so far (shared)
+    uint32_t* s_app;      // strings appended so far (shared, zero at first)
+    uint32_t* s_rare;     // rare strings listed so far (shared, zero at first)
     int* over;            // set when the stride has no room for one
 };
 
-// What a thread counts over its partitions.
+// What a thread counts over its partitions: the high word of the largest
+// pattern, the kept strings.
 struct InStats {
-    unsigned long long out_max;
-    uint32_t kept, above;
+    uint32_t hi_max, kept;
 };
 
-// Whether |c m| can exceed the threshold, from the high words of the patterns
-// (hm: m's with the exponent bias taken off, ht: the threshold's).  A pattern
-// is the logarithm up to (1+a)(1+b) against 1+a+b, at most 0.1716 of an
-// octave, and the low words and the rounding add at most 3 units: 0x2c140.
-// The bound needs a normal threshold; below that everything may pass.
-__device__ __forceinline__ bool child_may_pass(double c, int hm, int ht) {
-    const int hc = (int)(__double2hiint(c) & 0x7fffffff);
-    return hc + hm + 0x2c140 >= ht || ht < 0x00100000;
+// Whether a lone string's child can pass the threshold is decided on the high
+// words of the patterns of |c|, |m| and the threshold.  A pattern is the
+// logarithm up to (1+a)(1+b) against 1+a+b, at most 0.1716 of an octave, and the
+// low words and the rounding add at most 3 units: 0x2c140.  The bound needs a
+// normal threshold; below that everything may pass.
+
+// Predicated shared-memory steps of the main rows, without the branches that a
+// conditional atomic otherwise costs every row.
+__device__ __forceinline__ uint32_t exch_if(bool on, uint32_t* p, uint32_t v) {
+    uint32_t o;
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\tmov.u32 %0, 0;\n\t"
+                 "@p atom.shared.exch.b32 %0, [%1], %2;\n\t}"
+                 : "=r"(o) : "r"(smem_addr(p)), "r"(v), "r"((uint32_t)on) : "memory");
+    return o;
 }
 
-// One pass over n staged strings (keys(), vals() + shift; dup() cleared; a
-// barrier since).  kGathered: string i is the partition's src()[i].
-// sel_lo / sel_w: the candidate range of the select, width 0 when there is
-// none; push(hit, pattern - lo, index) takes the candidates (warp-wide).
-// Two barriers; the staging arrays are free again when it returns.
-template <int W, int BLOCK, bool kGathered, class Push>
-__device__ __forceinline__ void inplace_pass(uint32_t n, uint32_t shift, const GateArg<W>& g,
+__device__ __forceinline__ void list_if(bool on, uint32_t* count, uint16_t* list, uint32_t v) {
+    asm volatile("{\n\t.reg .pred p;\n\t.reg .u32 q;\n\t.reg .u16 h;\n\t"
+                 "setp.ne.u32 p, %3, 0;\n\tmov.u32 q, 0;\n\tcvt.u16.u32 h, %2;\n\t"
+                 "@p atom.shared.add.u32 q, [%0], 1;\n\tshl.b32 q, q, 1;\n\t"
+                 "add.u32 q, q, %1;\n\t@p st.shared.u16 [q], h;\n\t}"
+                 :: "r"(smem_addr(count)), "r"(smem_addr(list)), "r"(v), "r"((uint32_t)on)
+                 : "memory");
+}
+
+// One pass over n >= 1 strings: string i is the partition's i-th, or (kGathered)
+// its src()[i]-th.  *s_app and *s_rare are zero, and a barrier since.  thr: kept
+// is what lies above it; near_hi: kept strings up to this pattern are candidates
+// of the select (0: none), push(hit, pattern - thr - 1, index) takes them
+// (warp-wide).  kPlain: neither the identity's partition nor a weight cutoff
+// nor Q = I.  Three barriers; the shared arrays are free again when it returns.
+template <int W, int BLOCK, bool kGathered, bool kPlain, class Push>
+__device__ __forceinline__ void inplace_pass(uint32_t n, const GateArg<W>& g,
                                              unsigned long long pd_T, bool pd_ties,
                                              const PKey<W>& pd_key, double rnorm,
                                              unsigned long long thr, bool has_id, DevCtl* ctl,
                                              int nxt, uint32_t tag, const InPlace<W>& io,
-                                             InStats& st, unsigned long long sel_lo,
-                                             unsigned long long sel_hi, Push&& push) {
-    using A = InStage<W>;
-    double* vals = A::vals() + shift;
-    const uint32_t lane = threadIdx.x & 31u;
+                                             InStats& st, unsigned long long near_hi,
+                                             Push&& push) {
+    using A = InPass<W>;
+    constexpr int ROWS = A::C / BLOCK, GROUP = ROWS < 4 ? ROWS : 4;
+    // per row: slot (12 bits) | commutes | not the first to arrive in its
+    // chain | live, and (special) the identity or past the weight cutoff
+    constexpr uint32_t kComm = 1u << 12, kPrev = 1u << 13, kLive = 1u << 14, kSpecial = 1u << 15;
+    const uint32_t lane = threadIdx.x & 31u, w0 = threadIdx.x & ~31u;
     const unsigned int lt = (1u << lane) - 1u;
-    // A: live strings, normalised values, the chains of shared pair slots
-    for (uint32_t i0 = threadIdx.x & ~31u; i0 < n; i0 += BLOCK) {
-        const uint32_t i = i0 + lane;
-        uint32_t f = 0, prev = 0;
-        if (i < n) {
-            const PKey<W> K = A::keys()[i];
-            const double raw = vals[i];
-            const unsigned long long b = abs_pattern(raw);
-            bool live = b >= pd_T && b != 0ULL;   // pd_T == 0: no select pending
-            if (b == pd_T && !pd_ties) live = live && !key_less(pd_key, K);
-            double c = __dmul_rn(raw, rnorm);
-            if (has_id && key_is_zero(K)) {
-                c = 1.0;   // the identity's normalised value is exactly 1
-                if (!live) set_status(ctl, ST_TRACE_ZERO, 43);
-            }
-            vals[i] = live ? c : 0.0;
-            if (live) {
-                f = kInLive;
-                if (commutes(K, g)) {
-                    const uint32_t o = atomicExch(A::heads() + pair_slot(K, g),
-                                                  (tag << 11) | (i + 1u));
-                    prev = (o >> 11) == tag ? (o & kInPrev) : 0u;
-                    f |= kInComm | prev;
-                    if (prev) atomicOr(A::dup() + ((prev - 1u) >> 5), 1u << ((prev - 1u) & 31u));
-                }
-            }
-            A::next()[i] = (uint16_t)f;
-        }
-        const unsigned int m = __ballot_sync(0xffffffffu, prev != 0u);
-        if (m && lane == 0) atomicOr(A::dup() + (i0 >> 5), m);
-    }
-    __syncthreads();                                                  // (1) chains built
-    // B: every string that is alone in its slot (its partner is absent)
-    const int hm = (int)(__double2hiint(g.msh) & 0x7fffffff) - 0x3ff00000;
-    const int ht = (int)(thr >> 32);
-    const bool weigh = g.maxw < 64 * W;
+    const bool weigh = !kPlain && g.maxw < 64 * W;
+    const uint32_t me0 = (tag << 11) + threadIdx.x + 1u;   // + r * BLOCK: this thread's string of row r
+    const unsigned long long floor_T = pd_T ? pd_T - 1ULL : 0ULL;   // live: above it (a zero is no term)
     // the identity as the gate: every string is its own partner
     uint64_t qbits = 0;
 #pragma unroll
     for (int w = 0; w < W; ++w) qbits |= g.qx[w] | g.qz[w];
-    const bool self = qbits == 0;
-    uint16_t* rare = A::rare() + (threadIdx.x >> 5) * (A::C / (BLOCK / 32));
-    uint32_t n_rare = 0;
-    for (uint32_t i0 = threadIdx.x & ~31u; i0 < n; i0 += BLOCK) {
-        const uint32_t i = i0 + lane;
-        const bool in = i < n;
-        const uint32_t f = in ? A::next()[i] : 0u;
-        const double c = in ? vals[i] : 0.0;
-        const bool comm = (f & kInComm) != 0;
-        const bool dup = comm && (self || ((A::dup()[i0 >> 5] >> lane) & 1u));
-        double va = c;
-        if (comm) va = __dmul_rn(c, g.ch);
-        const unsigned int rb =
-            __ballot_sync(0xffffffffu, dup || (comm && child_may_pass(c, hm, ht)));
-        if ((rb >> lane) & 1u) rare[n_rare + __popc(rb & lt)] = (uint16_t)i;
-        n_rare += __popc(rb);
-        unsigned long long a = abs_pattern(va);
-        bool keep = (f & kInLive) && !dup && a > thr;
-        const uint32_t at = kGathered && in ? A::src()[i] : i;
-        if (weigh && keep) keep = light(A::keys()[i], g.maxw);
-        if (has_id && (f & kInLive) && !dup && key_is_zero(A::keys()[i])) {
-            ctl->norm[nxt] = va;
-            if (!keep) set_status(ctl, ST_TRACE_ZERO, 1);
-            keep = true;
+    const bool self = !kPlain && qbits == 0;
+    const PKey<W>* kp = io.keys + threadIdx.x;
+    const double* cp = io.cin + threadIdx.x;
+    // A: live strings, normalised values, the chains of shared slots (the
+    // loads of a group of rows first)
+    double c[ROWS];
+    uint32_t flags[(ROWS + 1) / 2];   // 16 bits a row
+#pragma unroll
+    for (int r = 0; r < (ROWS + 1) / 2; ++r) flags[r] = 0u;
+#pragma unroll
+    for (int r0 = 0; r0 < ROWS; r0 += GROUP) {
+        if (r0 * BLOCK + w0 >= n) break;   // whole warps
+        PKey<W> K[GROUP];
+#pragma unroll
+        for (int u = 0; u < GROUP; ++u) {
+            const int r = r0 + u;
+#pragma unroll
+            for (int w = 0; w < W; ++w) { K[u].x[w] = 0; K[u].z[w] = 0; }
+            c[r] = 0.0;
+            if (threadIdx.x + r * BLOCK < n) {
+                if (kGathered) {
+                    const uint32_t at = A::src()[threadIdx.x + r * BLOCK];
+                    K[u] = load_key_ca(io.keys + at);
+                    c[r] = io.cin[at];
+                } else {
+                    K[u] = load_key_ca(kp + r * BLOCK);
+                    c[r] = cp[r * BLOCK];
+                }
+            }
         }
-        if (in && !dup) __stcs(io.cout + at, keep ? va : 0.0);
-        if (!keep) a = 0ULL;
-        st.out_max = max(st.out_max, a);
-        st.kept += keep ? 1u : 0u;
-        if (sel_hi) {   // uniform
-            st.above += a > sel_hi ? 1u : 0u;
-            push(keep && a - sel_lo <= sel_hi - sel_lo, a - sel_lo, io.first + at);
+#pragma unroll
+        for (int u = 0; u < GROUP; ++u) {
+            const int r = r0 + u;
+            if (r * BLOCK + w0 >= n) break;   // whole warps
+            const unsigned long long b = abs_pattern(c[r]);   // 0 past the end
+            bool live = b > floor_T;
+            if (!pd_ties) live = live && (b != pd_T || !key_less(pd_key, K[u]));
+            c[r] = __dmul_rn(c[r], rnorm);
+            uint32_t f = 0;
+            if (!kPlain) {
+                if (has_id && threadIdx.x + r * BLOCK < n && key_is_zero(K[u])) {
+                    c[r] = 1.0;   // the identity's normalised value is exactly 1
+                    f = kSpecial;
+                    if (!live) set_status(ctl, ST_TRACE_ZERO, 43);
+                }
+                if (weigh && !light(K[u], g.maxw)) f = kSpecial;
+            }
+            const bool comm = live && commutes(K[u], g);
+            const uint32_t slot = A::slot(K[u], g);
+            const uint32_t d = exch_if(comm, A::heads() + slot, me0 + r * BLOCK) ^ (tag << 11);
+            const uint32_t prev = d <= kInPrev ? d : 0u;
+            if (comm) A::next()[threadIdx.x + r * BLOCK] = (uint16_t)prev;
+            f |= comm ? slot | kComm : 0u;
+            f |= prev ? kPrev : 0u;
+            f |= live ? kLive : 0u;
+            flags[r >> 1] |= f << (16 * (r & 1));
         }
     }
-    __syncwarp();
-    // C: this warp's rare strings, densely
-    for (uint32_t r0 = 0; r0 < n_rare; r0 += 32u) {
-        const bool in = r0 + lane < n_rare;
-        const uint32_t i = in ? rare[r0 + lane] : 0u;
-        PKey<W> K;
+    __syncthreads();                                                  // (1) chains built
+    // B: every string that is alone in its slot (its partner is absent).
+    // child_may_pass as one sum: the high words of |c| and |m| against the
+    // threshold's
+    const int ht = (int)(thr >> 32);
+    const int hm = ht < 0x00100000 ? 0x40000000
+                                   : (int)(__double2hiint(g.msh) & 0x7fffffff) - 0x3ff00000 + 0x2c140 - ht;
+    double* op = io.cout + threadIdx.x;
 #pragma unroll
-        for (int w = 0; w < W; ++w) { K.x[w] = 0; K.z[w] = 0; }
+    for (int r = 0; r < ROWS; ++r) {
+        if (r * BLOCK + w0 >= n) break;   // whole warps
+        const uint32_t f = flags[r >> 1] >> (16 * (r & 1));
+        const bool comm = (f & kComm) != 0;
+        const uint32_t me = me0 + r * BLOCK;
+        uint32_t head = me;
+        if (comm) head = A::heads()[f & 0xfffu];
+        bool dup = ((f & kPrev) | (head ^ me)) != 0u;
+        if (!kPlain) dup = dup || (self && comm);
+        const bool may = comm && (int)(__double2hiint(c[r]) & 0x7fffffff) + hm >= 0;
+        list_if(dup || may, io.s_rare, A::rare(), (threadIdx.x + r * BLOCK) | (dup ? 0x8000u : 0u));
+        double va = c[r];
+        if (comm) va = __dmul_rn(va, g.ch);
+        const unsigned long long a = abs_pattern(va);
+        bool keep = (f & kLive) && !dup && a > thr;
+        const bool in = threadIdx.x + r * BLOCK < n;
+        uint32_t at = threadIdx.x + r * BLOCK;
+        if (kGathered) at = A::src()[in ? at : 0u];
+        if (!kPlain && (f & kSpecial) && (f & kLive) && !dup) {
+            if (has_id && key_is_zero(load_key_ca(io.keys + at))) {
+                ctl->norm[nxt] = va;
+                if (!keep) set_status(ctl, ST_TRACE_ZERO, 1);
+                keep = true;
+            } else {
+                keep = false;
+            }
+        }
+        if (in && !dup) __stcs(kGathered ? io.cout + at : op + r * BLOCK, keep ? va : 0.0);
+        st.hi_max = max(st.hi_max, keep ? (uint32_t)(a >> 32) : 0u);
+        st.kept += keep ? 1u : 0u;
+        if (near_hi) {   // uniform
+            const bool hit = keep && a <= near_hi;
+            if (__any_sync(0xffffffffu, hit)) push(hit, a - thr - 1ULL, io.first + at);
+        }
+    }
+    __syncthreads();                                                  // (2) the list is complete
+    // C: the rare strings, densely (read again)
+    const uint32_t n_rare = *io.s_rare;
+    for (uint32_t r0 = w0; r0 < n_rare; r0 += BLOCK) {
+        const bool in = r0 + lane < n_rare;
+        const uint32_t e0 = in ? A::rare()[r0 + lane] : 0u;
+        const uint32_t i = e0 & 0x7fffu;
+        const bool dup = (e0 & 0x8000u) != 0;
+        const uint32_t at = kGathered && in ? A::src()[i] : i;
+        PKey<W> X;
+#pragma unroll
+        for (int w = 0; w < W; ++w) { X.x[w] = 0; X.z[w] = 0; }
         double va = 0.0, vb = 0.0;
-        bool ka = false, kb = false, dup = false;
-        uint32_t at = i;
+        bool ka = false, kb = false;
         if (in) {
-            K = A::keys()[i];
-            const double c = vals[i];
-            if (kGathered) at = A::src()[i];
-            dup = self || ((A::dup()[i >> 5] >> (i & 31u)) & 1u);
+            X = load_key_ca(io.keys + at);
+            const bool id = has_id && key_is_zero(X);
+            const double cx = id ? 1.0 : __dmul_rn(io.cin[at], rnorm);
             bool neg, found = false;
-            commute_sign(K, g, &neg);
+            commute_sign(X, g, &neg);
             const double m = __longlong_as_double(
                 __double_as_longlong(g.msh) ^ (neg ? (long long)0x8000000000000000ULL : 0LL));
-            double cq = 0.0;
             if (dup) {
-                // the chain of this slot; every string of it commutes
-                uint32_t e = A::heads()[pair_slot(K, g)] & kInPrev;
-                while (e) {
-                    // (a string is its own partner only for Q = I)
-                    if (key_is_partner(A::keys()[e - 1u], K, g)) {
+                // the chain of this slot; every string of it is live and
+                // commutes (a string is its own partner only for Q = I)
+                uint32_t e = A::heads()[A::slot(X, g)] & kInPrev;
+                double cq = 0.0;
+                for (uint32_t q = 0; e && q < n; ++q) {
+                    const uint32_t ea = kGathered ? A::src()[e - 1u] : e - 1u;
+                    const PKey<W> Y = load_key_ca(io.keys + ea);
+                    if (key_is_partner(Y, X, g)) {
                         found = true;
-                        cq = vals[e - 1u];
+                        cq = has_id && key_is_zero(Y) ? 1.0 : __dmul_rn(io.cin[ea], rnorm);
                         break;
                     }
-                    e = A::next()[e - 1u] & kInPrev;
+                    e = A::next()[e - 1u];
                 }
-                va = __dmul_rn(c, g.ch);
+                va = __dmul_rn(cx, g.ch);
                 if (found) va = __dadd_rn(va, __dmul_rn(cq, m));
-                ka = above(va, thr) && (!weigh || light(K, g.maxw));
-                if (has_id && key_is_zero(K)) {
+                ka = above(va, thr) && (!weigh || light(X, g.maxw));
+                if (id) {
                     ctl->norm[nxt] = va;
                     if (!ka) set_status(ctl, ST_TRACE_ZERO, 1);
                     ka = true;
@@ -222,8 +279,8 @@ __device__ __forceinline__ void inplace_pass(uint32_t n, uint32_t shift, const G
                 __stcs(io.cout + at, ka ? va : 0.0);
             }
             if (!found) {   // the child of a lone string
-                vb = __dmul_rn(c, m);
-                kb = above(vb, thr) && (!weigh || light(key_xor(K, g), g.maxw));
+                vb = __dmul_rn(cx, m);
+                kb = above(vb, thr) && (!weigh || light(key_xor(X, g), g.maxw));
             }
         }
         const unsigned int bb = __ballot_sync(0xffffffffu, kb);
@@ -234,7 +291,7 @@ __device__ __forceinline__ void inplace_pass(uint32_t n, uint32_t shift, const G
             pos = io.n + __shfl_sync(0xffffffffu, q, 0) + __popc(bb & lt);
             if (kb) {
                 if (pos < io.room) {
-                    store_key(io.keys + pos, key_xor(K, g));
+                    store_key(io.keys + pos, key_xor(X, g));
                     __stcs(io.cout + pos, vb);
                 } else {
                     *io.over = 1;
@@ -243,15 +300,78 @@ __device__ __forceinline__ void inplace_pass(uint32_t n, uint32_t shift, const G
             }
         }
         const unsigned long long a = ka ? abs_pattern(va) : 0ULL, b = kb ? abs_pattern(vb) : 0ULL;
-        st.out_max = max(st.out_max, max(a, b));
+        st.hi_max = max(st.hi_max, max((uint32_t)(a >> 32), (uint32_t)(b >> 32)));
         st.kept += (ka ? 1u : 0u) + (kb ? 1u : 0u);
-        if (sel_hi) {
-            st.above += (a > sel_hi ? 1u : 0u) + (b > sel_hi ? 1u : 0u);
-            push(ka && a - sel_lo <= sel_hi - sel_lo, a - sel_lo, io.first + at);
-            push(kb && b - sel_lo <= sel_hi - sel_lo, b - sel_lo, io.first + pos);
+        if (near_hi) {
+            push(ka && a <= near_hi, a - thr - 1ULL, io.first + at);
+            push(kb && b <= near_hi, b - thr - 1ULL, io.first + pos);
         }
     }
-    __syncthreads();                                                  // (2) staging free
+    __syncthreads();                                                  // (3) shared arrays free
+}
+
+// A partition of any size up to 65,535 strings: one pass, or its hash classes
+// one after another, each a list of indices (strings and partners agree on
+// the class).  Every thread calls it; *s_app and *s_rare are zero, and a
+// barrier since.  Returns whether it took sub-passes.
+template <int W, int BLOCK, class Push>
+__device__ __forceinline__ bool inplace_partition(const GateArg<W>& g, unsigned long long pd_T,
+                                                  bool pd_ties, const PKey<W>& pd_key,
+                                                  double rnorm, unsigned long long thr,
+                                                  bool has_id, DevCtl* ctl, int nxt, uint32_t* tag,
+                                                  const InPlace<W>& io, InStats& st,
+                                                  unsigned long long near_hi, uint32_t* s_n,
+                                                  Push&& push) {
+    using A = InPass<W>;
+    constexpr uint32_t C = A::C;
+    if (io.n == 0u) return false;
+    uint64_t qbits = 0;
+#pragma unroll
+    for (int w = 0; w < W; ++w) qbits |= g.qx[w] | g.qz[w];
+    const bool plain = !has_id && g.maxw >= 64 * W && qbits != 0;
+    if (io.n <= C) {
+        if (plain)
+            inplace_pass<W, BLOCK, false, true>(io.n, g, pd_T, pd_ties, pd_key, rnorm, thr, false,
+                                                ctl, nxt, ++*tag, io, st, near_hi, push);
+        else
+            inplace_pass<W, BLOCK, false, false>(io.n, g, pd_T, pd_ties, pd_key, rnorm, thr, has_id, ctl, nxt,
+                                      ++*tag, io, st, near_hi, push);
+        return false;
+    }
+    if (io.n > 0xffffu) {
+        if (threadIdx.x == 0) *io.over = 1;   // the gate is merged again
+        return true;
+    }
+    const uint32_t kc = (2u * io.n + C - 1u) / C;
+    for (uint32_t j = 0; j < kc; ++j) {
+        if (threadIdx.x == 0) *s_n = *io.s_rare = 0u;
+        __syncthreads();
+        for (uint32_t i = threadIdx.x; i < io.n; i += BLOCK) {
+            if (sub_pass(load_key_ca(io.keys + i), g, kc) != j) continue;
+            const uint32_t q = atomicAdd(s_n, 1u);
+            if (q < C) A::src()[q] = (uint16_t)i;
+            else *io.over = 1;
+        }
+        __syncthreads();
+        const uint32_t m = *s_n < C ? *s_n : C;
+        if (m == 0u) continue;   // uniform
+        inplace_pass<W, BLOCK, true, false>(m, g, pd_T, pd_ties, pd_key, rnorm, thr, has_id, ctl, nxt,
+                                     ++*tag, io, st, near_hi, push);
+    }
+    return true;
+}
+
+// CTAs per SM that the in-place merge's launch bound asks for.
+template <int W, int BLOCK>
+struct InOcc {
+    static constexpr int kMin = BLOCK <= 128 ? 8 : BLOCK == 256 ? 5 : 2;
+};
+
+// Heads clear of an earlier use of the shared memory, or of a tag that comes
+// round again (a barrier must follow).
+template <int W, int BLOCK>
+__device__ __forceinline__ void inplace_init() {
+    for (uint32_t i = threadIdx.x; i < (uint32_t)InPass<W>::S; i += BLOCK) InPass<W>::heads()[i] = 0u;
 }
 
 }  // namespace

@@ -33,57 +33,39 @@
 #include "itpp_gate_body.cuh"
 #include "itpp_launch.h"
 #include "itpp_stage.cuh"
+#include "itpp_inplace.cuh"
 
 namespace itpp {
 
 // Scatter the current state into the partitions of a window (force), or,
-// inside a window, only when the previous gate's partitions hold for that
-// gate alone; otherwise the next merge reads the previous merge's segments.
-// The state is a contiguous run of terms, or (after a partitioned merge)
-// the segments its descriptors list.
+// inside a window, only when the state has no partitions or they held for the
+// previous gate alone.  The state is a contiguous run, or the partitions of
+// a home; it goes to the other home.
 template <int W>
 __global__ void __launch_bounds__(256, W == 1 ? 6 : 4)
-k_part_scatter(Bufs<W> B, DevCtl* ctl, PKey<W>* pk, double* pc, unsigned int* cursor,
-               uint64_t pbuf_cap, uint32_t p_max, GateArg<W> g, PartFn<W> f, int force,
-               int n_sites, int target, const ChunkDesc* chunks0, const ChunkDesc* chunks1,
-               int redo) {
+k_part_scatter(Bufs<W> B, Homes<W> H, DevCtl* ctl, GateArg<W> g, PartFn<W> f, int force,
+               int n_sites, int target, int redo) {
     if (ctl->status) return;
     // the second launch of a gate's scatter runs only when the first one
     // found a partition's stride too small for the groups hashed to it; it
     // scatters by the gate's pair key (pairs always fit) into cleared cursors
-    if (redo) {
-        if (!ctl->scatter_over) return;
-        f.pair = 1;
-        force = 1;
-    }
+    if (redo && !ctl->scatter_over) return;
+    if (redo) f.pair = 1;
     const int cur = ctl->cur;
+    const bool run = force || redo || ctl->need_scatter || !ctl->home;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         // the next merge's counters
         ctl->count[cur ^ 1] = 0ULL;
-        ctl->alloc[cur ^ 1] = 0ULL;
-        ctl->nchunk[cur ^ 1] = 0u;
-        ctl->sp_above = 0ULL;
+        ctl->alloc = 0ULL;
         ctl->sp_ovf = 0;
+        ctl->over = 0;
+        ctl->scattered = run;
     }
-    if (!force && !ctl->need_scatter) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) ctl->part_from_scatter = 0;
-        return;
-    }
+    if (!run) return;
     const uint64_t n = live_count(ctl, cur);
-    // The merges of a window stage each partition's stored children, which
-    // hold the select's rejected ones until the predicate drops them: when
-    // the previous gate stored g times the terms it kept, aim the kept terms
-    // of a partition at target / g (at least target / 2) so that what the
-    // next merges stage stays near the target instead of passing the staging
-    // capacity.
-    int t_eff = target;
-    if (ctl->pend && n > 0 && ctl->pend_n > n) {
-        const uint64_t t = (uint64_t)target * n / ctl->pend_n;
-        t_eff = t < (uint64_t)(target / 2) ? target / 2 : (int)t;
-    }
     const bool fallback = redo || (!f.pair && !window_fits(n_sites, f.sites, n));
     if (fallback) f.pair = 1;
-    PartPlan pl = part_plan(n, pbuf_cap, p_max, t_eff);
+    PartPlan pl = part_plan(n, H.cap, H.part_max, target);
     if (!f.pair) {
         // a partition's stride holds a whole group (up to 4^sites strings,
         // the terms with one pattern outside the window), however the terms
@@ -91,330 +73,321 @@ k_part_scatter(Bufs<W> B, DevCtl* ctl, PKey<W>* pk, double* pc, unsigned int* cu
         // rely on the second scatter by pair key when a stride overflows
         const uint64_t gmax = 1ULL << (2 * f.sites);
         if (pl.R < gmax && gmax <= 2ULL * (uint64_t)target) {
-            const uint64_t P = pbuf_cap / gmax;
+            const uint64_t P = H.cap / gmax;
             pl.P = (uint32_t)(P > 0 ? P : 1);
-            pl.R = pbuf_cap / pl.P;
+            pl.R = H.cap / pl.P;
         }
     }
-    // the chunks of the previous merge's output
-    const bool seg = ctl->seg != 0;
-    const uint32_t n_chunks = ctl->nchunk[cur];
+    const bool home = ctl->home != 0;
+    const int a = home ? ctl->ha : cur;
+    const int to_b = home ? ctl->hb ^ 1 : 0, to_x = home ? ctl->hx ^ 1 : 0;
+    const int to_c = next3(ctl->hc);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
-        ctl->part_from_scatter = 1;
-        ctl->part_P = pl.P;
+        ctl->to_b = to_b;
+        ctl->to_x = to_x;
+        ctl->to_c = to_c;
+        ctl->to_P = pl.P;
+        ctl->to_R = pl.R;
+        if (!home) ctl->ha = cur;
         ctl->stat_scatters += 1;
-        if (fallback) ctl->part_over = 1;   // the partitions hold for this gate only
+        ctl->part_over = f.pair;   // such partitions hold for this gate only
     }
     const Pending<W> pd = pending_of<W>(ctl);
     // one loop for both layouts (a single copy of the scatter body): each
-    // output chunk of the previous merge by one CTA, or the contiguous run by
-    // the whole grid (with a deferred top-M select every stored term is
-    // scanned and its kept set applied)
-    const ChunkDesc* __restrict__ cin = cur ? chunks1 : chunks0;
-    uint64_t n_scan = n;
-    if (!seg && pd.on) n_scan = ctl->pend_n < ctl->buf_cap ? ctl->pend_n : ctl->buf_cap;
-    const uint32_t runs = seg ? n_chunks : 1u;
-    for (uint32_t s = seg ? blockIdx.x : 0u; s < runs; s += seg ? gridDim.x : 1u) {
-        const uint64_t off = seg ? cin[s].off : 0ULL;
-        const uint64_t cnt = seg ? (uint64_t)cin[s].cnt : n_scan;
-        const uint64_t first = seg ? 0ULL : (uint64_t)blockIdx.x * blockDim.x;
-        const uint64_t stride = seg ? (uint64_t)blockDim.x : (uint64_t)gridDim.x * blockDim.x;
-        scatter_run(B.key(cur) + off, B.coef(cur) + off, cnt, first, stride, pd, ctl, pk, pc,
-                    cursor, pl, g, f, &ctl->scatter_over);
+    // partition by one CTA, or the contiguous run by the whole grid
+    const StateRuns<W> r = state_runs(ctl, B, H);
+    for (uint32_t s = r.cnt ? blockIdx.x : 0u; s < r.P; s += r.cnt ? gridDim.x : 1u) {
+        const uint64_t off = (uint64_t)s * r.R;
+        const uint64_t cnt = r.cnt ? (r.cnt[s] < r.R ? (uint64_t)r.cnt[s] : r.R) : r.n;
+        const uint64_t first = r.cnt ? 0ULL : (uint64_t)blockIdx.x * blockDim.x;
+        const uint64_t stride = r.cnt ? (uint64_t)blockDim.x : (uint64_t)gridDim.x * blockDim.x;
+        scatter_run(r.keys + off, r.coef + off, cnt, first, stride, pd, ctl,
+                    H.keys(B, a, to_b), H.coef(B, a, to_x), H.cursors(to_c), pl, g, f,
+                    &ctl->scatter_over);
     }
 }
 
-
 // Between a gate's two scatter launches: when the first found a stride too
 // small, clear the cursors for the second.
-__global__ void k_scatter_clear(const DevCtl* ctl, unsigned int* cursor, uint32_t p_max) {
+template <int W>
+__global__ void k_scatter_clear(const DevCtl* ctl, Homes<W> H) {
     if (ctl->status || !ctl->scatter_over) return;
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < p_max; i += gridDim.x * blockDim.x)
+    unsigned int* cursor = H.cursors(ctl->to_c);
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < H.part_max;
+         i += gridDim.x * blockDim.x)
         cursor[i] = 0u;
 }
 
-// The gate's merge, one partition at a time per CTA.  The partition comes
-// from the scatter buffer (fixed stride, cursor) or is a segment the
-// previous gate of the window wrote (descriptor).  It is copied into shared
-// memory by two bulk (TMA) copies, keys and coefficients, completed on an
-// mbarrier; a later partition of the same CTA has been prefetched into L2.
-// One pass (stage_pass) then merges it, and its kept children go to one
-// contiguous segment of the CTA's output chunk, recorded as the partition's
-// descriptor for the next gate.  Chunks are claimed from the buffer's
-// allocator a few hundred partitions at a time, so no partition waits on a
-// global atomic.  A partition above the staging capacity is merged in
-// sub-passes: each gathers the strings of one hash class of the key with
-// the gate's sites cleared (which K and Q.K share) into the staging arrays.
-// With a top-M bound the children below the select's predicted range are
-// not written (retry_pass 0); k_merge_check then keeps that output when at
-// least cap_M children were kept, and otherwise the second launch
-// (retry_pass 1) merges the gate again in full from the same input.
+// Where this gate's input partitions are: where its scatter put them, or
+// where the previous gate left them.
+struct GateInput {
+    int a, b, x, c;
+    uint32_t P;
+    uint64_t R;
+};
+
+__device__ __forceinline__ GateInput gate_input(const DevCtl* ctl) {
+    GateInput in;
+    const bool s = ctl->scattered != 0;
+    in.a = ctl->ha;
+    in.b = s ? ctl->to_b : ctl->hb;
+    in.x = s ? ctl->to_x : ctl->hx;
+    in.c = s ? ctl->to_c : ctl->hc;
+    in.P = s ? ctl->to_P : ctl->part_P;
+    in.R = s ? ctl->to_R : ctl->part_R;
+    return in;
+}
+
+// The gate's merge, in place (itpp_inplace.cuh): persistent CTAs, one
+// partition at a time, a later partition of the same CTA prefetched into L2
+// by bulk (TMA) requests.  With a top-M bound the children at or
+// below the select's lower limit are left out; k_merge_check then keeps the
+// result when at least cap_M were kept and no partition's stride ran out, and
+// otherwise k_gate_part merges the gate again in full from the same input.
 template <int W, int BLOCK>
-__global__ void __launch_bounds__(BLOCK, (PartOcc<W, BLOCK>::kMin))
-k_gate_part(const PKey<W>* __restrict__ pk, const double* __restrict__ pc,
-            unsigned int* __restrict__ cursor, uint64_t pbuf_cap, PartDesc* desc0,
-            PartDesc* desc1, Bufs<W> B, DevCtl* ctl, GateArg<W> g, double delta,
-            uint64_t cap_out, uint64_t chunk, CandRegions cd, ChunkDesc* chunks0,
-            ChunkDesc* chunks1, uint32_t max_chunks, int retry_pass) {
-    using G = Stage<W>;
-    using A = PassArgs<W>;
-    constexpr uint32_t C = G::C;
-    __shared__ __align__(8) uint64_t s_bar;
-    __shared__ unsigned long long s_chunk, s_chsz, s_nout;
-    __shared__ uint32_t s_long, s_n;
-    __shared__ int s_stop;
-    __shared__ Pending<W> s_pd;
+__global__ void __launch_bounds__(BLOCK, (InOcc<W, BLOCK>::kMin))
+k_gate_inplace(Bufs<W> B, Homes<W> H, DevCtl* ctl, GateArg<W> g, double delta, CandRegions cd) {
+    using A = InPass<W>;
+    __shared__ unsigned long long s_T, s_thr, s_kept;
+    __shared__ PKey<W> s_tk;
     __shared__ double s_rnorm;
-    __shared__ unsigned long long s_thr;   // kept: pattern above this
+    __shared__ uint32_t s_long, s_n, s_app, s_rare;
+    __shared__ int s_stop, s_ties, s_over;
     const int cur = ctl->cur, nxt = cur ^ 1;
-    const bool from_scatter = ctl->part_from_scatter != 0;
-    const uint32_t P = ctl->part_P;
-    const uint64_t R = P ? pbuf_cap / P : 0;
-    const PartDesc* __restrict__ din = cur ? desc1 : desc0;
-    PartDesc* __restrict__ dout = cur ? desc0 : desc1;
-    const unsigned long long dbits = (unsigned long long)__double_as_longlong(delta);
+    const GateInput in = gate_input(ctl);
+    const uint64_t R = in.R;
     if (threadIdx.x == 0) {
         // one read of the status for the whole CTA (another CTA may set it
-        // meanwhile, and every thread must leave at the same point); the
-        // second launch of a gate runs only when the first one must be redone
-        s_stop = ctl->status || (retry_pass && !ctl->retry);
-        s_pd = pending_of<W>(ctl);
+        // meanwhile, and every thread must leave at the same point)
+        s_stop = ctl->status;
+        const Pending<W> pd = pending_of<W>(ctl);
+        s_T = pd.T;
+        s_ties = pd.all_ties;
+        s_tk = pd.tk;
         s_rnorm = ctl->rnorm[cur];
         g_cn = 0u;
         g_range[0] = ctl->sp_lo;
         g_range[1] = ctl->sp_hi;
-        s_nout = 0ULL;      // thread 0 counts the CTA's output and long partitions
+        s_kept = 0ULL;
         s_long = 0u;
-        mbar_init(&s_bar, 1);
-    }
-    if (threadIdx.x == 0) {
-        // children below the candidate range are left unwritten: when at
-        // least cap_M children lie at or above it (checked after the merge),
-        // the select would drop every one of them; otherwise the gate's
-        // merge runs again without this (retry_pass)
-        unsigned long long thr = dbits;
-        if (!retry_pass && g_range[1] != 0ULL && g_range[0] > 0ULL && g_range[0] - 1ULL > thr)
-            thr = g_range[0] - 1ULL;
+        s_over = 0;
+        const unsigned long long dbits = (unsigned long long)__double_as_longlong(delta);
+        const unsigned long long thr = ctl->sp_hi && ctl->sp_thr > dbits ? ctl->sp_thr : dbits;
         s_thr = thr;
-        if (blockIdx.x == 0 && !ctl->status && !retry_pass) ctl->drop_on = thr != dbits;
+        if (blockIdx.x == 0 && !ctl->status) {
+            ctl->drop_on = thr != dbits;
+            ctl->cand_regions = gridDim.x;
+        }
     }
-    pass_init<W, BLOCK>();
+    inplace_init<W, BLOCK>();
     __syncthreads();
     if (s_stop) return;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        ctl->cand_regions = gridDim.x;
-        ctl->seg = 1;          // the output is the P segments this merge writes
-        ctl->seg_P = P;
+    // the third cursor array (the previous gate's input) is the next scatter's
+    {
+        unsigned int* spare = H.cursors(next3(next3(in.c)));
+        for (uint32_t i = blockIdx.x * BLOCK + threadIdx.x; i < H.part_max; i += gridDim.x * BLOCK)
+            spare[i] = 0u;
     }
-    const Pending<W>& pd = s_pd;
-    const double rnorm = s_rnorm;
-    PKey<W>* __restrict__ kout = B.key(nxt);
-    double* __restrict__ cout = B.coef(nxt);
-    SelStats st{0ULL, 0u};
-    // this CTA's output chunk: [ch_start, ch_pos) written, [ch_pos, ch_end)
-    // free (the same on every thread)
-    unsigned long long ch_start = 0, ch_pos = 0, ch_end = 0;
-    uint32_t pass = 0, parity = 0;
-    const uint32_t p_id = identity_part<W>(P);
-    ChunkDesc* __restrict__ chunks_out = cur ? chunks0 : chunks1;
-    // record the written run of a chunk for the readers of the whole state
-    auto record_chunk = [&](unsigned long long start, unsigned long long end) {
-        if (end == start) return;
-        const unsigned int q = atomicAdd(&ctl->nchunk[nxt], 1u);
-        if (q < max_chunks) {
-            chunks_out[q].off = start;
-            chunks_out[q].cnt = (unsigned int)(end - start);
-        } else {
-            set_status(ctl, ST_CAPACITY, 46);
-        }
+    PKey<W>* keys = H.keys(B, in.a, in.b);
+    const double* cin = H.coef(B, in.a, in.x);
+    double* cout = H.coef(B, in.a, in.x ^ 1);
+    const unsigned int* cnt_in = H.cursors(in.c);
+    unsigned int* cnt_out = H.cursors(next3(in.c));
+    const uint32_t p_id = identity_part<W>(in.P);
+    auto push = [&](bool hit, unsigned long long v, uint64_t idx) {
+        cand_push(hit, v, idx, cd, &g_cn);
     };
-    // claim room for at least `need` terms (every thread calls it)
-    auto claim = [&](unsigned long long need) -> bool {
-        if (threadIdx.x == 0) {
-            record_chunk(ch_start, ch_pos);
-            const unsigned long long sz = need > chunk ? need : chunk;
-            const unsigned long long b = atomicAdd(&ctl->alloc[nxt], sz);
-            if (b + sz > cap_out) {
-                set_status(ctl, ST_CAPACITY, 2);
-                s_chunk = ~0ULL;
-            } else {
-                s_chunk = b;
-            }
-            s_chsz = sz;
-        }
-        __syncthreads();
-        const unsigned long long b = s_chunk;
-        if (b == ~0ULL) return false;
-        ch_start = b;
-        ch_pos = b;
-        ch_end = b + s_chsz;
-        return true;
-    };
-    for (uint32_t p = blockIdx.x; p < P; p += gridDim.x) {
-        const PKey<W>* kp;
-        const double* cp;
-        uint64_t np;
-        if (from_scatter) {
-            np = cursor[p];
-            if (np > R) np = R;
-            kp = pk + (uint64_t)p * R;
-            cp = pc + (uint64_t)p * R;
-        } else {
-            np = din[p].cnt;
-            kp = B.key(cur) + din[p].off;
-            cp = B.coef(cur) + din[p].off;
-        }
+    InStats st{0u, 0u};
+    uint32_t tag = 0;
+    uint32_t np = blockIdx.x < in.P ? cnt_in[blockIdx.x] : 0u;
+    for (uint32_t p = blockIdx.x; p < in.P; p += gridDim.x) {
+        InPlace<W> io;
+        io.n = np < R ? np : (uint32_t)R;
+        io.room = (uint32_t)(R < 0xffffffffULL ? R : 0xffffffffULL);
+        io.first = (uint64_t)p * R;
+        io.keys = keys + io.first;
+        io.cin = cin + io.first;
+        io.cout = cout + io.first;
+        io.s_app = &s_app;
+        io.s_rare = &s_rare;
+        io.over = &s_over;
         // warm L2 with the partition this CTA takes next
         const uint32_t pn = p + gridDim.x;
-        if (threadIdx.x == 0 && pn < P) {
-            uint64_t nn;
-            const PKey<W>* nk;
-            const double* nc;
-            if (from_scatter) {
-                nn = cursor[pn];
-                if (nn > R) nn = R;
-                nk = pk + (uint64_t)pn * R;
-                nc = pc + (uint64_t)pn * R;
-            } else {
-                nn = din[pn].cnt;
-                nk = B.key(cur) + din[pn].off;
-                nc = B.coef(cur) + din[pn].off;
-            }
+        np = pn < in.P ? cnt_in[pn] : 0u;
+        if (threadIdx.x == 0) {
+            s_app = s_rare = 0u;
+            const uint64_t nn = np < R ? np : R;
             if (nn) {
-                l2_prefetch_bulk(nk, nn * sizeof(PKey<W>));
-                l2_prefetch_bulk(nc, nn * sizeof(double));
+                l2_prefetch_bulk(keys + (uint64_t)pn * R, nn * sizeof(PKey<W>));
+                l2_prefetch_bulk(cin + (uint64_t)pn * R, nn * sizeof(double));
             }
         }
-        if (np <= C) {
-            // stage the partition: keys, and the coefficients from the 16-byte
-            // boundary at or below their start (one spare element when the
-            // segment starts at an odd element)
-            const uint32_t shift = (uint32_t)((reinterpret_cast<uint64_t>(cp) >> 3) & 1ULL);
-            if (np) {
-                if (threadIdx.x == 0) {
-                    const uint32_t kb = (uint32_t)(np * sizeof(PKey<W>));
-                    const uint32_t cb = (uint32_t)(((shift + np) * sizeof(double) + 15) & ~15ULL);
-                    fence_async_shared();
-                    mbar_expect(&s_bar, kb + cb);
-                    bulk_g2s(A::keys(), kp, kb, &s_bar);
-                    bulk_g2s(A::vals(), cp - shift, cb, &s_bar);
-                }
-                const bool ok = mbar_wait(&s_bar, parity, kWaitPolls);
-                if (__syncthreads_or(!ok)) {
-                    if (threadIdx.x == 0) {
-                        set_status(ctl, ST_TIMEOUT, 45);
-                        mbar_wait(&s_bar, parity, kWaitPolls);   // the copy in flight
-                    }
-                    __syncthreads();
-                    return;
-                }
-                parity ^= 1u;
-            }
-            ++pass;
-            // room for the most children the pass can have, claimed once the
-            // pairs are known: the rest of the current chunk, else a fresh one
-            // (the rest of the old one is left as a hole); the next partition
-            // starts right behind the kept ones
-            unsigned long long at = 0;
-            bool failed = false;
-            const uint32_t tot = stage_pass<W, BLOCK, PassRoom::kBound>(
-                (uint32_t)np, shift, g, pd, rnorm, s_thr, p == p_id, ctl, nxt, pass, kout, cout,
-                st, cd,
-                [&](uint32_t t) -> unsigned long long {
-                    if (ch_end - ch_pos < t && !claim(t)) {
-                        failed = true;
-                        return ~0ULL;
-                    }
-                    at = ch_pos;
-                    return at;
-                });
-            if (failed) return;
-            if (threadIdx.x == 0) {
-                dout[p].off = at;
-                dout[p].cnt = tot;
-                s_nout += tot;
-            }
-            ch_pos += tot;
-        } else {
-            // a long partition: sub-passes (merge_long), its children one
-            // segment; written in one round where room for 2 np of them is
-            // at hand or within a fresh chunk, else counted first and given
-            // exactly their number
-            unsigned long long pre = ~0ULL;
-            if (ch_end - ch_pos >= 2 * np) {
-                pre = ch_pos;
-            } else if (2 * np <= chunk) {
-                if (!claim(2 * np)) return;
-                pre = ch_pos;
-            }
-            unsigned long long at = pre;
-            bool failed = false;
-            const uint32_t done = merge_long<W, BLOCK>(
-                kp, cp, np, g, pd, rnorm, s_thr, p == p_id, ctl, nxt, &pass, kout, cout, st, cd,
-                pre,
-                [&](uint32_t t) -> unsigned long long {
-                    if (ch_end - ch_pos < t && !claim(t)) {
-                        failed = true;
-                        return ~0ULL;
-                    }
-                    at = ch_pos;
-                    return at;
-                },
-                nullptr, &s_n);
-            if (failed) return;
-            ch_pos += done;
-            if (threadIdx.x == 0) {
-                dout[p].off = at;
-                dout[p].cnt = done;
-                s_nout += done;
-                s_long += 1u;
-            }
+        __syncthreads();
+        const bool subs = inplace_partition<W, BLOCK>(g, s_T, s_ties != 0, s_tk, s_rnorm, s_thr,
+                                                      p == p_id, ctl, nxt, &tag, io, st,
+                                                      g_range[1], &s_n, push);
+        if (threadIdx.x == 0) {
+            const uint64_t c = (uint64_t)io.n + s_app;
+            cnt_out[p] = (unsigned int)(c < R ? c : R);
         }
+        if (subs && threadIdx.x == 0) s_long += 1u;
+        if (tag >= kHeadTagMax - 65536u) {   // tags start again
+            inplace_init<W, BLOCK>();
+            tag = 0;
+        }
+        __syncthreads();
     }
-    // one atomic per warp for the largest pattern and the count above the
-    // candidate range, one per CTA for the term count
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        st.out_max = max(st.out_max, __shfl_xor_sync(0xffffffffu, st.out_max, o));
-        st.above += __shfl_xor_sync(0xffffffffu, st.above, o);
-    }
+    // one atomic per warp for the largest pattern, one per CTA for the term
+    // count
+    const uint32_t hm = __reduce_max_sync(0xffffffffu, st.hi_max);
+    const uint32_t kept = __reduce_add_sync(0xffffffffu, st.kept);
     if ((threadIdx.x & 31) == 0) {
-        if (st.out_max) atomicMax(&ctl->out_max, st.out_max);
-        if (st.above) atomicAdd(&ctl->sp_above, (unsigned long long)st.above);
+        if (hm) atomicMax(&ctl->out_max, ((unsigned long long)hm << 32) | 0xffffffffULL);
+        if (kept) atomicAdd(&s_kept, (unsigned long long)kept);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        record_chunk(ch_start, ch_pos);
-        if (s_nout) atomicAdd(&ctl->count[nxt], s_nout);
+        if (s_kept) atomicAdd(&ctl->count[nxt], s_kept);
         if (s_long) atomicAdd(&ctl->stat_long, (unsigned long long)s_long);
+        if (s_over) ctl->over = 1;
         const uint32_t c = g_cn;
         cd.cnt[blockIdx.x] = c < cd.region ? c : (uint32_t)cd.region;
         if (c > cd.region) ctl->sp_ovf = 1;
     }
 }
 
-// After a merge that left the children below the candidate range unwritten:
-// with at least cap_M children kept, the select keeps cap_M of them and every
-// unwritten one lay below them all; with fewer, the unwritten ones are
-// needed, so the merge's output is discarded and the gate's merge runs again
-// in full (its input, the partitions or the previous gate's segments, is
-// still in place).
+// After a merge that left children out: with at least cap_M kept, the select
+// keeps cap_M of them and every one left out lay below them all; with fewer
+// they are needed.  Then, and when a partition's stride ran out, the gate's
+// merge is done again in full (its input is still in place).
 __global__ void k_merge_check(DevCtl* ctl, uint64_t cap_M) {
     if (threadIdx.x != 0 || ctl->status) return;
     const int nxt = ctl->cur ^ 1;
     ctl->retry = 0;
     ctl->scatter_over = 0;   // the gate's scatters are done
-    if (ctl->drop_on && ctl->count[nxt] < cap_M) {
+    if (ctl->over || (ctl->drop_on && ctl->count[nxt] < cap_M)) {
         ctl->retry = 1;
         ctl->count[nxt] = 0ULL;
-        ctl->alloc[nxt] = 0ULL;
-        ctl->nchunk[nxt] = 0u;
-        ctl->sp_above = 0ULL;
+        ctl->alloc = 0ULL;
         ctl->sp_ovf = 0;
+        ctl->cand_regions = 0;
         ctl->out_max = 0ULL;
         ctl->stat_retry += 1ULL;
     }
     ctl->drop_on = 0;
+}
+
+// The gate's merge again, in full, into a contiguous run of the free buffer:
+// one partition at a time per CTA, its children counted, then claimed (one
+// atomic a partition) and written.  Lists no candidates: the select passes
+// over the state.
+template <int W, int BLOCK>
+__global__ void __launch_bounds__(BLOCK, (PartOcc<W, BLOCK>::kMin))
+k_gate_part(Bufs<W> B, Homes<W> H, DevCtl* ctl, GateArg<W> g, double delta, uint64_t cap_out) {
+    using A = PassArgs<W>;
+    __shared__ unsigned long long s_at;
+    __shared__ uint32_t s_n;
+    __shared__ int s_stop;
+    __shared__ Pending<W> s_pd;
+    __shared__ double s_rnorm;
+    const int cur = ctl->cur, nxt = cur ^ 1;
+    if (threadIdx.x == 0) {
+        s_stop = ctl->status || !ctl->retry;
+        s_pd = pending_of<W>(ctl);
+        s_rnorm = ctl->rnorm[cur];
+        g_cn = 0u;
+        g_range[0] = g_range[1] = 0ULL;
+    }
+    __syncthreads();
+    if (s_stop) return;
+    pass_init<W, BLOCK>();
+    __syncthreads();
+    const GateInput in = gate_input(ctl);
+    const unsigned long long dbits = (unsigned long long)__double_as_longlong(delta);
+    const PKey<W>* keys = H.keys(B, in.a, in.b);
+    const double* cin = H.coef(B, in.a, in.x);
+    PKey<W>* kout = B.key(in.a);
+    double* cout = B.coef(in.a);
+    const uint32_t p_id = identity_part<W>(in.P);
+    {   // the first try's cursors: the next scatter's
+        unsigned int* spare = H.cursors(next3(in.c));
+        for (uint32_t i = blockIdx.x * BLOCK + threadIdx.x; i < H.part_max; i += gridDim.x * BLOCK)
+            spare[i] = 0u;
+    }
+    auto room = [&](uint32_t n_out) -> unsigned long long {
+        if (threadIdx.x == 0) {
+            unsigned long long at = n_out ? atomicAdd(&ctl->alloc, (unsigned long long)n_out) : 0ULL;
+            if (at + n_out > cap_out) {
+                set_status(ctl, ST_CAPACITY, 2);
+                at = ~0ULL;
+            }
+            s_at = at;
+        }
+        __syncthreads();
+        return s_at;
+    };
+    SelStats st{0ULL, 0u};
+    const CandRegions none{};
+    uint32_t pass = 0;
+    for (uint32_t p = blockIdx.x; p < in.P; p += gridDim.x) {
+        uint64_t np = H.cursors(in.c)[p];
+        if (np > in.R) np = in.R;
+        const PKey<W>* kp = keys + (uint64_t)p * in.R;
+        const double* cp = cin + (uint64_t)p * in.R;
+        if (np <= (uint64_t)Stage<W>::C) {
+            ++pass;   // (merge_long numbers its own: consecutive passes alternate)
+            for (uint32_t i = threadIdx.x; i < np; i += BLOCK) {
+                A::keys()[i] = load_key_stream(kp + i);
+                A::vals()[i] = __ldcs(cp + i);
+            }
+            __syncthreads();
+            stage_pass<W, BLOCK, PassRoom::kExact>((uint32_t)np, 0u, g, s_pd, s_rnorm, dbits,
+                                                   p == p_id, ctl, nxt, pass, kout, cout, st, none,
+                                                   room);
+        } else {
+            merge_long<W, BLOCK>(kp, cp, np, g, s_pd, s_rnorm, dbits, p == p_id, ctl, nxt, &pass,
+                                 kout, cout, st, none, ~0ULL, room, nullptr, &s_n);
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        st.out_max = max(st.out_max, __shfl_xor_sync(0xffffffffu, st.out_max, o));
+    if ((threadIdx.x & 31) == 0 && st.out_max) atomicMax(&ctl->out_max, st.out_max);
+}
+
+// After the merge: where the state is now, then the buffer switch, normaliser,
+// statistics and bound of every gate (post_one).
+__global__ void k_part_post(DevCtl* ctl, uint64_t cap_M, int cap_policy) {
+    __shared__ int s_active;
+    if (ctl->status) return;
+    if (threadIdx.x == 0) {
+        if (ctl->scattered) {
+            ctl->home = 1;
+            ctl->hb = ctl->to_b;
+            ctl->hx = ctl->to_x;
+            ctl->hc = ctl->to_c;
+            ctl->part_P = ctl->to_P;
+            ctl->part_R = ctl->to_R;
+        }
+        if (ctl->retry) {
+            ctl->home = 0;
+            ctl->count[ctl->cur ^ 1] = ctl->alloc;
+        } else {
+            ctl->hx ^= 1;
+            ctl->hc = next3(ctl->hc);
+        }
+        s_active = post_one(ctl, cap_M, cap_policy);
+        const int cur = ctl->cur, a = ctl->ha;
+        if (!ctl->home && cur != a) {   // the run is in buffer a
+            ctl->count[a] = ctl->count[cur];
+            ctl->norm[a] = ctl->norm[cur];
+            ctl->rnorm[a] = ctl->rnorm[cur];
+            ctl->cur = a;
+        }
+    }
+    __syncthreads();
+    if (s_active)
+        for (int b = threadIdx.x; b < kSelBins; b += blockDim.x) ctl->sel_hist[b] = 0ULL;
 }
 
 // ---------------------------------------------------------------------------
@@ -458,50 +431,58 @@ static PartFn<W> part_fn_of(const HostGate& h) {
 }
 
 template <int W>
+static Homes<W> homes_of(const DeviceState& s) {
+    Homes<W> h;
+    h.kp = reinterpret_cast<PKey<W>*>(s.part_keys);
+    h.cp = s.part_coef;
+    h.cnt = s.part_cursor;
+    h.part_max = s.part_max;
+    h.cap = s.part_cap < s.buf_cap ? s.part_cap : s.buf_cap;
+    return h;
+}
+
+template <int W>
 static cudaError_t scatter_w(const DeviceState& s, const HostGate& h, int force, cudaStream_t st) {
-    // every gate: the merge leaves the cursors as they are (a gate whose
-    // merge runs again reads its partitions twice), and whether this gate
-    // scatters is decided on the device
-    cudaError_t e = cudaMemsetAsync(s.part_cursor, 0, (size_t)s.part_max * sizeof(unsigned int), st);
-    if (e != cudaSuccess) return e;
     uint64_t gs = (s.buf_cap + 255) / 256;
     const uint64_t lim = (uint64_t)s.num_sms * 8;
     if (gs > lim) gs = lim;
     if (gs < 1) gs = 1;
     for (int redo = 0; redo < 2; ++redo) {
-        if (redo) k_scatter_clear<<<s.num_sms, 256, 0, st>>>(s.ctl, s.part_cursor, s.part_max);
-        k_part_scatter<W><<<(int)gs, 256, 0, st>>>(pbufs_of<W>(s), s.ctl,
-                                                   reinterpret_cast<PKey<W>*>(s.part_keys),
-                                                   s.part_coef, s.part_cursor, s.part_cap,
-                                                   s.part_max, gate_of<W>(h), part_fn_of<W>(h),
-                                                   force, s.n, s.part_target, s.chunks[0],
-                                                   s.chunks[1], redo);
+        if (redo) k_scatter_clear<W><<<s.num_sms, 256, 0, st>>>(s.ctl, homes_of<W>(s));
+        k_part_scatter<W><<<(int)gs, 256, 0, st>>>(pbufs_of<W>(s), homes_of<W>(s), s.ctl,
+                                                   gate_of<W>(h), part_fn_of<W>(h), force, s.n,
+                                                   s.part_target, redo);
     }
     return cudaGetLastError();
 }
 
 template <int W, int BLOCK>
 static cudaError_t merge_wb(const DeviceState& s, const GateArg<W>& g, cudaStream_t st) {
-    static int per_sm = 0;
-    constexpr size_t smem = Stage<W>::kBytes;
+    static int per_sm = 0, per_sm_full = 0;
+    constexpr size_t smem = InPass<W>::kBytes, smem_full = Stage<W>::kBytes;
     if (!per_sm) {
-        cudaFuncSetAttribute(k_gate_part<W, BLOCK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
         // shared memory for every resident CTA's staging rather than L1
+        cudaFuncSetAttribute(k_gate_inplace<W, BLOCK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)smem);
+        cudaFuncSetAttribute(k_gate_inplace<W, BLOCK>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                             (int)cudaSharedmemCarveoutMaxShared);
+        cudaFuncSetAttribute(k_gate_part<W, BLOCK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)smem_full);
         cudaFuncSetAttribute(k_gate_part<W, BLOCK>, cudaFuncAttributePreferredSharedMemoryCarveout,
                              (int)cudaSharedmemCarveoutMaxShared);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gate_part<W, BLOCK>, BLOCK, smem);
-        if (per_sm < 1) per_sm = 1;
+        int n = 0;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_gate_part<W, BLOCK>, BLOCK, smem_full);
+        per_sm_full = n > 0 ? n : 1;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_gate_inplace<W, BLOCK>, BLOCK, smem);
+        per_sm = n > 0 ? n : 1;
     }
     int grid = s.num_sms * per_sm;
     if (grid > s.max_ctas) grid = s.max_ctas;   // one candidate region per CTA
-    for (int pass = 0; pass < 2; ++pass) {
-        k_gate_part<W, BLOCK><<<grid, BLOCK, smem, st>>>(
-            reinterpret_cast<const PKey<W>*>(s.part_keys), s.part_coef, s.part_cursor, s.part_cap,
-            s.part_desc[0], s.part_desc[1], pbufs_of<W>(s), s.ctl, g, s.delta, s.buf_cap,
-            s.chunk, s.cand, s.chunks[0], s.chunks[1], s.max_chunks, pass);
-        if (pass == 0) k_merge_check<<<1, 32, 0, st>>>(s.ctl, s.cap_M);
-    }
+    k_gate_inplace<W, BLOCK><<<grid, BLOCK, smem, st>>>(pbufs_of<W>(s), homes_of<W>(s), s.ctl, g,
+                                                        s.delta, s.cand);
+    k_merge_check<<<1, 32, 0, st>>>(s.ctl, s.cap_M);
+    k_gate_part<W, BLOCK><<<s.num_sms * per_sm_full, BLOCK, smem_full, st>>>(
+        pbufs_of<W>(s), homes_of<W>(s), s.ctl, g, s.delta, s.buf_cap);
     return cudaGetLastError();
 }
 
@@ -521,6 +502,11 @@ static cudaError_t merge_w(const DeviceState& s, const HostGate& h, cudaStream_t
 cudaError_t launch_part_scatter(const DeviceState& s, const HostGate& h, int force,
                                 cudaStream_t st) {
     return s.W == 1 ? scatter_w<1>(s, h, force, st) : scatter_w<2>(s, h, force, st);
+}
+
+cudaError_t launch_part_post(const DeviceState& s, cudaStream_t st) {
+    k_part_post<<<1, 256, 0, st>>>(s.ctl, s.cap_M, s.cap_policy);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_part_merge(const DeviceState& s, const HostGate& h, cudaStream_t st) {
@@ -562,28 +548,6 @@ void plan_windows(int W, std::vector<HostGate>& gates) {
         }
         k = e;
     }
-}
-
-// A merge CTA claims output room in chunks of about an eighth of its share
-// of a bounded state (at most 2^16 terms), or exactly a partition's children
-// when they need more.  What the chunks leave unused is the rest of each
-// CTA's last chunk and, each time a partition did not fit, the rest of the
-// chunk it left (less than that partition's children, at most a quarter of
-// a chunk of at least four times the largest pass's children): the state
-// buffers' slack covers two chunks per CTA and three quarters of the bound
-// for the second, above the 2 cap_M children a merge writes at most.  A
-// bound too small for such chunks (0 returned) makes every claim exact: one
-// claim per partition, nothing left unused.
-uint64_t merge_chunk(uint64_t cap_M, int max_ctas, int W) {
-    uint64_t c = cap_M / (8ULL * (uint64_t)(max_ctas > 0 ? max_ctas : 1));
-    uint64_t p = 16;
-    while (p * 2 <= c && p < (1ULL << 16)) p *= 2;
-    const uint64_t least = 4ULL * 2ULL * (uint64_t)(W == 1 ? Stage<1>::C : Stage<2>::C);
-    return p < least ? 0ULL : p;
-}
-
-uint64_t merge_slack(uint64_t cap_M, int max_ctas, int W) {
-    return 2ULL * (uint64_t)max_ctas * merge_chunk(cap_M, max_ctas, W) + cap_M / 4 * 3 + 4096;
 }
 
 int partition_target_default(int W) {

@@ -10,11 +10,12 @@
 //
 //   scatter   (a window's first gate) the state into the window's partitions
 //   merge     the gate over every partition, in place (itpp_inplace.cuh)
-//   select    the team's first CTA: statistics, the next normaliser, the
-//             top-M threshold from the candidates the merge listed, published
-//             for the next gate; the others clear cursors meanwhile
+//   select    the team's first CTA, once all have arrived: statistics, the next
+//             normaliser, the top-M threshold from the candidates the merge
+//             listed, published for the next gate
 //
-// that is two barriers per gate inside a window.  The rest is rare and decided
+// so inside a window a gate costs one arrival of every CTA and one word that
+// all of them wait for.  The rest is rare and decided
 // on the device: a threshold outside the listed range takes radix passes over
 // the state by the whole team; a merge that left children out which the bound
 // then needed, or that ran out of a partition's stride, is done again from its
@@ -37,7 +38,9 @@ namespace {
 
 constexpr int kBlock = 256;
 constexpr int kDigit = 11, kBins = 1 << kDigit;   // radix digit of the select
-constexpr uint32_t kFinal = 256;                  // strings ranked one per thread
+constexpr uint32_t kFinal = 128;                  // values ranked one per thread
+constexpr size_t kScratch = 16384;                 // shared scratch of a select, behind the pass's arrays
+constexpr uint32_t kOneCta = 4096;                // candidates the first CTA selects among
 constexpr uint32_t kPushBuf = 512;                // candidates a CTA lists in shared memory
 constexpr int kRangeShift = 45;                   // first candidate range: T +- about 1/128 of T
 
@@ -46,15 +49,17 @@ struct Pub {
     unsigned long long T;        // pending select: kept at or above this pattern (0: none)
     uint64_t tk[4];              // ... and at it up to this key
     unsigned long long lo, hi;   // candidate range of the next gate (hi == 0: none)
+    unsigned long long thr;      // children at or below this pattern are left out
     unsigned long long n;        // logical terms
+    unsigned long long base, range, rank;   // a select by the team: values pattern - base
     double rnorm;
-    int all_ties, stop, full, rescatter;
+    int all_ties, stop, full, rescatter, redo, pad;
 };
 
 // Written by every CTA during a gate; one set per gate parity, one for the
 // merge that is done again.
 struct Acc {
-    unsigned long long kept, above, out_max, alloc;
+    unsigned long long kept, out_max, alloc, pad;
     unsigned int cand_n, over, n_long, scatter_over;
 };
 
@@ -63,12 +68,13 @@ struct Acc {
 struct RunShared {
     unsigned int bar;            // arrivals at the team's barrier so far
     unsigned int dead;           // a wait ran out
+    unsigned int seq;            // publications so far
+    unsigned int pad0;
     Pub pub;
     Acc acc[2][2];
-    unsigned int sel_n;          // full select: candidates gathered
+    unsigned int sel_n;          // select by the team: entries gathered
     unsigned int pad;
-    unsigned long long sel_prefix, sel_mask, sel_k, sel_count;
-    unsigned int hist[kBins];
+    unsigned int hist[3][kBins];
 };
 
 size_t run_shared_bytes() { return (sizeof(RunShared) + 255) / 256 * 256; }
@@ -77,46 +83,94 @@ size_t run_shared_head() { return offsetof(RunShared, pub); }
 namespace {
 
 // ---------------------------------------------------------------------------
-// Team barrier
+// Arrivals and publications
 // ---------------------------------------------------------------------------
 struct Team {
     RunShared* rs;
     uint32_t rank, size;
-    uint32_t target;   // arrivals that complete the next barrier
+    uint32_t target;   // arrivals that complete the current phase
+    uint32_t seq;      // publications so far
 };
 
-// False: the wait ran out (about ten seconds) here or elsewhere in the team;
-// the caller leaves the kernel.  Every thread calls it.
-__device__ __forceinline__ bool team_barrier(Team& t, DevCtl* ctl) {
-    __shared__ int s_ok;
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int ok = 1;
-        t.target += t.size;
-        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" :: "l"(&t.rs->bar) : "memory");
-        uint32_t it = 0;
-        for (;;) {
-            uint32_t v;
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&t.rs->bar) : "memory");
-            if ((int32_t)(v - t.target) >= 0) break;
-            if (++it > 64u) {
-                __nanosleep(it > 4096u ? 1000u : 32u);
-                if (it > 10000000u || *(volatile unsigned int*)&t.rs->dead) {
-                    set_status(ctl, ST_TIMEOUT, 60);
-                    *(volatile unsigned int*)&t.rs->dead = 1u;
-                    ok = 0;
-                    break;
-                }
+// One thread waits for *p to reach v (in wrapping order); false after about
+// ten seconds here, or when another wait of the team ran out.
+__device__ __forceinline__ bool wait_for(const unsigned int* p, uint32_t v, RunShared* rs,
+                                         DevCtl* ctl) {
+    for (uint32_t it = 0;; ++it) {
+        uint32_t x;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(x) : "l"(p) : "memory");
+        if ((int32_t)(x - v) >= 0) return true;
+        if (it > 2048u) {
+            __nanosleep(it > 16384u ? 1000u : 64u);
+            if (it > 10000000u || *(volatile unsigned int*)&rs->dead) {
+                set_status(ctl, ST_TIMEOUT, 60);
+                *(volatile unsigned int*)&rs->dead = 1u;
+                return false;
             }
         }
-        __threadfence();
-        s_ok = ok;
+    }
+}
+
+// This CTA's writes so far are done; every thread calls it.
+__device__ __forceinline__ void team_arrive(Team& t) {
+    t.target += t.size;
+    __syncthreads();   // the release below covers every thread's writes before it
+    if (threadIdx.x == 0) {
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" :: "l"(&t.rs->bar) : "memory");
+    }
+}
+
+// Wait until every CTA of the team has arrived; every thread calls it.  False:
+// the wait ran out and the caller leaves the kernel.
+__device__ __forceinline__ bool team_wait(const Team& t, DevCtl* ctl) {
+    __shared__ int s_ok;
+    if (threadIdx.x == 0) {
+        s_ok = wait_for(&t.rs->bar, t.target, t.rs, ctl);
     }
     __syncthreads();
     const int ok = s_ok;
     __syncthreads();
     return ok != 0;
+}
+
+__device__ __forceinline__ bool team_barrier(Team& t, DevCtl* ctl) {
+    team_arrive(t);
+    return team_wait(t, ctl);
+}
+
+// Publish a block prepared in shared memory (the first CTA's first warp, whose
+// thread 0 wrote it, calls it).
+__device__ __forceinline__ void publish(const Team& t, const Pub* s_next) {
+    constexpr int N = sizeof(Pub) / 8;
+    __syncwarp();
+    if (threadIdx.x < N)
+        __stcg(reinterpret_cast<unsigned long long*>(&t.rs->pub) + threadIdx.x,
+               reinterpret_cast<const unsigned long long*>(s_next)[threadIdx.x]);
+    __syncwarp();
+    if (threadIdx.x == 0)
+        asm volatile("st.release.gpu.global.u32 [%0], %1;" :: "l"(&t.rs->seq), "r"(t.seq + 1u) : "memory");
+}
+
+// Wait for the next publication and copy it (every thread calls it).
+__device__ __forceinline__ bool take_pub(Team& t, DevCtl* ctl, Pub* s_pub) {
+    static_assert(sizeof(Pub) % 8 == 0 && sizeof(Pub) <= 256, "one load per lane");
+    constexpr int N = sizeof(Pub) / 8;
+    __shared__ int s_ok;
+    t.seq += 1u;
+    __syncthreads();   // the last one's readers are done
+    if (threadIdx.x < 32) {
+        int ok = 0;
+        if (threadIdx.x == 0) {
+            ok = wait_for(&t.rs->seq, t.seq, t.rs, ctl);
+            s_ok = ok;
+        }
+        __syncwarp();
+        if (threadIdx.x < N)
+            reinterpret_cast<unsigned long long*>(s_pub)[threadIdx.x] =
+                __ldcg(reinterpret_cast<const unsigned long long*>(&t.rs->pub) + threadIdx.x);
+    }
+    __syncthreads();
+    return s_ok != 0;
 }
 
 // ---------------------------------------------------------------------------
@@ -219,13 +273,11 @@ __device__ __forceinline__ void pick_bin(const uint32_t* h, uint32_t k, uint32_t
     __syncthreads();
 }
 
-// Bits [off, off + kDigit) of a key, words in comparison order, off counted
-// from the top of word 0; a digit may end early at a word's end (width out).
+// Bits [off, off + wd) of a key, counted from the top of word 0 in comparison
+// order, within one word.
 template <int W>
-__device__ __forceinline__ uint32_t key_digit(const PKey<W>& k, int off, int* width) {
+__device__ __forceinline__ uint32_t key_digit(const PKey<W>& k, int off, int wd) {
     const int w = off >> 6, in = off & 63;
-    const int wd = 64 - in < kDigit ? 64 - in : kDigit;
-    *width = wd;
     uint64_t word = 0;
 #pragma unroll
     for (int j = 0; j < 2 * W; ++j) if (j == w) word = j < W ? k.x[j] : k.z[j - W];
@@ -233,32 +285,56 @@ __device__ __forceinline__ uint32_t key_digit(const PKey<W>& k, int off, int* wi
 }
 
 // prefix, top: the bits of v from `top` up already agree with prefix.  Every
-// thread calls it; *tk receives the largest kept key at the threshold.
-// ties/tie_cap: global scratch for a long list of equal values.
+// thread calls it; *tk receives the largest kept key at the threshold when
+// some of its ties are dropped.  ties: global scratch for a long list of equal
+// values.  What bounds it is latency, a pass over a few thousand candidates
+// being about a microsecond: so the values are read once (up to 4,096 stay in
+// registers), a digit usually leaves few enough to rank by counting, and keys
+// are read for ties alone.
 template <int W>
 __device__ SelOut select_list(const unsigned long long* gv, const uint32_t* gidx, uint64_t n,
                               uint64_t k, unsigned long long prefix, unsigned long long mask,
                               int top, const PKey<W>* keys, PKey<W>* ties, PKey<W>* tk,
                               DevCtl* ctl) {
-    // scratch, behind one another in the staging memory
-    uint32_t* h = reinterpret_cast<uint32_t*>(g_stage);                     // kBins
-    unsigned long long* fv = reinterpret_cast<unsigned long long*>(h + kBins);
-    PKey<W>* fk = reinterpret_cast<PKey<W>*>(fv + kFinal);
+    constexpr int kReg = (int)kOneCta / kBlock;
+    constexpr uint32_t kTieMax = 512 / W;   // keys held in shared memory
+    uint32_t* h = reinterpret_cast<uint32_t*>(g_stage + InPass<W>::kBytes);                     // kBins
+    PKey<W>* sk = reinterpret_cast<PKey<W>*>(h + kBins);                    // kTieMax
+    unsigned long long* fv = reinterpret_cast<unsigned long long*>(sk);     // kFinal
+    uint32_t* fi = reinterpret_cast<uint32_t*>(fv + kFinal);
+    PKey<W>* fk = reinterpret_cast<PKey<W>*>(fi + kFinal);
+    static_assert(kBins * 4 + kTieMax * sizeof(PKey<W>) <= kScratch, "scratch");
+    static_assert(kFinal * (12 + sizeof(PKey<W>)) <= kTieMax * sizeof(PKey<W>), "scratch");
     __shared__ uint32_t s_w[kBlock / 32], s_n, s_gt, s_eq;
     __shared__ PickOut s_pick;
-    __shared__ SelOut s_out;
+    __shared__ unsigned long long s_T;
     __shared__ uint64_t s_tk[4];
     const uint32_t lane = threadIdx.x & 31u;
+    const unsigned int lt = (1u << lane) - 1u;
+    const bool held = n <= (uint64_t)(kReg * kBlock);
+    unsigned long long rv[kReg];
+#pragma unroll
+    for (int u = 0; u < kReg; ++u) {
+        const uint32_t j = u * kBlock + threadIdx.x;
+        rv[u] = held && j < n ? __ldcg(gv + j) : ~prefix;
+    }
     uint64_t cnt = n;          // entries that match the prefix
     uint32_t rank = (uint32_t)k;
     while (cnt > kFinal && top > 0) {
         const int shift = top > kDigit ? top - kDigit : 0;
+        const uint32_t dmask = (1u << (top - shift)) - 1u;
         for (int b = threadIdx.x; b < kBins; b += kBlock) h[b] = 0u;
         __syncthreads();
-        const uint32_t dmask = (1u << (top - shift)) - 1u;
-        for (uint64_t j = threadIdx.x; j < n; j += kBlock) {
-            const unsigned long long v = __ldcg(gv + j);
-            if ((v & mask) == prefix) atomicAdd(&h[(uint32_t)(v >> shift) & dmask], 1u);
+        if (held) {
+#pragma unroll
+            for (int u = 0; u < kReg; ++u)
+                if (u * kBlock + threadIdx.x < n && (rv[u] & mask) == prefix)
+                    atomicAdd(&h[(uint32_t)(rv[u] >> shift) & dmask], 1u);
+        } else {
+            for (uint64_t j = threadIdx.x; j < n; j += kBlock) {
+                const unsigned long long v = __ldcg(gv + j);
+                if ((v & mask) == prefix) atomicAdd(&h[(uint32_t)(v >> shift) & dmask], 1u);
+            }
         }
         __syncthreads();
         pick_bin<true>(h, rank, s_w, &s_pick);
@@ -269,35 +345,116 @@ __device__ SelOut select_list(const unsigned long long* gv, const uint32_t* gidx
         top = shift;
         __syncthreads();
     }
-    // a long list of exact ties: by key digits, from a list of their keys
-    bool by_key = false;
-    int off = 0;
-    uint64_t kpre[2 * W];   // key bits fixed so far
+    SelOut o;
+    o.v = prefix;
+    o.all_ties = 1;
+    if (threadIdx.x == 0) s_n = s_gt = s_eq = 0u;
+    __syncthreads();
+    if (cnt > kFinal && rank == cnt) return o;   // a class of equal values, all kept
+    if (cnt <= kFinal) {
+        // the entries left: value and place
+        auto take = [&](uint64_t j, unsigned long long v) {
+            if ((v & mask) == prefix) {
+                const uint32_t q = atomicAdd(&s_n, 1u);
+                if (q < kFinal) {
+                    fv[q] = v;
+                    fi[q] = (uint32_t)j;
+                }
+            }
+        };
+        if (held) {
 #pragma unroll
-    for (int w = 0; w < 2 * W; ++w) kpre[w] = 0;
-    uint64_t n_tie = 0;
-    if (cnt > kFinal) {
-        if (rank == cnt) {   // every one of them is kept
-            SelOut o;
-            o.v = prefix;
-            o.all_ties = 1;
+            for (int u = 0; u < kReg; ++u)
+                if (u * kBlock + threadIdx.x < n) take(u * kBlock + threadIdx.x, rv[u]);
+        } else {
+            for (uint64_t j = threadIdx.x; j < n; j += kBlock) take(j, __ldcg(gv + j));
+        }
+        __syncthreads();
+        const uint32_t m = s_n;
+        if (m > kFinal || rank < 1u || rank > m) {   // uniform; the list agrees with the counts
+            if (threadIdx.x == 0) set_status(ctl, ST_STATE, 61);
+            __syncthreads();
             return o;
         }
-        by_key = true;
-        n_tie = cnt;
-        if (threadIdx.x == 0) s_n = 0u;
-        __syncthreads();
-        for (uint64_t j0 = threadIdx.x & ~31u; j0 < n; j0 += kBlock) {
-            const uint64_t j = j0 + lane;
-            const bool hit = j < n && (__ldcg(gv + j) & mask) == prefix;
-            const unsigned int m = __ballot_sync(0xffffffffu, hit);
-            if (!m) continue;
-            uint32_t q = 0;
-            if (lane == 0) q = atomicAdd(&s_n, (uint32_t)__popc(m));
-            q = __shfl_sync(0xffffffffu, q, 0) + __popc(m & ((1u << lane) - 1u));
-            if (hit) ties[q] = load_key_stream(keys + __ldcg(gidx + j));
+        uint32_t gt = 0, eq = 0;
+        unsigned long long v = 0;
+        if (threadIdx.x < m) {
+            v = fv[threadIdx.x];
+#pragma unroll 4
+            for (uint32_t j = 0; j < m; ++j) {
+                const unsigned long long u = fv[j];
+                gt += u > v ? 1u : 0u;
+                eq += u == v ? 1u : 0u;
+            }
+            if (gt < rank && rank <= gt + eq) {   // the same values from every tie
+                s_T = v;
+                s_gt = gt;
+                s_eq = eq;
+            }
         }
         __syncthreads();
+        const uint32_t need = rank - s_gt, ne = s_eq;
+        o.v = s_T;
+        o.all_ties = need == ne;
+        if (o.all_ties) {
+            __syncthreads();
+            return o;
+        }
+        // some ties are dropped: the need-th smallest key among them
+        if (threadIdx.x == 0) s_n = 0u;
+        __syncthreads();
+        if (threadIdx.x < m && v == o.v) {
+            const PKey<W> key = load_key_stream(keys + __ldcg(gidx + fi[threadIdx.x]));
+            fk[atomicAdd(&s_n, 1u)] = key;
+        }
+        __syncthreads();
+        if (threadIdx.x < ne) {
+            const PKey<W> key = fk[threadIdx.x];
+            uint32_t before = 0;
+            for (uint32_t j = 0; j < ne; ++j) before += key_less(fk[j], key) ? 1u : 0u;
+            if (before == need - 1u) {
+#pragma unroll
+                for (int w = 0; w < W; ++w) {
+                    s_tk[w] = key.x[w];
+                    s_tk[W + w] = key.z[w];
+                }
+            }
+        }
+    } else {
+        // a long class of equal values of which some are dropped: the rank-th
+        // smallest key, by key digits over a list of the keys (in shared
+        // memory when it fits)
+        o.all_ties = 0;
+        const uint32_t nt = (uint32_t)cnt;
+        const bool local = nt <= kTieMax;
+        auto put = [&](uint64_t j, bool hit) {   // whole warps
+            const unsigned int m = __ballot_sync(0xffffffffu, hit);
+            if (!m) return;
+            uint32_t q = 0;
+            if (lane == 0) q = atomicAdd(&s_n, (uint32_t)__popc(m));
+            q = __shfl_sync(0xffffffffu, q, 0) + __popc(m & lt);
+            if (hit && q < nt) {
+                const PKey<W> key = load_key_stream(keys + __ldcg(gidx + j));
+                if (local) sk[q] = key;
+                else ties[q] = key;
+            }
+        };
+        if (held) {
+#pragma unroll
+            for (int u = 0; u < kReg; ++u) {
+                const uint32_t j = u * kBlock + threadIdx.x;
+                put(j, j < n && (rv[u] & mask) == prefix);
+            }
+        } else {
+            for (uint64_t j0 = threadIdx.x & ~31u; j0 < n; j0 += kBlock)
+                put(j0 + lane, j0 + lane < n && (__ldcg(gv + j0 + lane) & mask) == prefix);
+        }
+        __syncthreads();
+        const PKey<W>* list = local ? sk : ties;
+        uint64_t kpre[2 * W];   // key bits fixed so far
+#pragma unroll
+        for (int w = 0; w < 2 * W; ++w) kpre[w] = 0;
+        int off = 0;
         auto matches = [&](const PKey<W>& key) {
             const int full = off >> 6, r = off & 63;
             bool ok = true;
@@ -309,18 +466,14 @@ __device__ SelOut select_list(const unsigned long long* gv, const uint32_t* gidx
             }
             return ok;
         };
-        while (cnt > kFinal && off < 128 * W) {
+        uint32_t left = nt;
+        while (left > 1u && off < 128 * W) {
             for (int b = threadIdx.x; b < kBins; b += kBlock) h[b] = 0u;
             __syncthreads();
-            int wd = kDigit;
-            for (uint64_t j = threadIdx.x; j < n_tie; j += kBlock) {
-                const PKey<W> key = load_key_stream(ties + j);
-                const uint32_t d = key_digit(key, off, &wd);
-                if (matches(key)) atomicAdd(&h[d], 1u);
-            }
-            {   // the digit's width, also for threads that saw no key
-                const PKey<W> z{};
-                key_digit(z, off, &wd);
+            int wd = 64 - (off & 63) < kDigit ? 64 - (off & 63) : kDigit;
+            for (uint32_t j = threadIdx.x; j < nt; j += kBlock) {
+                const PKey<W> key = list[j];
+                if (matches(key)) atomicAdd(&h[key_digit(key, off, wd)], 1u);
             }
             __syncthreads();
             pick_bin<false>(h, rank, s_w, &s_pick);
@@ -329,79 +482,23 @@ __device__ SelOut select_list(const unsigned long long* gv, const uint32_t* gidx
             for (int v = 0; v < 2 * W; ++v)
                 if (v == w) kpre[v] |= (uint64_t)s_pick.digit << (64 - in - wd);
             rank = s_pick.k_in;
-            cnt = s_pick.count;
+            left = s_pick.count;
             off += wd;
             __syncthreads();
         }
-        // the strings that remain (distinct keys: at most kFinal)
-        if (threadIdx.x == 0) s_n = 0u;
-        __syncthreads();
-        for (uint64_t j = threadIdx.x; j < n_tie; j += kBlock) {
-            const PKey<W> key = load_key_stream(ties + j);
+        // the one key that matches (keys are distinct)
+        for (uint32_t j = threadIdx.x; j < nt; j += kBlock) {
+            const PKey<W> key = list[j];
             if (matches(key)) {
-                const uint32_t q = atomicAdd(&s_n, 1u);
-                if (q < kFinal) {
-                    fk[q] = key;
-                    fv[q] = prefix;
-                }
-            }
-        }
-    } else {
-        if (threadIdx.x == 0) s_n = 0u;
-        __syncthreads();
-        for (uint64_t j = threadIdx.x; j < n; j += kBlock) {
-            const unsigned long long v = __ldcg(gv + j);
-            if ((v & mask) == prefix) {
-                const uint32_t q = atomicAdd(&s_n, 1u);
-                if (q < kFinal) {
-                    fv[q] = v;
-                    fk[q] = load_key_stream(keys + __ldcg(gidx + j));
+#pragma unroll
+                for (int w = 0; w < W; ++w) {
+                    s_tk[w] = key.x[w];
+                    s_tk[W + w] = key.z[w];
                 }
             }
         }
     }
-    if (threadIdx.x == 0) s_gt = s_eq = 0u;
     __syncthreads();
-    const uint32_t m = s_n;
-    if (m > kFinal || rank < 1u || rank > m) {   // uniform; the lists always agree with the counts
-        if (threadIdx.x == 0) set_status(ctl, ST_STATE, 61);
-        __syncthreads();
-        SelOut o;
-        o.v = prefix;
-        o.all_ties = 1;
-        return o;
-    }
-    // one string per thread: how many come before it
-    bool mine = false;
-    unsigned long long v = 0;
-    if (threadIdx.x < m) {
-        v = fv[threadIdx.x];
-        const PKey<W> key = fk[threadIdx.x];
-        uint32_t before = 0;
-        for (uint32_t j = 0; j < m; ++j) {
-            const unsigned long long u = fv[j];
-            if (u > v) ++before;
-            else if (u == v && key_less(fk[j], key)) ++before;
-        }
-        mine = before == rank - 1u;
-        if (mine) {
-            s_out.v = v;
-            for (int w = 0; w < W; ++w) {
-                s_tk[w] = key.x[w];
-                s_tk[W + w] = key.z[w];
-            }
-        }
-    }
-    __syncthreads();
-    if (threadIdx.x < m) {
-        if (v > s_out.v) atomicAdd(&s_gt, 1u);
-        if (v == s_out.v) atomicAdd(&s_eq, 1u);
-    }
-    __syncthreads();
-    SelOut o;
-    o.v = s_out.v;
-    // by_key: the strings outside the final set also tie, and some are dropped
-    o.all_ties = !by_key && rank - s_gt == s_eq;
 #pragma unroll
     for (int w = 0; w < W; ++w) { tk->x[w] = s_tk[w]; tk->z[w] = s_tk[W + w]; }
     __syncthreads();
@@ -411,32 +508,34 @@ __device__ SelOut select_list(const unsigned long long* gv, const uint32_t* gidx
 // ---------------------------------------------------------------------------
 // The run
 // ---------------------------------------------------------------------------
+// The prediction's state between gates (kept by the first CTA's thread 0, in
+// the control block between launches).
+struct Predict {
+    unsigned long long tprev;
+    int shift, reason;
+    unsigned long long cands, range, full;   // statistics
+};
+
 // The candidate range around the threshold predicted for the next gate: C +-
 // 2^s in pattern units, narrower when the list ran long, wider when the
 // threshold fell outside.  C is this threshold moved by what the next gate's
-// moved in the last layer, or, without that, carried into the next gate's
+// moved in the last layer (dn), or, without that, carried into the next gate's
 // scale.
-template <int W>
-__device__ void next_range(const RunArgs<W>& a, DevCtl* ctl, long long* drift, int n_drift, int k,
-                           unsigned long long T, double rnorm, int reason, uint32_t cn,
-                           unsigned long long range, Pub* p) {
-    const int gi = n_drift > 0 ? (a.gate0 + k) % n_drift : 0;
-    const int gn = n_drift > 0 ? (a.gate0 + k + 1) % n_drift : 0;
-    const unsigned long long Tp = ctl->sp_tprev;
-    if (n_drift > 0) drift[gi] = Tp ? (long long)(T - Tp) : 0LL;
-    ctl->sp_tprev = T;
-    ctl->stat_cands += cn;
-    ctl->stat_range = range;
-    int sft = ctl->sp_shift ? ctl->sp_shift : kRangeShift;
-    switch (reason) {
-        case 0: if (cn > a.cand_hi) sft -= 1; break;
+__device__ __forceinline__ void next_range(Predict* q, uint64_t cand_hi, long long* drift_now,
+                                           long long dn, unsigned long long T, double rnorm,
+                                           uint32_t cn, unsigned long long dbits, Pub* p) {
+    if (drift_now) *drift_now = q->tprev ? (long long)(T - q->tprev) : 0LL;
+    q->tprev = T;
+    q->cands += cn;
+    int sft = q->shift ? q->shift : kRangeShift;
+    switch (q->reason) {
+        case 0: if (cn > cand_hi) sft -= 1; break;
         case 1: sft = kRangeShift; break;
         case 2: sft -= 2; break;
         default: sft += 1; break;
     }
-    sft = sft < 8 ? 8 : (sft > 60 ? 60 : sft);
-    ctl->sp_shift = sft;
-    const long long dn = n_drift > 0 ? drift[gn] : 0LL;
+    sft = sft < 8 ? 8 : (sft > kRangeShiftMax ? kRangeShiftMax : sft);
+    q->shift = sft;
     unsigned long long C;
     if (dn != 0LL) {
         const long long c = (long long)T + dn;
@@ -444,9 +543,10 @@ __device__ void next_range(const RunArgs<W>& a, DevCtl* ctl, long long* drift, i
     } else {
         C = abs_pattern(__dmul_rn(__longlong_as_double((long long)T), rnorm));
     }
-    const unsigned long long h = 1ULL << sft;
-    p->lo = C > h ? C - h : 0ULL;
-    p->hi = C + h;
+    const SelRange r = sel_range(C, sft, dbits);
+    p->thr = r.thr;
+    p->lo = r.thr + 1ULL;
+    p->hi = r.hi;
 }
 
 template <int W>
@@ -461,8 +561,10 @@ __device__ __forceinline__ GateArg<W> gate_arg_of(const RunGate<W>& r, int maxw)
     return g;
 }
 
+// The partition function of the window of level `lv` that starts at a gate,
+// or of its pair key (lv < 0).
 template <int W>
-__device__ __forceinline__ PartFn<W> part_fn_of(const RunGate<W>& r) {
+__device__ __forceinline__ PartFn<W> part_fn_of(const RunGate<W>& r, int lv) {
     PartFn<W> f;
     bool found = false;
 #pragma unroll
@@ -473,11 +575,20 @@ __device__ __forceinline__ PartFn<W> part_fn_of(const RunGate<W>& r) {
         found = found || m;
     }
 #pragma unroll
-    for (int w = 0; w < W; ++w) { f.kx[w] = ~r.win[w]; f.kz[w] = ~r.win[w]; }
-    f.pair = r.pair;
-    f.sites = r.sites;
+    for (int w = 0; w < W; ++w) {
+        const uint64_t win = lv < 0 ? 0ULL : (lv ? r.win[1][w] : r.win[0][w]);
+        f.kx[w] = ~win;
+        f.kz[w] = ~win;
+    }
+    f.pair = lv < 0;
+    f.sites = lv < 0 ? 0 : (lv ? r.sites[1] : r.sites[0]);
     return f;
 }
+
+// Cursors lie a line apart: a scatter makes an atomic per term, and those on
+// one line follow one another (20 us against 5 us for 2^18 terms into 608
+// partitions with packed cursors).
+constexpr uint32_t kPad = kRunPad;
 
 // The instance's arrays (by compare-select: a dynamic index into an array of
 // pointers would put it in local memory).
@@ -485,23 +596,32 @@ template <int W>
 struct Arrays {
     PKey<W>*k0, *k1, *kp;
     double *c0, *c1, *cp;
-    unsigned int *n0, *n1;
-    int a;   // the contiguous state's buffer at the start
+    unsigned int* n0;   // three cursor arrays of `pm` entries, kPad apart
+    uint32_t pm;
+    int a;              // the contiguous state's buffer at the start
     __device__ __forceinline__ PKey<W>* run_keys(int b) const { return b ? k1 : k0; }
     __device__ __forceinline__ double* run_coef(int b) const { return b ? c1 : c0; }
     __device__ __forceinline__ PKey<W>* home(int h) const { return h ? run_keys(a ^ 1) : kp; }
     __device__ __forceinline__ double* coef(int x) const { return x ? run_coef(a ^ 1) : cp; }
-    __device__ __forceinline__ unsigned int* cnt(int p) const { return p ? n1 : n0; }
+    __device__ __forceinline__ unsigned int* cnt(int p) const { return n0 + (uint64_t)p * pm * kPad; }
 };
 
+// Which window a scatter at this gate prepares: the long one (level 0) while
+// the groups, the strings with one pattern outside it, are small (as the
+// separate scatter decides it), else the three-site one (level 1), whose
+// groups of at most 64 strings balance over partitions whatever the state,
+// if there are a few groups to a partition; else the gate's pair key (-1).  A
+// single partition holds any window.
 template <int W>
-__device__ __forceinline__ void read_pub(const RunShared* rs, Pub* s_pub) {
-    static_assert(sizeof(Pub) % 8 == 0, "words");
-    constexpr int N = sizeof(Pub) / 8;
-    if (threadIdx.x < N)
-        reinterpret_cast<unsigned long long*>(s_pub)[threadIdx.x] =
-            __ldcg(reinterpret_cast<const unsigned long long*>(&rs->pub) + threadIdx.x);
-    __syncthreads();
+__device__ __forceinline__ int window_level(const RunGate<W>& r, int n_sites, uint64_t n,
+                                            uint64_t parts) {
+    if (r.len[0] > 0 && (parts == 1 || window_fits(n_sites, r.sites[0], n))) return 0;
+    if (r.len[1] > 0) {
+        const int free_bits = 2 * (n_sites - r.sites[1]);
+        if (free_bits >= 40 || (1ULL << (free_bits < 0 ? 0 : free_bits)) >= 4ULL * parts)
+            return 1;
+    }
+    return -1;
 }
 
 // Run gates [0, n_gates) n_layers times on one instance.  Returns false when
@@ -509,9 +629,9 @@ __device__ __forceinline__ void read_pub(const RunShared* rs, Pub* s_pub) {
 template <int W>
 __device__ bool run_instance(const RunArgs<W>& a, const RunGate<W>* gates, int n_gates, int inst,
                              Team& team) {
-    using A = InStage<W>;
+    using A = InPass<W>;
     constexpr uint32_t C = A::C;
-    __shared__ Pub s_pub;
+    __shared__ Pub s_pub, s_next;
     // raw storage: a shared variable gets no constructor, and GateArg has a
     // default member initialiser
     __shared__ __align__(16) unsigned char s_g_raw[sizeof(GateArg<W>)];
@@ -519,11 +639,19 @@ __device__ bool run_instance(const RunArgs<W>& a, const RunGate<W>* gates, int n
     __shared__ PartFn<W> s_f;
     __shared__ unsigned long long s_cv[kPushBuf];
     __shared__ uint32_t s_ci[kPushBuf];
-    __shared__ uint32_t s_cn, s_cs, s_app, s_n, s_base32;
+    __shared__ uint32_t s_cn, s_cs, s_app, s_rare, s_n;
     __shared__ int s_over;
-    __shared__ unsigned long long s_red[kBlock / 32], s_at;
-    __shared__ uint32_t s_kept[kBlock / 32], s_above[kBlock / 32], s_w[kBlock / 32];
-    __shared__ unsigned long long s_stat[8];   // first CTA: statistics of the run
+    __shared__ unsigned long long s_at;
+    __shared__ uint32_t s_red[kBlock / 32], s_kept[kBlock / 32], s_w[kBlock / 32];
+    // first CTA: statistics of the run, counters of the gate
+    __shared__ unsigned long long s_stat[8];
+    __shared__ Acc s_acc;
+    __shared__ double s_norm, s_rnorm;
+    __shared__ int s_status;
+    __shared__ long long s_dn;
+    __shared__ Predict s_pred;
+    __shared__ PickOut s_pick;
+    __shared__ unsigned int s_long;
 
     DevCtl* ctl = a.ctl + inst;
     RunShared* rs = team.rs;
@@ -535,8 +663,8 @@ __device__ bool run_instance(const RunArgs<W>& a, const RunGate<W>* gates, int n
     arr.c0 = a.c[0] + (uint64_t)inst * a.buf_stride;
     arr.c1 = a.c[1] + (uint64_t)inst * a.buf_stride;
     arr.cp = a.cp + (uint64_t)inst * a.part_stride;
-    arr.n0 = a.cnt + (uint64_t)inst * 2 * a.part_max;
-    arr.n1 = arr.n0 + a.part_max;
+    arr.n0 = a.cnt + (uint64_t)inst * 3 * a.part_max * kPad;
+    arr.pm = a.part_max;
     arr.a = ctl->cur;
     // candidates and ties share the merge table's memory
     char* scr = static_cast<char*>(a.scratch) + (uint64_t)inst * a.scratch_stride;
@@ -549,42 +677,45 @@ __device__ bool run_instance(const RunArgs<W>& a, const RunGate<W>* gates, int n
 
     const PushList pl{s_cv, s_ci, &s_cn, &s_cs, cand_v, cand_i, nullptr, a.cand_cap};
 
-    // start: the published state from the control block, both cursor arrays
+    // start: the published state from the control block, the cursor arrays
     // zero, no chain head of an earlier use
     if (threadIdx.x < 8) s_stat[threadIdx.x] = 0ULL;
-    for (uint32_t i = threadIdx.x; i < (uint32_t)A::S; i += kBlock) A::heads()[i] = 0u;
-    for (uint32_t i = team.rank * kBlock + threadIdx.x; i < a.part_max; i += team.size * kBlock) {
-        arr.n0[i] = 0u;
-        arr.n1[i] = 0u;
+    inplace_init<W, kBlock>();
+    for (uint32_t i = team.rank * kBlock + threadIdx.x; i < 3u * a.part_max; i += team.size * kBlock)
+        arr.n0[(uint64_t)i * kPad] = 0u;
+    if (leader && threadIdx.x == 0) {
+        Pub& first = s_next;
+        memset(rs->acc, 0, sizeof rs->acc);
+        memset(&first, 0, sizeof first);
+        first.all_ties = 1;
+        first.lo = ctl->sp_lo;
+        first.hi = ctl->sp_hi;
+        first.thr = ctl->sp_thr > a.delta_bits ? ctl->sp_thr : a.delta_bits;
+        s_pred.tprev = ctl->sp_tprev;
+        s_pred.shift = ctl->sp_shift;
+        s_pred.reason = 1;
+        s_pred.cands = s_pred.range = s_pred.full = 0ULL;
+        first.n = live_count(ctl, arr.a);
+        first.rnorm = ctl->rnorm[arr.a];
+        first.stop = ctl->status != 0;
+        first.rescatter = 1;
     }
+    if (leader)
+        for (int b = threadIdx.x; b < 3 * kBins; b += kBlock) rs->hist[0][b] = 0u;
+    team_arrive(team);
     if (leader) {
-        for (int b = threadIdx.x; b < kBins; b += kBlock) rs->hist[b] = 0u;
-        if (threadIdx.x == 0) {
-            Pub p;
-            p.T = 0;
-            p.all_ties = 1;
-            for (int w = 0; w < 4; ++w) p.tk[w] = 0;
-            p.lo = ctl->sp_lo;
-            p.hi = ctl->sp_hi;
-            p.n = live_count(ctl, arr.a);
-            p.rnorm = ctl->rnorm[arr.a];
-            p.stop = ctl->status != 0;
-            p.full = 0;
-            p.rescatter = 1;
-            rs->pub = p;
-            memset(rs->acc, 0, sizeof rs->acc);
-        }
+        if (!team_wait(team, ctl)) return false;
+        if (threadIdx.x < 32) publish(team, &s_next);
     }
-    if (!team_barrier(team, ctl)) return false;
-    read_pub<W>(rs, &s_pub);
+    if (!take_pub(team, ctl, &s_pub)) return false;
 
     uint32_t tag = 0, pass = 0;
-    int layout = 0, hb = 0, cx = 0, par = 0, run_buf = arr.a;
+    int layout = 0, hb = 0, cx = 0, ci = 0, run_buf = arr.a;
     bool any = false;                   // a gate ran
-    uint64_t run_n = s_pub.n;           // terms stored there
+    uint64_t run_n = s_pub.n;           // terms stored in the contiguous run
     uint32_t P = 0;
-    uint64_t R = 0;
-    bool over_one = false;              // the partitions hold for one gate only
+    uint64_t R = 0, n_scat = 0;         // stride; terms at the last scatter
+    int win_end = 0;                    // the partitions hold for the gates before this one
     const int total = n_gates * a.n_layers;
     for (int gi = 0; gi < total; ++gi) {
         const int k = gi % n_gates;
@@ -592,7 +723,6 @@ __device__ bool run_instance(const RunArgs<W>& a, const RunGate<W>* gates, int n
         if (s_pub.stop) break;          // uniform over the team
         if (threadIdx.x == 0) {
             s_g = gate_arg_of<W>(gates[k], a.maxw);
-            s_f = part_fn_of<W>(gates[k]);
             s_cn = s_cs = 0u;
             s_over = 0;
         }
@@ -604,186 +734,129 @@ __device__ bool run_instance(const RunArgs<W>& a, const RunGate<W>* gates, int n
         __syncthreads();
         Acc* acc = &rs->acc[np_][0];
         // ---- scatter ----------------------------------------------------
-        if (gi == 0 || layout == 0 || over_one || gates[k].start || s_pub.rescatter) {
-            bool pair = s_f.pair || !window_fits(sites, s_f.sites, n_in);
-            for (int tries = 0; tries < 2; ++tries) {
-                // at least a partition for every CTA of the team, of no fewer
-                // than kMinPart terms, so that a small state uses the chip
-                uint64_t want = (n_in + a.target - 1) / a.target;
-                const uint64_t most = (n_in + a.min_part - 1) / a.min_part;
-                const uint64_t wide = most < team.size ? most : team.size;
-                if (want < wide) want = wide;
-                if (want < 1) want = 1;
-                if (want > a.part_max) want = a.part_max;
-                if (!pair) {   // a stride holds a whole group (up to 4^sites strings)
-                    const uint64_t gmax = 1ULL << (2 * s_f.sites);
-                    if (a.home_cap / want < gmax) want = a.home_cap / gmax > 0 ? a.home_cap / gmax : 1;
-                }
-                P = (uint32_t)want;
-                R = a.home_cap / P;
-                PartPlan plan;
-                plan.P = P;
-                plan.R = R;
+        if (layout == 0 || gi >= win_end || s_pub.rescatter) {
+            // at least a partition for every CTA of the team, of no fewer
+            // than min_part terms, so that a small state uses the chip
+            uint64_t want = (n_in + a.target - 1) / a.target;
+            const uint64_t most = (n_in + a.min_part - 1) / a.min_part;
+            const uint64_t wide = most < team.size ? most : team.size;
+            if (want < wide) want = wide;
+            if (want < 1) want = 1;
+            if (want > a.part_max) want = a.part_max;
+            const int lv0 = window_level<W>(gates[k], sites, n_in, want);
+            for (int lv = lv0;; lv = -1) {
+                if (threadIdx.x == 0) s_f = part_fn_of<W>(gates[k], lv);
+                __syncthreads();
                 PartFn<W> f = s_f;
-                f.pair = pair ? 1 : 0;
+                uint64_t np = want;
+                if (lv >= 0) {   // a stride holds a whole group (up to 4^sites strings)
+                    const uint64_t gmax = 1ULL << (2 * f.sites);
+                    if (a.home_cap / np < gmax) np = a.home_cap / gmax > 0 ? a.home_cap / gmax : 1;
+                }
+                const uint32_t oldP = P;
+                const uint64_t oldR = R;
+                PartPlan plan;
+                plan.P = (uint32_t)np;
+                plan.R = a.home_cap / np;
                 Pending<W> pd;
                 pd.on = s_pub.T != 0ULL;
                 pd.all_ties = s_pub.all_ties != 0;
                 pd.T = s_pub.T;
                 pd.tk = tk;
                 const int dh = layout == 0 ? 0 : hb ^ 1, dx = layout == 0 ? 0 : cx ^ 1;
+                const int dc = next3(ci);
                 int* over = reinterpret_cast<int*>(&acc->scatter_over);
                 if (layout == 0) {
                     scatter_run<W>(arr.run_keys(run_buf), arr.run_coef(run_buf), run_n,
                                    (uint64_t)team.rank * kBlock, (uint64_t)team.size * kBlock, pd,
-                                   ctl, arr.home(dh), arr.coef(dx), arr.cnt(par ^ 1), plan, g, f,
-                                   over);
+                                   ctl, arr.home(dh), arr.coef(dx), arr.cnt(dc), plan, g, f, over, kPad);
                 } else {
-                    const uint32_t oldP = s_base32;
-                    const uint64_t oldR = a.home_cap / oldP;
                     for (uint32_t p = team.rank; p < oldP; p += team.size) {
-                        const uint64_t c = __ldcg(arr.cnt(par) + p);
+                        const uint64_t c = __ldcg(arr.cnt(ci) + (uint64_t)p * kPad);
                         scatter_run<W>(arr.home(hb) + p * oldR, arr.coef(cx) + p * oldR, c, 0,
-                                       kBlock, pd, ctl, arr.home(dh), arr.coef(dx),
-                                       arr.cnt(par ^ 1), plan, g, f, over);
+                                       kBlock, pd, ctl, arr.home(dh), arr.coef(dx), arr.cnt(dc),
+                                       plan, g, f, over, kPad);
                     }
                 }
                 if (!team_barrier(team, ctl)) return false;
                 if (leader && threadIdx.x == 0) s_stat[4] += 1;
-                if (pair || !__ldcg(&acc->scatter_over)) {
+                if (lv < 0 || !__ldcg(&acc->scatter_over)) {
                     hb = dh;
                     cx = dx;
-                    par ^= 1;
+                    ci = dc;
                     layout = 1;
+                    P = plan.P;
+                    R = plan.R;
+                    n_scat = n_in;
+                    win_end = gi + (lv < 0 ? 1 : (lv ? gates[k].len[1] : gates[k].len[0]));
                     break;
                 }
                 // a window group passed a stride: again, by the pair key
                 for (uint32_t i = team.rank * kBlock + threadIdx.x; i < a.part_max;
                      i += team.size * kBlock)
-                    arr.cnt(par ^ 1)[i] = 0u;
-                pair = true;
+                    arr.cnt(dc)[(uint64_t)i * kPad] = 0u;
                 if (!team_barrier(team, ctl)) return false;
             }
-            over_one = pair;
-            if (threadIdx.x == 0) s_base32 = P;
-            __syncthreads();
         }
         // ---- merge, in place --------------------------------------------
         const unsigned long long dbits = a.delta_bits;
-        const bool drop = s_pub.hi != 0ULL && s_pub.lo > 0ULL && s_pub.lo - 1ULL > dbits;
-        const unsigned long long thr = drop ? s_pub.lo - 1ULL : dbits;
+        const unsigned long long thr = s_pub.thr;
+        const bool drop = thr > dbits;
         const uint32_t p_id = identity_part<W>(P);
         PushList push_to = pl;
         push_to.gn = &acc->cand_n;
         auto push = [&](bool hit, unsigned long long v, uint64_t idx) {
             push_cand(push_to, hit, v, idx);
         };
-        InStats st{0ULL, 0u, 0u};
+        InStats st{0u, 0u};
         uint32_t n_long = 0;
+        // the third cursor array (two gates back) is the next scatter's
+        for (uint32_t i = team.rank * kBlock + threadIdx.x; i < a.part_max; i += team.size * kBlock)
+            arr.cnt(next3(next3(ci)))[(uint64_t)i * kPad] = 0u;
         for (uint32_t p = team.rank; p < P; p += team.size) {
-            const uint32_t np = __ldcg(arr.cnt(par) + p);
+            const uint32_t np = __ldcg(arr.cnt(ci) + (uint64_t)p * kPad);
             InPlace<W> io;
             io.first = (uint64_t)p * R;
             io.keys = arr.home(hb) + io.first;
+            io.cin = arr.coef(cx) + io.first;
             io.cout = arr.coef(cx ^ 1) + io.first;
             io.n = np < R ? np : (uint32_t)R;
             io.room = (uint32_t)(R < 0xffffffffULL ? R : 0xffffffffULL);
             io.s_app = &s_app;
+            io.s_rare = &s_rare;
             io.over = &s_over;
-            const double* cin = arr.coef(cx) + io.first;
-            if (threadIdx.x == 0) s_app = 0u;
-            if (io.n <= C) {
-                // stage: all loads of a thread before its stores
-                constexpr int U = (int)(C / kBlock);
-                PKey<W> kk[U];
-                double cc[U];
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const uint32_t i = u * kBlock + threadIdx.x;
-                    if (i < io.n) {
-                        kk[u] = load_key_stream(io.keys + i);
-                        cc[u] = __ldcs(cin + i);
-                    }
-                }
-                if (threadIdx.x < C / 32) A::dup()[threadIdx.x] = 0u;
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const uint32_t i = u * kBlock + threadIdx.x;
-                    if (i < io.n) {
-                        A::keys()[i] = kk[u];
-                        A::vals()[i] = cc[u];
-                    }
-                }
-                __syncthreads();
-                inplace_pass<W, kBlock, false>(io.n, 0u, g, s_pub.T, s_pub.all_ties != 0, tk,
-                                               s_pub.rnorm, thr, p == p_id, ctl, np_, ++tag, io, st,
-                                               s_pub.lo, s_pub.hi, push);
-            } else if (io.n <= 0xffffu) {
-                // a partition above the staging capacity: its hash classes one
-                // after another, each gathered with the strings' indices
-                const uint32_t kc = (2u * io.n + C - 1u) / C;
+            if (threadIdx.x == 0) s_app = s_rare = 0u;
+            __syncthreads();
+            if (inplace_partition<W, kBlock>(g, s_pub.T, s_pub.all_ties != 0, tk, s_pub.rnorm, thr,
+                                             p == p_id, ctl, np_, &tag, io, st, s_pub.hi, &s_n, push))
                 ++n_long;
-                for (uint32_t j = 0; j < kc; ++j) {
-                    if (threadIdx.x == 0) s_n = 0u;
-                    if (threadIdx.x < C / 32) A::dup()[threadIdx.x] = 0u;
-                    __syncthreads();
-                    for (uint32_t i = threadIdx.x; i < io.n; i += kBlock) {
-                        const PKey<W> K = load_key_stream(io.keys + i);
-                        if (sub_pass(K, g, kc) != j) continue;
-                        const uint32_t q = atomicAdd(&s_n, 1u);
-                        if (q < C) {
-                            A::keys()[q] = K;
-                            A::vals()[q] = __ldcs(cin + i);
-                            A::src()[q] = (uint16_t)i;
-                        } else {
-                            s_over = 1;   // the merge is done again
-                        }
-                    }
-                    __syncthreads();
-                    const uint32_t m = s_n < C ? s_n : C;
-                    inplace_pass<W, kBlock, true>(m, 0u, g, s_pub.T, s_pub.all_ties != 0, tk,
-                                                  s_pub.rnorm, thr, p == p_id, ctl, np_, ++tag, io,
-                                                  st, s_pub.lo, s_pub.hi, push);
-                }
-            } else {
-                if (threadIdx.x == 0) s_over = 1;
-                __syncthreads();
-            }
             if (threadIdx.x == 0) {
                 const uint64_t c = (uint64_t)io.n + s_app;
-                arr.cnt(par ^ 1)[p] = (unsigned int)(c < R ? c : R);
+                arr.cnt(next3(ci))[(uint64_t)p * kPad] = (unsigned int)(c < R ? c : R);
             }
             if (tag >= kHeadTagMax - 65536u) {   // tags start again
-                __syncthreads();
-                for (uint32_t i = threadIdx.x; i < (uint32_t)A::S; i += kBlock) A::heads()[i] = 0u;
+                inplace_init<W, kBlock>();
                 tag = 0;
             }
             __syncthreads();
         }
         // the CTA's counts and candidates
-        auto flush = [&](Acc* to, InStats& s) {
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                s.out_max = max(s.out_max, __shfl_xor_sync(0xffffffffu, s.out_max, o));
-                s.above += __shfl_xor_sync(0xffffffffu, s.above, o);
-                s.kept += __shfl_xor_sync(0xffffffffu, s.kept, o);
-            }
+        auto flush = [&](Acc* to, const InStats& s) {
+            const uint32_t hm = __reduce_max_sync(0xffffffffu, s.hi_max);
+            const uint32_t kw = __reduce_add_sync(0xffffffffu, s.kept);
             if ((threadIdx.x & 31) == 0) {
-                s_red[threadIdx.x >> 5] = s.out_max;
-                s_kept[threadIdx.x >> 5] = s.kept;
-                s_above[threadIdx.x >> 5] = s.above;
+                s_red[threadIdx.x >> 5] = hm;
+                s_kept[threadIdx.x >> 5] = kw;
             }
             __syncthreads();
             if (threadIdx.x == 0) {
-                unsigned long long mx = 0, kept = 0, above = 0;
+                uint32_t mx = 0, kept = 0;
                 for (int w = 0; w < kBlock / 32; ++w) {
                     mx = max(mx, s_red[w]);
                     kept += s_kept[w];
-                    above += s_above[w];
                 }
-                if (mx) atomicMax(&to->out_max, mx);
-                if (kept) atomicAdd(&to->kept, kept);
-                if (above) atomicAdd(&to->above, above);
+                if (mx) atomicMax(&to->out_max, ((unsigned long long)mx << 32) | 0xffffffffULL);
+                if (kept) atomicAdd(&to->kept, (unsigned long long)kept);
                 if (s_over) atomicExch(&to->over, 1u);
                 if (n_long) atomicAdd(&to->n_long, n_long);
                 s_n = s_cs ? atomicAdd(&to->cand_n, s_cs) : 0u;
@@ -796,13 +869,128 @@ __device__ bool run_instance(const RunArgs<W>& a, const RunGate<W>* gates, int n
                     cand_i[b + j] = s_ci[j];
                 }
         };
+        // how this gate's and the next gate's thresholds moved in the last layer
+        long long* drift_now = n_drift > 0 ? drift + (a.gate0 + k) % n_drift : nullptr;
+        const long long* drift_next = n_drift > 0 ? drift + (a.gate0 + k + 1) % n_drift : nullptr;
+        // the first CTA, once every CTA has arrived (s_acc read): statistics,
+        // normaliser, bound, threshold; published for all
+        auto lead_gate = [&](bool redone) {
+            const unsigned long long kept = redone ? s_acc.alloc : s_acc.kept;
+            const bool active = a.cap_policy == 1 && kept > a.cap_M;
+            const unsigned long long lo = s_pub.lo, hi = s_pub.hi;
+            const uint32_t cn = redone ? 0u : s_acc.cand_n;
+            // kept children above the range: all that were not listed
+            const unsigned long long above = kept - cn, omax = s_acc.out_max;
+            // why not the listed candidates: 1 no range, 2 list too long,
+            // 3 threshold above the range, 4 below it
+            const int reason = hi == 0ULL ? 1 : redone ? 4 : cn > a.cand_cap ? 2
+                               : above >= a.cap_M ? 3 : above + cn < a.cap_M ? 4 : 0;
+            const int failed = s_status;
+            SelOut so{0ULL, 1};
+            PKey<W> key{};
+            const bool listed = active && reason == 0 && !failed;
+            // a long list is first cut down by the whole team
+            const bool fast = listed && (cn <= kOneCta || cn > a.cand_cap / 4);
+            if (fast)
+                so = select_list<W>(cand_v, cand_i, cn, a.cap_M - above, 0ULL, 0ULL,
+                                    hi > lo ? 64 - __clzll((long long)(hi - lo)) : 0,
+                                    arr.home(hb), ties, &key, ctl);
+            if (threadIdx.x == 0) {
+                constexpr unsigned long long kInfBits = 0x7ff0000000000000ULL;
+                if (omax >= kInfBits) set_status(ctl, ST_STATE, 4);
+                if (abs_pattern(s_norm) >= kInfBits) set_status(ctl, ST_STATE, 5);
+                if (a.cap_policy == 0 && kept > a.cap_M) set_status(ctl, ST_CAPACITY, 1);
+                Pub& p = s_next;
+                p.rnorm = s_rnorm;
+                p.n = active ? a.cap_M : kept;
+                p.T = fast ? so.v + lo : 0ULL;
+                p.all_ties = fast ? so.all_ties : 1;
+#pragma unroll
+                for (int w = 0; w < 4; ++w) p.tk[w] = 0;
+                if (fast && !so.all_ties) {
+#pragma unroll
+                    for (int w = 0; w < W; ++w) { p.tk[w] = key.x[w]; p.tk[W + w] = key.z[w]; }
+                }
+                // 1: radix passes over the state, 2: over the candidates
+                p.full = !active || fast || failed ? 0 : listed ? 2 : 1;
+                p.base = listed ? lo : a.delta_bits;
+                p.range = listed ? hi - lo : omax > a.delta_bits ? omax - a.delta_bits : 0ULL;
+                p.rank = listed ? a.cap_M - above : a.cap_M;
+                p.redo = 0;
+                p.pad = 0;
+                p.lo = lo;
+                p.hi = hi;
+                p.thr = s_pub.thr;
+                // a state that doubled since its scatter: more partitions, before
+                // they outgrow the staging
+                p.rescatter = !redone && p.n > 2ULL * n_scat && p.n > (C / 2) * (uint64_t)P;
+                p.stop = failed || omax >= kInfBits || abs_pattern(s_norm) >= kInfBits ||
+                         (a.cap_policy == 0 && kept > a.cap_M) ||
+                         (fast && *(volatile int*)&ctl->status != 0);
+                if (a.log) a.log[gi] = p.stop ? ~0ULL : p.n;
+                s_stat[0] += 1;
+                s_stat[1] += n_in;
+                s_stat[2] += p.n;
+                if (p.n > s_stat[3]) s_stat[3] = p.n;
+                s_stat[5] += active ? 1 : 0;
+                s_stat[6] += redone ? 1 : 0;
+                s_stat[7] += s_long;
+                if (active) {
+                    s_pred.reason = reason;
+                    s_pred.range = hi - lo;
+                }
+                if (fast)
+                    next_range(&s_pred, a.cand_hi, drift_now, s_dn, p.T, p.rnorm, cn, a.delta_bits, &p);
+                s_pred.full += p.full == 1 ? 1 : 0;
+                if (p.full) rs->sel_n = 0u;
+            }
+            if (threadIdx.x < 32) publish(team, &s_next);
+        };
+        // the counters of a finished merge, one load per lane
+        auto read_acc = [&](const Acc* from, Acc* to) {
+            constexpr int N = sizeof(Acc) / 8;
+            if (threadIdx.x < N)
+                reinterpret_cast<unsigned long long*>(to)[threadIdx.x] =
+                    __ldcg(reinterpret_cast<const unsigned long long*>(from) + threadIdx.x);
+            else if (threadIdx.x == 32) {
+                s_norm = *(volatile double*)&ctl->norm[np_];
+                s_rnorm = __ddiv_rn(1.0, s_norm);
+            } else if (threadIdx.x == 64)
+                s_dn = drift_next ? *drift_next : 0LL;
+            else if (threadIdx.x == 33)
+                s_status = *(volatile int*)&ctl->status;
+            else if (threadIdx.x == 34)
+                s_long = *(volatile unsigned int*)&rs->acc[np_][0].n_long;
+            else if (threadIdx.x >= 96 && threadIdx.x < 96 + 2 * N)
+                // the next gate's counters (every CTA is done with them)
+                reinterpret_cast<unsigned long long*>(&rs->acc[np_ ^ 1][0])[threadIdx.x - 96] = 0ULL;
+            __syncthreads();
+        };
         flush(acc, st);
-        if (!team_barrier(team, ctl)) return false;
-        unsigned long long kept = __ldcg(&acc->kept);
-        bool redo = __ldcg(&acc->over) != 0u || (drop && kept < a.cap_M);
+        team_arrive(team);
+        if (leader) {
+            if (!team_wait(team, ctl)) return false;
+            read_acc(acc, &s_acc);
+            // children left out that the bound may need, or a stride that had
+            // no room: the merge is done again
+            if (s_acc.over != 0u || (drop && s_acc.kept < a.cap_M)) {
+                if (threadIdx.x == 0) {
+                    s_next = s_pub;
+                    s_next.redo = 1;
+                }
+                if (threadIdx.x < 32) publish(team, &s_next);
+            } else {
+                lead_gate(false);
+            }
+        }
+        if (!take_pub(team, ctl, &s_pub)) return false;
+        const bool redo = s_pub.redo != 0;
         if (redo) {
             // again in full from the same input, into a contiguous run
             acc = &rs->acc[np_][1];
+            for (uint32_t i = team.rank * kBlock + threadIdx.x; i < a.part_max;
+                 i += team.size * kBlock)
+                arr.cnt(next3(ci))[(uint64_t)i * kPad] = 0u;   // the first try's counts
             push_to.gn = &acc->cand_n;
             if (threadIdx.x == 0) {
                 s_cn = s_cs = 0u;
@@ -836,12 +1024,12 @@ __device__ bool run_instance(const RunArgs<W>& a, const RunGate<W>* gates, int n
             SelStats ss{0ULL, 0u};
             const CandRegions none{};
             for (uint32_t p = team.rank; p < P; p += team.size) {
-                uint64_t np = __ldcg(arr.cnt(par) + p);
+                uint64_t np = __ldcg(arr.cnt(ci) + (uint64_t)p * kPad);
                 if (np > R) np = R;
                 const PKey<W>* kp = arr.home(hb) + (uint64_t)p * R;
                 const double* cp = arr.coef(cx) + (uint64_t)p * R;
-                ++pass;
                 if (np <= (uint64_t)Stage<W>::C) {
+                    ++pass;   // (merge_long numbers its own: consecutive passes alternate)
                     for (uint32_t i = threadIdx.x; i < np; i += kBlock) {
                         PassArgs<W>::keys()[i] = load_key_stream(kp + i);
                         PassArgs<W>::vals()[i] = __ldcs(cp + i);
@@ -857,191 +1045,133 @@ __device__ bool run_instance(const RunArgs<W>& a, const RunGate<W>* gates, int n
                 }
             }
             n_long = 0;
-            InStats s2{ss.out_max, 0u, 0u};
+            const InStats s2{(uint32_t)(__reduce_max_sync(0xffffffffu, (uint32_t)(ss.out_max >> 32))), 0u};
             flush(acc, s2);
-            for (uint32_t i = threadIdx.x; i < (uint32_t)A::S; i += kBlock) A::heads()[i] = 0u;
+            inplace_init<W, kBlock>();
             tag = 0;
-            if (!team_barrier(team, ctl)) return false;
-            kept = __ldcg(&acc->alloc);
+            team_arrive(team);
             layout = 0;
             run_buf = arr.a;
-            run_n = kept;
+            if (leader) {
+                if (!team_wait(team, ctl)) return false;
+                read_acc(acc, &s_acc);
+                lead_gate(true);
+            }
+            if (!take_pub(team, ctl, &s_pub)) return false;
+            run_n = __ldcg(&acc->alloc);
         } else {
             cx ^= 1;
-            par ^= 1;
+            ci = next3(ci);
         }
-        // ---- post and select --------------------------------------------
-        // the spare cursors: the next scatter's
-        for (uint32_t i = team.rank * kBlock + threadIdx.x; i < a.part_max; i += team.size * kBlock)
-            arr.cnt(par ^ 1)[i] = 0u;
-        if (layout == 0)
-            for (uint32_t i = team.rank * kBlock + threadIdx.x; i < a.part_max;
-                 i += team.size * kBlock)
-                arr.cnt(par)[i] = 0u;
-        bool active = false;
-        if (leader) {
-            if (a.cap_policy == 1 && kept > a.cap_M) active = true;
-            unsigned long long lo = s_pub.lo, hi = s_pub.hi;
-            const uint32_t cn = redo ? 0u : __ldcg(&acc->cand_n);
-            const unsigned long long above = redo ? 0ULL : __ldcg(&acc->above);
-            const unsigned long long omax = __ldcg(&acc->out_max);
-            const double norm = *(volatile double*)&ctl->norm[np_];
-            // why not the listed candidates: 1 no range, 2 list too long,
-            // 3 threshold above the range, 4 below it
-            const int reason = (hi == 0ULL || redo) ? (redo && hi ? 4 : 1)
-                               : cn > a.cand_cap ? 2 : above >= a.cap_M ? 3
-                               : above + cn < a.cap_M ? 4 : 0;
-            const int failed = *(volatile int*)&ctl->status;
-            SelOut so{0ULL, 1};
-            PKey<W> key{};
-            const bool fast = active && reason == 0 && !failed;
-            if (fast)
-                so = select_list<W>(cand_v, cand_i, cn, a.cap_M - above, 0ULL, 0ULL,
-                                    hi > lo ? 64 - __clzll((long long)(hi - lo)) : 0,
-                                    arr.home(hb), ties, &key, ctl);
-            if (threadIdx.x == 0) {
-                constexpr unsigned long long kInfBits = 0x7ff0000000000000ULL;
-                if (omax >= kInfBits) set_status(ctl, ST_STATE, 4);
-                if (abs_pattern(norm) >= kInfBits) set_status(ctl, ST_STATE, 5);
-                if (a.cap_policy == 0 && kept > a.cap_M) set_status(ctl, ST_CAPACITY, 1);
-                Pub p;
-                p.rnorm = __ddiv_rn(1.0, norm);
-                p.n = active ? a.cap_M : kept;
-                p.T = fast ? so.v + lo : 0ULL;
-                p.all_ties = fast ? so.all_ties : 1;
-                for (int w = 0; w < 4; ++w) p.tk[w] = 0;
-                if (fast)
-                    for (int w = 0; w < W; ++w) { p.tk[w] = key.x[w]; p.tk[W + w] = key.z[w]; }
-                p.full = active && !fast && !failed;
-                p.lo = lo;
-                p.hi = hi;
-                p.rescatter = 0;
-                // a state that grew several times since its scatter
-                if (layout == 1 && p.n > 2ULL * a.target * P) p.rescatter = 1;
-                p.stop = *(volatile int*)&ctl->status != 0;
-                if (a.log) a.log[gi] = p.stop ? ~0ULL : p.n;
-                s_stat[0] += 1;
-                s_stat[1] += n_in;
-                s_stat[2] += p.n;
-                if (p.n > s_stat[3]) s_stat[3] = p.n;
-                s_stat[5] += active ? 1 : 0;
-                s_stat[6] += redo ? 1 : 0;
-                s_stat[7] += __ldcg(&rs->acc[np_][0].n_long);
-                ctl->sp_reason = reason;
-                if (fast) next_range(a, ctl, drift, n_drift, k, p.T, p.rnorm, reason, cn, hi - lo, &p);
-                if (p.full) {   // the team takes radix passes over the state
-                    ctl->stat_sel_full += 1;
-                    const unsigned long long top = omax > dbits ? omax - dbits : 0ULL;
-                    rs->sel_prefix = 0ULL;
-                    rs->sel_mask = 0ULL;
-                    rs->sel_k = a.cap_M;
-                    rs->sel_count = kept;
-                    rs->sel_n = 0u;
-                    p.T = top;   // the passes' value range (T itself comes after them)
-                }
-                memset(&rs->acc[np_ ^ 1][0], 0, sizeof rs->acc[0]);
-                rs->pub = p;
-            }
-        }
-        if (!team_barrier(team, ctl)) return false;
-        read_pub<W>(rs, &s_pub);
-        {
-            if (s_pub.full && !s_pub.stop) {
-                int top = s_pub.T ? 64 - __clzll((long long)s_pub.T) : 0;
-                // every stored value: v = pattern - delta's
-                auto each = [&](auto&& f) {
-                    if (layout == 0) {
-                        const double* c = arr.run_coef(run_buf);
-                        for (uint64_t i = (uint64_t)team.rank * kBlock + (threadIdx.x & ~31u);
-                             i < run_n; i += (uint64_t)team.size * kBlock) {
-                            const uint64_t j = i + (threadIdx.x & 31u);
-                            const unsigned long long b = j < run_n ? abs_pattern(__ldcs(c + j)) : 0ULL;
-                            f(b > dbits, b - dbits, j);
-                        }
-                    } else {
-                        for (uint32_t p = team.rank; p < P; p += team.size) {
-                            const uint32_t n = __ldcg(arr.cnt(par) + p);
-                            const double* c = arr.coef(cx) + (uint64_t)p * R;
-                            for (uint32_t i = threadIdx.x & ~31u; i < n; i += kBlock) {
-                                const uint32_t j = i + (threadIdx.x & 31u);
-                                const unsigned long long b = j < n ? abs_pattern(__ldcs(c + j)) : 0ULL;
-                                f(b > dbits, b - dbits, (uint64_t)p * R + j);
-                            }
+        // ---- a threshold outside the listed range, or a long list: radix
+        // passes by the whole team, every CTA picking the digit for itself ----
+        if (s_pub.full && !s_pub.stop) {
+            const bool of_list = s_pub.full == 2;
+            const unsigned long long base = s_pub.base;
+            const uint32_t cn = of_list ? __ldcg(&acc->cand_n) : 0u;
+            // every value: f(in, pattern - base, place), whole warps
+            auto each = [&](auto&& f) {
+                const uint32_t lane = threadIdx.x & 31u;
+                if (of_list || layout == 0) {
+                    const double* c = arr.run_coef(run_buf);
+                    const uint64_t n = of_list ? cn : run_n;
+                    for (uint64_t i = (uint64_t)team.rank * kBlock + (threadIdx.x & ~31u); i < n;
+                         i += (uint64_t)team.size * kBlock) {
+                        const uint64_t j = i + lane;
+                        if (of_list) {
+                            f(j < n, j < n ? __ldcg(cand_v + j) : 0ULL,
+                              j < n ? (uint64_t)__ldcg(cand_i + j) : 0ULL);
+                        } else {
+                            const unsigned long long b = j < n ? abs_pattern(__ldcs(c + j)) : 0ULL;
+                            f(b > base, b - base, j);
                         }
                     }
-                };
-                uint32_t* h = reinterpret_cast<uint32_t*>(g_stage);
-                for (;;) {
-                    const unsigned long long prefix = __ldcg(&rs->sel_prefix),
-                                             mask = __ldcg(&rs->sel_mask),
-                                             count = __ldcg(&rs->sel_count);
-                    if (top <= 0 || (mask && count <= 4096ULL)) break;
-                    const int shift = top > kDigit ? top - kDigit : 0;
-                    const uint32_t dmask = (1u << (top - shift)) - 1u;
-                    for (int b = threadIdx.x; b < kBins; b += kBlock) h[b] = 0u;
-                    __syncthreads();
-                    each([&](bool in, unsigned long long v, uint64_t) {
-                        if (in && (v & mask) == prefix)
-                            atomicAdd(&h[(uint32_t)(v >> shift) & dmask], 1u);
-                    });
-                    __syncthreads();
-                    for (int b = threadIdx.x; b < kBins; b += kBlock)
-                        if (h[b]) atomicAdd(&rs->hist[b], h[b]);
-                    if (!team_barrier(team, ctl)) return false;
-                    if (leader) {
-                        __shared__ PickOut s_p;
-                        for (int b = threadIdx.x; b < kBins; b += kBlock) {
-                            h[b] = __ldcg(&rs->hist[b]);
-                            rs->hist[b] = 0u;
-                        }
-                        __syncthreads();
-                        pick_bin<true>(h, (uint32_t)__ldcg(&rs->sel_k), s_w, &s_p);
-                        if (threadIdx.x == 0) {
-                            rs->sel_prefix = prefix | ((unsigned long long)s_p.digit << shift);
-                            rs->sel_mask = mask | ((unsigned long long)dmask << shift);
-                            rs->sel_k = s_p.k_in;
-                            rs->sel_count = s_p.count;
+                } else {
+                    for (uint32_t p = team.rank; p < P; p += team.size) {
+                        const uint32_t n = __ldcg(arr.cnt(ci) + (uint64_t)p * kPad);
+                        const double* c = arr.coef(cx) + (uint64_t)p * R;
+                        for (uint32_t i = threadIdx.x & ~31u; i < n; i += kBlock) {
+                            const uint32_t j = i + lane;
+                            const unsigned long long b = j < n ? abs_pattern(__ldcs(c + j)) : 0ULL;
+                            f(b > base, b - base, (uint64_t)p * R + j);
                         }
                     }
-                    top = shift;
-                    if (!team_barrier(team, ctl)) return false;
                 }
-                const unsigned long long prefix = __ldcg(&rs->sel_prefix),
-                                         mask = __ldcg(&rs->sel_mask);
-                PushList gp = pl;
-                gp.gn = &rs->sel_n;
-                if (threadIdx.x == 0) s_cn = kPushBuf;   // straight to the global list
+            };
+            uint32_t* h = reinterpret_cast<uint32_t*>(g_stage + InPass<W>::kBytes);
+            unsigned long long prefix = 0ULL, mask = 0ULL;
+            uint32_t rank = (uint32_t)s_pub.rank, count = 0xffffffffu;
+            int top = s_pub.range ? 64 - __clzll((long long)s_pub.range) : 0;
+            for (int q = 0; top > 0 && count > kOneCta; ++q) {
+                const int shift = top > kDigit ? top - kDigit : 0;
+                const uint32_t dmask = (1u << (top - shift)) - 1u;
+                uint32_t* hist = rs->hist[q % 3];
+                uint32_t* spare = rs->hist[(q + 1) % 3];
+                for (int b = threadIdx.x; b < kBins; b += kBlock) h[b] = 0u;
+                for (uint32_t b = team.rank * kBlock + threadIdx.x; b < (uint32_t)kBins;
+                     b += team.size * kBlock)
+                    spare[b] = 0u;
                 __syncthreads();
-                each([&](bool in, unsigned long long v, uint64_t idx) {
-                    push_cand(gp, in && (v & mask) == prefix, v, idx);
+                each([&](bool in, unsigned long long v, uint64_t) {
+                    if (in && (v & mask) == prefix)
+                        atomicAdd(&h[(uint32_t)(v >> shift) & dmask], 1u);
                 });
+                __syncthreads();
+                for (int b = threadIdx.x; b < kBins; b += kBlock)
+                    if (h[b]) atomicAdd(hist + b, h[b]);
                 if (!team_barrier(team, ctl)) return false;
-                if (leader) {
-                    PKey<W> key{};
-                    const uint32_t cn = __ldcg(&rs->sel_n);
-                    SelOut so{0ULL, 1};
-                    if (cn > a.cand_cap) {
-                        if (threadIdx.x == 0) set_status(ctl, ST_CAPACITY, 63);
-                    } else {
-                        so = select_list<W>(cand_v, cand_i, cn, __ldcg(&rs->sel_k), prefix, mask,
-                                            top, layout == 0 ? arr.run_keys(run_buf) : arr.home(hb),
-                                            ties, &key, ctl);
-                    }
-                    if (threadIdx.x == 0) {
-                        Pub p = s_pub;
-                        p.T = so.v + dbits;
-                        p.all_ties = so.all_ties;
-                        for (int w = 0; w < W; ++w) { p.tk[w] = key.x[w]; p.tk[W + w] = key.z[w]; }
-                        p.full = 0;
-                        p.stop = *(volatile int*)&ctl->status != 0;
-                        next_range(a, ctl, drift, n_drift, k, p.T, p.rnorm, ctl->sp_reason, cn,
-                                   s_pub.T, &p);
-                        rs->pub = p;
-                    }
-                }
-                if (!team_barrier(team, ctl)) return false;
-                read_pub<W>(rs, &s_pub);
+                for (int b = threadIdx.x; b < kBins; b += kBlock) h[b] = __ldcg(hist + b);
+                __syncthreads();
+                pick_bin<true>(h, rank, s_w, &s_pick);
+                prefix |= (unsigned long long)s_pick.digit << shift;
+                mask |= (unsigned long long)dmask << shift;
+                rank = s_pick.k_in;
+                count = s_pick.count;
+                top = shift;
+                __syncthreads();
             }
+            // the values left, for the first CTA (those of the list beside it)
+            PushList gp = pl;
+            unsigned long long* lv = of_list ? reinterpret_cast<unsigned long long*>(ties) : cand_v;
+            uint32_t* li = of_list ? reinterpret_cast<uint32_t*>(lv + cn) : cand_i;
+            gp.gv = lv;
+            gp.gidx = li;
+            gp.gn = &rs->sel_n;
+            if (threadIdx.x == 0) s_cn = kPushBuf;   // straight to the global list
+            __syncthreads();
+            each([&](bool in, unsigned long long v, uint64_t idx) {
+                push_cand(gp, in && (v & mask) == prefix, v, idx);
+            });
+            team_arrive(team);
+            if (leader) {
+                if (!team_wait(team, ctl)) return false;
+                for (int b = threadIdx.x; b < 3 * kBins; b += kBlock) rs->hist[0][b] = 0u;
+                PKey<W> key{};
+                const uint32_t ln = __ldcg(&rs->sel_n);
+                SelOut so{0ULL, 1};
+                if (ln > a.cand_cap) {
+                    if (threadIdx.x == 0) set_status(ctl, ST_CAPACITY, 63);
+                } else {
+                    PKey<W>* tl = of_list ? reinterpret_cast<PKey<W>*>(cand_v) : ties;
+                    so = select_list<W>(lv, li, ln, rank, prefix, mask, top,
+                                        layout == 0 ? arr.run_keys(run_buf) : arr.home(hb), tl,
+                                        &key, ctl);
+                }
+                if (threadIdx.x == 0) {
+                    Pub& p = s_next;
+                    p = s_pub;
+                    p.T = so.v + base;
+                    p.all_ties = so.all_ties;
+                    if (!so.all_ties)
+                        for (int w = 0; w < W; ++w) { p.tk[w] = key.x[w]; p.tk[W + w] = key.z[w]; }
+                    p.full = 0;
+                    p.stop = *(volatile int*)&ctl->status != 0;
+                    next_range(&s_pred, a.cand_hi, drift_now, s_dn, p.T, p.rnorm, of_list ? cn : ln,
+                               a.delta_bits, &p);
+                }
+                if (threadIdx.x < 32) publish(team, &s_next);
+            }
+            if (!take_pub(team, ctl, &s_pub)) return false;
         }
         any = true;
     }
@@ -1061,8 +1191,8 @@ __device__ bool run_instance(const RunArgs<W>& a, const RunGate<W>* gates, int n
         const uint32_t runs = layout == 1 ? P : 1u;
         for (uint32_t p = layout == 1 ? team.rank : 0u; p < runs; p += layout == 1 ? team.size : 1u) {
             const PKey<W>* ki = layout == 1 ? arr.home(hb) + (uint64_t)p * R : arr.run_keys(run_buf);
-            const double* ci = layout == 1 ? arr.coef(cx) + (uint64_t)p * R : arr.run_coef(run_buf);
-            const uint64_t n = layout == 1 ? __ldcg(arr.cnt(par) + p) : run_n;
+            const double* vi = layout == 1 ? arr.coef(cx) + (uint64_t)p * R : arr.run_coef(run_buf);
+            const uint64_t n = layout == 1 ? __ldcg(arr.cnt(ci) + (uint64_t)p * kPad) : run_n;
             const uint64_t first = layout == 1 ? 0ULL : (uint64_t)team.rank * kBlock;
             const uint64_t step = layout == 1 ? (uint64_t)kBlock : (uint64_t)team.size * kBlock;
             for (uint64_t i0 = first; i0 < n; i0 += step) {
@@ -1072,7 +1202,7 @@ __device__ bool run_instance(const RunArgs<W>& a, const RunGate<W>* gates, int n
                 bool keep = false;
                 if (i < n) {
                     K = load_key_stream(ki + i);
-                    c = __ldcs(ci + i);
+                    c = __ldcs(vi + i);
                     keep = abs_pattern(c) != 0ULL &&
                            cap_keep(K, c, s_pub.T, s_pub.all_ties != 0, tk);
                     if (!keep && key_is_zero(K)) set_status(ctl, ST_TRACE_ZERO, 3);
@@ -1097,12 +1227,18 @@ __device__ bool run_instance(const RunArgs<W>& a, const RunGate<W>* gates, int n
         ctl->norm[out_buf] = norm;
         ctl->rnorm[out_buf] = s_pub.rnorm;
         ctl->pend = 0;
-        ctl->seg = 0;
+        ctl->home = 0;
         ctl->need_scatter = 0;
         ctl->part_over = 0;
         ctl->sel_active = 0;
         ctl->sp_lo = s_pub.lo;
         ctl->sp_hi = s_pub.hi;
+        ctl->sp_thr = s_pub.thr;
+        ctl->sp_tprev = s_pred.tprev;
+        ctl->sp_shift = s_pred.shift;
+        ctl->stat_cands += s_pred.cands;
+        if (s_pred.range) ctl->stat_range = s_pred.range;
+        ctl->stat_sel_full += s_pred.full;
         ctl->out_max = 0;
         const unsigned int gen = ctl->gen + (unsigned int)s_stat[0];
         if (gen < ctl->gen) set_status(ctl, ST_STATE, 1);   // generation counter wrapped
@@ -1137,6 +1273,7 @@ k_run(const RunArgs<W> a, const __grid_constant__ RunChunk<W> chunk) {
     }
     team.rs = reinterpret_cast<RunShared*>(static_cast<char*>(a.shared) + (uint64_t)t * a.shared_stride);
     team.target = 0;
+    team.seq = 0;
     for (int inst = (int)t; inst < a.B; inst += (int)teams) {
         const RunGate<W>* gates = a.gates ? a.gates + (uint64_t)inst * a.max_gates : chunk.g;
         const int n = a.gates ? a.n_gates[inst] : a.one_gates;
@@ -1147,8 +1284,14 @@ k_run(const RunArgs<W> a, const __grid_constant__ RunChunk<W> chunk) {
 }  // namespace
 
 template <int W>
+static constexpr size_t run_smem() {
+    return InPass<W>::kBytes + kScratch > Stage<W>::kBytes ? InPass<W>::kBytes + kScratch
+                                                           : Stage<W>::kBytes;
+}
+
+template <int W>
 static int run_fit_w() {
-    constexpr size_t smem = InStage<W>::kBytes;
+    constexpr size_t smem = run_smem<W>();
     cudaFuncSetAttribute(k_run<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     cudaFuncSetAttribute(k_run<W>, cudaFuncAttributePreferredSharedMemoryCarveout,
                          (int)cudaSharedmemCarveoutMaxShared);
@@ -1163,7 +1306,7 @@ template <int W>
 cudaError_t launch_run(const RunArgs<W>& a, const RunChunk<W>& chunk, int grid, cudaStream_t st) {
     void* args[2] = {const_cast<RunArgs<W>*>(&a), const_cast<RunChunk<W>*>(&chunk)};
     return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(&k_run<W>), dim3(grid),
-                                       dim3(kBlock), args, InStage<W>::kBytes, st);
+                                       dim3(kBlock), args, run_smem<W>(), st);
 }
 
 template cudaError_t launch_run<1>(const RunArgs<1>&, const RunChunk<1>&, int, cudaStream_t);

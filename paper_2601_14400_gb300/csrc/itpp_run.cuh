@@ -10,21 +10,55 @@
 
 namespace itpp {
 
-// One gate as the run reads it.
+// One gate as the run reads it, with the windows a scatter at this gate can
+// prepare: the gates from here on that act on at most so many sites (level 0:
+// the longest windows, level 1: three sites), len 0 when this gate alone acts
+// on more.
 template <int W>
 struct RunGate {
     uint64_t qx[W], qz[W];
-    uint64_t win[W];     // sites of its window
+    uint64_t win[2][W];
     double ch, msh;
-    int pair, sites;     // pair-key mode; sites of the window
-    int start, pad;      // first gate of its window
+    uint8_t len[2], sites[2];
+    uint8_t pad[4];
 };
+
+// Sites of the two window levels.
+constexpr int run_sites(int W, int level) { return level ? 3 : (W == 1 ? 5 : 4); }
+
+// The windows that start at each of n gates of a schedule (which repeats).
+template <int W>
+void plan_run_windows(RunGate<W>* g, int n) {
+    for (int lv = 0; lv < 2; ++lv)
+        for (int k = 0; k < n; ++k) {
+            uint64_t s[W] = {};
+            int len = 0, sites = 0;
+            for (int j = 0; j < n && len < 255; ++j) {
+                const RunGate<W>& q = g[(k + j) % n];
+                uint64_t t[W];
+                int c = 0;
+                for (int w = 0; w < W; ++w) {
+                    t[w] = s[w] | q.qx[w] | q.qz[w];
+                    c += __builtin_popcountll(t[w]);
+                }
+                if (c > run_sites(W, lv)) break;
+                for (int w = 0; w < W; ++w) s[w] = t[w];
+                sites = c;
+                ++len;
+            }
+            g[k].len[lv] = (uint8_t)len;
+            g[k].sites[lv] = (uint8_t)sites;
+            for (int w = 0; w < W; ++w) g[k].win[lv][w] = s[w];
+        }
+}
 
 // The gates of a launch as a kernel argument: the host keeps no device copy
 // of them that a change of the coefficients or a captured launch could race.
 constexpr int kRunChunk = 256;
 // Smallest mean partition a scatter aims for to give every CTA one.
 constexpr int kRunMinPart = 128;
+// Distance of two partition cursors (words).
+constexpr int kRunPad = 32;
 template <int W>
 struct RunChunk {
     RunGate<W> g[kRunChunk];
@@ -36,7 +70,7 @@ struct RunArgs {
     double* c[2];
     PKey<W>* kp;
     double* cp;
-    unsigned int* cnt;            // [B][2][part_max]
+    unsigned int* cnt;            // [B][3][part_max], kRunPad apart
     DevCtl* ctl;                  // [B]
     void* scratch;                // [B] candidates and ties (the merge table's memory)
     void* shared;                 // [teams] RunShared

@@ -46,26 +46,6 @@ __device__ __forceinline__ void sel_geometry(const DevCtl* ctl, unsigned long lo
     *sh = bits > kSelBits ? bits - kSelBits : 0;
 }
 
-// Stored terms of the current buffer: chunk s is [off, off + cnt) when the
-// buffer is segmented (a partitioned merge wrote it), else one run of n.
-struct StateRuns {
-    const ChunkDesc* din;
-    bool seg;
-    uint32_t P;
-    uint64_t n;
-};
-
-__device__ __forceinline__ StateRuns state_runs(const DevCtl* ctl, const ChunkDesc* chunks0,
-                                                const ChunkDesc* chunks1) {
-    StateRuns r;
-    const int cur = ctl->cur;
-    r.din = cur ? chunks1 : chunks0;
-    r.seg = ctl->seg != 0;
-    r.P = ctl->nchunk[cur];
-    r.n = live_count(ctl, cur);
-    return r;
-}
-
 __device__ __forceinline__ unsigned long long sel_value(double c, unsigned long long lo) {
     const unsigned long long b = abs_bits(c);
     return b > lo ? b - lo : 0ULL;
@@ -146,7 +126,8 @@ k_sel_begin(DevCtl* ctl, CandRegions cr, unsigned long long* cand_v, uint32_t* c
     uint32_t tot;
     const uint32_t off = block_exclusive_scan<1024>(c, &tot, s_scan);
     s_off[threadIdx.x] = off;
-    const unsigned long long above = ctl->sp_above;
+    // kept children above the range: all that were not listed
+    const unsigned long long above = ctl->count[ctl->cur] - tot;
     const int reason = ctl->sp_hi == 0ULL ? 1
                        : (ctl->sp_ovf || tot > cand_cap) ? 2
                        : above >= cap_M ? 3
@@ -191,7 +172,7 @@ k_sel_begin(DevCtl* ctl, CandRegions cr, unsigned long long* cand_v, uint32_t* c
 // ---------------------------------------------------------------------------
 template <int W>
 __global__ void __launch_bounds__(256, 4)
-k_sel_hist(Bufs<W> B, DevCtl* ctl, const ChunkDesc* desc0, const ChunkDesc* desc1) {
+k_sel_hist(Bufs<W> B, Homes<W> H, DevCtl* ctl) {
     __shared__ unsigned int h[kSelBins];
     __shared__ unsigned long long s_part[256];
     __shared__ int s_last;
@@ -202,21 +183,21 @@ k_sel_hist(Bufs<W> B, DevCtl* ctl, const ChunkDesc* desc0, const ChunkDesc* desc
     sel_geometry(ctl, lo, &sh);
     for (int b = threadIdx.x; b < kSelBins; b += blockDim.x) h[b] = 0u;
     __syncthreads();
-    const int cur = ctl->cur;
-    const StateRuns rs = state_runs(ctl, desc0, desc1);
+    const StateRuns<W> rs = state_runs(ctl, B, H);
     // the coefficients' bit patterns, read as integers (no floating point)
     const unsigned long long* __restrict__ c =
-        reinterpret_cast<const unsigned long long*>(B.coef(cur));
+        reinterpret_cast<const unsigned long long*>(rs.coef);
     auto count = [&](unsigned long long raw) {
         const unsigned long long b = raw & 0x7fffffffffffffffULL;   // |c| pattern
+        if (!b) return;   // a zero is no term
         unsigned long long d = (b > lo ? b - lo : 0ULL) >> sh;
         if (d > (unsigned long long)(kSelBins - 1)) d = kSelBins - 1;   // not reached: hi is the max
         atomicAdd(&h[d], 1u);
     };
-    if (rs.seg) {
+    if (rs.cnt) {
         for (uint32_t s = blockIdx.x; s < rs.P; s += gridDim.x) {
-            const uint64_t off = rs.din[s].off;
-            const uint32_t cnt = rs.din[s].cnt;
+            const uint64_t off = (uint64_t)s * rs.R;
+            const uint32_t cnt = rs.cnt[s] < rs.R ? rs.cnt[s] : (uint32_t)rs.R;
             for (uint32_t j = threadIdx.x; j < cnt; j += blockDim.x) count(__ldcs(c + off + j));
         }
     } else {
@@ -321,18 +302,17 @@ __device__ __forceinline__ void gather_one(bool hit, unsigned long long x, uint6
 
 template <int W>
 __global__ void __launch_bounds__(256)
-k_sel_gather(Bufs<W> B, DevCtl* ctl, const ChunkDesc* desc0, const ChunkDesc* desc1,
-             unsigned long long* cand_v, uint32_t* cand_idx, uint64_t cand_cap) {
+k_sel_gather(Bufs<W> B, Homes<W> H, DevCtl* ctl, unsigned long long* cand_v,
+             uint32_t* cand_idx, uint64_t cand_cap) {
     __shared__ unsigned long long st_v[kStage];
     __shared__ uint32_t st_i[kStage];
     __shared__ unsigned int s_claimed, s_staged;
     __shared__ unsigned long long s_base;
     if (!ctl->sel_active || ctl->status || ctl->sel_fast) return;
-    const int cur = ctl->cur;
-    const StateRuns rs = state_runs(ctl, desc0, desc1);
+    const StateRuns<W> rs = state_runs(ctl, B, H);
     const unsigned long long lo = ctl->sel_lo;
     const unsigned long long prefix = ctl->sel_prefix, mask = ctl->sel_mask;
-    const double* __restrict__ c = B.coef(cur);
+    const double* __restrict__ c = rs.coef;
     const GatherStage gs{st_v, st_i, &s_claimed, &s_staged};
     if (threadIdx.x == 0) {
         s_claimed = 0u;
@@ -340,15 +320,15 @@ k_sel_gather(Bufs<W> B, DevCtl* ctl, const ChunkDesc* desc0, const ChunkDesc* de
     }
     __syncthreads();
     // whole warps iterate together (the claims are warp-wide)
-    if (rs.seg) {
+    if (rs.cnt) {
         for (uint32_t s = blockIdx.x; s < rs.P; s += gridDim.x) {
-            const uint64_t off = rs.din[s].off;
-            const uint32_t cnt = rs.din[s].cnt;
+            const uint64_t off = (uint64_t)s * rs.R;
+            const uint32_t cnt = rs.cnt[s] < rs.R ? rs.cnt[s] : (uint32_t)rs.R;
             for (uint32_t j0 = 0; j0 < cnt; j0 += blockDim.x) {
                 const uint32_t j = j0 + threadIdx.x;
                 const double v = j < cnt ? __ldcs(c + off + j) : 0.0;
                 const unsigned long long x = sel_value(v, lo);
-                gather_one(j < cnt && (x & mask) == prefix, x, off + j, gs, ctl, cand_v, cand_idx,
+                gather_one(j < cnt && v != 0.0 && (x & mask) == prefix, x, off + j, gs, ctl, cand_v, cand_idx,
                            cand_cap);
             }
         }
@@ -443,14 +423,16 @@ k_sel_vpass(DevCtl* ctl, const unsigned long long* cand_v, int p) {
 // ---------------------------------------------------------------------------
 template <int W>
 __global__ void __launch_bounds__(256)
-k_sel_tcollect(Bufs<W> B, DevCtl* ctl, const unsigned long long* cand_v,
+k_sel_tcollect(Bufs<W> B, Homes<W> H, DevCtl* ctl, const unsigned long long* cand_v,
                const uint32_t* cand_idx, PKey<W>* tie_list, uint64_t tie_cap) {
     constexpr int kT = 1024;
     __shared__ PKey<W> st[kT];
     __shared__ unsigned int s_n;
     __shared__ unsigned long long s_base;
     if (!tie_select_needed(ctl)) return;
-    const int cur = ctl->cur;
+    const StateRuns<W> rs = state_runs(ctl, B, H);
+    const PKey<W>* keys = rs.keys;
+    const uint64_t held = rs.cnt ? rs.P * rs.R : rs.n;
     const unsigned long long nc = ctl->sel_cand_n, T = ctl->sel_prefix;
     if (threadIdx.x == 0) s_n = 0u;
     __syncthreads();
@@ -458,8 +440,12 @@ k_sel_tcollect(Bufs<W> B, DevCtl* ctl, const unsigned long long* cand_v,
          j0 < nc; j0 += (unsigned long long)gridDim.x * blockDim.x) {
         const unsigned long long j = j0 + threadIdx.x;
         if (j < nc && cand_v[j] == T) {
-            const unsigned int q = atomicAdd(&s_n, 1u);
-            st[q] = load_key(B.key(cur) + cand_idx[j]);
+            if (cand_idx[j] < held) {
+                const unsigned int q = atomicAdd(&s_n, 1u);
+                st[q] = load_key(keys + cand_idx[j]);
+            } else {
+                set_status(ctl, ST_STATE, 34);   // not reached
+            }
         }
         __syncthreads();
         const unsigned int m = s_n;
@@ -578,7 +564,7 @@ __device__ void bitonic_sort_keys(PKey<W>* a, int n_pad) {
 template <int W>
 __global__ void __launch_bounds__(1024)
 k_sel_finish(DevCtl* ctl, const PKey<W>* tie_list, uint64_t cap_M, uint64_t cand_hi,
-             long long* drift, int n_drift, int gate) {
+             long long* drift, int n_drift, int gate, unsigned long long delta_bits) {
     __shared__ PKey<W> s_ties[SmallTies<W>::kMax];
     __shared__ unsigned int s_cnt;
     if (!ctl->sel_active) return;
@@ -616,7 +602,11 @@ k_sel_finish(DevCtl* ctl, const PKey<W>* tie_list, uint64_t cap_M, uint64_t cand
             __syncthreads();
             bitonic_sort_keys<W>(s_ties, n_pad);
             if (threadIdx.x == 0) {
-                const unsigned long long r = ctl->sel_tie_state == 2 ? 1ULL : ctl->sel_tie_k;
+                unsigned long long r = ctl->sel_tie_state == 2 ? 1ULL : ctl->sel_tie_k;
+                if (r < 1ULL || r > m) {   // not reached: the list agrees with the counts
+                    set_status(ctl, ST_STATE, 33);
+                    r = 1ULL;
+                }
                 const PKey<W> tk = s_ties[r - 1];
                 for (int w = 0; w < W; ++w) {
                     ctl->sel_tie_key[w] = tk.x[w];
@@ -660,7 +650,7 @@ k_sel_finish(DevCtl* ctl, const PKey<W>* tie_list, uint64_t cap_M, uint64_t cand
             case 2: sft -= 2; break;
             default: sft += 1; break;
         }
-        sft = sft < 8 ? 8 : (sft > 60 ? 60 : sft);
+        sft = sft < 8 ? 8 : (sft > kRangeShiftMax ? kRangeShiftMax : sft);
         ctl->sp_shift = sft;
         const long long dn = n_drift > 0 ? drift[gn] : 0LL;
         unsigned long long C;
@@ -670,9 +660,10 @@ k_sel_finish(DevCtl* ctl, const PKey<W>* tie_list, uint64_t cap_M, uint64_t cand
         } else {
             C = abs_pattern(__dmul_rn(__longlong_as_double((long long)T), ctl->rnorm[cur]));
         }
-        const unsigned long long h = 1ULL << sft;
-        ctl->sp_lo = C > h ? C - h : 0ULL;
-        ctl->sp_hi = C + h;
+        SelRange r = sel_range(C, sft, delta_bits);
+        ctl->sp_thr = r.thr;
+        ctl->sp_lo = r.thr + 1ULL;
+        ctl->sp_hi = r.hi;
     }
 }
 
@@ -719,19 +710,25 @@ static cudaError_t select_w(const DeviceState& s, cudaStream_t st, int gate) {
     std::memcpy(&lo, &s.delta, sizeof lo);   // delta >= +0: its pattern bounds every kept |c|
     const SelScratch<W> sc = sel_scratch<W>(s);
     const Bufs<W> B = sel_bufs<W>(s);
+    Homes<W> H;
+    H.kp = reinterpret_cast<PKey<W>*>(s.part_keys);
+    H.cp = s.part_coef;
+    H.cnt = s.part_cursor;
+    H.part_max = s.part_max;
+    H.cap = 0;
     k_sel_begin<<<s.num_sms, 1024, 0, st>>>(s.ctl, s.cand, sc.cand_v, sc.cand_idx, sc.cand_cap,
                                             s.cap_M, lo);
-    k_sel_hist<W><<<s.num_sms * 4, 256, 0, st>>>(B, s.ctl, s.chunks[0], s.chunks[1]);
-    k_sel_gather<W><<<s.num_sms * 4, 256, 0, st>>>(B, s.ctl, s.chunks[0], s.chunks[1],
-                                                   sc.cand_v, sc.cand_idx, sc.cand_cap);
+    k_sel_hist<W><<<s.num_sms * 4, 256, 0, st>>>(B, H, s.ctl);
+    k_sel_gather<W><<<s.num_sms * 4, 256, 0, st>>>(B, H, s.ctl, sc.cand_v, sc.cand_idx,
+                                                   sc.cand_cap);
     for (int p = 1; p <= kVPasses; ++p)    // 13-bit digits cover any 63-bit range
         k_sel_vpass<<<s.num_sms, 1024, 0, st>>>(s.ctl, sc.cand_v, p);
-    k_sel_tcollect<W><<<s.num_sms * 2, 256, 0, st>>>(B, s.ctl, sc.cand_v, sc.cand_idx, sc.ties,
+    k_sel_tcollect<W><<<s.num_sms * 2, 256, 0, st>>>(B, H, s.ctl, sc.cand_v, sc.cand_idx, sc.ties,
                                                      sc.tie_cap);
     for (int p = 0; p < 8 * W; ++p)
         k_sel_tpass<W><<<s.num_sms, 1024, 0, st>>>(s.ctl, sc.ties, p);
     k_sel_finish<W><<<1, 1024, 0, st>>>(s.ctl, sc.ties, s.cap_M, s.cand_hi, s.sp_drift,
-                                        s.sp_drift ? s.layer_gates : 0, gate);
+                                        s.sp_drift ? s.layer_gates : 0, gate, lo);
     return cudaGetLastError();
 }
 

@@ -116,7 +116,7 @@ __device__ __forceinline__ void scatter_run(const PKey<W>* __restrict__ kin,
                                             DevCtl* ctl, PKey<W>* pk, double* pc,
                                             unsigned int* cursor, const PartPlan& pl,
                                             const GateArg<W>& g, const PartFn<W>& f,
-                                            int* over) {
+                                            int* over, uint32_t pad = 1u) {
     // whole warps iterate together (the cursor claim below is warp-wide);
     // U items per thread per round, their loads issued before any claim
     constexpr int U = 4;
@@ -150,7 +150,7 @@ __device__ __forceinline__ void scatter_run(const PKey<W>* __restrict__ kin,
             const unsigned int peers = __match_any_sync(0xffffffffu, p);
             const int leader = __ffs(peers) - 1;
             unsigned int base = 0;
-            if (live[u] && (threadIdx.x & 31) == leader) base = atomicAdd(cursor + p, __popc(peers));
+            if (live[u] && (threadIdx.x & 31) == leader) base = atomicAdd(cursor + (uint64_t)p * pad, __popc(peers));
             base = __shfl_sync(0xffffffffu, base, leader);
             if (live[u]) {
                 const unsigned int pos = base + __popc(peers & lt);
@@ -339,14 +339,11 @@ __device__ __forceinline__ bool commute_sign(const PKey<W>& k, const GateArg<W>&
     return (a & 1) == 0;
 }
 
-// Slot of a commuting string in the pair table: a multilinear hash of the key
-// with the gate's bits cleared, on which K and Q.K agree (32-bit multiplies:
-// the 64-bit ones cost four times as many issue slots).
+// Multilinear hash of the key with the gate's bits cleared, on which K and Q.K
+// agree; its high bits are a slot (32-bit multiplies: the 64-bit ones cost four
+// times as many issue slots).
 template <int W>
-__device__ __forceinline__ uint32_t pair_slot(const PKey<W>& K, const GateArg<W>& g) {
-    constexpr uint32_t S = StageGeom<W>::kSlots;
-    constexpr int kBits = S == 2048 ? 11 : 10;
-    static_assert(S == (1u << kBits), "slots");
+__device__ __forceinline__ uint32_t pair_hash(const PKey<W>& K, const GateArg<W>& g) {
     uint32_t h = 0;
 #pragma unroll
     for (int w = 0; w < W; ++w) {
@@ -354,7 +351,15 @@ __device__ __forceinline__ uint32_t pair_slot(const PKey<W>& K, const GateArg<W>
         h = h * 0x2c1b3c6du + (uint32_t)mx * 0x9e3779b1u + (uint32_t)(mx >> 32) * 0x85ebca77u +
             (uint32_t)mz * 0xc2b2ae3du + (uint32_t)(mz >> 32) * 0x27d4eb2fu;
     }
-    return h >> (32 - kBits);
+    return h;
+}
+
+template <int W>
+__device__ __forceinline__ uint32_t pair_slot(const PKey<W>& K, const GateArg<W>& g) {
+    constexpr uint32_t S = StageGeom<W>::kSlots;
+    constexpr int kBits = S == 2048 ? 11 : 10;
+    static_assert(S == (1u << kBits), "slots");
+    return pair_hash(K, g) >> (32 - kBits);
 }
 
 // Pair table of one pass.  A commuting string K and its partner Q.K agree
@@ -536,14 +541,10 @@ __device__ __forceinline__ void pass_children(uint32_t n_pair, uint32_t n_throug
     }
 }
 
-// How a pass learns where its children go.  kBound: room(most) is asked for
-// the most children the pass can have (live pass-through strings once,
-// pairs twice: at most twice the live strings, so the claims of a gate never
-// exceed twice its input), before any child is computed; what stays unused
-// behind the kept ones is the caller's.  kExact: the children are counted
-// first and room(kept) gives a run with no holes (the batch's contiguous
-// output).  kCount: they are counted only.
-enum class PassRoom { kBound, kExact, kCount };
+// How a pass learns where its children go.  kExact: the children are counted
+// first and room(kept) gives a run with no holes.  kCount: they are counted
+// only.  kAt: the caller holds room for all of them at room().
+enum class PassRoom { kAt, kExact, kCount };
 
 // One pass of the gate over n staged strings.
 //
@@ -618,7 +619,7 @@ __device__ __forceinline__ uint32_t stage_pass(uint32_t n, uint32_t shift, const
         g_kept[par ^ 1u] = 0u;
     }
     uint32_t* kept = &g_kept[par];
-    if (kRoom == PassRoom::kBound) {
+    if (kRoom == PassRoom::kAt) {
         const unsigned long long base = room(n_through + 2u * n_pair);
         if (base != ~0ULL)
             pass_children<W, BLOCK, true, true>(n_pair, n_through, shift, g, dbits, has_id, ctl,
@@ -706,7 +707,7 @@ __device__ __forceinline__ uint32_t merge_long(const PKey<W>* kp, const double* 
             *pass += 1u;
             if (write) {
                 const unsigned long long at = base + done;
-                done += stage_pass<W, BLOCK, PassRoom::kBound>(
+                done += stage_pass<W, BLOCK, PassRoom::kAt>(
                     n, 0u, g, pd, rnorm, dbits, has_id, ctl, nxt, *pass, kout, cout, st, cd,
                     [at](uint32_t) { return at; });
             } else {
