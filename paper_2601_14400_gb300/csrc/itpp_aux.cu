@@ -47,28 +47,38 @@ __device__ __forceinline__ PKey<W> key_from_planes(const uint64_t* x, const uint
 // Expectation values: <O> = sum_j w_j c_{P_j} (identity coefficient one).
 // ---------------------------------------------------------------------------
 
-// One CTA: deterministic open-addressing table of the observable strings
-// (first occurrence of each distinct string), zeroed value slots.
+// One CTA: open-addressing table of the observable strings, entry = the first
+// occurrence of its string, and zeroed value slots.  Which slot a string lands
+// in depends on the order of arrival, its entry does not: equal strings meet in
+// one slot and the smallest index stays.  What bounds it is the latency of a
+// few dependent accesses per string; one thread inserting them one after
+// another took 490 us for 2,080 strings, all threads at once take a few.
 template <int W>
-__global__ void k_obs_prep(const uint64_t* ox, const uint64_t* oz, int m, int tsize, int* tab,
-                           int* first, double* vals, DevCtl* ctl) {
+__global__ void __launch_bounds__(1024)
+k_obs_prep(const uint64_t* ox, const uint64_t* oz, int m, int tsize, int* tab, int* first,
+           double* vals, DevCtl* ctl) {
     for (int t = threadIdx.x; t < tsize; t += blockDim.x) tab[t] = -1;
     for (int j = threadIdx.x; j < m; j += blockDim.x) vals[j] = 0.0;
     __syncthreads();
-    if (threadIdx.x != 0) return;
     const uint64_t mask = (uint64_t)tsize - 1;
-    for (int j = 0; j < m; ++j) {
+    for (int j = threadIdx.x; j < m; j += blockDim.x) {
         const PKey<W> K = key_from_planes<W>(ox, oz, (uint64_t)j);
         uint64_t h = key_hash(K) & mask;
         int p = 0;
         for (; p < tsize; ++p) {
-            const int e = tab[h];
-            if (e < 0) { tab[h] = j; first[j] = j; break; }
-            if (key_eq(key_from_planes<W>(ox, oz, (uint64_t)e), K)) { first[j] = e; break; }
+            const int e = atomicCAS(tab + h, -1, j);
+            if (e < 0) break;
+            if (key_eq(key_from_planes<W>(ox, oz, (uint64_t)e), K)) {
+                atomicMin(tab + h, j);
+                break;
+            }
             h = (h + 1) & mask;
         }
+        first[j] = (int)h;   // its slot, for now
         if (p == tsize) set_status(ctl, ST_HASH_PROBE, 3);
     }
+    __syncthreads();
+    for (int j = threadIdx.x; j < m; j += blockDim.x) first[j] = __ldcg(tab + first[j]);
 }
 
 // Stream the state once; each term looks its key up in the observable
@@ -139,7 +149,7 @@ template <int W>
 static cudaError_t expect_w(const DeviceState& s, const uint64_t* ox, const uint64_t* oz,
                             const double* ow, int m, int tsize, int* tab, int* first,
                             double* vals, double* out, cudaStream_t st) {
-    k_obs_prep<W><<<1, 256, 0, st>>>(ox, oz, m, tsize, tab, first, vals, s.ctl);
+    k_obs_prep<W><<<1, 1024, 0, st>>>(ox, oz, m, tsize, tab, first, vals, s.ctl);
     k_obs_scan<W><<<grid_for(s, s.buf_cap, 256, 8), 256, 0, st>>>(
         bufsa_of<W>(s), s.ctl, ox, oz, tsize, tab, vals);
     k_obs_reduce<<<1, 256, 0, st>>>(m, first, vals, ow, out);

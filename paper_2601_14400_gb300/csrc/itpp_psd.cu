@@ -16,7 +16,10 @@
 // table (under a generation of its own), then one pass over the state
 // looks up O_j.P for every commuting observable string.  Sums are
 // compensated per thread, then reduced in a fixed order, so the result does
-// not depend on scheduling.
+// not depend on scheduling.  Few of the strings O_j.P are in the state (a few in
+// a hundred for the chains), so a bitmap of the state's hashes, about 8 to 16
+// bits a term, is asked first: a 4-byte read that mostly hits L1 instead of a
+// random 32- or 64-byte table slot.
 #include "itpp_common.cuh"
 #include "itpp_gate_body.cuh"
 #include "itpp_launch.h"
@@ -38,27 +41,55 @@ static Bufs<W> psd_bufs(const DeviceState& s) {
 }
 
 // A fresh table generation for the state's terms (never equal to a gate's).
-__global__ void k_psd_begin(DevCtl* ctl) {
-    if (threadIdx.x != 0 || ctl->status) return;
+// Clears the filter.
+template <int W>
+__global__ void k_psd_begin(Bufs<W> B, DevCtl* ctl, size_t fbytes) {
+    if (ctl->status) return;
+    uint4* f = reinterpret_cast<uint4*>(B.key(ctl->cur ^ 1));
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < fbytes / 16;
+         i += (size_t)gridDim.x * blockDim.x)
+        f[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (blockIdx.x != 0 || threadIdx.x != 0) return;
     ctl->gen = ctl->gen + 1u;
     if (ctl->gen == 0u) set_status(ctl, ST_STATE, 60);
 }
 
-// Every term of the state, normalised, into the table.
+// Bits of the filter for n terms: the power of two between 8 and 16 a term.
+__device__ __forceinline__ uint32_t filter_shift(uint64_t n) {
+    int b = 64 - __clzll((long long)(n | 7ULL));   // n < 2^b
+    b += 3;
+    return 32u - (uint32_t)(b < 31 ? b : 31);        // the hash's top bits
+}
+
+template <int W>
+__device__ __forceinline__ uint32_t filter_hash(const PKey<W>& K) {
+    uint32_t h = 0x51ed270bu;
+#pragma unroll
+    for (int w = 0; w < W; ++w)
+        h = h * 0x2c1b3c6du + (uint32_t)K.x[w] * 0x9e3779b1u + (uint32_t)(K.x[w] >> 32) * 0x85ebca77u +
+            (uint32_t)K.z[w] * 0xc2b2ae3du + (uint32_t)(K.z[w] >> 32) * 0x27d4eb2fu;
+    return h;
+}
+
+// Every term of the state, normalised, into the table and the filter.
 template <int W>
 __global__ void __launch_bounds__(kPB)
 k_psd_build(Bufs<W> B, DevCtl* ctl, Slot<W>* table, uint64_t slots, int load_pct,
             int probe_limit) {
     if (ctl->status) return;
     const int cur = ctl->cur;
+    uint32_t* filter = reinterpret_cast<uint32_t*>(B.key(cur ^ 1));
     const uint64_t n = live_count(ctl, cur);
     const double rnorm = ctl->rnorm[cur];
     const unsigned gen = ctl->gen;
     const uint64_t mask = table_mask(n, slots, load_pct);
+    const uint32_t fs = filter_shift(n);
     int probes = 0;
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (uint64_t)gridDim.x * blockDim.x) {
         const PKey<W> K = load_key(B.key(cur) + i);
+        const uint32_t fb = filter_hash(K) >> fs;
+        atomicOr(filter + (fb >> 5), 1u << (fb & 31u));
         const double c = normalised(B.coef(cur)[i], rnorm, key_is_zero(K));
         if (!table_insert(table, mask, gen, K, c, (uint32_t)i, probe_limit, &probes))
             set_status(ctl, ST_HASH_PROBE, 61);
@@ -70,6 +101,23 @@ __device__ __forceinline__ void kahan_add(double& s, double& comp, double v) {
     const double t = __dadd_rn(s, y);
     comp = __dsub_rn(__dsub_rn(t, s), y);
     s = t;
+}
+
+constexpr int kObs = 8;   // observable strings looked up together
+
+template <int W>
+__device__ __forceinline__ GateArg<W> obs_gate(const uint64_t* __restrict__ ox,
+                                               const uint64_t* __restrict__ oz, int j) {
+    GateArg<W> o;
+    int yy = 0;
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+        o.qx[w] = __ldg(ox + (size_t)j * W + w);
+        o.qz[w] = __ldg(oz + (size_t)j * W + w);
+        yy += __popcll(o.qx[w] & o.qz[w]);
+    }
+    o.qyy = yy & 3;
+    return o;
 }
 
 // One pass over the state: purity and the commuting-pair overlap; per-block
@@ -87,29 +135,37 @@ k_psd_pairs(Bufs<W> B, DevCtl* ctl, const Slot<W>* table, uint64_t slots, int lo
         const double rnorm = ctl->rnorm[cur];
         const unsigned gen = ctl->gen;
         const uint64_t mask = table_mask(n, slots, load_pct);
+        const uint32_t* __restrict__ filter = reinterpret_cast<const uint32_t*>(B.key(cur ^ 1));
+        const uint32_t fs = filter_shift(n);
         int probes = 0;
         for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
              i += (uint64_t)gridDim.x * blockDim.x) {
             const PKey<W> P = load_key(B.key(cur) + i);
             const double cp = normalised(B.coef(cur)[i], rnorm, key_is_zero(P));
             kahan_add(den, cd, __dmul_rn(cp, cp));
-            for (int j = 0; j < m; ++j) {
-                GateArg<W> o;
-                int yy = 0;
+            for (int j0 = 0; j0 < m; j0 += kObs) {
+                // the filter's words of a group of strings, all in flight
+                uint32_t word[kObs], bit[kObs];
 #pragma unroll
-                for (int w = 0; w < W; ++w) {
-                    o.qx[w] = __ldg(ox + (size_t)j * W + w);
-                    o.qz[w] = __ldg(oz + (size_t)j * W + w);
-                    yy += __popcll(o.qx[w] & o.qz[w]);
+                for (int u = 0; u < kObs; ++u) {
+                    const int j = j0 + u < m ? j0 + u : m - 1;
+                    const GateArg<W> o = obs_gate<W>(ox, oz, j);
+                    const uint32_t fb = filter_hash(key_xor(P, o)) >> fs;
+                    bit[u] = 1u << (fb & 31u);
+                    word[u] = 0u;
+                    if (j0 + u < m && commutes(P, o)) word[u] = __ldg(filter + (fb >> 5));
                 }
-                o.qyy = yy & 3;
-                if (!commutes(P, o)) continue;
-                double cr;
-                if (!table_find(table, mask, gen, key_xor(P, o), &cr, probe_limit, ctl, &probes))
-                    continue;
-                const double pair = __dmul_rn(cp, cr);
-                const double v = __dmul_rn(__ldg(ow + j), pair);
-                kahan_add(num, cn, product_negative(P, o) ? -v : v);
+#pragma unroll
+                for (int u = 0; u < kObs; ++u) {
+                    if (!(word[u] & bit[u])) continue;
+                    const GateArg<W> o = obs_gate<W>(ox, oz, j0 + u);
+                    double cr;
+                    if (!table_find(table, mask, gen, key_xor(P, o), &cr, probe_limit, ctl, &probes))
+                        continue;
+                    const double pair = __dmul_rn(cp, cr);
+                    const double v = __dmul_rn(__ldg(ow + j0 + u), pair);
+                    kahan_add(num, cn, product_negative(P, o) ? -v : v);
+                }
             }
         }
     }
@@ -129,18 +185,42 @@ k_psd_pairs(Bufs<W> B, DevCtl* ctl, const Slot<W>* table, uint64_t slots, int lo
     }
 }
 
-// The blocks' partials in block order (compensated); the ratio; the next
-// gate gets a fresh table generation.
-__global__ void k_psd_final(DevCtl* ctl, const double* partials, int n_part, double* out) {
-    if (threadIdx.x != 0) return;
+// The blocks' partials, compensated per thread over a fixed stride, then in a
+// fixed tree (one thread adding 1,216 of them in turn took 376 us: every step
+// of a compensated sum waits for the last); the ratio; the next gate gets a
+// fresh table generation.
+__global__ void __launch_bounds__(kPB)
+k_psd_final(DevCtl* ctl, const double* partials, int n_part, double* out) {
+    __shared__ double s_s[2][kPB], s_c[2][kPB];
     double num = 0.0, cn = 0.0, den = 0.0, cd = 0.0;
-    for (int b = 0; b < n_part; ++b) {
+    for (int b = threadIdx.x; b < n_part; b += kPB) {
         kahan_add(num, cn, partials[2 * b]);
         kahan_add(den, cd, partials[2 * b + 1]);
     }
-    out[0] = __ddiv_rn(num, den);
-    out[1] = num;
-    out[2] = den;
+    s_s[0][threadIdx.x] = num;
+    s_c[0][threadIdx.x] = cn;
+    s_s[1][threadIdx.x] = den;
+    s_c[1][threadIdx.x] = cd;
+    __syncthreads();
+    for (int o = kPB / 2; o > 0; o >>= 1) {
+        if (threadIdx.x < o) {
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                // add (sum_b - comp_b) into (sum_a, comp_a), one compensated step
+                const double a = s_s[k][threadIdx.x];
+                const double y = __dsub_rn(s_s[k][threadIdx.x + o],
+                                           __dadd_rn(s_c[k][threadIdx.x], s_c[k][threadIdx.x + o]));
+                const double t = __dadd_rn(a, y);
+                s_c[k][threadIdx.x] = __dsub_rn(__dsub_rn(t, a), y);
+                s_s[k][threadIdx.x] = t;
+            }
+        }
+        __syncthreads();
+    }
+    if (threadIdx.x != 0) return;
+    out[0] = __ddiv_rn(s_s[0][0], s_s[1][0]);
+    out[1] = s_s[0][0];
+    out[2] = s_s[1][0];
     if (!ctl->status) {
         ctl->gen = ctl->gen + 1u;
         if (ctl->gen == 0u) set_status(ctl, ST_STATE, 62);
@@ -156,14 +236,18 @@ static cudaError_t psd_w(const DeviceState& s, const uint64_t* d_ox, const uint6
     const size_t slot = W == 1 ? 32 : 64;
     cudaError_t e = cudaMemsetAsync(s.table, 0, (size_t)s.table_slots * slot, st);
     if (e != cudaSuccess) return e;
-    k_psd_begin<<<1, 32, 0, st>>>(s.ctl);
+    // the filter lies in the other buffer's keys, free between gates: two bytes
+    // a term at most, and those hold 16 or more (which of the two is the other
+    // one the device knows)
+    const size_t fbytes = ((size_t)s.cap_M * 2 + 15) / 16 * 16;
+    k_psd_begin<<<s.num_sms * 4, 256, 0, st>>>(psd_bufs<W>(s), s.ctl, fbytes);
     Slot<W>* table = static_cast<Slot<W>*>(s.table);
     k_psd_build<W><<<s.num_sms * 8, kPB, 0, st>>>(psd_bufs<W>(s), s.ctl, table, s.table_slots,
                                                  s.load_pct, s.probe_limit);
     k_psd_pairs<W><<<n_part, kPB, 0, st>>>(psd_bufs<W>(s), s.ctl, table, s.table_slots,
                                           s.load_pct, s.probe_limit, d_ox, d_oz, d_ow, m,
                                           d_partials);
-    k_psd_final<<<1, 32, 0, st>>>(s.ctl, d_partials, n_part, d_out);
+    k_psd_final<<<1, kPB, 0, st>>>(s.ctl, d_partials, n_part, d_out);
     return cudaGetLastError();
 }
 
