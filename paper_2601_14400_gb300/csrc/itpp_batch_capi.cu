@@ -1,6 +1,8 @@
 // itpp_batch_capi.cu -- C ABI of the batched propagation (include/itpp.h):
-// many independent ITPP instances advanced in shared launches, one CUDA
-// graph per Trotter layer.
+// many independent ITPP instances advanced together: a team of CTAs per
+// instance in one launch (merge_path 0), or shared launches replayed as one CUDA
+// graph per Trotter layer (merge_path 2).
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <new>
@@ -9,6 +11,7 @@
 #include "itpp.h"
 #include "itpp_common.cuh"
 #include "itpp_launch.h"
+#include "itpp_run.cuh"
 
 using namespace itpp;
 
@@ -26,6 +29,14 @@ struct itpp_batch_ctx {
     uint64_t launches = 0;
     std::vector<unsigned char> h_ctl;   // one DevCtl head, for reads
     int load_floor = 50;                // lowest table load the allocation allows
+    // run kernel: gates, sites, teams, their shared blocks, threshold drifts
+    void* run_gates = nullptr;          // RunGate<W>[B * max_gates]
+    int* run_sites = nullptr;           // [B]
+    uint4* run_teams = nullptr;         // [grid]
+    void* run_shared = nullptr;
+    long long* run_drift = nullptr;     // [B * (max_gates + 1)]
+    int run_grid = 0, run_n_teams = 0, run_fit_ctas = 0;
+    int max_weight = 0;
     bool target_fixed = false;          // partition size given by the caller
 };
 
@@ -33,6 +44,7 @@ namespace {
 
 constexpr size_t kHead = offsetof(DevCtl, sel_hist);
 constexpr int kTargetMin = 150;   // smallest mean partition size the autotuner tries
+constexpr int kMinPartMin = 64;   // smallest lower limit of it
 
 uint64_t next_pow2(uint64_t v) {
     uint64_t s = 1;
@@ -60,6 +72,11 @@ void free_batch(itpp_batch_ctx* h) {
     if (s.part_keys) cudaFree(s.part_keys);
     if (s.part_coef) cudaFree(s.part_coef);
     if (s.part_cursor) cudaFree(s.part_cursor);
+    if (h->run_gates) cudaFree(h->run_gates);
+    if (h->run_sites) cudaFree(h->run_sites);
+    if (h->run_teams) cudaFree(h->run_teams);
+    if (h->run_shared) cudaFree(h->run_shared);
+    if (h->run_drift) cudaFree(h->run_drift);
     if (s.ctls) cudaFree(s.ctls);
     if (s.gates) cudaFree(s.gates);
     if (s.n_gates) cudaFree(s.n_gates);
@@ -123,30 +140,131 @@ itpp_status read_head(itpp_batch_ctx* h, int b, DevCtl* out) {
     return ITPP_OK;
 }
 
-// Reset every instance to the identity (statistics cleared, partition
-// cursors zero).
+// Reset every instance to the identity (statistics cleared).
 itpp_status reset_all(itpp_batch_ctx* h) {
     const BatchState& s = h->s;
-    if (s.part_cursor &&
-        cudaMemsetAsync(s.part_cursor, 0, (size_t)s.B * s.part_max * sizeof(unsigned int),
-                        h->stream) != cudaSuccess)
-        return ITPP_ERR_CUDA;
     for (int b = 0; b < s.B; ++b)
         if (launch_reset_identity(view(h, b), h->stream) != cudaSuccess) return ITPP_ERR_CUDA;
     return ITPP_OK;
 }
 
-// The partition merge's CTAs per SM: the requested count, at most what fits
-// at the current block size (0: what fits).
-void fit_merge(BatchState& s, int want) {
-    const int fit = batch_merge_fit(s.W, s.main_block);
-    s.merge_ctas = (want > 0 && want < fit) ? want : fit;
+// Which CTAs work on which instance: every instance its team, of a size in
+// proportion to its gates (a layer ends with the slowest team), at most one
+// CTA per smallest partition; with more instances than CTAs every CTA is a
+// team and takes one instance after another.
+itpp_status plan_teams(itpp_batch_ctx* h) {
+    const BatchState& s = h->s;
+    const int per_sm = s.team_ctas > 0 && s.team_ctas < h->run_fit_ctas ? s.team_ctas : h->run_fit_ctas;
+    const long long ctas = (long long)s.num_sms * per_sm;
+    std::vector<uint4> t;
+    if ((long long)s.B >= ctas) {
+        for (long long c = 0; c < ctas; ++c)
+            t.push_back(make_uint4((unsigned)c, 0u, 1u, (unsigned)ctas));
+        h->run_n_teams = (int)ctas;
+    } else {
+        long long sum = 0;
+        for (int g : h->n_gates) sum += g;
+        const long long most = (long long)(s.cap_M / (uint64_t)s.min_part) + 1;
+        for (int b = 0; b < s.B; ++b) {
+            long long size = 1 + (sum ? (ctas - s.B) * h->n_gates[(size_t)b] / sum : 0);
+            size = std::min(size, most);
+            for (long long r = 0; r < size; ++r)
+                t.push_back(make_uint4((unsigned)b, (unsigned)r, (unsigned)size, (unsigned)s.B));
+        }
+        h->run_n_teams = s.B;
+    }
+    h->run_grid = (int)t.size();
+    return cudaMemcpyAsync(h->run_teams, t.data(), t.size() * sizeof(uint4), cudaMemcpyHostToDevice,
+                           h->stream) == cudaSuccess &&
+                   cudaStreamSynchronize(h->stream) == cudaSuccess
+               ? ITPP_OK : ITPP_ERR_CUDA;
+}
+
+// n_layers layers of every instance in one launch.
+template <int W>
+itpp_status run_batch(itpp_batch_ctx* h, int n_layers) {
+    const BatchState& s = h->s;
+    RunArgs<W> a{};
+    for (int i = 0; i < 2; ++i) {
+        a.k[i] = static_cast<PKey<W>*>(s.keys[i]);
+        a.c[i] = s.coef[i];
+    }
+    a.kp = static_cast<PKey<W>*>(s.part_keys);
+    a.cp = s.part_coef;
+    a.cnt = s.part_cursor;
+    a.ctl = s.ctls;
+    a.scratch = s.table;
+    a.shared = h->run_shared;
+    a.drift = h->run_drift;
+    a.n = h->run_sites;
+    a.gates = static_cast<const RunGate<W>*>(h->run_gates);
+    a.n_gates = s.n_gates;
+    a.team_of = h->run_teams;
+    a.buf_stride = s.buf_cap;
+    a.part_stride = s.part_cap;
+    a.scratch_stride = s.table_slots * (W == 1 ? 32 : 64);
+    a.shared_stride = run_shared_bytes();
+    a.buf_cap = s.buf_cap;
+    a.home_cap = std::min(s.part_cap, s.buf_cap);
+    a.cand_cap = std::min<uint64_t>(a.scratch_stride / (12 + sizeof(PKey<W>)) - 64, a.home_cap);
+    a.tie_off = (a.cand_cap * 12 + 255) / 256 * 256;
+    a.cap_M = s.cap_M;
+    a.cand_hi = std::max<uint64_t>(1024, s.cap_M / 16);
+    std::memcpy(&a.delta_bits, &s.delta, sizeof a.delta_bits);
+    a.part_max = s.part_max;
+    a.drift_stride = s.max_gates + 1;
+    a.drift_gates = s.max_gates;
+    a.B = s.B;
+    a.max_gates = s.max_gates;
+    a.n_layers = n_layers;
+    a.target = s.part_target;
+    a.min_part = s.min_part;
+    a.cap_policy = s.cap_policy;
+    a.maxw = h->max_weight ? h->max_weight : (1 << 30);
+    static const RunChunk<W> none{};
+    if (cudaMemset2DAsync(h->run_shared, a.shared_stride, 0, run_shared_head(),
+                          (size_t)h->run_n_teams, h->stream) != cudaSuccess ||
+        launch_run<W>(a, none, h->run_grid, h->stream) != cudaSuccess) {
+        cudaGetLastError();
+        return ITPP_ERR_CUDA;
+    }
+    h->launches += 1;
+    return ITPP_OK;
+}
+
+itpp_status run_layers(itpp_batch_ctx* h, int n_layers) {
+    // at most a few thousand gates a launch (it holds the GPU's CTA slots)
+    const int most = std::max(1, 4096 / std::max(1, h->s.max_gates));
+    for (int l = 0; l < n_layers && h->s.max_gates > 0; l += most) {
+        const int nl = std::min(most, n_layers - l);
+        const itpp_status st = h->s.W == 1 ? run_batch<1>(h, nl) : run_batch<2>(h, nl);
+        if (st) return st;
+    }
+    return ITPP_OK;
+}
+
+// The gates of every instance with the windows that start at each.
+template <int W>
+void fill_run_gates(RunGate<W>* dst, int max_g, const GateArg<W>* src, const std::vector<int>& n) {
+    for (size_t b = 0; b < n.size(); ++b) {
+        RunGate<W>* g = dst + b * (size_t)max_g;
+        for (int j = 0; j < n[b]; ++j) {
+            const GateArg<W>& q = src[b * (size_t)max_g + (size_t)j];
+            for (int w = 0; w < W; ++w) {
+                g[j].qx[w] = q.qx[w];
+                g[j].qz[w] = q.qz[w];
+            }
+            g[j].ch = q.ch;
+            g[j].msh = q.msh;
+        }
+        plan_run_windows(g, n[b]);
+    }
 }
 
 // Capture one Trotter layer (every gate step, all instances per launch) as
 // the handle's graph, if it has none.
 itpp_status capture_layer(itpp_batch_ctx* h) {
-    if (h->layer) return ITPP_OK;
+    if (h->layer || h->s.merge_path == 0) return ITPP_OK;
     cudaGraph_t g = nullptr;
     if (cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess)
         return ITPP_ERR_CUDA;
@@ -178,7 +296,8 @@ itpp_status time_shape(itpp_batch_ctx* h, int probe_layers, double* ms) {
     if (cudaEventCreate(&a) != cudaSuccess) return ITPP_ERR_CUDA;
     if (cudaEventCreate(&b) != cudaSuccess) { cudaEventDestroy(a); return ITPP_ERR_CUDA; }
     cudaEventRecord(a, h->stream);
-    for (int l = 0; l < probe_layers; ++l) cudaGraphLaunch(h->layer, h->stream);
+    if (h->s.merge_path == 0) run_layers(h, probe_layers);
+    else for (int l = 0; l < probe_layers; ++l) cudaGraphLaunch(h->layer, h->stream);
     cudaEventRecord(b, h->stream);
     float f = 0.f;
     const bool ok = cudaEventSynchronize(b) == cudaSuccess &&
@@ -246,20 +365,22 @@ itpp_status itpp_batch_create(int B, const int* n, const int* n_gates, const uin
     s.cap_M = p->cap_M;
     s.buf_cap = 2 * p->cap_M;
     s.cap_policy = p->cap_policy;
+    h->max_weight = p->max_weight;
     s.merge_path = p->merge_path;
     s.delta = p->delta + 0.0;   // -0 becomes +0 (the threshold compares bit patterns)
     s.load_pct = p->table_load_pct ? p->table_load_pct : 50;
     if (s.load_pct < 10 || s.load_pct > 75) { free_batch(h); delete h; return ITPP_ERR_ARG; }
     if (s.merge_path == 0) {
-        // scatter buffer per instance (even: a staging copy may start one
-        // element below an odd partition start); cursors for the smallest
-        // partition size the autotuner tries
+        // a home per instance, and cursors for the smallest partition sizes the
+        // autotuner tries
         h->target_fixed = p->partition_target != 0;
         s.part_target = p->partition_target ? p->partition_target : partition_target_default(W);
+        s.min_part = kRunMinPart;
         s.part_cap = 2 * p->cap_M + p->cap_M / 2 + 4096;
         s.part_cap += s.part_cap & 1ULL;
-        const int t_min = h->target_fixed ? s.part_target : kTargetMin;
-        s.part_max = partition_max(p->cap_M, t_min < s.part_target ? t_min : s.part_target);
+        const int t_min = std::min(h->target_fixed ? s.part_target : kTargetMin, s.part_target);
+        s.part_max = partition_max(p->cap_M, t_min) + 1;
+        h->run_fit_ctas = run_fit(W);
     }
     // auto sizing leaves room for the autotuner to try loads down to 25 %
     const int load_for_size = p->table_load_pct ? (s.load_pct < 50 ? s.load_pct : 50) : 25;
@@ -270,6 +391,10 @@ itpp_status itpp_batch_create(int B, const int* n, const int* n_gates, const uin
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     s.num_sms = sms;
+    if (s.merge_path == 0)   // a partition for every CTA of a team
+        s.part_max = (uint32_t)std::max<uint64_t>(
+            s.part_max, std::min<uint64_t>((uint64_t)sms * h->run_fit_ctas,
+                                           p->cap_M / (uint64_t)kMinPartMin + 1) + 1);
 
     const size_t gsz = W == 1 ? sizeof(GateArg<1>) : sizeof(GateArg<2>);
     std::vector<unsigned char> gates((size_t)B * (max_g > 0 ? max_g : 1) * gsz, 0);
@@ -295,7 +420,20 @@ itpp_status itpp_batch_create(int B, const int* n, const int* n_gates, const uin
         ok &= ok && cudaMalloc(reinterpret_cast<void**>(&s.part_coef),
                                ((size_t)B * s.part_cap + 2) * 8) == cudaSuccess;
         ok &= ok && cudaMalloc(reinterpret_cast<void**>(&s.part_cursor),
-                               (size_t)B * s.part_max * sizeof(unsigned int)) == cudaSuccess;
+                               (size_t)B * 3 * s.part_max * kRunPad * sizeof(unsigned int)) ==
+                        cudaSuccess;
+        const size_t ctas = (size_t)sms * h->run_fit_ctas;
+        const size_t rg = W == 1 ? sizeof(RunGate<1>) : sizeof(RunGate<2>);
+        const size_t nd = (size_t)B * (max_g + 1) * sizeof(long long);
+        ok &= ok && cudaMalloc(&h->run_gates, (size_t)B * (max_g > 0 ? max_g : 1) * rg) == cudaSuccess;
+        ok &= ok && cudaMalloc(reinterpret_cast<void**>(&h->run_sites), (size_t)B * sizeof(int)) ==
+                        cudaSuccess;
+        ok &= ok && cudaMalloc(reinterpret_cast<void**>(&h->run_teams), ctas * sizeof(uint4)) ==
+                        cudaSuccess;
+        ok &= ok && cudaMalloc(&h->run_shared, std::min<size_t>(ctas, (size_t)B) *
+                                                   run_shared_bytes()) == cudaSuccess;
+        ok &= ok && cudaMalloc(reinterpret_cast<void**>(&h->run_drift), nd) == cudaSuccess;
+        ok &= ok && cudaMemsetAsync(h->run_drift, 0, nd, h->stream) == cudaSuccess;
     }
     ok &= ok && cudaMalloc(reinterpret_cast<void**>(&s.ctls), (size_t)B * sizeof(DevCtl)) == cudaSuccess;
     ok &= ok && cudaMalloc(&s.gates, gates.size()) == cudaSuccess;
@@ -316,10 +454,21 @@ itpp_status itpp_batch_create(int B, const int* n, const int* n_gates, const uin
     ok &= cudaMemsetAsync(s.table, 0, (size_t)B * s.table_slots * slot, h->stream) == cudaSuccess;
     ok &= cudaMemsetAsync(s.ctls, 0, (size_t)B * sizeof(DevCtl), h->stream) == cudaSuccess;
     ok &= cudaMemsetAsync(s.item_prefix, 0, 4 * (size_t)(B + 1) * sizeof(unsigned long long), h->stream) == cudaSuccess;
-    if (s.merge_path == 0) {
-        ok &= cudaMemsetAsync(s.part_cursor, 0, (size_t)B * s.part_max * sizeof(unsigned int),
+    std::vector<unsigned char> rgates;
+    if (s.merge_path == 0 && ok) {
+        const size_t rg = W == 1 ? sizeof(RunGate<1>) : sizeof(RunGate<2>);
+        rgates.assign((size_t)B * (max_g > 0 ? max_g : 1) * rg, 0);
+        if (W == 1)
+            fill_run_gates<1>(reinterpret_cast<RunGate<1>*>(rgates.data()), max_g,
+                              reinterpret_cast<const GateArg<1>*>(gates.data()), h->n_gates);
+        else
+            fill_run_gates<2>(reinterpret_cast<RunGate<2>*>(rgates.data()), max_g,
+                              reinterpret_cast<const GateArg<2>*>(gates.data()), h->n_gates);
+        ok &= cudaMemcpyAsync(h->run_gates, rgates.data(), rgates.size(), cudaMemcpyHostToDevice,
                               h->stream) == cudaSuccess;
-        fit_merge(s, 0);
+        ok &= cudaMemcpyAsync(h->run_sites, n, (size_t)B * sizeof(int), cudaMemcpyHostToDevice,
+                              h->stream) == cudaSuccess;
+        ok &= plan_teams(h) == ITPP_OK;
     }
     for (int b = 0; b < B && ok; ++b) {
         DeviceState d = view(h, b);
@@ -349,6 +498,10 @@ itpp_status itpp_batch_destroy(itpp_batch_handle h) {
 itpp_status itpp_batch_apply_trotter_layer(itpp_batch_handle h, int n_layers) {
     if (!h || n_layers < 0) return ITPP_ERR_ARG;
     if (h->sticky) return h->sticky;
+    if (h->s.merge_path == 0) {
+        const itpp_status st = run_layers(h, n_layers);
+        return st == ITPP_OK ? ITPP_OK : h->sticky = st;
+    }
     // one layer (every gate step, all instances per launch) as a graph
     if (n_layers > 0 && capture_layer(h) != ITPP_OK) return h->sticky = ITPP_ERR_CUDA;
     for (int l = 0; l < n_layers; ++l) {
@@ -363,16 +516,18 @@ itpp_status itpp_batch_autotune(itpp_batch_handle h, int probe_layers, itpp_tune
     if (h->sticky) return h->sticky;
     BatchState& s = h->s;
     const bool part = s.merge_path == 0;
-    // a shape: block, CTAs per SM of the merge (partitioned: 0 = what fits)
-    // or of the branch-emit kernel, CTAs per SM of the scatter or table
-    // build, table load (global table) or mean partition size (partitioned)
+    // a shape: block, CTAs per SM (partitioned: 0 = what fits) or of the
+    // branch-emit kernel, CTAs per SM of the table build or (partitioned) the
+    // smallest mean partition in units of 16 terms, table load (global table)
+    // or mean partition size (partitioned)
     struct Shape { int mb, mg, ig, load, target; };
     auto install = [&](const Shape& c) {
         s.main_block = c.mb;
         if (part) {
-            fit_merge(s, c.mg);
-            s.scatter_grid = c.ig;
+            s.team_ctas = c.mg;
+            s.min_part = 16 * c.ig;
             s.part_target = c.target;
+            plan_teams(h);
         } else {
             s.main_grid = c.mg;
             s.insert_grid = c.ig;
@@ -399,9 +554,9 @@ itpp_status itpp_batch_autotune(itpp_batch_handle h, int probe_layers, itpp_tune
     };
     // one parameter at a time, each from the best shape so far
     const int blocks[3] = {128, 256, 512};
-    for (int v : blocks) if (v != best.mb) { Shape c = best; c.mb = v; if ((st = try_shape(c))) return h->sticky = st; }
+    if (!part) for (int v : blocks) if (v != best.mb) { Shape c = best; c.mb = v; if ((st = try_shape(c))) return h->sticky = st; }
     if (part) {
-        const int mgs[3] = {2, 4, 0}, sgs[3] = {4, 8, 16};
+        const int mgs[4] = {1, 2, 3, 0}, sgs[3] = {4, 8, 16};
         const int t1[4] = {350, 500, 700, 1000}, t2[3] = {150, 300, 450};
         for (int v : mgs) if (v != best.mg) { Shape c = best; c.mg = v; if ((st = try_shape(c))) return h->sticky = st; }
         for (int v : sgs) if (v != best.ig) { Shape c = best; c.ig = v; if ((st = try_shape(c))) return h->sticky = st; }
@@ -431,7 +586,7 @@ itpp_status itpp_batch_autotune(itpp_batch_handle h, int probe_layers, itpp_tune
     if (out) {
         std::memset(out, 0, sizeof(*out));
         out->main_block = best.mb;
-        out->main_grid = part ? s.merge_ctas : best.mg;
+        out->main_grid = part ? (best.mg ? best.mg : h->run_fit_ctas) : best.mg;
         out->insert_grid = best.ig;
         out->table_load_pct = part ? 0 : best.load;
         out->partition_target = part ? best.target : 0;
@@ -475,11 +630,12 @@ itpp_status itpp_batch_get_stats(itpp_batch_handle h, int b, itpp_stats* o) {
     o->cap_events = c->stat_cap;
     o->count = c->count[c->cur];
     o->table_probes = c->stat_probes;
-    o->repartitions = 0;
-    o->select_candidates = 0;
-    o->select_range = 0;
-    o->select_full = 0;
-    o->long_partitions = 0;
+    o->repartitions = c->stat_scatters;
+    o->select_candidates = c->stat_cands;
+    o->select_range = c->stat_range;
+    o->select_full = c->stat_sel_full;
+    o->long_partitions = c->stat_long;
+    o->merge_retries = c->stat_retry;
     o->error_site = c->status ? c->err_info : 0;
     o->kernel_launches = h->launches;
     return (itpp_status)c->status;

@@ -101,22 +101,59 @@ __device__ __forceinline__ void list_if(bool on, uint32_t* count, uint16_t* list
                  : "memory");
 }
 
+// A thread's strings of a pass (row r: string r * BLOCK + thread), zero past the
+// end.
+template <int W, int BLOCK>
+struct InRows {
+    static constexpr int N = InPass<W>::C / BLOCK;
+    PKey<W> K[N];
+    double c[N];
+};
+
+template <int W, int BLOCK, bool kGathered>
+__device__ __forceinline__ void load_rows(InRows<W, BLOCK>& rows, const PKey<W>* keys,
+                                          const double* cin, uint32_t n) {
+    const PKey<W>* kp = keys + threadIdx.x;
+    const double* cp = cin + threadIdx.x;
+#pragma unroll
+    for (int r = 0; r < InRows<W, BLOCK>::N; ++r) {
+#pragma unroll
+        for (int w = 0; w < W; ++w) { rows.K[r].x[w] = 0; rows.K[r].z[w] = 0; }
+        rows.c[r] = 0.0;
+        if (threadIdx.x + r * BLOCK < n) {
+            if (kGathered) {
+                const uint32_t at = InPass<W>::src()[threadIdx.x + r * BLOCK];
+                rows.K[r] = load_key_ca(keys + at);
+                rows.c[r] = cin[at];
+            } else {
+                rows.K[r] = load_key_ca(kp + r * BLOCK);
+                rows.c[r] = cp[r * BLOCK];
+            }
+        }
+    }
+}
+
 // One pass over n >= 1 strings: string i is the partition's i-th, or (kGathered)
-// its src()[i]-th.  *s_app and *s_rare are zero, and a barrier since.  thr: kept
-// is what lies above it; near_hi: kept strings up to this pattern are candidates
-// of the select (0: none), push(hit, pattern - thr - 1, index) takes them
-// (warp-wide).  kPlain: neither the identity's partition nor a weight cutoff
-// nor Q = I.  Three barriers; the shared arrays are free again when it returns.
-template <int W, int BLOCK, bool kGathered, bool kPlain, class Push>
+// its src()[i]-th; rows holds them.  *s_app and *s_rare are zero (seen by every
+// thread after the first barrier here).  thr: kept is what lies above it;
+// near_hi: kept strings up to this pattern are candidates of the select (0:
+// none), push(hit, pattern - thr - 1, index) takes them (warp-wide).  kPlain:
+// neither the identity's partition nor a weight cutoff nor Q = I.  then() is
+// called when the rows are done with and before the rare strings are: the
+// caller loads its next ones there, so that their latency is not waited for.
+// Three barriers; the shared arrays are free again when it returns.
+template <int W, int BLOCK, bool kGathered, bool kPlain, class Push, class Then>
 __device__ __forceinline__ void inplace_pass(uint32_t n, const GateArg<W>& g,
                                              unsigned long long pd_T, bool pd_ties,
                                              const PKey<W>& pd_key, double rnorm,
                                              unsigned long long thr, bool has_id, DevCtl* ctl,
                                              int nxt, uint32_t tag, const InPlace<W>& io,
                                              InStats& st, unsigned long long near_hi,
-                                             Push&& push) {
+                                             InRows<W, BLOCK>& rows, Push&& push, Then&& then) {
     using A = InPass<W>;
-    constexpr int ROWS = A::C / BLOCK, GROUP = ROWS < 4 ? ROWS : 4;
+    constexpr int ROWS = InRows<W, BLOCK>::N;
+    PKey<W>(&K)[ROWS] = rows.K;
+    double(&c)[ROWS] = rows.c;
     // per row: slot (12 bits) | commutes | not the first to arrive in its
     // chain | live, and (special) the identity or past the weight cutoff
     constexpr uint32_t kComm = 1u << 12, kPrev = 1u << 13, kLive = 1u << 14, kSpecial = 1u << 15;
@@ -130,62 +167,35 @@ __device__ __forceinline__ void inplace_pass(uint32_t n, const GateArg<W>& g,
 #pragma unroll
     for (int w = 0; w < W; ++w) qbits |= g.qx[w] | g.qz[w];
     const bool self = !kPlain && qbits == 0;
-    const PKey<W>* kp = io.keys + threadIdx.x;
-    const double* cp = io.cin + threadIdx.x;
-    // A: live strings, normalised values, the chains of shared slots (the
-    // loads of a group of rows first)
-    double c[ROWS];
+    // A: live strings, normalised values, the chains of shared slots
     uint32_t flags[(ROWS + 1) / 2];   // 16 bits a row
 #pragma unroll
     for (int r = 0; r < (ROWS + 1) / 2; ++r) flags[r] = 0u;
 #pragma unroll
-    for (int r0 = 0; r0 < ROWS; r0 += GROUP) {
-        if (r0 * BLOCK + w0 >= n) break;   // whole warps
-        PKey<W> K[GROUP];
-#pragma unroll
-        for (int u = 0; u < GROUP; ++u) {
-            const int r = r0 + u;
-#pragma unroll
-            for (int w = 0; w < W; ++w) { K[u].x[w] = 0; K[u].z[w] = 0; }
-            c[r] = 0.0;
-            if (threadIdx.x + r * BLOCK < n) {
-                if (kGathered) {
-                    const uint32_t at = A::src()[threadIdx.x + r * BLOCK];
-                    K[u] = load_key_ca(io.keys + at);
-                    c[r] = io.cin[at];
-                } else {
-                    K[u] = load_key_ca(kp + r * BLOCK);
-                    c[r] = cp[r * BLOCK];
-                }
+    for (int r = 0; r < ROWS; ++r) {
+        if (r * BLOCK + w0 >= n) break;   // whole warps
+        const unsigned long long b = abs_pattern(c[r]);   // 0 past the end
+        bool live = b > floor_T;
+        if (!pd_ties) live = live && (b != pd_T || !key_less(pd_key, K[r]));
+        c[r] = __dmul_rn(c[r], rnorm);
+        uint32_t f = 0;
+        if (!kPlain) {
+            if (has_id && threadIdx.x + r * BLOCK < n && key_is_zero(K[r])) {
+                c[r] = 1.0;   // the identity's normalised value is exactly 1
+                f = kSpecial;
+                if (!live) set_status(ctl, ST_TRACE_ZERO, 43);
             }
+            if (weigh && !light(K[r], g.maxw)) f = kSpecial;
         }
-#pragma unroll
-        for (int u = 0; u < GROUP; ++u) {
-            const int r = r0 + u;
-            if (r * BLOCK + w0 >= n) break;   // whole warps
-            const unsigned long long b = abs_pattern(c[r]);   // 0 past the end
-            bool live = b > floor_T;
-            if (!pd_ties) live = live && (b != pd_T || !key_less(pd_key, K[u]));
-            c[r] = __dmul_rn(c[r], rnorm);
-            uint32_t f = 0;
-            if (!kPlain) {
-                if (has_id && threadIdx.x + r * BLOCK < n && key_is_zero(K[u])) {
-                    c[r] = 1.0;   // the identity's normalised value is exactly 1
-                    f = kSpecial;
-                    if (!live) set_status(ctl, ST_TRACE_ZERO, 43);
-                }
-                if (weigh && !light(K[u], g.maxw)) f = kSpecial;
-            }
-            const bool comm = live && commutes(K[u], g);
-            const uint32_t slot = A::slot(K[u], g);
-            const uint32_t d = exch_if(comm, A::heads() + slot, me0 + r * BLOCK) ^ (tag << 11);
-            const uint32_t prev = d <= kInPrev ? d : 0u;
-            if (comm) A::next()[threadIdx.x + r * BLOCK] = (uint16_t)prev;
-            f |= comm ? slot | kComm : 0u;
-            f |= prev ? kPrev : 0u;
-            f |= live ? kLive : 0u;
-            flags[r >> 1] |= f << (16 * (r & 1));
-        }
+        const bool comm = live && commutes(K[r], g);
+        const uint32_t slot = A::slot(K[r], g);
+        const uint32_t d = exch_if(comm, A::heads() + slot, me0 + r * BLOCK) ^ (tag << 11);
+        const uint32_t prev = d <= kInPrev ? d : 0u;
+        if (comm) A::next()[threadIdx.x + r * BLOCK] = (uint16_t)prev;
+        f |= comm ? slot | kComm : 0u;
+        f |= prev ? kPrev : 0u;
+        f |= live ? kLive : 0u;
+        flags[r >> 1] |= f << (16 * (r & 1));
     }
     __syncthreads();                                                  // (1) chains built
     // B: every string that is alone in its slot (its partner is absent).
@@ -231,6 +241,7 @@ __device__ __forceinline__ void inplace_pass(uint32_t n, const GateArg<W>& g,
             if (__any_sync(0xffffffffu, hit)) push(hit, a - thr - 1ULL, io.first + at);
         }
     }
+    then();
     __syncthreads();                                                  // (2) the list is complete
     // C: the rare strings, densely (read again)
     const uint32_t n_rare = *io.s_rare;
@@ -312,19 +323,23 @@ __device__ __forceinline__ void inplace_pass(uint32_t n, const GateArg<W>& g,
 
 // A partition of any size up to 65,535 strings: one pass, or its hash classes
 // one after another, each a list of indices (strings and partners agree on
-// the class).  Every thread calls it; *s_app and *s_rare are zero, and a
-// barrier since.  Returns whether it took sub-passes.
-template <int W, int BLOCK, class Push>
+// the class).  Every thread calls it, with the partition in rows when one pass
+// holds it; *s_app and *s_rare are zero.  Returns whether it took sub-passes.
+template <int W, int BLOCK, class Push, class Then>
 __device__ __forceinline__ bool inplace_partition(const GateArg<W>& g, unsigned long long pd_T,
                                                   bool pd_ties, const PKey<W>& pd_key,
                                                   double rnorm, unsigned long long thr,
                                                   bool has_id, DevCtl* ctl, int nxt, uint32_t* tag,
                                                   const InPlace<W>& io, InStats& st,
                                                   unsigned long long near_hi, uint32_t* s_n,
-                                                  Push&& push) {
+                                                  InRows<W, BLOCK>& rows, Push&& push,
+                                                  Then&& then) {
     using A = InPass<W>;
     constexpr uint32_t C = A::C;
-    if (io.n == 0u) return false;
+    if (io.n == 0u) {
+        then();
+        return false;
+    }
     uint64_t qbits = 0;
 #pragma unroll
     for (int w = 0; w < W; ++w) qbits |= g.qx[w] | g.qz[w];
@@ -332,14 +347,16 @@ __device__ __forceinline__ bool inplace_partition(const GateArg<W>& g, unsigned 
     if (io.n <= C) {
         if (plain)
             inplace_pass<W, BLOCK, false, true>(io.n, g, pd_T, pd_ties, pd_key, rnorm, thr, false,
-                                                ctl, nxt, ++*tag, io, st, near_hi, push);
+                                                ctl, nxt, ++*tag, io, st, near_hi, rows, push, then);
         else
-            inplace_pass<W, BLOCK, false, false>(io.n, g, pd_T, pd_ties, pd_key, rnorm, thr, has_id, ctl, nxt,
-                                      ++*tag, io, st, near_hi, push);
+            inplace_pass<W, BLOCK, false, false>(io.n, g, pd_T, pd_ties, pd_key, rnorm, thr, has_id,
+                                                 ctl, nxt, ++*tag, io, st, near_hi, rows, push,
+                                                 then);
         return false;
     }
     if (io.n > 0xffffu) {
         if (threadIdx.x == 0) *io.over = 1;   // the gate is merged again
+        then();
         return true;
     }
     const uint32_t kc = (2u * io.n + C - 1u) / C;
@@ -355,16 +372,18 @@ __device__ __forceinline__ bool inplace_partition(const GateArg<W>& g, unsigned 
         __syncthreads();
         const uint32_t m = *s_n < C ? *s_n : C;
         if (m == 0u) continue;   // uniform
+        load_rows<W, BLOCK, true>(rows, io.keys, io.cin, m);
         inplace_pass<W, BLOCK, true, false>(m, g, pd_T, pd_ties, pd_key, rnorm, thr, has_id, ctl, nxt,
-                                     ++*tag, io, st, near_hi, push);
+                                            ++*tag, io, st, near_hi, rows, push, [] {});
     }
+    then();
     return true;
 }
 
 // CTAs per SM that the in-place merge's launch bound asks for.
 template <int W, int BLOCK>
 struct InOcc {
-    static constexpr int kMin = BLOCK <= 128 ? 8 : BLOCK == 256 ? 5 : 2;
+    static constexpr int kMin = BLOCK <= 128 ? 6 : BLOCK == 256 ? 4 : 2;
 };
 
 // Heads clear of an earlier use of the shared memory, or of a tag that comes

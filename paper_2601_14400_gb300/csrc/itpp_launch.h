@@ -148,25 +148,21 @@ struct BatchState {
     // launch shape (autotuned): branch-emit block (x2 items per thread), grid
     // multipliers (CTAs per SM) of the branch-emit and table-build kernels
     int main_block = 256, main_grid = 4, insert_grid = 8;
-    // merge_path 0 (partitioned merge): per instance a scatter buffer of
-    // part_cap terms in at most part_max pair-key partitions; the merge's
-    // CTAs per SM (0: as many as fit) and the scatter's, and the mean
-    // partition size (autotuned); merge_path 2: the global table above
+    // merge_path 0 (the run kernel, a team of CTAs per instance): per instance
+    // a home of part_cap terms, at most part_max partitions of mean size
+    // part_target (at least min_part where the team would be idle), CTAs per SM
+    // (0: as many as fit); merge_path 2: the global table above
     int merge_path = 0;
     void* part_keys = nullptr;                    // [B * part_cap] keys
     double* part_coef = nullptr;                  // [B * part_cap + 2]
-    unsigned int* part_cursor = nullptr;          // [B * part_max]
+    unsigned int* part_cursor = nullptr;          // [B * 3 * part_max], padded
     uint64_t part_cap = 0;
     uint32_t part_max = 0;
-    int part_target = 0, merge_ctas = 0, scatter_grid = 8;
+    int part_target = 0, min_part = 0, team_ctas = 0;
 };
 
 // Gate `step` of the layer for every instance that has one.
 cudaError_t launch_batch_step(const BatchState& s, int step, cudaStream_t st);
-// CTAs per SM of the batch's partition merge that fit, for W mask words and
-// `block` threads per CTA (sets the kernel's shared-memory attributes: call
-// it before capturing a layer).
-int batch_merge_fit(int W, int block);
 int batch_step_launches(const BatchState& s);
 
 }  // namespace itpp

@@ -147,7 +147,7 @@ __device__ __forceinline__ GateInput gate_input(const DevCtl* ctl) {
 template <int W, int BLOCK>
 __global__ void __launch_bounds__(BLOCK, (InOcc<W, BLOCK>::kMin))
 k_gate_inplace(Bufs<W> B, Homes<W> H, DevCtl* ctl, GateArg<W> g, double delta, CandRegions cd) {
-    using A = InPass<W>;
+    constexpr uint32_t C = InPass<W>::C;
     __shared__ unsigned long long s_T, s_thr, s_kept;
     __shared__ PKey<W> s_tk;
     __shared__ double s_rnorm;
@@ -171,6 +171,7 @@ k_gate_inplace(Bufs<W> B, Homes<W> H, DevCtl* ctl, GateArg<W> g, double delta, C
         s_kept = 0ULL;
         s_long = 0u;
         s_over = 0;
+        s_app = s_rare = 0u;
         const unsigned long long dbits = (unsigned long long)__double_as_longlong(delta);
         const unsigned long long thr = ctl->sp_hi && ctl->sp_thr > dbits ? ctl->sp_thr : dbits;
         s_thr = thr;
@@ -199,10 +200,19 @@ k_gate_inplace(Bufs<W> B, Homes<W> H, DevCtl* ctl, GateArg<W> g, double delta, C
     };
     InStats st{0u, 0u};
     uint32_t tag = 0;
-    uint32_t np = blockIdx.x < in.P ? cnt_in[blockIdx.x] : 0u;
+    InRows<W, BLOCK> rows;
+    auto stored = [&](uint32_t p) -> uint32_t {
+        const uint32_t c = p < in.P ? cnt_in[p] : 0u;
+        return c < R ? c : (uint32_t)R;
+    };
+    auto load = [&](uint32_t p, uint32_t n) {   // (a longer one is gathered later)
+        if (n && n <= C) load_rows<W, BLOCK, false>(rows, keys + (uint64_t)p * R, cin + (uint64_t)p * R, n);
+    };
+    uint32_t np = stored(blockIdx.x), np2 = stored(blockIdx.x + gridDim.x);
+    load(blockIdx.x, np);
     for (uint32_t p = blockIdx.x; p < in.P; p += gridDim.x) {
         InPlace<W> io;
-        io.n = np < R ? np : (uint32_t)R;
+        io.n = np;
         io.room = (uint32_t)(R < 0xffffffffULL ? R : 0xffffffffULL);
         io.first = (uint64_t)p * R;
         io.keys = keys + io.first;
@@ -211,31 +221,30 @@ k_gate_inplace(Bufs<W> B, Homes<W> H, DevCtl* ctl, GateArg<W> g, double delta, C
         io.s_app = &s_app;
         io.s_rare = &s_rare;
         io.over = &s_over;
-        // warm L2 with the partition this CTA takes next
-        const uint32_t pn = p + gridDim.x;
-        np = pn < in.P ? cnt_in[pn] : 0u;
-        if (threadIdx.x == 0) {
-            s_app = s_rare = 0u;
-            const uint64_t nn = np < R ? np : R;
-            if (nn) {
-                l2_prefetch_bulk(keys + (uint64_t)pn * R, nn * sizeof(PKey<W>));
-                l2_prefetch_bulk(cin + (uint64_t)pn * R, nn * sizeof(double));
-            }
+        // warm L2 with the partition after the next
+        const uint32_t pn = p + gridDim.x, pf = pn + gridDim.x;
+        np = np2;
+        np2 = stored(pf);
+        if (threadIdx.x == 0 && np2) {
+            l2_prefetch_bulk(keys + (uint64_t)pf * R, np2 * sizeof(PKey<W>));
+            l2_prefetch_bulk(cin + (uint64_t)pf * R, np2 * sizeof(double));
         }
-        __syncthreads();
         const bool subs = inplace_partition<W, BLOCK>(g, s_T, s_ties != 0, s_tk, s_rnorm, s_thr,
                                                       p == p_id, ctl, nxt, &tag, io, st,
-                                                      g_range[1], &s_n, push);
+                                                      g_range[1], &s_n, rows, push,
+                                                      [&] { load(pn, np); });
         if (threadIdx.x == 0) {
+            // (the others use these again only after the next pass's barrier)
             const uint64_t c = (uint64_t)io.n + s_app;
             cnt_out[p] = (unsigned int)(c < R ? c : R);
+            s_app = s_rare = 0u;
+            if (subs) s_long += 1u;
         }
-        if (subs && threadIdx.x == 0) s_long += 1u;
         if (tag >= kHeadTagMax - 65536u) {   // tags start again
             inplace_init<W, BLOCK>();
             tag = 0;
+            __syncthreads();
         }
-        __syncthreads();
     }
     // one atomic per warp for the largest pattern, one per CTA for the term
     // count

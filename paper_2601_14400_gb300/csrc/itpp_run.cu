@@ -672,7 +672,7 @@ __device__ bool run_instance(const RunArgs<W>& a, const RunGate<W>* gates, int n
     uint32_t* cand_i = reinterpret_cast<uint32_t*>(scr + a.cand_cap * 8);
     PKey<W>* ties = reinterpret_cast<PKey<W>*>(scr + a.tie_off);
     long long* drift = a.drift + (uint64_t)inst * (a.drift_stride);
-    const int n_drift = a.drift_gates;
+    const int n_drift = a.gates ? n_gates : a.drift_gates;
     const int sites = a.n ? a.n[inst] : a.one_n;
 
     const PushList pl{s_cv, s_ci, &s_cn, &s_cs, cand_v, cand_i, nullptr, a.cand_cap};
@@ -723,7 +723,7 @@ __device__ bool run_instance(const RunArgs<W>& a, const RunGate<W>* gates, int n
         if (s_pub.stop) break;          // uniform over the team
         if (threadIdx.x == 0) {
             s_g = gate_arg_of<W>(gates[k], a.maxw);
-            s_cn = s_cs = 0u;
+            s_cn = s_cs = s_app = s_rare = 0u;
             s_over = 0;
         }
         const GateArg<W>& g = s_g;
@@ -813,32 +813,46 @@ __device__ bool run_instance(const RunArgs<W>& a, const RunGate<W>* gates, int n
         // the third cursor array (two gates back) is the next scatter's
         for (uint32_t i = team.rank * kBlock + threadIdx.x; i < a.part_max; i += team.size * kBlock)
             arr.cnt(next3(next3(ci)))[(uint64_t)i * kPad] = 0u;
+        InRows<W, kBlock> rows;
+        auto stored = [&](uint32_t p) -> uint32_t {
+            const uint32_t c = p < P ? __ldcg(arr.cnt(ci) + (uint64_t)p * kPad) : 0u;
+            return c < R ? c : (uint32_t)R;
+        };
+        auto load = [&](uint32_t p, uint32_t n) {   // (a longer one is gathered later)
+            if (n && n <= C)
+                load_rows<W, kBlock, false>(rows, arr.home(hb) + (uint64_t)p * R,
+                                            arr.coef(cx) + (uint64_t)p * R, n);
+        };
+        uint32_t np = stored(team.rank);
         for (uint32_t p = team.rank; p < P; p += team.size) {
-            const uint32_t np = __ldcg(arr.cnt(ci) + (uint64_t)p * kPad);
+            load(p, np);
             InPlace<W> io;
             io.first = (uint64_t)p * R;
             io.keys = arr.home(hb) + io.first;
             io.cin = arr.coef(cx) + io.first;
             io.cout = arr.coef(cx ^ 1) + io.first;
-            io.n = np < R ? np : (uint32_t)R;
+            io.n = np;
             io.room = (uint32_t)(R < 0xffffffffULL ? R : 0xffffffffULL);
             io.s_app = &s_app;
             io.s_rare = &s_rare;
             io.over = &s_over;
-            if (threadIdx.x == 0) s_app = s_rare = 0u;
-            __syncthreads();
+            const uint32_t pn = p + team.size;
+            np = stored(pn);
             if (inplace_partition<W, kBlock>(g, s_pub.T, s_pub.all_ties != 0, tk, s_pub.rnorm, thr,
-                                             p == p_id, ctl, np_, &tag, io, st, s_pub.hi, &s_n, push))
+                                             p == p_id, ctl, np_, &tag, io, st, s_pub.hi, &s_n, rows,
+                                             push, [] {}))
                 ++n_long;
             if (threadIdx.x == 0) {
+                // (the others use these again only after the next pass's barrier)
                 const uint64_t c = (uint64_t)io.n + s_app;
                 arr.cnt(next3(ci))[(uint64_t)p * kPad] = (unsigned int)(c < R ? c : R);
+                s_app = s_rare = 0u;
             }
             if (tag >= kHeadTagMax - 65536u) {   // tags start again
                 inplace_init<W, kBlock>();
                 tag = 0;
+                __syncthreads();
             }
-            __syncthreads();
         }
         // the CTA's counts and candidates
         auto flush = [&](Acc* to, const InStats& s) {
