@@ -19,7 +19,12 @@
 // not depend on scheduling.  Few of the strings O_j.P are in the state (a few in
 // a hundred for the chains), so a bitmap of the state's hashes, about 8 to 16
 // bits a term, is asked first: a 4-byte read that mostly hits L1 instead of a
-// random 32- or 64-byte table slot.
+// random 32- or 64-byte table slot.  What
+// passes it goes on a queue per warp and is looked up and summed 32 at a time: a
+// warp holds the double-precision pipe for every instruction however few of its
+// lanes have a pair (448 us for 2^18 terms and 63 strings when each lane did its
+// own, 190 us this way).  Each pair {P, O_j.P} is taken once, from the member without O_j's
+// lowest bit, and counts twice.
 #include "itpp_common.cuh"
 #include "itpp_gate_body.cuh"
 #include "itpp_launch.h"
@@ -106,6 +111,30 @@ __device__ __forceinline__ void kahan_add(double& s, double& comp, double v) {
 constexpr int kObs = 8;   // observable strings looked up together
 
 template <int W>
+__device__ __forceinline__ bool obs_is_identity(const GateArg<W>& o) {
+    uint64_t q = 0;
+#pragma unroll
+    for (int w = 0; w < W; ++w) q |= o.qx[w] | o.qz[w];
+    return q == 0ULL;
+}
+
+// Of the pair {P, O.P}: the member without O's lowest bit (any P for O = I,
+// which is its own partner).
+template <int W>
+__device__ __forceinline__ bool first_of_pair(const PKey<W>& P, const GateArg<W>& o) {
+    uint64_t bit = 0;
+    bool found = false;
+#pragma unroll
+    for (int w = 0; w < 2 * W; ++w) {
+        const uint64_t q = w < W ? o.qx[w] : o.qz[w - W];
+        const uint64_t k = w < W ? P.x[w] : P.z[w - W];
+        if (!found) bit = k & q & (~q + 1ULL);
+        found = found || q != 0ULL;
+    }
+    return bit == 0ULL;
+}
+
+template <int W>
 __device__ __forceinline__ GateArg<W> obs_gate(const uint64_t* __restrict__ ox,
                                                const uint64_t* __restrict__ oz, int j) {
     GateArg<W> o;
@@ -128,6 +157,8 @@ k_psd_pairs(Bufs<W> B, DevCtl* ctl, const Slot<W>* table, uint64_t slots, int lo
             int probe_limit, const uint64_t* __restrict__ ox, const uint64_t* __restrict__ oz,
             const double* __restrict__ ow, int m, double* partials) {
     __shared__ double s_num[kPB], s_den[kPB];
+    __shared__ uint32_t s_qi[kPB / 32][64];   // queue: term, string
+    __shared__ uint32_t s_qj[kPB / 32][64];
     double num = 0.0, cn = 0.0, den = 0.0, cd = 0.0;
     if (!ctl->status) {
         const int cur = ctl->cur;
@@ -137,37 +168,74 @@ k_psd_pairs(Bufs<W> B, DevCtl* ctl, const Slot<W>* table, uint64_t slots, int lo
         const uint64_t mask = table_mask(n, slots, load_pct);
         const uint32_t* __restrict__ filter = reinterpret_cast<const uint32_t*>(B.key(cur ^ 1));
         const uint32_t fs = filter_shift(n);
+        const uint32_t lane = threadIdx.x & 31u;
+        const unsigned int lt = (1u << lane) - 1u;
+        uint32_t* qi = s_qi[threadIdx.x >> 5];
+        uint32_t* qj = s_qj[threadIdx.x >> 5];
+        uint32_t qn = 0;   // queued, the same on every lane
         int probes = 0;
-        for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-             i += (uint64_t)gridDim.x * blockDim.x) {
-            const PKey<W> P = load_key(B.key(cur) + i);
-            const double cp = normalised(B.coef(cur)[i], rnorm, key_is_zero(P));
-            kahan_add(den, cd, __dmul_rn(cp, cp));
-            for (int j0 = 0; j0 < m; j0 += kObs) {
-                // the filter's words of a group of strings, all in flight
-                uint32_t word[kObs], bit[kObs];
-#pragma unroll
-                for (int u = 0; u < kObs; ++u) {
-                    const int j = j0 + u < m ? j0 + u : m - 1;
-                    const GateArg<W> o = obs_gate<W>(ox, oz, j);
-                    const uint32_t fb = filter_hash(key_xor(P, o)) >> fs;
-                    bit[u] = 1u << (fb & 31u);
-                    word[u] = 0u;
-                    if (j0 + u < m && commutes(P, o)) word[u] = __ldg(filter + (fb >> 5));
-                }
-#pragma unroll
-                for (int u = 0; u < kObs; ++u) {
-                    if (!(word[u] & bit[u])) continue;
-                    const GateArg<W> o = obs_gate<W>(ox, oz, j0 + u);
-                    double cr;
-                    if (!table_find(table, mask, gen, key_xor(P, o), &cr, probe_limit, ctl, &probes))
-                        continue;
-                    const double pair = __dmul_rn(cp, cr);
-                    const double v = __dmul_rn(__ldg(ow + j0 + u), pair);
+        // the first `take` entries of the queue, one per lane
+        auto drain = [&](uint32_t take) {
+            __syncwarp();
+            if (lane < take) {
+                const uint64_t i = qi[lane];
+                const int j = (int)qj[lane];
+                const GateArg<W> o = obs_gate<W>(ox, oz, j);
+                const PKey<W> P = load_key(B.key(cur) + i);
+                double cr;
+                if (table_find(table, mask, gen, key_xor(P, o), &cr, probe_limit, ctl, &probes)) {
+                    const double cp = normalised(B.coef(cur)[i], rnorm, key_is_zero(P));
+                    // (doubling is exact; the identity is its own partner)
+                    const double w = __ldg(ow + j);
+                    const double v = __dmul_rn(obs_is_identity(o) ? w : w + w, __dmul_rn(cp, cr));
                     kahan_add(num, cn, product_negative(P, o) ? -v : v);
                 }
             }
+            __syncwarp();
+            if (lane + take < qn) {
+                qi[lane] = qi[lane + take];   // take is 32 here: the halves are apart
+                qj[lane] = qj[lane + take];
+            }
+            __syncwarp();
+            qn -= take;
+        };
+        // whole warps iterate together
+        for (uint64_t i0 = (uint64_t)blockIdx.x * kPB + (threadIdx.x & ~31u); i0 < n;
+             i0 += (uint64_t)gridDim.x * kPB) {
+            const uint64_t i = i0 + lane;
+            PKey<W> P;
+#pragma unroll
+            for (int w = 0; w < W; ++w) { P.x[w] = 0; P.z[w] = 0; }
+            if (i < n) {
+                P = load_key(B.key(cur) + i);
+                const double cp = normalised(B.coef(cur)[i], rnorm, key_is_zero(P));
+                kahan_add(den, cd, __dmul_rn(cp, cp));
+            }
+            for (int j0 = 0; j0 < m; j0 += kObs) {
+                // the filter's words of a group of strings, all in flight
+                uint32_t word[kObs];
+#pragma unroll
+                for (int u = 0; u < kObs; ++u) {
+                    const GateArg<W> o = obs_gate<W>(ox, oz, j0 + u < m ? j0 + u : m - 1);
+                    const uint32_t fb = filter_hash(key_xor(P, o)) >> fs;
+                    const bool ask = i < n && j0 + u < m && first_of_pair(P, o) && commutes(P, o);
+                    word[u] = ask ? __ldg(filter + (fb >> 5)) >> (fb & 31u) : 0u;
+                }
+#pragma unroll
+                for (int u = 0; u < kObs; ++u) {
+                    const bool hit = word[u] & 1u;
+                    const unsigned int h = __ballot_sync(0xffffffffu, hit);
+                    if (!h) continue;
+                    if (hit) {
+                        qi[qn + __popc(h & lt)] = (uint32_t)i;
+                        qj[qn + __popc(h & lt)] = (uint32_t)(j0 + u);
+                    }
+                    qn += __popc(h);
+                    if (qn >= 32u) drain(32u);
+                }
+            }
         }
+        if (qn) drain(qn);
     }
     s_num[threadIdx.x] = num;
     s_den[threadIdx.x] = den;
