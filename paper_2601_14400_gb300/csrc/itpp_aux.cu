@@ -311,6 +311,9 @@ template <int W>
 static cudaError_t import_w(const DeviceState& s, const uint64_t* x, const uint64_t* z,
                             const double* c, uint64_t count, cudaStream_t st) {
     const int g = grid_for(s, count, 256, 8);
+    // stale contents (the selects keep lists in this memory) must not read as tags
+    cudaError_t e = cudaMemsetAsync(s.table, 0, (size_t)s.table_slots * sizeof(Slot<W>), st);
+    if (e != cudaSuccess) return e;
     k_import_begin<<<1, 32, 0, st>>>(s.ctl, count);
     k_import<W><<<g, 256, 0, st>>>(bufsa_of<W>(s), s.ctl, x, z, c, count, s.n,
                                    reinterpret_cast<Slot<W>*>(s.table), s.table_slots,

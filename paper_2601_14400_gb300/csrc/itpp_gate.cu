@@ -401,10 +401,6 @@ static cudaError_t cap_w(const DeviceState& s, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_cap_select(const DeviceState& s, cudaStream_t st) {
-    return s.W == 1 ? cap_select_w<1>(s, st) : cap_select_w<2>(s, st);
-}
-
 int cap_launches(const DeviceState& s) {
     return s.merge_deferred ? select_deferred_launches(s.W) : 5 * 2 + 1 + 8 * s.W * 2 + 3;
 }

@@ -94,12 +94,14 @@ __device__ __forceinline__ StateRuns<W> state_runs(const DevCtl* ctl, const Bufs
 // ---------------------------------------------------------------------------
 // Merge-table probe
 // ---------------------------------------------------------------------------
-template <int W>
+// kFresh: the table was written in this launch (behind a barrier).
+template <int W, bool kFresh = false>
 __device__ __forceinline__ bool table_find(const Slot<W>* __restrict__ table, uint64_t mask,
                                            unsigned gen, const PKey<W>& P, double* c,
                                            int probe_limit, DevCtl* ctl, int* probes,
                                            uint32_t* idx = nullptr) {
     uint64_t h = key_hash(P) & mask;
+    auto ld = [](const ulonglong2* a) { return kFresh ? __ldcg(a) : __ldg(a); };
     for (int p = 0; p < probe_limit; ++p) {
         const Slot<W>* s = table + h;
         const ulonglong2* v = reinterpret_cast<const ulonglong2*>(s);
@@ -107,14 +109,14 @@ __device__ __forceinline__ bool table_find(const Slot<W>* __restrict__ table, ui
         double cc;
         unsigned tag;
         if constexpr (W == 1) {
-            ulonglong2 a = __ldg(v), b = __ldg(v + 1);
+            ulonglong2 a = ld(v), b = ld(v + 1);
             k.x[0] = a.x;
             k.z[0] = a.y;
             cc = __longlong_as_double((long long)b.x);
             tag = (unsigned)(b.y & 0xffffffffULL);
             if (idx) *idx = (uint32_t)(b.y >> 32);
         } else {
-            ulonglong2 a = __ldg(v), b = __ldg(v + 1), d = __ldg(v + 2);
+            ulonglong2 a = ld(v), b = ld(v + 1), d = ld(v + 2);
             k.x[0] = a.x; k.x[1] = a.y;
             k.z[0] = b.x; k.z[1] = b.y;
             cc = __longlong_as_double((long long)d.x);
@@ -167,7 +169,7 @@ __device__ __forceinline__ bool table_insert(Slot<W>* table, uint64_t mask, unsi
 }
 
 // Partner lookup in the global merge table.
-template <int W>
+template <int W, bool kFresh = false>
 struct GlobalLookup {
     const Slot<W>* table;
     uint64_t mask;
@@ -176,7 +178,7 @@ struct GlobalLookup {
     DevCtl* ctl;
     int* probes;
     __device__ __forceinline__ bool find(const PKey<W>& P, double* c, uint32_t* idx) const {
-        return table_find(table, mask, gen, P, c, probe_limit, ctl, probes, idx);
+        return table_find<W, kFresh>(table, mask, gen, P, c, probe_limit, ctl, probes, idx);
     }
 };
 
@@ -207,7 +209,12 @@ struct StepMaps {
     unsigned long long* id_pos;   // output position of the identity
 };
 
-template <int W, int BLOCK, int IPT, bool REC = false, class Lookup = GlobalLookup<W>>
+struct NoSink {
+    __device__ __forceinline__ void operator()(double) const {}
+};
+
+template <int W, int BLOCK, int IPT, bool REC = false, class Lookup = GlobalLookup<W>,
+          class Sink = NoSink>
 __device__ __forceinline__ void gate_tile(uint64_t t, uint64_t n,
                                           const PKey<W>* __restrict__ kin,
                                           const double* __restrict__ cin,
@@ -217,7 +224,8 @@ __device__ __forceinline__ void gate_tile(uint64_t t, uint64_t n,
                                           unsigned long long dbits, uint64_t cap_out,
                                           uint32_t* s_scan, unsigned long long* s_base,
                                           StepMaps maps = StepMaps{nullptr, nullptr, nullptr,
-                                                                   nullptr}) {
+                                                                   nullptr},
+                                          const Sink& sink = Sink()) {
     constexpr uint64_t TILE = (uint64_t)BLOCK * IPT;
     PKey<W> K[IPT];
     double va[IPT], vb[IPT];
@@ -298,11 +306,13 @@ __device__ __forceinline__ void gate_tile(uint64_t t, uint64_t n,
         if ((flags >> (2 * j)) & 1u) {
             store_key_stream(kout + pos, K[j]);
             __stcs(cout + pos, va[j]);
+            sink(va[j]);
             ++pos;
         }
         if ((flags >> (2 * j + 1)) & 1u) {
             store_key_stream(kout + pos, key_xor(K[j], g));
             __stcs(cout + pos, vb[j]);
+            sink(vb[j]);
             ++pos;
         }
     }

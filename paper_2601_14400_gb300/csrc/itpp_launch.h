@@ -89,9 +89,6 @@ void plan_windows(int W, std::vector<HostGate>& gates);
 // select predicts the next threshold from the same gate of the last layer).
 cudaError_t launch_cap(const DeviceState& s, cudaStream_t st, int gate = 0);
 int cap_launches(const DeviceState& s);
-// The select part only (threshold and tie key in the control block, no
-// compaction): used where the kept set is compacted elsewhere.
-cudaError_t launch_cap_select(const DeviceState& s, cudaStream_t st);
 // The top-M select of the partitioned merge (itpp_select.cu): leaves the
 // kept set as a predicate for the next gate's reads.
 cudaError_t launch_select_deferred(const DeviceState& s, cudaStream_t st, int gate);
