@@ -134,9 +134,10 @@ struct AdjSweep {
 
 // Recompute a segment's steps, recording the output positions, by one
 // persistent launch.  A step is a few tens of microseconds of work at most;
-// made of 35 launches (reset, table, merge, five radix passes over |c| and
-// eight over the ties of two launches each, compaction) it took 170 us at 2^18
-// terms, nearly all of it between launches.  Here it is
+// it was made of 35 launches (reset, table, merge, five radix passes over |c|
+// and eight over the ties of two launches each, compaction), with four more in
+// the reverse sweep: 273 us a step of both at 2^18 terms, nearly all of it
+// between launches.  Persistent, they take 64 and 22 us.  Here a step is
 //
 //   merge      every input's children against the table, with a histogram of
 //              |c| around the last threshold (512 bins an octave)
@@ -145,7 +146,9 @@ struct AdjSweep {
 //   select     the first CTA, among the list
 //   compact    the kept terms, which enter the next step's table at once
 //
-// with a barrier after each.
+// with a barrier after each.  What bounds it is latency, one tile a CTA: the
+// merge 30 us (two lookups one after the other, histogram), compaction 22, the
+// list and the select 11.
 template <int W>
 __global__ void __launch_bounds__(kBlock, 4) k_adj_recompute(const AdjSweep<W> a) {
     __shared__ __align__(16) unsigned char s_scratch[kScratch];
@@ -429,8 +432,8 @@ __global__ void k_adj_wsum(const int* first, const double* w, int m, double* wsu
 // The reverse sweep over a segment by one persistent launch: mu_{s-1} from
 // nu_s through the recorded output positions, with the partial sums of
 // df/dtheta_s, and of the next step's dot = sum_{j != I} mu[j] u[j] (nu_I =
-// -dot / D) from the values just made.  One barrier a step: four launches, of
-// which two add up 512 partials in one block, took 17 us a step at 2^18 terms.
+// -dot / D) from the values just made.  One barrier a step, where
+// four launches were.
 // The grid and so the order of the sums are fixed by the sizes.
 template <int W>
 __global__ void __launch_bounds__(kBlock, 4)

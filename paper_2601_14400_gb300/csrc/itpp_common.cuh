@@ -59,6 +59,23 @@ constexpr int kSelBins = 1 << kSelBits;
 constexpr int kTieBits = 16;                 // radix digit of the tie (key) select
 constexpr int kTieBins = 1 << kTieBits;
 
+// First in the shared block of a team of CTAs (itpp_team.cuh); zero before a
+// launch.
+struct TeamHead {
+    unsigned int bar;    // arrivals at the team's barrier so far
+    unsigned int dead;   // a wait ran out
+    unsigned int seq;    // publications so far
+    unsigned int pad;
+};
+constexpr int kDigit = 11, kBins = 1 << kDigit;   // radix digit of a select by a team
+
+// The partitioned merge's select (itpp_select.cu): cleared after every gate.
+struct SelTeam {
+    TeamHead head;
+    unsigned int list_n;             // values gathered for the first CTA
+    unsigned int hist[3][kBins];
+};
+
 // Device-resident control block: everything that changes from gate to gate
 // lives here, so a sequence of gates can be launched (or captured) without
 // the host knowing any count.
@@ -144,6 +161,7 @@ struct DevCtl {
     unsigned int sel_done;
     unsigned long long sel_hist[kSelBins];
     unsigned long long tie_hist[kTieBins];
+    SelTeam sel;
 };
 
 // Terms held by buffer b, clamped to the buffer (after a device error the

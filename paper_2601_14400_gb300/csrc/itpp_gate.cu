@@ -402,7 +402,7 @@ static cudaError_t cap_w(const DeviceState& s, cudaStream_t st) {
 }
 
 int cap_launches(const DeviceState& s) {
-    return s.merge_deferred ? select_deferred_launches(s.W) : 5 * 2 + 1 + 8 * s.W * 2 + 3;
+    return s.merge_deferred ? 3 : 5 * 2 + 1 + 8 * s.W * 2 + 3;
 }
 
 template <int W>

@@ -92,7 +92,7 @@ int cap_launches(const DeviceState& s);
 // The top-M select of the partitioned merge (itpp_select.cu): leaves the
 // kept set as a predicate for the next gate's reads.
 cudaError_t launch_select_deferred(const DeviceState& s, cudaStream_t st, int gate);
-int select_deferred_launches(int W);
+uint64_t select_list_cap(const DeviceState& s);   // candidates it can take
 // Apply a deferred top-M select and gather the state's partitions into one
 // contiguous run; a no-op when neither is there.
 cudaError_t launch_materialize(const DeviceState& s, cudaStream_t st);

@@ -29,6 +29,8 @@
 // least cap_M children lie at or above the range; otherwise the merge runs
 // again in full), and the select (itpp_select.cu) then works on that short
 // list instead of passing over every coefficient.
+#include <cstring>
+
 #include "itpp_common.cuh"
 #include "itpp_gate_body.cuh"
 #include "itpp_launch.h"
@@ -365,10 +367,24 @@ k_gate_part(Bufs<W> B, Homes<W> H, DevCtl* ctl, GateArg<W> g, double delta, uint
 }
 
 // After the merge: where the state is now, then the buffer switch, normaliser,
-// statistics and bound of every gate (post_one).
-__global__ void k_part_post(DevCtl* ctl, uint64_t cap_M, int cap_policy) {
-    __shared__ int s_active;
+// statistics and bound of every gate (post_one), and the way to the top-M
+// threshold (itpp_select.cu): the merge's candidates when the cap_M-th largest
+// value lies among them, else passes over the state.
+__global__ void __launch_bounds__(256)
+k_part_post(DevCtl* ctl, CandRegions cd, uint64_t cap_M, int cap_policy, uint64_t cand_cap,
+            unsigned long long delta_bits) {
+    __shared__ uint32_t s_scan[256 / 32];
     if (ctl->status) return;
+    const uint32_t nreg = ctl->cand_regions < 1024u ? ctl->cand_regions : 1024u;
+    uint32_t c = 0, tot;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const uint32_t r = u * 256u + threadIdx.x;
+        c += r < nreg ? cd.cnt[r] : 0u;
+    }
+    block_exclusive_scan<256>(c, &tot, s_scan);
+    unsigned int* team = reinterpret_cast<unsigned int*>(&ctl->sel);
+    for (uint32_t b = threadIdx.x; b < sizeof(SelTeam) / 4; b += 256u) team[b] = 0u;
     if (threadIdx.x == 0) {
         if (ctl->scattered) {
             ctl->home = 1;
@@ -385,18 +401,38 @@ __global__ void k_part_post(DevCtl* ctl, uint64_t cap_M, int cap_policy) {
             ctl->hx ^= 1;
             ctl->hc = next3(ctl->hc);
         }
-        s_active = post_one(ctl, cap_M, cap_policy);
+        const int active = post_one(ctl, cap_M, cap_policy);
         const int cur = ctl->cur, a = ctl->ha;
+        const unsigned long long kept = ctl->count[cur];
         if (!ctl->home && cur != a) {   // the run is in buffer a
-            ctl->count[a] = ctl->count[cur];
+            ctl->count[a] = kept;
             ctl->norm[a] = ctl->norm[cur];
             ctl->rnorm[a] = ctl->rnorm[cur];
             ctl->cur = a;
         }
+        if (active) {
+            // kept children above the range: all that were not listed
+            const unsigned long long above = kept - tot;
+            const int reason = ctl->sp_hi == 0ULL ? 1
+                               : (ctl->sp_ovf || tot > cand_cap) ? 2
+                               : above >= cap_M ? 3
+                               : above + tot < cap_M ? 4 : 0;
+            const bool fast = reason == 0;
+            const unsigned long long range = ctl->sp_hi - ctl->sp_lo;
+            ctl->sel_fast = fast ? 1 : 0;
+            ctl->sp_reason = reason;
+            ctl->sel_prefix = 0ULL;
+            ctl->sel_mask = 0ULL;
+            ctl->sel_lo = fast ? ctl->sp_lo : delta_bits;
+            ctl->sel_cand_n = fast ? tot : 0ULL;
+            if (fast) {
+                ctl->sel_top = range ? 64 - __clzll((long long)range) : 0;
+                ctl->sel_k = cap_M - above;
+            } else {
+                ctl->stat_sel_full += 1;
+            }
+        }
     }
-    __syncthreads();
-    if (s_active)
-        for (int b = threadIdx.x; b < kSelBins; b += blockDim.x) ctl->sel_hist[b] = 0ULL;
 }
 
 // ---------------------------------------------------------------------------
@@ -514,7 +550,9 @@ cudaError_t launch_part_scatter(const DeviceState& s, const HostGate& h, int for
 }
 
 cudaError_t launch_part_post(const DeviceState& s, cudaStream_t st) {
-    k_part_post<<<1, 256, 0, st>>>(s.ctl, s.cap_M, s.cap_policy);
+    unsigned long long dbits;
+    std::memcpy(&dbits, &s.delta, sizeof dbits);   // delta >= +0: it bounds every kept pattern
+    k_part_post<<<1, 256, 0, st>>>(s.ctl, s.cand, s.cap_M, s.cap_policy, select_list_cap(s), dbits);
     return cudaGetLastError();
 }
 

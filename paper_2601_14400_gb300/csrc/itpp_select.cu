@@ -4,30 +4,31 @@
 //
 // The values selected on are the 63-bit magnitude patterns b of the raw
 // coefficients (monotone in |c|), offset by sel_lo: v = b - sel_lo.  Two ways
-// to the threshold:
+// to the threshold, which k_part_post chooses between:
 //   fast   the merge compared every kept child with a range [lo, hi] around
-//          the previous gate's threshold, counted the children above hi and
-//          listed those inside; when the cap_M-th largest lies inside
-//          (above < cap_M <= above + listed), k_sel_begin compacts the
-//          merge's per-CTA lists and the digits of v are resolved over that
-//          list alone (sel_lo = lo);
+//          the predicted threshold, counted the children above hi and listed
+//          those inside, per CTA; the cap_M-th largest lies inside
+//          (above < cap_M <= above + listed; sel_lo = lo);
 //   full   otherwise (no range yet, the threshold moved outside it, a list
 //          overflowed): k_sel_hist takes the first 13-bit digit over every
 //          stored coefficient, with sel_lo = delta's pattern and the digit
 //          scaled to the largest pattern the merge wrote (bits [sh, sh+13)
 //          of v, sh = max(0, bitlen(hi - lo) - 13)), so the values spread over
 //          thousands of bins; k_sel_gather lists the terms of the picked digit.
-// Then, on the list: k_sel_vpass resolves the remaining digits of v;
-// k_sel_tcollect / k_sel_tpass / k_sel_finish select among exact ties by key
-// (a bitonic sort in shared memory, or 16-bit radix passes over a long tie
-// list), and k_sel_finish records the kept set as the predicate (threshold,
-// tie key) that the next gate's reads apply, and the next gate's range.  No
-// CTA waits for another: each multi-block pass ends in its last CTA.
+// k_sel_resolve then finishes on the list, one cooperative launch: digits of v
+// and then of the keys of exact ties by all CTAs, with a barrier after each,
+// until few enough values are left for the first CTA, which records the kept
+// set as the predicate (threshold, tie key) that the next gate's reads apply,
+// and the next gate's range.  In its place were 5 launches for the digits of
+// v, 8 or 16 for those of a key and 3 more, a few microseconds each whether
+// they had work or not: 117 us a gate at 2^23 terms (W = 1), 154 us at 2^22
+// (W = 2).
 #include <cstring>
 
 #include "itpp_common.cuh"
 #include "itpp_gate_body.cuh"
 #include "itpp_launch.h"
+#include "itpp_team.cuh"
 
 namespace itpp {
 
@@ -107,64 +108,6 @@ __device__ __forceinline__ void pick_digit(const void* hist, unsigned long long 
         }
     }
     __syncthreads();
-}
-
-// ---------------------------------------------------------------------------
-// 0. Fast or full: when the cap_M-th largest value lies in the merge's
-// candidate range, compact the merge's per-CTA lists into the candidate list
-// (every CTA computes the region offsets and the decision from the same
-// counts; block 0 alone writes the select state).
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(1024)
-k_sel_begin(DevCtl* ctl, CandRegions cr, unsigned long long* cand_v, uint32_t* cand_idx,
-            uint64_t cand_cap, uint64_t cap_M, unsigned long long delta_bits) {
-    __shared__ uint32_t s_scan[32];
-    __shared__ uint32_t s_off[1024];
-    if (!ctl->sel_active || ctl->status) return;
-    const unsigned int nreg = ctl->cand_regions < 1024u ? ctl->cand_regions : 1024u;
-    const uint32_t c = threadIdx.x < nreg ? cr.cnt[threadIdx.x] : 0u;
-    uint32_t tot;
-    const uint32_t off = block_exclusive_scan<1024>(c, &tot, s_scan);
-    s_off[threadIdx.x] = off;
-    // kept children above the range: all that were not listed
-    const unsigned long long above = ctl->count[ctl->cur] - tot;
-    const int reason = ctl->sp_hi == 0ULL ? 1
-                       : (ctl->sp_ovf || tot > cand_cap) ? 2
-                       : above >= cap_M ? 3
-                       : above + tot < cap_M ? 4 : 0;
-    const bool fast = reason == 0;
-    __syncthreads();
-    if (fast) {
-        for (unsigned int r = blockIdx.x; r < nreg; r += gridDim.x) {
-            const uint32_t n = cr.cnt[r], o = s_off[r];
-            const uint64_t rb = (uint64_t)r * cr.region;
-            for (uint32_t j = threadIdx.x; j < n; j += blockDim.x) {
-                cand_v[o + j] = cr.v[rb + j];
-                cand_idx[o + j] = cr.idx[rb + j];
-            }
-        }
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        ctl->sel_fast = fast ? 1 : 0;
-        ctl->sp_reason = reason;
-        ctl->sel_prefix = 0ULL;
-        ctl->sel_mask = 0ULL;
-        if (fast) {
-            const int top = bit_length(ctl->sp_hi - ctl->sp_lo);
-            ctl->sel_lo = ctl->sp_lo;
-            ctl->sel_top = top;
-            ctl->sel_k = cap_M - above;
-            ctl->sel_cand_n = tot;
-            if (top == 0) {          // a range of one value: every candidate ties
-                ctl->sel_ties = tot;
-                ctl->sel_tie_k = cap_M - above;
-            }
-        } else {
-            ctl->sel_lo = delta_bits;
-            ctl->sel_cand_n = 0ULL;
-            ctl->stat_sel_full += 1;
-        }
-    }
 }
 
 // ---------------------------------------------------------------------------
@@ -256,7 +199,6 @@ k_sel_hist(Bufs<W> B, Homes<W> H, DevCtl* ctl) {
 // immaterial: every later pass histograms them and the ties are sorted by key.
 // ---------------------------------------------------------------------------
 constexpr int kStage = 3072;      // staged candidates per CTA (36 KB)
-constexpr int kVPasses = 5;       // 13-bit passes over v: 5 x 13 >= 63 bits
 constexpr int kRangeShift0 = 45;  // the first candidate range: T +- about 1/128 of T
 
 struct GatherStage {
@@ -369,301 +311,254 @@ k_sel_gather(Bufs<W> B, Homes<W> H, DevCtl* ctl, unsigned long long* cand_v,
 }
 
 // ---------------------------------------------------------------------------
-// 3. The remaining digits of v over the candidates, one per launch; the
-// last CTA picks.  Pass p covers bits [max(0, top - 13p), top - 13(p-1)),
-// top = sel_top (the bits below the first digit on the full path, every bit
-// of the range on the fast path).
+// 3. The rest of the select on the list: every CTA's candidates of the merge
+// where they are (fast), or the gathered list (full).
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(1024)
-k_sel_vpass(DevCtl* ctl, const unsigned long long* cand_v, int p) {
-    __shared__ unsigned int h[kSelBins];
-    __shared__ unsigned long long s_part[1024];
-    __shared__ int s_last;
-    __shared__ Pick s_pick;
-    if (!ctl->sel_active || ctl->status) return;
-    const int sh = ctl->sel_top;
-    if (sh - kSelBits * (p - 1) <= 0) return;          // every bit already fixed
-    const int shift = sh - kSelBits * p > 0 ? sh - kSelBits * p : 0;
-    const unsigned long long nc = ctl->sel_cand_n;
-    const unsigned long long prefix = ctl->sel_prefix, mask = ctl->sel_mask;
-    for (int b = threadIdx.x; b < kSelBins; b += blockDim.x) h[b] = 0u;
-    __syncthreads();
-    for (unsigned long long j = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; j < nc;
-         j += (unsigned long long)gridDim.x * blockDim.x) {
-        const unsigned long long v = cand_v[j];
-        if ((v & mask) == prefix) atomicAdd(&h[(v >> shift) & (kSelBins - 1)], 1u);
-    }
-    __syncthreads();
-    for (int b = threadIdx.x; b < kSelBins; b += blockDim.x)
-        if (h[b]) atomicAdd(&ctl->sel_hist[b], (unsigned long long)h[b]);
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) s_last = atomicAdd(&ctl->sel_done, 1u) == gridDim.x - 1;
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    pick_digit<1024, true>(ctl->sel_hist, ctl->sel_k, s_part, &s_pick);
-    if (threadIdx.x == 0) {
-        const Pick pk = s_pick;
-        ctl->sel_prefix = prefix | ((unsigned long long)pk.digit << shift);
-        ctl->sel_mask = mask | ((unsigned long long)(kSelBins - 1) << shift);
-        ctl->sel_k = pk.k_in;
-        if (shift == 0) {
-            ctl->sel_ties = pk.count;
-            ctl->sel_tie_k = pk.k_in;
-        }
-        ctl->sel_done = 0u;
-    }
-    for (int b = threadIdx.x; b < kSelBins; b += blockDim.x) ctl->sel_hist[b] = 0ULL;
-}
-
-// ---------------------------------------------------------------------------
-// 4. Ties: the keys of the candidates exactly at the threshold (only when
-// some of them are dropped), staged per CTA like the candidates.
-// ---------------------------------------------------------------------------
-template <int W>
-__global__ void __launch_bounds__(256)
-k_sel_tcollect(Bufs<W> B, Homes<W> H, DevCtl* ctl, const unsigned long long* cand_v,
-               const uint32_t* cand_idx, PKey<W>* tie_list, uint64_t tie_cap) {
-    constexpr int kT = 1024;
-    __shared__ PKey<W> st[kT];
-    __shared__ unsigned int s_n;
-    __shared__ unsigned long long s_base;
-    if (!tie_select_needed(ctl)) return;
-    const StateRuns<W> rs = state_runs(ctl, B, H);
-    const PKey<W>* keys = rs.keys;
-    const uint64_t held = rs.cnt ? rs.P * rs.R : rs.n;
-    const unsigned long long nc = ctl->sel_cand_n, T = ctl->sel_prefix;
-    if (threadIdx.x == 0) s_n = 0u;
-    __syncthreads();
-    for (unsigned long long j0 = (unsigned long long)blockIdx.x * blockDim.x;
-         j0 < nc; j0 += (unsigned long long)gridDim.x * blockDim.x) {
-        const unsigned long long j = j0 + threadIdx.x;
-        if (j < nc && cand_v[j] == T) {
-            if (cand_idx[j] < held) {
-                const unsigned int q = atomicAdd(&s_n, 1u);
-                st[q] = load_key(keys + cand_idx[j]);
-            } else {
-                set_status(ctl, ST_STATE, 34);   // not reached
-            }
-        }
-        __syncthreads();
-        const unsigned int m = s_n;
-        if (m > kT - 256) {
-            if (threadIdx.x == 0) s_base = atomicAdd(&ctl->sel_tie_n, (unsigned long long)m);
-            __syncthreads();
-            for (unsigned int t = threadIdx.x; t < m; t += blockDim.x) {
-                if (s_base + t < tie_cap) tie_list[s_base + t] = st[t];
-                else set_status(ctl, ST_CAPACITY, 32);
-            }
-            __syncthreads();
-            if (threadIdx.x == 0) s_n = 0u;
-        }
-        __syncthreads();
-    }
-    const unsigned int m = s_n;
-    if (m) {
-        if (threadIdx.x == 0) s_base = atomicAdd(&ctl->sel_tie_n, (unsigned long long)m);
-        __syncthreads();
-        for (unsigned int t = threadIdx.x; t < m; t += blockDim.x) {
-            if (s_base + t < tie_cap) tie_list[s_base + t] = st[t];
-            else set_status(ctl, ST_CAPACITY, 32);
-        }
-    }
-}
-
-// ---------------------------------------------------------------------------
-// 5. Key passes over a long tie list (16-bit digits from word 0), one per
-// launch, the last CTA picking; they stop once at most kSmallTies keys
-// share the picked prefix (state 3), which the final block then sorts.
-// ---------------------------------------------------------------------------
-template <int W>
-struct SmallTies {
-    static constexpr int kMax = 2048 / W;    // 32 KB of keys
+struct SelPredict {   // the next gate's range
+    uint64_t cap_M, cand_hi;
+    long long* drift;
+    int n_drift, gate;
+    unsigned long long delta_bits;
 };
 
+// One thread: the kept set as the next gate's predicate, and its range.
 template <int W>
-__global__ void __launch_bounds__(1024)
-k_sel_tpass(DevCtl* ctl, const PKey<W>* tie_list, int p) {
-    __shared__ unsigned long long s_part[1024];
-    __shared__ int s_last;
-    if (!tie_select_needed(ctl) || ctl->sel_tie_state != 0) return;
-    if (p == 0 && ctl->sel_ties <= (unsigned long long)SmallTies<W>::kMax) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) ctl->sel_tie_state = 3;   // small already
-        return;
-    }
-    tie_hist_range<W>(ctl, tie_list, p, (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x,
-                      ctl->sel_tie_n, (unsigned long long)gridDim.x * blockDim.x);
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) s_last = atomicAdd(&ctl->sel_done, 1u) == gridDim.x - 1;
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    // the digit (ascending) holding the sel_tie_k-th smallest key
-    constexpr int PER = kTieBins / 1024;
-    const int t = threadIdx.x;
-    unsigned long long sum = 0;
-    for (int j = 0; j < PER; ++j) sum += __ldcg(&ctl->tie_hist[PER * t + j]);
-    const unsigned long long incl = scan_nt<1024>(sum, s_part);
-    unsigned long long run = incl - sum;
-    const unsigned long long k = ctl->sel_tie_k;
-    const int wi = p / 4, shift = 48 - 16 * (p % 4);
-    if (run < k && k <= incl) {
-        for (int j = 0; j < PER; ++j) {
-            const unsigned long long hv = __ldcg(&ctl->tie_hist[PER * t + j]);
-            if (run < k && k <= run + hv) {
-                ctl->sel_tie_k = k - run;
-                ctl->sel_tie_key[wi] |= (unsigned long long)(PER * t + j) << shift;
-                ctl->sel_tie_pass = p + 1;
-                if (p == 8 * W - 1) ctl->sel_tie_state = 1;                 // every bit fixed
-                else if (hv == 1) ctl->sel_tie_state = 2;                   // a unique key
-                else if (hv <= (unsigned long long)SmallTies<W>::kMax) ctl->sel_tie_state = 3;
-            }
-            run += hv;
+__device__ __forceinline__ void sel_finish(DevCtl* ctl, unsigned long long T, bool all_ties,
+                                           const PKey<W>& tk, const SelPredict& q) {
+    const int cur = ctl->cur;
+    ctl->pend = 1;
+    ctl->pend_n = ctl->count[cur];
+    ctl->pend_T = T;
+    ctl->pend_all_ties = all_ties;
+    for (int w = 0; w < 4; ++w) ctl->pend_tie_key[w] = 0ULL;
+    if (!all_ties)
+        for (int w = 0; w < W; ++w) {
+            ctl->pend_tie_key[w] = tk.x[w];
+            ctl->pend_tie_key[W + w] = tk.z[w];
         }
+    ctl->count[cur] = q.cap_M;   // the logical term count
+    ctl->stat_cands += ctl->sel_cand_n;
+    const unsigned long long lo = ctl->sel_lo;
+    ctl->stat_range = ctl->sel_fast ? ctl->sp_hi - ctl->sp_lo
+                                    : (ctl->sel_hi > lo ? ctl->sel_hi - lo : 0ULL);
+    // the next gate's candidate range: C +- 2^s in pattern units (a
+    // relative width of about 2^(s-52)), narrower when the list ran long
+    // or overflowed, wider when the threshold fell outside.  Its centre C:
+    // this threshold moved by what the next gate's threshold moved in the
+    // last layer (the schedule repeats every layer), or, without that,
+    // carried into the next gate's scale (the next gate reads the state
+    // rescaled by 1/c_I, rnorm of the buffer this gate wrote).
+    const unsigned long long Tp = ctl->sp_tprev;
+    const int gi = q.n_drift > 0 ? q.gate % q.n_drift : 0;
+    const int gn = q.n_drift > 0 ? (q.gate + 1) % q.n_drift : 0;
+    if (q.n_drift > 0) q.drift[gi] = Tp ? (long long)(T - Tp) : 0LL;
+    ctl->sp_tprev = T;
+    int sft = ctl->sp_shift ? ctl->sp_shift : kRangeShift0;
+    switch (ctl->sel_fast ? 0 : ctl->sp_reason) {
+        case 0: if (ctl->sel_cand_n > q.cand_hi) sft -= 1; break;
+        case 1: sft = kRangeShift0; break;
+        case 2: sft -= 2; break;
+        default: sft += 1; break;
     }
-    __syncthreads();
-    for (int b = t; b < kTieBins; b += blockDim.x) ctl->tie_hist[b] = 0ULL;
-    if (t == 0) ctl->sel_done = 0u;
-}
-
-// ---------------------------------------------------------------------------
-// 6. One block: the last key digits by a shared-memory sort, then the
-// predicate.
-// ---------------------------------------------------------------------------
-template <int W>
-__device__ __forceinline__ PKey<W> key_max() {
-    PKey<W> k;
-#pragma unroll
-    for (int w = 0; w < W; ++w) { k.x[w] = ~0ULL; k.z[w] = ~0ULL; }
-    return k;
-}
-
-// Ascending bitonic sort of n_pad (a power of two) keys in shared memory.
-template <int W>
-__device__ void bitonic_sort_keys(PKey<W>* a, int n_pad) {
-    for (int k = 2; k <= n_pad; k <<= 1) {
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = threadIdx.x; i < n_pad; i += blockDim.x) {
-                const int l = i ^ j;
-                if (l > i) {
-                    const bool up = (i & k) == 0;
-                    const PKey<W> x = a[i], y = a[l];
-                    if (up ? key_less(y, x) : key_less(x, y)) {
-                        a[i] = y;
-                        a[l] = x;
-                    }
-                }
-            }
-            __syncthreads();
-        }
+    sft = sft < 8 ? 8 : (sft > kRangeShiftMax ? kRangeShiftMax : sft);
+    ctl->sp_shift = sft;
+    const long long dn = q.n_drift > 0 ? q.drift[gn] : 0LL;
+    unsigned long long C;
+    if (dn != 0LL) {
+        const long long c = (long long)T + dn;
+        C = c > 0 ? (unsigned long long)c : 0ULL;
+    } else {
+        C = abs_pattern(__dmul_rn(__longlong_as_double((long long)T), ctl->rnorm[cur]));
     }
+    const SelRange r = sel_range(C, sft, q.delta_bits);
+    ctl->sp_thr = r.thr;
+    ctl->sp_lo = r.thr + 1ULL;
+    ctl->sp_hi = r.hi;
+    ctl->sel_active = 0;
 }
 
+// CTAs of the launch per SM: two read a list of a few hundred thousand values
+// in a few rounds; a barrier grows with every CTA.
+constexpr int kResolvePerSm = 2;
+
 template <int W>
-__global__ void __launch_bounds__(1024)
-k_sel_finish(DevCtl* ctl, const PKey<W>* tie_list, uint64_t cap_M, uint64_t cand_hi,
-             long long* drift, int n_drift, int gate, unsigned long long delta_bits) {
-    __shared__ PKey<W> s_ties[SmallTies<W>::kMax];
-    __shared__ unsigned int s_cnt;
+__global__ void __launch_bounds__(kBlock, kResolvePerSm)
+k_sel_resolve(Bufs<W> B, Homes<W> H, DevCtl* ctl, CandRegions cr, unsigned long long* cand_v,
+              uint32_t* cand_idx, PKey<W>* ties, SelPredict q) {
+    __shared__ __align__(16) unsigned char s_scratch[kScratch];
+    __shared__ uint32_t s_off[1024];
+    __shared__ uint32_t s_scan[kBlock / 32];
+    __shared__ PickOut s_pick;
+    uint32_t* s_hist = reinterpret_cast<uint32_t*>(s_scratch);
     if (!ctl->sel_active) return;
+    const bool first = blockIdx.x == 0;
     if (ctl->status) {
-        __syncthreads();
-        if (threadIdx.x == 0) ctl->sel_active = 0;
+        if (first && threadIdx.x == 0) ctl->sel_active = 0;
         return;
     }
-    const bool all_ties = ctl->sel_k == ctl->sel_ties;
-    if (!all_ties && ctl->sel_tie_state != 1) {
-        // the keys sharing the picked prefix (state 3, or the unique key of
-        // state 2), sorted; the tie_k-th smallest is the largest kept key
-        const int p = ctl->sel_tie_pass;   // key digits fixed so far
-        uint64_t pre[2 * W];
+    const uint64_t n = ctl->sel_cand_n;
+    // few values: the first CTA alone, among them all
+    if (!first && n <= kOneCta) return;
+    const bool fast = ctl->sel_fast != 0;
+    const unsigned long long lo = ctl->sel_lo;
+    unsigned long long prefix = ctl->sel_prefix, mask = ctl->sel_mask, rank = ctl->sel_k;
+    int top = ctl->sel_top;
+    TeamOf<SelTeam> team{&ctl->sel, blockIdx.x, gridDim.x, 0u, 0u};
+    const PKey<W>* keys = state_runs(ctl, B, H).keys;
+    const unsigned long long* sv = fast ? cr.v : cand_v;
+    const uint32_t* si = fast ? cr.idx : cand_idx;
+    uint32_t nreg = 0;
+    if (fast) {   // where each CTA's candidates start
+        nreg = ctl->cand_regions < 1024u ? ctl->cand_regions : 1024u;
+        uint32_t c[4], sum = 0, tot;
 #pragma unroll
-        for (int w = 0; w < 2 * W; ++w) pre[w] = ctl->sel_tie_key[w];
-        if (threadIdx.x == 0) s_cnt = 0u;
-        __syncthreads();
-        const unsigned long long nt = ctl->sel_tie_n;
-        for (unsigned long long j = threadIdx.x; j < nt; j += blockDim.x) {
-            const PKey<W> k = tie_list[j];
-            if (tie_prefix_match<W>(k, pre, p)) {
-                const unsigned int q = atomicAdd(&s_cnt, 1u);
-                if (q < (unsigned int)SmallTies<W>::kMax) s_ties[q] = k;
-            }
+        for (int u = 0; u < 4; ++u) {
+            const uint32_t r = threadIdx.x * 4u + u;
+            c[u] = r < nreg ? cr.cnt[r] : 0u;
+            sum += c[u];
+        }
+        uint32_t at = block_exclusive_scan<kBlock>(sum, &tot, s_scan);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            s_off[threadIdx.x * 4u + u] = at;
+            at += c[u];
         }
         __syncthreads();
-        const unsigned int m = s_cnt;
-        if (m > (unsigned int)SmallTies<W>::kMax || m == 0u) {
-            if (threadIdx.x == 0) set_status(ctl, ST_STATE, 31);
-        } else {
-            int n_pad = 1;
-            while (n_pad < (int)m) n_pad <<= 1;
-            for (int i = (int)m + threadIdx.x; i < n_pad; i += blockDim.x) s_ties[i] = key_max<W>();
+    }
+    // place of the j-th value (j < n)
+    auto place = [&](uint64_t j) -> uint64_t {
+        if (!fast) return j;
+        uint32_t r = 0;   // the last region that starts at or before j
+#pragma unroll
+        for (uint32_t b = 512u; b > 0u; b >>= 1)
+            if (s_off[r + b] <= (uint32_t)j) r += b;
+        if (r >= nreg) r = nreg - 1u;   // (empty ones at the end start at n)
+        return (uint64_t)r * cr.region + (j - s_off[r]);
+    };
+    const uint64_t tid = (uint64_t)blockIdx.x * kBlock + threadIdx.x;
+    const uint64_t all = (uint64_t)(n <= kOneCta ? 1u : gridDim.x) * kBlock;
+    // f(value, place) for every value that matches, its loads four at a time
+    auto each = [&](auto&& f) {
+        constexpr int U = 4;
+        for (uint64_t j0 = tid; j0 < n; j0 += U * all) {
+            uint64_t at[U];
+            unsigned long long v[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const uint64_t j = j0 + u * all;
+                at[u] = j < n ? place(j) : 0ULL;
+                v[u] = j < n ? __ldcg(sv + at[u]) : ~prefix;
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (j0 + u * all < n && (v[u] & mask) == prefix) f(v[u], at[u]);
+        }
+    };
+    uint64_t cnt = n;
+    int koff = 0;          // key bits fixed
+    uint64_t kpre[2 * W];
+#pragma unroll
+    for (int w = 0; w < 2 * W; ++w) kpre[w] = 0;
+    auto key_matches = [&](const PKey<W>& key) {
+        const int full = koff >> 6, r = koff & 63;
+        bool ok = true;
+#pragma unroll
+        for (int w = 0; w < 2 * W; ++w) {
+            const uint64_t word = w < W ? key.x[w] : key.z[w - W];
+            if (w < full) ok = ok && word == kpre[w];
+            else if (w == full && r) ok = ok && (word >> (64 - r)) == (kpre[w] >> (64 - r));
+        }
+        return ok;
+    };
+    if (n > kOneCta) {
+        for (int hb = 0; cnt > kOneCta; hb = (hb + 1) % 3) {
+            const bool by_key = top == 0;
+            if (by_key && (rank == cnt && koff == 0)) break;   // every tie is kept
+            if (koff >= 128 * W) break;                        // (keys are distinct)
+            for (int b = threadIdx.x; b < kBins; b += kBlock) s_hist[b] = 0u;
             __syncthreads();
-            bitonic_sort_keys<W>(s_ties, n_pad);
-            if (threadIdx.x == 0) {
-                unsigned long long r = ctl->sel_tie_state == 2 ? 1ULL : ctl->sel_tie_k;
-                if (r < 1ULL || r > m) {   // not reached: the list agrees with the counts
-                    set_status(ctl, ST_STATE, 33);
-                    r = 1ULL;
-                }
-                const PKey<W> tk = s_ties[r - 1];
-                for (int w = 0; w < W; ++w) {
-                    ctl->sel_tie_key[w] = tk.x[w];
-                    ctl->sel_tie_key[W + w] = tk.z[w];
-                }
+            const int wd = by_key ? (64 - (koff & 63) < kDigit ? 64 - (koff & 63) : kDigit)
+                                  : (top > kDigit ? kDigit : top);
+            if (!by_key) {
+                const int shift = top - wd;
+                each([&](unsigned long long v, uint64_t) {
+                    atomicAdd(&s_hist[(uint32_t)(v >> shift) & ((1u << wd) - 1u)], 1u);
+                });
+            } else {
+                each([&](unsigned long long, uint64_t at) {
+                    const PKey<W> key = load_key_stream(keys + __ldcg(si + at));
+                    if (key_matches(key)) atomicAdd(&s_hist[key_digit(key, koff, wd)], 1u);
+                });
+            }
+            __syncthreads();
+            for (int b = threadIdx.x; b < kBins; b += kBlock)
+                if (s_hist[b]) atomicAdd(&ctl->sel.hist[hb][b], s_hist[b]);
+            if (!team_barrier(team, ctl)) return;
+            for (int b = threadIdx.x; b < kBins; b += kBlock) {
+                s_hist[b] = __ldcg(&ctl->sel.hist[hb][b]);
+                if (first) ctl->sel.hist[(hb + 2) % 3][b] = 0u;   // read before this barrier
+            }
+            if (threadIdx.x == 0) s_pick = PickOut{0u, 1u, 0u};
+            __syncthreads();
+            if (by_key) pick_bin<false>(s_hist, (uint32_t)rank, s_scan, &s_pick);
+            else pick_bin<true>(s_hist, (uint32_t)rank, s_scan, &s_pick);
+            const PickOut o = s_pick;
+            __syncthreads();
+            rank = o.k_in;
+            cnt = o.count;
+            if (by_key) {
+                const int w = koff >> 6, in = koff & 63;
+#pragma unroll
+                for (int u = 0; u < 2 * W; ++u)
+                    if (u == w) kpre[u] |= (uint64_t)o.digit << (64 - in - wd);
+                koff += wd;
+            } else {
+                top -= wd;
+                prefix |= (unsigned long long)o.digit << top;
+                mask |= (unsigned long long)((1u << wd) - 1u) << top;
             }
         }
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        const int cur = ctl->cur;
-        const unsigned long long lo = ctl->sel_lo;
-        const unsigned long long T = ctl->sel_prefix + lo;   // the threshold's pattern
-        // the kept set, applied where the next gate reads the state
-        ctl->pend = 1;
-        ctl->pend_n = ctl->count[cur];
-        ctl->pend_T = T;
-        ctl->pend_all_ties = all_ties;
-        for (int w = 0; w < 4; ++w) ctl->pend_tie_key[w] = all_ties ? 0ULL : ctl->sel_tie_key[w];
-        ctl->count[cur] = cap_M;   // the logical term count
-        ctl->sel_active = 0;
-        ctl->stat_cands += ctl->sel_cand_n;
-        ctl->stat_range = ctl->sel_fast ? ctl->sp_hi - ctl->sp_lo
-                                        : (ctl->sel_hi > lo ? ctl->sel_hi - lo : 0ULL);
-        // the next gate's candidate range: C +- 2^s in pattern units (a
-        // relative width of about 2^(s-52)), narrower when the list ran long
-        // or overflowed, wider when the threshold fell outside.  Its centre C:
-        // this threshold moved by what the next gate's threshold moved in the
-        // last layer (the schedule repeats every layer), or, without that,
-        // carried into the next gate's scale (the next gate reads the state
-        // rescaled by 1/c_I, rnorm of the buffer this gate wrote).
-        const unsigned long long Tp = ctl->sp_tprev;
-        const int gi = n_drift > 0 ? gate % n_drift : 0;
-        const int gn = n_drift > 0 ? (gate + 1) % n_drift : 0;
-        if (n_drift > 0) drift[gi] = Tp ? (long long)(T - Tp) : 0LL;
-        ctl->sp_tprev = T;
-        int sft = ctl->sp_shift ? ctl->sp_shift : kRangeShift0;
-        switch (ctl->sel_fast ? 0 : ctl->sp_reason) {
-            case 0: if (ctl->sel_cand_n > cand_hi) sft -= 1; break;
-            case 1: sft = kRangeShift0; break;
-            case 2: sft -= 2; break;
-            default: sft += 1; break;
+    if (cnt > kOneCta) {   // a long class of ties, all kept
+        if (first && threadIdx.x == 0) {
+            const PKey<W> none{};
+            sel_finish(ctl, prefix + lo, true, none, q);
         }
-        sft = sft < 8 ? 8 : (sft > kRangeShiftMax ? kRangeShiftMax : sft);
-        ctl->sp_shift = sft;
-        const long long dn = n_drift > 0 ? drift[gn] : 0LL;
-        unsigned long long C;
-        if (dn != 0LL) {
-            const long long c = (long long)T + dn;
-            C = c > 0 ? (unsigned long long)c : 0ULL;
+        return;
+    }
+    // the values left, for the first CTA
+    unsigned long long* lv = cand_v;
+    uint32_t* li = cand_idx;
+    if (!fast && n > kOneCta) {   // the merge's lists are free
+        lv = cr.v;
+        li = cr.idx;
+    }
+    if (fast || n > kOneCta) {
+        each([&](unsigned long long v, uint64_t at) {
+            const uint32_t idx = __ldcg(si + at);
+            if (koff && !key_matches(load_key_stream(keys + idx))) return;
+            const uint32_t p = atomicAdd(&ctl->sel.list_n, 1u);
+            if (p < kOneCta) {
+                lv[p] = v;
+                li[p] = idx;
+            }
+        });
+        if (n > kOneCta) {
+            team_arrive(team);
+            if (!first) return;
+            if (!team_wait(team, ctl)) return;
         } else {
-            C = abs_pattern(__dmul_rn(__longlong_as_double((long long)T), ctl->rnorm[cur]));
+            __syncthreads();
         }
-        SelRange r = sel_range(C, sft, delta_bits);
-        ctl->sp_thr = r.thr;
-        ctl->sp_lo = r.thr + 1ULL;
-        ctl->sp_hi = r.hi;
+        cnt = __ldcg(&ctl->sel.list_n);
+        if (cnt > kOneCta) cnt = kOneCta;
+    }
+    PKey<W> tk{};
+    const SelOut so = select_list<W>(s_scratch, lv, li, cnt, rank, prefix, mask, top, keys, ties,
+                                     &tk, ctl, koff > 0);
+    if (threadIdx.x == 0) {
+        if (ctl->status) ctl->sel_active = 0;
+        else sel_finish(ctl, so.v + lo, so.all_ties != 0, tk, q);
     }
 }
 
@@ -716,19 +611,18 @@ static cudaError_t select_w(const DeviceState& s, cudaStream_t st, int gate) {
     H.cnt = s.part_cursor;
     H.part_max = s.part_max;
     H.cap = 0;
-    k_sel_begin<<<s.num_sms, 1024, 0, st>>>(s.ctl, s.cand, sc.cand_v, sc.cand_idx, sc.cand_cap,
-                                            s.cap_M, lo);
     k_sel_hist<W><<<s.num_sms * 4, 256, 0, st>>>(B, H, s.ctl);
     k_sel_gather<W><<<s.num_sms * 4, 256, 0, st>>>(B, H, s.ctl, sc.cand_v, sc.cand_idx,
                                                    sc.cand_cap);
-    for (int p = 1; p <= kVPasses; ++p)    // 13-bit digits cover any 63-bit range
-        k_sel_vpass<<<s.num_sms, 1024, 0, st>>>(s.ctl, sc.cand_v, p);
-    k_sel_tcollect<W><<<s.num_sms * 2, 256, 0, st>>>(B, H, s.ctl, sc.cand_v, sc.cand_idx, sc.ties,
-                                                     sc.tie_cap);
-    for (int p = 0; p < 8 * W; ++p)
-        k_sel_tpass<W><<<s.num_sms, 1024, 0, st>>>(s.ctl, sc.ties, p);
-    k_sel_finish<W><<<1, 1024, 0, st>>>(s.ctl, sc.ties, s.cap_M, s.cand_hi, s.sp_drift,
-                                        s.sp_drift ? s.layer_gates : 0, gate, lo);
+    SelPredict q{s.cap_M, s.cand_hi, s.sp_drift, s.sp_drift ? s.layer_gates : 0, gate, lo};
+    CandRegions cr = s.cand;
+    DevCtl* ctl = s.ctl;
+    void* args[8] = {const_cast<Bufs<W>*>(&B), &H, &ctl, &cr, const_cast<unsigned long long**>(&sc.cand_v),
+                     const_cast<uint32_t**>(&sc.cand_idx), const_cast<PKey<W>**>(&sc.ties), &q};
+    cudaError_t e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(&k_sel_resolve<W>),
+                                                dim3(s.num_sms * kResolvePerSm), dim3(kBlock),
+                                                args, 0, st);
+    if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
 
@@ -738,6 +632,8 @@ cudaError_t launch_select_deferred(const DeviceState& s, cudaStream_t st, int ga
     return s.W == 1 ? select_w<1>(s, st, gate) : select_w<2>(s, st, gate);
 }
 
-int select_deferred_launches(int W) { return 4 + kVPasses + 8 * W + 1; }
+uint64_t select_list_cap(const DeviceState& s) {
+    return s.W == 1 ? sel_scratch<1>(s).cand_cap : sel_scratch<2>(s).cand_cap;
+}
 
 }  // namespace itpp

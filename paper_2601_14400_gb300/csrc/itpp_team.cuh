@@ -11,18 +11,9 @@
 namespace itpp {
 
 constexpr int kBlock = 256;
-constexpr int kDigit = 11, kBins = 1 << kDigit;   // radix digit of the select
 constexpr uint32_t kFinal = 128;                  // values ranked one per thread
 constexpr size_t kScratch = 16384;                // shared scratch of a select
 constexpr uint32_t kOneCta = 4096;                // candidates one CTA selects among
-
-// First in a team's shared block; zero before a launch.
-struct TeamHead {
-    unsigned int bar;    // arrivals at the team's barrier so far
-    unsigned int dead;   // a wait ran out
-    unsigned int seq;    // publications so far
-    unsigned int pad;
-};
 
 // ---------------------------------------------------------------------------
 // Arrivals
@@ -154,7 +145,8 @@ __device__ __forceinline__ uint32_t key_digit(const PKey<W>& k, int off, int wd)
     return (uint32_t)((word >> (64 - in - wd)) & ((1ULL << wd) - 1ULL));
 }
 
-// prefix, top: the bits of v from `top` up already agree with prefix.  Every
+// prefix, top: the bits of v from `top` up already agree with prefix.  more:
+// there are further ties beyond the list, all dropped.  Every
 // thread calls it; *tk receives the largest kept key at the threshold when
 // some of its ties are dropped.  ties: global scratch for a long list of equal
 // values.  What bounds it is latency, a pass over a few thousand candidates
@@ -165,7 +157,7 @@ template <int W>
 __device__ SelOut select_list(unsigned char* scratch, const unsigned long long* gv, const uint32_t* gidx, uint64_t n,
                               uint64_t k, unsigned long long prefix, unsigned long long mask,
                               int top, const PKey<W>* keys, PKey<W>* ties, PKey<W>* tk,
-                              DevCtl* ctl) {
+                              DevCtl* ctl, bool more = false) {
     constexpr int kReg = (int)kOneCta / kBlock;
     constexpr uint32_t kTieMax = 512 / W;   // keys held in shared memory
     uint32_t* h = reinterpret_cast<uint32_t*>(scratch);                    // kBins
@@ -220,7 +212,7 @@ __device__ SelOut select_list(unsigned char* scratch, const unsigned long long* 
     o.all_ties = 1;
     if (threadIdx.x == 0) s_n = s_gt = s_eq = 0u;
     __syncthreads();
-    if (cnt > kFinal && rank == cnt) return o;   // a class of equal values, all kept
+    if (cnt > kFinal && rank == cnt && !more) return o;   // a class of equal values, all kept
     if (cnt <= kFinal) {
         // the entries left: value and place
         auto take = [&](uint64_t j, unsigned long long v) {
@@ -265,7 +257,7 @@ __device__ SelOut select_list(unsigned char* scratch, const unsigned long long* 
         __syncthreads();
         const uint32_t need = rank - s_gt, ne = s_eq;
         o.v = s_T;
-        o.all_ties = need == ne;
+        o.all_ties = need == ne && !more;
         if (o.all_ties) {
             __syncthreads();
             return o;
