@@ -36,6 +36,7 @@ struct itpp_batch_ctx {
     void* run_shared = nullptr;
     long long* run_drift = nullptr;     // [B * (max_gates + 1)]
     int run_grid = 0, run_n_teams = 0, run_fit_ctas = 0;
+    bool run_wide = false;
     int max_weight = 0;
     bool target_fixed = false;          // partition size given by the caller
 };
@@ -224,7 +225,7 @@ itpp_status run_batch(itpp_batch_ctx* h, int n_layers) {
     static const RunChunk<W> none{};
     if (cudaMemset2DAsync(h->run_shared, a.shared_stride, 0, run_shared_head(),
                           (size_t)h->run_n_teams, h->stream) != cudaSuccess ||
-        launch_run<W>(a, none, h->run_grid, h->stream) != cudaSuccess) {
+        launch_run<W>(a, none, h->run_grid, h->run_wide, h->stream) != cudaSuccess) {
         cudaGetLastError();
         return ITPP_ERR_CUDA;
     }
@@ -380,7 +381,8 @@ itpp_status itpp_batch_create(int B, const int* n, const int* n_gates, const uin
         s.part_cap += s.part_cap & 1ULL;
         const int t_min = std::min(h->target_fixed ? s.part_target : kTargetMin, s.part_target);
         s.part_max = partition_max(p->cap_M, t_min) + 1;
-        h->run_fit_ctas = run_fit(W);
+        h->run_wide = (uint64_t)B * p->cap_M > kRunWide;
+        h->run_fit_ctas = run_fit(W, h->run_wide);
     }
     // auto sizing leaves room for the autotuner to try loads down to 25 %
     const int load_for_size = p->table_load_pct ? (s.load_pct < 50 ? s.load_pct : 50) : 25;

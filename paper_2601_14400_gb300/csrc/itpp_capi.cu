@@ -122,8 +122,11 @@ cudaError_t clear_cursors(itpp_ctx* h) {
                            h->stream);
 }
 
-// Bounds up to this run a layer in one launch (itpp_run.cu).
-constexpr uint64_t kRunMax = 1ULL << 21;
+// Bounds up to this run a layer in one launch (itpp_run_impl.cuh).  A layer of
+// the 64-site chain takes 9.4 ms that way and 12.1 by separate launches at 2^20,
+// 13.1 and 13.7 at 2^21, 21.5 and 18.1 at 2^22; one of the 11 x 11 lattice 22.9
+// and 28.0 at 2^19, 32.8 and 34.7 at 2^20, 64.1 and 44.4 at 2^21.
+constexpr uint64_t kRunMax = 1ULL << 20;
 
 // Gates [k0, k0 + n) n_layers times in one launch (n <= kRunChunk).
 template <int W>
@@ -179,7 +182,7 @@ itpp_status run_launch(itpp_ctx* h, int k0, int n, int n_layers, unsigned long l
     h->contiguous = true;
     itpp_detail_touch(h);
     if (cudaMemsetAsync(h->run_shared, 0, run_shared_head(), h->stream) != cudaSuccess ||
-        launch_run<W>(a, ch, h->run_grid, h->stream) != cudaSuccess)
+        launch_run<W>(a, ch, h->run_grid, false, h->stream) != cudaSuccess)
         return cuda_fail(h);
     h->launches += 1;
     return ITPP_OK;
@@ -474,7 +477,10 @@ itpp_status itpp_create(int n, const uint64_t* gate_x, const uint64_t* gate_z,
     s.load_pct = p->table_load_pct ? p->table_load_pct : 50;
     // defaults: 512 x 2 for the partitioned merge (a whole partition in
     // registers), 256 x 2 for the global-table merge
-    s.block = p->block_threads ? p->block_threads : 256;
+    // partitions of two-word strings are half as large: the lattice's merge takes
+    // 94 us at 2^22 terms with 128 threads, 111 with 256; the chain's 1133 and
+    // 1076 us at 2^26
+    s.block = p->block_threads ? p->block_threads : (p->merge_path == 0 && W == 2) ? 128 : 256;
     s.ipt = p->items_per_thread ? p->items_per_thread : 2;
     s.merge_deferred = p->merge_path == 0;
     s.probe_limit = 4096;
@@ -565,7 +571,7 @@ itpp_status itpp_create(int n, const uint64_t* gate_x, const uint64_t* gate_z,
         // CTAs as there can be partitions, at most what fits
         if (p->cap_M <= kRunMax && (p->block_threads == 0 || p->block_threads == 256)) {
             const uint64_t parts = p->cap_M / kRunMinPart + 1;
-            h->run_grid = (int)std::min<uint64_t>((uint64_t)sms * run_fit(W), parts);
+            h->run_grid = (int)std::min<uint64_t>((uint64_t)sms * run_fit(W, false), parts);
             h->run_part_max = (uint32_t)std::max<uint64_t>(p->cap_M / s.part_target + 2,
                                                            (uint64_t)h->run_grid + 1);
             ok &= ok && cudaMalloc(&h->run_shared, run_shared_bytes()) == cudaSuccess;

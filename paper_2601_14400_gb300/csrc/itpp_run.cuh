@@ -93,10 +93,28 @@ struct RunArgs {
 // Bytes of one team's shared block, and of its head that a launch clears.
 size_t run_shared_bytes();
 size_t run_shared_head();
+// The kernel with few CTAs per SM (3; 2 with two mask words), or the wide one
+// with one more.  The register file is shared out: the first spills little
+// (104 bytes against 888 with two words), the second hides more latency.  For
+// one propagation of 2^16 or 2^18 terms a layer takes 3.21 and 3.14 ms with the
+// first, 3.55 and 3.45 with the second; at 2^20 both 9.3.  Batches of 4 x 2^16
+// and 16 x 2^14: 64.1 and 39.8 ms with the first, 68.1 and 41.6 with the second;
+// 8 x 2^16 and 64 x 2^14: 77.2 and 69.4 against 72.1 and 60.7.
+template <int W, bool kWide> int run_fit_as();
+template <int W, bool kWide>
+cudaError_t launch_run_as(const RunArgs<W>& a, const RunChunk<W>& chunk, int grid, cudaStream_t st);
+extern template int run_fit_as<1, true>();
+extern template int run_fit_as<2, true>();
+extern template cudaError_t launch_run_as<1, true>(const RunArgs<1>&, const RunChunk<1>&, int, cudaStream_t);
+extern template cudaError_t launch_run_as<2, true>(const RunArgs<2>&, const RunChunk<2>&, int, cudaStream_t);
+// A batch of more terms than this runs on the wide one.
+constexpr uint64_t kRunWide = 1ULL << 18;
+
 // CTAs per SM that fit.
-int run_fit(int W);
+int run_fit(int W, bool wide);
 // A cooperative launch (the CTAs of a team wait for one another).
 template <int W>
-cudaError_t launch_run(const RunArgs<W>& a, const RunChunk<W>& chunk, int grid, cudaStream_t st);
+cudaError_t launch_run(const RunArgs<W>& a, const RunChunk<W>& chunk, int grid, bool wide,
+                       cudaStream_t st);
 
 }  // namespace itpp

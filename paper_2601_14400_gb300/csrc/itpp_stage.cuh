@@ -17,13 +17,17 @@ namespace {
 
 // Partition geometry per word count: the mean partition size the scatter
 // aims for, and the largest window (sites; a group holds at most 4^sites
-// terms).
+// terms).  A pass has fixed costs and a partition beyond its capacity goes in
+// sub-passes.  Merge per gate of the 64-site chain at 2^23 terms: 144, 136, 128
+// and 144 us for targets of 500, 600, 700 and 850; of the 11 x 11 lattice at
+// 2^22: 98, 94, 99 and 120 us for 300, 350, 400 and 440.  Windows of 6 or 7 sites
+// instead of 5: a layer of 230 and 235 ms instead of 234 at 2^26.
 template <int W> struct PartGeom;
 template <> struct PartGeom<1> {
     static constexpr int kTarget = 700, kWinSites = 5;
 };
 template <> struct PartGeom<2> {
-    static constexpr int kTarget = 300, kWinSites = 4;
+    static constexpr int kTarget = 350, kWinSites = 4;
 };
 
 struct PartPlan {
