@@ -44,7 +44,7 @@ namespace itpp {
 // previous gate alone.  The state is a contiguous run, or the partitions of
 // a home; it goes to the other home.
 template <int W>
-__global__ void __launch_bounds__(256, W == 1 ? 6 : 4)
+__global__ void __launch_bounds__(256, 4)
 k_part_scatter(Bufs<W> B, Homes<W> H, DevCtl* ctl, GateArg<W> g, PartFn<W> f, int force,
                int n_sites, int target, int redo) {
     if (ctl->status) return;

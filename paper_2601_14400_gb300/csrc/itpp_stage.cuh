@@ -142,6 +142,9 @@ __device__ __forceinline__ void scatter_run(const PKey<W>* __restrict__ kin,
                 live[u] = abs_pattern(c[u]) != 0ULL;   // a zero is no term
             }
         }
+        // partitions and claims of all items before the first position is used:
+        // their atomics are in flight together
+        uint32_t part[U], peers[U], base[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             if (live[u] && pd.on && !cap_keep(K[u], c[u], pd.T, pd.all_ties, pd.tk)) {
@@ -150,23 +153,28 @@ __device__ __forceinline__ void scatter_run(const PKey<W>* __restrict__ kin,
             }
             // one cursor claim per distinct partition in the warp: terms of
             // one group arrive together and would otherwise serialise on it
-            const uint32_t p = live[u] ? part_of(K[u], g, f, pl.P) : 0xffffffffu;
-            const unsigned int peers = __match_any_sync(0xffffffffu, p);
-            const int leader = __ffs(peers) - 1;
-            unsigned int base = 0;
-            if (live[u] && (threadIdx.x & 31) == leader) base = atomicAdd(cursor + (uint64_t)p * pad, __popc(peers));
-            base = __shfl_sync(0xffffffffu, base, leader);
-            if (live[u]) {
-                const unsigned int pos = base + __popc(peers & lt);
-                if (pos < pl.R) {
-                    const uint64_t d = (uint64_t)p * pl.R + pos;
-                    store_key(pk + d, K[u]);
-                    pc[d] = c[u];
-                } else if (!f.pair) {
-                    *over = 1;   // the gate scatters again by its pair key
-                } else {
-                    set_status(ctl, ST_CAPACITY, 40);
-                }
+            part[u] = live[u] ? part_of(K[u], g, f, pl.P) : 0xffffffffu;
+            peers[u] = __match_any_sync(0xffffffffu, part[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            base[u] = 0;
+            if (live[u] && !(peers[u] & lt))
+                base[u] = atomicAdd(cursor + (uint64_t)part[u] * pad, __popc(peers[u]));
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const uint32_t b = __shfl_sync(0xffffffffu, base[u], __ffs(peers[u]) - 1);
+            if (!live[u]) continue;
+            const unsigned int pos = b + __popc(peers[u] & lt);
+            if (pos < pl.R) {
+                const uint64_t d = (uint64_t)part[u] * pl.R + pos;
+                store_key(pk + d, K[u]);
+                pc[d] = c[u];
+            } else if (!f.pair) {
+                *over = 1;   // the gate scatters again by its pair key
+            } else {
+                set_status(ctl, ST_CAPACITY, 40);
             }
         }
     }
