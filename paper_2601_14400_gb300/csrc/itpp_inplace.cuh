@@ -27,20 +27,25 @@ namespace itpp {
 
 namespace {
 
+// Slots of the separate kernel's passes, where shared memory has room for them:
+// a string that shares its slot with another that is not its partner is looked
+// at twice (700 strings in 4,096 slots: 15 %, in 8,192: 8 %).  Merge per gate of
+// the 64-site chain at 2^26 terms 1074 us with 4,096, 1024 with 8,192.
+constexpr int kLargeBits = 13;
+
 // Geometry and shared memory of one pass: up to kItems strings, each read from
 // global memory into registers (nothing is staged: the rare ones are read
 // again, from L1 or L2), the heads of the chains of strings that share a slot,
 // the chain links, the index of a gathered string (sub-passes) and the list of
 // rare strings.
-template <int W>
+template <int W, int BITS = 12>
 struct InPass {
-    static constexpr int C = StageGeom<W>::kItems, S = 4096, kSlotBits = 12;
+    static constexpr int C = StageGeom<W>::kItems, kSlotBits = BITS, S = 1 << BITS;
     static constexpr size_t kHeads = 0;
     static constexpr size_t kNext = kHeads + sizeof(uint32_t) * S;
     static constexpr size_t kSrc = kNext + sizeof(uint16_t) * C;
     static constexpr size_t kRare = kSrc + sizeof(uint16_t) * C;
     static constexpr size_t kBytes = (kRare + sizeof(uint16_t) * C + 15) / 16 * 16;
-    static_assert(S == (1 << kSlotBits), "slots");
     __device__ __forceinline__ static uint32_t* heads() { return reinterpret_cast<uint32_t*>(g_stage + kHeads); }
     __device__ __forceinline__ static uint16_t* next() { return reinterpret_cast<uint16_t*>(g_stage + kNext); }
     __device__ __forceinline__ static uint16_t* src() { return reinterpret_cast<uint16_t*>(g_stage + kSrc); }
@@ -112,7 +117,8 @@ struct InRows {
 
 template <int W, int BLOCK, bool kGathered>
 __device__ __forceinline__ void load_rows(InRows<W, BLOCK>& rows, const PKey<W>* keys,
-                                          const double* cin, uint32_t n) {
+                                          const double* cin, uint32_t n,
+                                          const uint16_t* src = nullptr) {
     const PKey<W>* kp = keys + threadIdx.x;
     const double* cp = cin + threadIdx.x;
 #pragma unroll
@@ -122,7 +128,7 @@ __device__ __forceinline__ void load_rows(InRows<W, BLOCK>& rows, const PKey<W>*
         rows.c[r] = 0.0;
         if (threadIdx.x + r * BLOCK < n) {
             if (kGathered) {
-                const uint32_t at = InPass<W>::src()[threadIdx.x + r * BLOCK];
+                const uint32_t at = src[threadIdx.x + r * BLOCK];
                 rows.K[r] = load_key_ca(keys + at);
                 rows.c[r] = cin[at];
             } else {
@@ -142,7 +148,7 @@ __device__ __forceinline__ void load_rows(InRows<W, BLOCK>& rows, const PKey<W>*
 // called when the rows are done with and before the rare strings are: the
 // caller loads its next ones there, so that their latency is not waited for.
 // Three barriers; the shared arrays are free again when it returns.
-template <int W, int BLOCK, bool kGathered, bool kPlain, class Push, class Then>
+template <int W, int BLOCK, int BITS, bool kGathered, bool kPlain, class Push, class Then>
 __device__ __forceinline__ void inplace_pass(uint32_t n, const GateArg<W>& g,
                                              unsigned long long pd_T, bool pd_ties,
                                              const PKey<W>& pd_key, double rnorm,
@@ -150,13 +156,15 @@ __device__ __forceinline__ void inplace_pass(uint32_t n, const GateArg<W>& g,
                                              int nxt, uint32_t tag, const InPlace<W>& io,
                                              InStats& st, unsigned long long near_hi,
                                              InRows<W, BLOCK>& rows, Push&& push, Then&& then) {
-    using A = InPass<W>;
+    using A = InPass<W, BITS>;
     constexpr int ROWS = InRows<W, BLOCK>::N;
     PKey<W>(&K)[ROWS] = rows.K;
     double(&c)[ROWS] = rows.c;
-    // per row: slot (12 bits) | commutes | not the first to arrive in its
-    // chain | live, and (special) the identity or past the weight cutoff
-    constexpr uint32_t kComm = 1u << 12, kPrev = 1u << 13, kLive = 1u << 14, kSpecial = 1u << 15;
+    // per row: slot | commutes | not the first to arrive in its chain | live,
+    // and (special) the identity or past the weight cutoff; two rows a word
+    // where they fit
+    constexpr uint32_t kComm = 1u << BITS, kPrev = 2u << BITS, kLive = 4u << BITS, kSpecial = 8u << BITS;
+    constexpr int PER = BITS <= 12 ? 2 : 1;
     const uint32_t lane = threadIdx.x & 31u, w0 = threadIdx.x & ~31u;
     const unsigned int lt = (1u << lane) - 1u;
     const bool weigh = !kPlain && g.maxw < 64 * W;
@@ -168,9 +176,9 @@ __device__ __forceinline__ void inplace_pass(uint32_t n, const GateArg<W>& g,
     for (int w = 0; w < W; ++w) qbits |= g.qx[w] | g.qz[w];
     const bool self = !kPlain && qbits == 0;
     // A: live strings, normalised values, the chains of shared slots
-    uint32_t flags[(ROWS + 1) / 2];   // 16 bits a row
+    uint32_t flags[(ROWS + PER - 1) / PER];
 #pragma unroll
-    for (int r = 0; r < (ROWS + 1) / 2; ++r) flags[r] = 0u;
+    for (int r = 0; r < (ROWS + PER - 1) / PER; ++r) flags[r] = 0u;
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) {
         if (r * BLOCK + w0 >= n) break;   // whole warps
@@ -195,7 +203,7 @@ __device__ __forceinline__ void inplace_pass(uint32_t n, const GateArg<W>& g,
         f |= comm ? slot | kComm : 0u;
         f |= prev ? kPrev : 0u;
         f |= live ? kLive : 0u;
-        flags[r >> 1] |= f << (16 * (r & 1));
+        flags[r / PER] |= f << (16 * (r % PER));
     }
     __syncthreads();                                                  // (1) chains built
     // B: every string that is alone in its slot (its partner is absent).
@@ -208,11 +216,11 @@ __device__ __forceinline__ void inplace_pass(uint32_t n, const GateArg<W>& g,
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) {
         if (r * BLOCK + w0 >= n) break;   // whole warps
-        const uint32_t f = flags[r >> 1] >> (16 * (r & 1));
+        const uint32_t f = flags[r / PER] >> (16 * (r % PER));
         const bool comm = (f & kComm) != 0;
         const uint32_t me = me0 + r * BLOCK;
         uint32_t head = me;
-        if (comm) head = A::heads()[f & 0xfffu];
+        if (comm) head = A::heads()[f & (uint32_t)(A::S - 1)];
         bool dup = ((f & kPrev) | (head ^ me)) != 0u;
         if (!kPlain) dup = dup || (self && comm);
         const bool may = comm && (int)(__double2hiint(c[r]) & 0x7fffffff) + hm >= 0;
@@ -325,7 +333,7 @@ __device__ __forceinline__ void inplace_pass(uint32_t n, const GateArg<W>& g,
 // one after another, each a list of indices (strings and partners agree on
 // the class).  Every thread calls it, with the partition in rows when one pass
 // holds it; *s_app and *s_rare are zero.  Returns whether it took sub-passes.
-template <int W, int BLOCK, class Push, class Then>
+template <int W, int BLOCK, int BITS, class Push, class Then>
 __device__ __forceinline__ bool inplace_partition(const GateArg<W>& g, unsigned long long pd_T,
                                                   bool pd_ties, const PKey<W>& pd_key,
                                                   double rnorm, unsigned long long thr,
@@ -334,7 +342,7 @@ __device__ __forceinline__ bool inplace_partition(const GateArg<W>& g, unsigned 
                                                   unsigned long long near_hi, uint32_t* s_n,
                                                   InRows<W, BLOCK>& rows, Push&& push,
                                                   Then&& then) {
-    using A = InPass<W>;
+    using A = InPass<W, BITS>;
     constexpr uint32_t C = A::C;
     if (io.n == 0u) {
         then();
@@ -346,10 +354,10 @@ __device__ __forceinline__ bool inplace_partition(const GateArg<W>& g, unsigned 
     const bool plain = !has_id && g.maxw >= 64 * W && qbits != 0;
     if (io.n <= C) {
         if (plain)
-            inplace_pass<W, BLOCK, false, true>(io.n, g, pd_T, pd_ties, pd_key, rnorm, thr, false,
+            inplace_pass<W, BLOCK, BITS, false, true>(io.n, g, pd_T, pd_ties, pd_key, rnorm, thr, false,
                                                 ctl, nxt, ++*tag, io, st, near_hi, rows, push, then);
         else
-            inplace_pass<W, BLOCK, false, false>(io.n, g, pd_T, pd_ties, pd_key, rnorm, thr, has_id,
+            inplace_pass<W, BLOCK, BITS, false, false>(io.n, g, pd_T, pd_ties, pd_key, rnorm, thr, has_id,
                                                  ctl, nxt, ++*tag, io, st, near_hi, rows, push,
                                                  then);
         return false;
@@ -372,8 +380,8 @@ __device__ __forceinline__ bool inplace_partition(const GateArg<W>& g, unsigned 
         __syncthreads();
         const uint32_t m = *s_n < C ? *s_n : C;
         if (m == 0u) continue;   // uniform
-        load_rows<W, BLOCK, true>(rows, io.keys, io.cin, m);
-        inplace_pass<W, BLOCK, true, false>(m, g, pd_T, pd_ties, pd_key, rnorm, thr, has_id, ctl, nxt,
+        load_rows<W, BLOCK, true>(rows, io.keys, io.cin, m, A::src());
+        inplace_pass<W, BLOCK, BITS, true, false>(m, g, pd_T, pd_ties, pd_key, rnorm, thr, has_id, ctl, nxt,
                                             ++*tag, io, st, near_hi, rows, push, [] {});
     }
     then();
@@ -388,9 +396,10 @@ struct InOcc {
 
 // Heads clear of an earlier use of the shared memory, or of a tag that comes
 // round again (a barrier must follow).
-template <int W, int BLOCK>
+template <int W, int BLOCK, int BITS>
 __device__ __forceinline__ void inplace_init() {
-    for (uint32_t i = threadIdx.x; i < (uint32_t)InPass<W>::S; i += BLOCK) InPass<W>::heads()[i] = 0u;
+    for (uint32_t i = threadIdx.x; i < (uint32_t)InPass<W, BITS>::S; i += BLOCK)
+        InPass<W, BITS>::heads()[i] = 0u;
 }
 
 }  // namespace

@@ -149,7 +149,7 @@ __device__ __forceinline__ GateInput gate_input(const DevCtl* ctl) {
 template <int W, int BLOCK>
 __global__ void __launch_bounds__(BLOCK, (InOcc<W, BLOCK>::kMin))
 k_gate_inplace(Bufs<W> B, Homes<W> H, DevCtl* ctl, GateArg<W> g, double delta, CandRegions cd) {
-    constexpr uint32_t C = InPass<W>::C;
+    constexpr uint32_t C = InPass<W, kLargeBits>::C;
     __shared__ unsigned long long s_T, s_thr, s_kept;
     __shared__ PKey<W> s_tk;
     __shared__ double s_rnorm;
@@ -182,7 +182,7 @@ k_gate_inplace(Bufs<W> B, Homes<W> H, DevCtl* ctl, GateArg<W> g, double delta, C
             ctl->cand_regions = gridDim.x;
         }
     }
-    inplace_init<W, BLOCK>();
+    inplace_init<W, BLOCK, kLargeBits>();
     __syncthreads();
     if (s_stop) return;
     // the third cursor array (the previous gate's input) is the next scatter's
@@ -231,7 +231,7 @@ k_gate_inplace(Bufs<W> B, Homes<W> H, DevCtl* ctl, GateArg<W> g, double delta, C
             l2_prefetch_bulk(keys + (uint64_t)pf * R, np2 * sizeof(PKey<W>));
             l2_prefetch_bulk(cin + (uint64_t)pf * R, np2 * sizeof(double));
         }
-        const bool subs = inplace_partition<W, BLOCK>(g, s_T, s_ties != 0, s_tk, s_rnorm, s_thr,
+        const bool subs = inplace_partition<W, BLOCK, kLargeBits>(g, s_T, s_ties != 0, s_tk, s_rnorm, s_thr,
                                                       p == p_id, ctl, nxt, &tag, io, st,
                                                       g_range[1], &s_n, rows, push,
                                                       [&] { load(pn, np); });
@@ -243,7 +243,7 @@ k_gate_inplace(Bufs<W> B, Homes<W> H, DevCtl* ctl, GateArg<W> g, double delta, C
             if (subs) s_long += 1u;
         }
         if (tag >= kHeadTagMax - 65536u) {   // tags start again
-            inplace_init<W, BLOCK>();
+            inplace_init<W, BLOCK, kLargeBits>();
             tag = 0;
             __syncthreads();
         }
@@ -504,7 +504,7 @@ static cudaError_t scatter_w(const DeviceState& s, const HostGate& h, int force,
 template <int W, int BLOCK>
 static cudaError_t merge_wb(const DeviceState& s, const GateArg<W>& g, cudaStream_t st) {
     static int per_sm = 0, per_sm_full = 0;
-    constexpr size_t smem = InPass<W>::kBytes, smem_full = Stage<W>::kBytes;
+    constexpr size_t smem = InPass<W, kLargeBits>::kBytes, smem_full = Stage<W>::kBytes;
     if (!per_sm) {
         // shared memory for every resident CTA's staging rather than L1
         cudaFuncSetAttribute(k_gate_inplace<W, BLOCK>, cudaFuncAttributeMaxDynamicSharedMemorySize,

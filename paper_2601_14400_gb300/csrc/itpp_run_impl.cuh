@@ -327,7 +327,7 @@ __device__ bool run_instance(const RunArgs<W>& a, const RunGate<W>* gates, int n
     // start: the published state from the control block, the cursor arrays
     // zero, no chain head of an earlier use
     if (threadIdx.x < 8) s_stat[threadIdx.x] = 0ULL;
-    inplace_init<W, kBlock>();
+    inplace_init<W, kBlock, 12>();
     for (uint32_t i = team.rank * kBlock + threadIdx.x; i < 3u * a.part_max; i += team.size * kBlock)
         arr.n0[(uint64_t)i * kPad] = 0u;
     if (leader && threadIdx.x == 0) {
@@ -485,7 +485,7 @@ __device__ bool run_instance(const RunArgs<W>& a, const RunGate<W>* gates, int n
             io.over = &s_over;
             const uint32_t pn = p + team.size;
             np = stored(pn);
-            if (inplace_partition<W, kBlock>(g, s_pub.T, s_pub.all_ties != 0, tk, s_pub.rnorm, thr,
+            if (inplace_partition<W, kBlock, 12>(g, s_pub.T, s_pub.all_ties != 0, tk, s_pub.rnorm, thr,
                                              p == p_id, ctl, np_, &tag, io, st, s_pub.hi, &s_n, rows,
                                              push, [] {}))
                 ++n_long;
@@ -496,7 +496,7 @@ __device__ bool run_instance(const RunArgs<W>& a, const RunGate<W>* gates, int n
                 s_app = s_rare = 0u;
             }
             if (tag >= kHeadTagMax - 65536u) {   // tags start again
-                inplace_init<W, kBlock>();
+                inplace_init<W, kBlock, 12>();
                 tag = 0;
                 __syncthreads();
             }
@@ -708,7 +708,7 @@ __device__ bool run_instance(const RunArgs<W>& a, const RunGate<W>* gates, int n
             n_long = 0;
             const InStats s2{(uint32_t)(__reduce_max_sync(0xffffffffu, (uint32_t)(ss.out_max >> 32))), 0u};
             flush(acc, s2);
-            inplace_init<W, kBlock>();
+            inplace_init<W, kBlock, 12>();
             tag = 0;
             team_arrive(team);
             layout = 0;
