@@ -218,6 +218,7 @@ __global__ void k_import_begin(DevCtl* ctl, uint64_t count) {
         ctl->pend = 0;
         ctl->home = 0;
         ctl->need_scatter = ctl->part_over = ctl->scattered = ctl->over = 0;
+        ctl->ticket = 0;
         ctl->sp_lo = ctl->sp_hi = ctl->sp_thr = 0;
         ctl->sp_shift = 0;
         ctl->sp_tprev = 0;
@@ -356,6 +357,7 @@ __global__ void k_reset_identity(BufsA<W> B, DevCtl* ctl) {
         ctl->pend = 0;
         ctl->home = 0;
         ctl->need_scatter = ctl->part_over = ctl->scattered = ctl->over = 0;
+        ctl->ticket = 0;
         ctl->sp_lo = ctl->sp_hi = ctl->sp_thr = 0;
         ctl->sp_shift = 0;
         ctl->sp_tprev = 0;

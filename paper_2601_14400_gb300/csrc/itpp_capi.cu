@@ -256,7 +256,7 @@ itpp_status launch_one_gate(itpp_ctx* h, int k) {
     // scatter, merge, post (partitioned: also the scatter's clear and second
     // launch, the merge's check and the merge in full, which return at once
     // unless the scatter or the merge must be redone)
-    h->launches += h->p.merge_path == 0 ? 7 : 3;
+    h->launches += h->p.merge_path == 0 ? 5 : 3;
     if (e == cudaSuccess && h->s.cap_policy == 1) {
         EventPair* ev2 = prof_begin(h, 2);
         e = launch_cap(h->s, h->stream, k);

@@ -131,6 +131,7 @@ struct DevCtl {
     int part_over;                   // this gate's partitions hold for this gate only
     int need_scatter;                // ... so the next gate re-partitions
     int over;                        // the merge found no room in a partition's stride
+    unsigned int ticket;             // CTAs of a launch that are done (the last clears it)
     unsigned long long alloc;        // terms a merge done again, or a gather, has written
     // top-M select folded into the merge: children at or below sp_thr are
     // left out, kept ones in [sp_lo = sp_thr + 1, sp_hi] (a range around the

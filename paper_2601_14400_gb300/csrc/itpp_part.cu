@@ -39,6 +39,18 @@
 
 namespace itpp {
 
+// Is this the last CTA of the launch to get here?  (One thread; what the CTA
+// wrote before the barrier ahead of it is then seen by the last one.)
+__device__ __forceinline__ bool last_cta(DevCtl* ctl) {
+    __threadfence();
+    const bool last = atomicAdd(&ctl->ticket, 1u) == gridDim.x - 1u;
+    if (last) {
+        ctl->ticket = 0u;
+        __threadfence();
+    }
+    return last;
+}
+
 // Scatter the current state into the partitions of a window (force), or,
 // inside a window, only when the state has no partitions or they held for the
 // previous gate alone.  The state is a contiguous run, or the partitions of
@@ -107,17 +119,36 @@ k_part_scatter(Bufs<W> B, Homes<W> H, DevCtl* ctl, GateArg<W> g, PartFn<W> f, in
                     H.keys(B, a, to_b), H.coef(B, a, to_x), H.cursors(to_c), pl, g, f,
                     &ctl->scatter_over);
     }
+    if (redo) return;
+    // when a stride was too small, the last CTA clears the cursors for the
+    // second launch
+    __shared__ int s_clear;
+    __syncthreads();
+    if (threadIdx.x == 0) s_clear = last_cta(ctl) && *(volatile int*)&ctl->scatter_over;
+    __syncthreads();
+    if (s_clear)
+        for (uint32_t i = threadIdx.x; i < H.part_max; i += blockDim.x)
+            H.cursors(__ldcg(&ctl->to_c))[i] = 0u;   // (read again: one register less over the loop)
 }
 
-// Between a gate's two scatter launches: when the first found a stride too
-// small, clear the cursors for the second.
-template <int W>
-__global__ void k_scatter_clear(const DevCtl* ctl, Homes<W> H) {
-    if (ctl->status || !ctl->scatter_over) return;
-    unsigned int* cursor = H.cursors(ctl->to_c);
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < H.part_max;
-         i += gridDim.x * blockDim.x)
-        cursor[i] = 0u;
+// After a merge that left children out: with at least cap_M kept, the select
+// keeps cap_M of them and every one left out lay below them all; with fewer
+// they are needed.  Then, and when a partition's stride ran out, the gate's
+// merge is done again in full (its input is still in place).  One thread.
+__device__ __forceinline__ void merge_check(DevCtl* ctl, uint64_t cap_M) {
+    const int nxt = ctl->cur ^ 1;
+    ctl->retry = 0;
+    ctl->scatter_over = 0;   // the gate's scatters are done
+    if (__ldcg(&ctl->over) || (__ldcg(&ctl->drop_on) && __ldcg(&ctl->count[nxt]) < cap_M)) {
+        ctl->retry = 1;
+        ctl->count[nxt] = 0ULL;
+        ctl->alloc = 0ULL;
+        ctl->sp_ovf = 0;
+        ctl->cand_regions = 0;
+        ctl->out_max = 0ULL;
+        ctl->stat_retry += 1ULL;
+    }
+    ctl->drop_on = 0;
 }
 
 // Where this gate's input partitions are: where its scatter put them, or
@@ -148,7 +179,8 @@ __device__ __forceinline__ GateInput gate_input(const DevCtl* ctl) {
 // otherwise k_gate_part merges the gate again in full from the same input.
 template <int W, int BLOCK>
 __global__ void __launch_bounds__(BLOCK, (InOcc<W, BLOCK>::kMin))
-k_gate_inplace(Bufs<W> B, Homes<W> H, DevCtl* ctl, GateArg<W> g, double delta, CandRegions cd) {
+k_gate_inplace(Bufs<W> B, Homes<W> H, DevCtl* ctl, GateArg<W> g, double delta, CandRegions cd,
+               uint64_t cap_M) {
     constexpr uint32_t C = InPass<W, kLargeBits>::C;
     __shared__ unsigned long long s_T, s_thr, s_kept;
     __shared__ PKey<W> s_tk;
@@ -264,28 +296,8 @@ k_gate_inplace(Bufs<W> B, Homes<W> H, DevCtl* ctl, GateArg<W> g, double delta, C
         const uint32_t c = g_cn;
         cd.cnt[blockIdx.x] = c < cd.region ? c : (uint32_t)cd.region;
         if (c > cd.region) ctl->sp_ovf = 1;
+        if (last_cta(ctl)) merge_check(ctl, cap_M);
     }
-}
-
-// After a merge that left children out: with at least cap_M kept, the select
-// keeps cap_M of them and every one left out lay below them all; with fewer
-// they are needed.  Then, and when a partition's stride ran out, the gate's
-// merge is done again in full (its input is still in place).
-__global__ void k_merge_check(DevCtl* ctl, uint64_t cap_M) {
-    if (threadIdx.x != 0 || ctl->status) return;
-    const int nxt = ctl->cur ^ 1;
-    ctl->retry = 0;
-    ctl->scatter_over = 0;   // the gate's scatters are done
-    if (ctl->over || (ctl->drop_on && ctl->count[nxt] < cap_M)) {
-        ctl->retry = 1;
-        ctl->count[nxt] = 0ULL;
-        ctl->alloc = 0ULL;
-        ctl->sp_ovf = 0;
-        ctl->cand_regions = 0;
-        ctl->out_max = 0ULL;
-        ctl->stat_retry += 1ULL;
-    }
-    ctl->drop_on = 0;
 }
 
 // The gate's merge again, in full, into a contiguous run of the free buffer:
@@ -493,7 +505,6 @@ static cudaError_t scatter_w(const DeviceState& s, const HostGate& h, int force,
     if (gs > lim) gs = lim;
     if (gs < 1) gs = 1;
     for (int redo = 0; redo < 2; ++redo) {
-        if (redo) k_scatter_clear<W><<<s.num_sms, 256, 0, st>>>(s.ctl, homes_of<W>(s));
         k_part_scatter<W><<<(int)gs, 256, 0, st>>>(pbufs_of<W>(s), homes_of<W>(s), s.ctl,
                                                    gate_of<W>(h), part_fn_of<W>(h), force, s.n,
                                                    s.part_target, redo);
@@ -524,8 +535,7 @@ static cudaError_t merge_wb(const DeviceState& s, const GateArg<W>& g, cudaStrea
     int grid = s.num_sms * per_sm;
     if (grid > s.max_ctas) grid = s.max_ctas;   // one candidate region per CTA
     k_gate_inplace<W, BLOCK><<<grid, BLOCK, smem, st>>>(pbufs_of<W>(s), homes_of<W>(s), s.ctl, g,
-                                                        s.delta, s.cand);
-    k_merge_check<<<1, 32, 0, st>>>(s.ctl, s.cap_M);
+                                                        s.delta, s.cand, s.cap_M);
     k_gate_part<W, BLOCK><<<s.num_sms * per_sm_full, BLOCK, smem_full, st>>>(
         pbufs_of<W>(s), homes_of<W>(s), s.ctl, g, s.delta, s.buf_cap);
     return cudaGetLastError();
