@@ -1,4 +1,5 @@
-// itpp_part.cu -- the per-gate merge with the table in shared memory.
+// itpp_part.cu -- a gate of a large state by separate launches: the partitioned
+// merge, in place.
 //
 // A gate's merge only pairs a string K with its partner QK (Sec. II.B: a
 // commuting string keeps cosh(theta) of itself and sends -sinh(theta) s to QK).
@@ -6,28 +7,26 @@
 // sites S, and group the state by the key with the sites of S cleared: K, QK
 // and every child under any gate of the window share that group.  The state
 // is scattered once per window into hash partitions of that masked key (one
-// streaming pass, one atomic per term on the partition's cursor), and then
-// every gate of the window runs a persistent kernel that takes one partition
-// at a time per CTA: the partition is staged in shared memory by bulk (TMA)
-// copies, each commuting string joins its partner {K, QK} in a shared-memory
-// table, one string of each pair computes both merged children, and the kept
-// children of the partition are written as one contiguous segment of an
-// output chunk the CTA holds (room claimed once their number is known, a
-// global atomic every few partitions).  The segments, listed by the partition
-// descriptors, are the partitions of the next gate of the window, so no
-// scatter runs between the gates of a window.  A group holds at most 4^|S|
-// terms; a partition above the staging capacity is merged in sub-passes,
-// each taking the pairs of one hash class of the key with the gate's sites
-// cleared, so no partition size forces a re-partition.  A gate acting on more
-// sites than a window allows is a window of its own, partitioned by its pair
-// key (the member of {K, QK} with the gate's lowest bit clear).
+// streaming pass, one atomic per term on the partition's cursor), and every
+// gate of the window then runs over the partitions where they lie
+// (itpp_inplace.cuh): a string keeps its place, its coefficient goes to the
+// same place of a second array (zero: no term any more), and the few new
+// strings are appended to the partition's stride, so keys are written only
+// where they are new and no scatter runs between the gates of a window.  A
+// group holds at most 4^|S| terms; a partition above a pass's capacity is
+// merged in sub-passes, each taking the pairs of one hash class of the key with
+// the gate's sites cleared, so no partition size forces a re-partition.  A gate
+// acting on more sites than a window allows is a window of its own,
+// partitioned by its pair key (the member of {K, QK} with the gate's lowest bit
+// clear).
 //
 // The top-M select (Sec. II.C, term bound) is folded into the merge: every
 // kept child is compared with a range around the threshold predicted for the
-// gate; the merge counts the children above it, lists those inside it and
-// leaves those below it unwritten (they are dropped by the select whenever at
-// least cap_M children lie at or above the range; otherwise the merge runs
-// again in full), and the select (itpp_select.cu) then works on that short
+// gate; the merge counts the kept children, lists those inside the range and
+// leaves out those below it (they are dropped by the select whenever at least
+// cap_M children lie at or above the range; otherwise, and when a stride ran
+// out, k_gate_part merges again in full from the unchanged input into a
+// contiguous run), and the select (itpp_select.cu) then works on that short
 // list instead of passing over every coefficient.
 #include <cstring>
 
@@ -174,7 +173,7 @@ __device__ __forceinline__ GateInput gate_input(const DevCtl* ctl) {
 // The gate's merge, in place (itpp_inplace.cuh): persistent CTAs, one
 // partition at a time, a later partition of the same CTA prefetched into L2
 // by bulk (TMA) requests.  With a top-M bound the children at or
-// below the select's lower limit are left out; k_merge_check then keeps the
+// below the select's lower limit are left out; merge_check then keeps the
 // result when at least cap_M were kept and no partition's stride ran out, and
 // otherwise k_gate_part merges the gate again in full from the same input.
 template <int W, int BLOCK>
@@ -318,8 +317,6 @@ k_gate_part(Bufs<W> B, Homes<W> H, DevCtl* ctl, GateArg<W> g, double delta, uint
         s_stop = ctl->status || !ctl->retry;
         s_pd = pending_of<W>(ctl);
         s_rnorm = ctl->rnorm[cur];
-        g_cn = 0u;
-        g_range[0] = g_range[1] = 0ULL;
     }
     __syncthreads();
     if (s_stop) return;
@@ -349,8 +346,7 @@ k_gate_part(Bufs<W> B, Homes<W> H, DevCtl* ctl, GateArg<W> g, double delta, uint
         __syncthreads();
         return s_at;
     };
-    SelStats st{0ULL, 0u};
-    const CandRegions none{};
+    SelStats st{0ULL};
     uint32_t pass = 0;
     for (uint32_t p = blockIdx.x; p < in.P; p += gridDim.x) {
         uint64_t np = H.cursors(in.c)[p];
@@ -364,12 +360,11 @@ k_gate_part(Bufs<W> B, Homes<W> H, DevCtl* ctl, GateArg<W> g, double delta, uint
                 A::vals()[i] = __ldcs(cp + i);
             }
             __syncthreads();
-            stage_pass<W, BLOCK, PassRoom::kExact>((uint32_t)np, 0u, g, s_pd, s_rnorm, dbits,
-                                                   p == p_id, ctl, nxt, pass, kout, cout, st, none,
-                                                   room);
+            stage_pass<W, BLOCK, PassRoom::kExact>((uint32_t)np, g, s_pd, s_rnorm, dbits,
+                                                   p == p_id, ctl, nxt, pass, kout, cout, st, room);
         } else {
             merge_long<W, BLOCK>(kp, cp, np, g, s_pd, s_rnorm, dbits, p == p_id, ctl, nxt, &pass,
-                                 kout, cout, st, none, ~0ULL, room, nullptr, &s_n);
+                                 kout, cout, st, room, &s_n);
         }
     }
 #pragma unroll

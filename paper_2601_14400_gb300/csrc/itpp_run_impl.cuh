@@ -682,8 +682,7 @@ __device__ bool run_instance(const RunArgs<W>& a, const RunGate<W>* gates, int n
                 __syncthreads();
                 return s_at;
             };
-            SelStats ss{0ULL, 0u};
-            const CandRegions none{};
+            SelStats ss{0ULL};
             for (uint32_t p = team.rank; p < P; p += team.size) {
                 uint64_t np = __ldcg(arr.cnt(ci) + (uint64_t)p * kPad);
                 if (np > R) np = R;
@@ -696,13 +695,12 @@ __device__ bool run_instance(const RunArgs<W>& a, const RunGate<W>* gates, int n
                         PassArgs<W>::vals()[i] = __ldcs(cp + i);
                     }
                     __syncthreads();
-                    stage_pass<W, kBlock, PassRoom::kExact>((uint32_t)np, 0u, g, pd, s_pub.rnorm,
+                    stage_pass<W, kBlock, PassRoom::kExact>((uint32_t)np, g, pd, s_pub.rnorm,
                                                             dbits, p == p_id, ctl, np_, pass, kout,
-                                                            cout, ss, none, room);
+                                                            cout, ss, room);
                 } else {
                     merge_long<W, kBlock>(kp, cp, np, g, pd, s_pub.rnorm, dbits, p == p_id, ctl,
-                                          np_, &pass, kout, cout, ss, none, ~0ULL, room, nullptr,
-                                          &s_n);
+                                          np_, &pass, kout, cout, ss, room, &s_n);
                 }
             }
             n_long = 0;

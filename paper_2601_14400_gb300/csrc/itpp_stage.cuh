@@ -1,9 +1,10 @@
-// itpp_stage.cuh -- the partition merge's device building blocks, shared by
-// the single propagation (itpp_part.cu) and the batched one (itpp_batch.cu):
-// the partition function and plan, bulk (TMA) copies into shared memory on
-// an mbarrier, the staged pass of one gate over one partition (pair table,
-// merged children, threshold, write), and the sub-passes of a partition
-// above the staging capacity.
+// itpp_stage.cuh -- building blocks of the partitioned merge, shared by the
+// separate kernels (itpp_part.cu) and the run kernel (itpp_run_impl.cuh): the
+// partition function and plan, the scatter, and the merge in full of a
+// partition staged in shared memory (pair table, merged children, threshold,
+// write into a contiguous run), which is what a gate falls back to when the
+// in-place merge (itpp_inplace.cuh) left out children that the bound then
+// needed, or ran out of a partition's stride.
 #pragma once
 
 #include "itpp_common.cuh"
@@ -192,54 +193,8 @@ __device__ __forceinline__ void l2_prefetch_bulk(const void* p, uint64_t bytes) 
                          : "memory");
 }
 
-// ---------------------------------------------------------------------------
-// Bulk (TMA) copies into shared memory, completed on an mbarrier.  A copy
-// needs 16-byte aligned addresses and a size that is a multiple of 16 bytes.
-// ---------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
     return (uint32_t)__cvta_generic_to_shared(p);
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(smem_addr(bar)), "r"(count)
-                 : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-}
-
-// Arrive on the barrier and announce `bytes` of copies that complete it.
-__device__ __forceinline__ void mbar_expect(uint64_t* bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
-                 :: "r"(smem_addr(bar)), "r"(bytes) : "memory");
-}
-
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes,
-                                         uint64_t* bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes "
-                 "[%0], [%1], %2, [%3];"
-                 :: "r"(smem_addr(dst)), "l"(src), "r"(bytes), "r"(smem_addr(bar)) : "memory");
-}
-
-// Generic-proxy accesses to shared memory made before this fence are ordered
-// before later bulk copies into it.
-__device__ __forceinline__ void fence_async_shared() {
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-
-// Wait for the barrier's phase `parity` to complete, at most `limit` polls
-// (each poll may itself suspend the thread for a while).  False: timed out.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint32_t limit) {
-    const uint32_t a = smem_addr(bar);
-    for (uint32_t it = 0; it < limit; ++it) {
-        uint32_t done;
-        // the thread sleeps in the wait until the phase completes or the
-        // hint (nanoseconds) runs out, instead of polling
-        asm volatile("{\n\t.reg .pred p;\n\t"
-                     "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-                     "selp.u32 %0, 1, 0, p;\n\t}"
-                     : "=r"(done) : "r"(a), "r"(parity), "r"(1000000u) : "memory");
-        if (done) return true;
-    }
-    return false;
 }
 
 // Sub-pass of a long partition's commuting string: a hash of the key with
@@ -297,15 +252,14 @@ template <> struct StageGeom<1> { static constexpr int kItems = 1024, kSlots = 2
 template <> struct StageGeom<2> { static constexpr int kItems = 512, kSlots = 1024; };
 
 // Dynamic shared memory of the merge: the staged keys, their values (raw
-// coefficient in, normalised coefficient after the join; two spare slots let
-// a copy start at the 16-byte boundary below an odd element), the pair table
-// and the pass's work list.
+// coefficient in, normalised coefficient after the join), the pair table and
+// the pass's work list.
 template <int W>
 struct Stage {
     static constexpr int C = StageGeom<W>::kItems, S = StageGeom<W>::kSlots;
     static constexpr size_t kKeys = 0;
     static constexpr size_t kVals = kKeys + sizeof(PKey<W>) * C;
-    static constexpr size_t kTab = kVals + sizeof(double) * (C + 2);
+    static constexpr size_t kTab = kVals + sizeof(double) * C;
     static constexpr size_t kList = kTab + sizeof(uint32_t) * S;
     static constexpr size_t kBytes = (kList + sizeof(uint16_t) * C + 15) / 16 * 16;
     static_assert(kVals % 16 == 0 && kTab % 16 == 0, "alignment");
@@ -321,11 +275,6 @@ __shared__ unsigned long long g_range[2];   // candidate range [lo, hi] (hi == 0
 // per pass (indexed by its parity): the work list's lengths (pairs in the low
 // half, pass-through strings in the high half) and the children kept so far
 __shared__ uint32_t g_lists[2], g_kept[2];
-
-// Waits on a staging copy's barrier before the CTA gives up: each wait
-// sleeps up to a millisecond, and a copy of a few tens of kilobytes completes
-// within microseconds; this bound is seconds.
-constexpr uint32_t kWaitPolls = 4096u;
 
 // Commutation and the sign of Q P = s R in one pass over the masks.  Site by
 // site Q and P anticommute where bit (x qz ^ z qx) is set, and there their
@@ -408,11 +357,9 @@ __device__ __forceinline__ bool pair_enter(const PKey<W>& K, const GateArg<W>& g
     return false;
 }
 
-// Statistics of the kept children for the top-M select: the largest
-// pattern, the count above the candidate range, the candidates inside it.
+// Of the kept children: the largest pattern.
 struct SelStats {
     unsigned long long out_max;
-    uint32_t above;
 };
 
 template <int W>
@@ -420,7 +367,7 @@ struct PassArgs {
     __device__ __forceinline__ static PKey<W>* keys() {
         return reinterpret_cast<PKey<W>*>(g_stage + Stage<W>::kKeys);
     }
-    __device__ __forceinline__ static double* vals() {   // item i at vals()[shift + i]
+    __device__ __forceinline__ static double* vals() {
         return reinterpret_cast<double*>(g_stage + Stage<W>::kVals);
     }
     __device__ __forceinline__ static uint32_t* tab() {
@@ -450,8 +397,7 @@ template <int W, bool kWrite>
 __device__ __forceinline__ void emit_children(bool ka, bool kb, const PKey<W>& K,
                                               const GateArg<W>& g, double va, double vb,
                                               PKey<W>* kout, double* cout, uint64_t base,
-                                              uint32_t* kept, SelStats& st,
-                                              const CandRegions& cd) {
+                                              uint32_t* kept, SelStats& st) {
     const unsigned int ba = __ballot_sync(0xffffffffu, ka), bb = __ballot_sync(0xffffffffu, kb);
     const uint32_t na = __popc(ba), tot = na + __popc(bb);
     if (!tot) return;
@@ -474,27 +420,19 @@ __device__ __forceinline__ void emit_children(bool ka, bool kb, const PKey<W>& K
         b = abs_pattern(vb);
     }
     st.out_max = max(st.out_max, max(a, b));
-    const unsigned long long hi = g_range[1];
-    if (hi) {   // uniform
-        const unsigned long long lo = g_range[0], w = hi - lo;
-        st.above += (a > hi ? 1u : 0u) + (b > hi ? 1u : 0u);
-        // a - lo <= w on unsigned values: lo <= a <= hi (a kept child has a > 0)
-        cand_push(ka && a - lo <= w, a - lo, pa, cd, &g_cn);
-        cand_push(kb && b - lo <= w, b - lo, pb, cd, &g_cn);
-    }
 }
 
 // Phase B of a pass: the work list, pairs first (whole warps), then the
 // strings that pass through.  kWrite: store the kept children from `base` on;
 // kClear: leave the pair table free for the next pass.
 template <int W, int BLOCK, bool kWrite, bool kClear>
-__device__ __forceinline__ void pass_children(uint32_t n_pair, uint32_t n_through, uint32_t shift,
+__device__ __forceinline__ void pass_children(uint32_t n_pair, uint32_t n_through,
                                               const GateArg<W>& g, unsigned long long dbits,
                                               bool has_id, DevCtl* ctl, int nxt, PKey<W>* kout,
                                               double* cout, uint64_t base, uint32_t* kept,
-                                              SelStats& st, const CandRegions& cd) {
+                                              SelStats& st) {
     using A = PassArgs<W>;
-    const double* vals = A::vals() + shift;
+    const double* vals = A::vals();
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t pair_end = (n_pair + 31u) & ~31u;
     for (uint32_t j0 = threadIdx.x & ~31u; j0 < pair_end + n_through; j0 += BLOCK) {
@@ -549,7 +487,7 @@ __device__ __forceinline__ void pass_children(uint32_t n_pair, uint32_t n_throug
                 }
             }
         }
-        emit_children<W, kWrite>(ka, kb, K, g, va, vb, kout, cout, base, kept, st, cd);
+        emit_children<W, kWrite>(ka, kb, K, g, va, vb, kout, cout, base, kept, st);
     }
 }
 
@@ -572,22 +510,18 @@ enum class PassRoom { kAt, kExact, kCount };
 //
 // What bounds it: instruction issue, and the double-precision pipe (about two
 // lanes per clock and SM on GB300, a whole warp's slot for every instruction
-// however few lanes take part).  Hence the work list: over the strings
-// themselves only the quarter or so that owns a pair would be active in the
-// six double-precision instructions.  Against a per-string second phase, a
-// block scan and a third, writing phase this issues about a third of the
-// instructions and waits twice per partition instead of three times.
+// however few lanes take part): hence the work list.
 // Two barriers (and any the room call takes); returns the kept children
 // (the same on every thread).  `pass` numbers the CTA's passes: counters
 // alternate by its parity.
 template <int W, int BLOCK, PassRoom kRoom, class Room>
-__device__ __forceinline__ uint32_t stage_pass(uint32_t n, uint32_t shift, const GateArg<W>& g,
+__device__ __forceinline__ uint32_t stage_pass(uint32_t n, const GateArg<W>& g,
                                                const Pending<W>& pd, double rnorm,
                                                unsigned long long dbits, bool has_id, DevCtl* ctl,
                                                int nxt, uint32_t pass, PKey<W>* kout, double* cout,
-                                               SelStats& st, const CandRegions& cd, Room&& room) {
+                                               SelStats& st, Room&& room) {
     using A = PassArgs<W>;
-    double* vals = A::vals() + shift;
+    double* vals = A::vals();
     const uint32_t lane = threadIdx.x & 31u, par = pass & 1u;
     const unsigned int lt = (1u << lane) - 1u;
     for (uint32_t i0 = threadIdx.x & ~31u; i0 < n; i0 += BLOCK) {   // whole warps
@@ -634,19 +568,19 @@ __device__ __forceinline__ uint32_t stage_pass(uint32_t n, uint32_t shift, const
     if (kRoom == PassRoom::kAt) {
         const unsigned long long base = room(n_through + 2u * n_pair);
         if (base != ~0ULL)
-            pass_children<W, BLOCK, true, true>(n_pair, n_through, shift, g, dbits, has_id, ctl,
-                                                nxt, kout, cout, base, kept, st, cd);
+            pass_children<W, BLOCK, true, true>(n_pair, n_through, g, dbits, has_id, ctl,
+                                                nxt, kout, cout, base, kept, st);
         __syncthreads();                                              // (2) staging free
         return *kept;
     }
     if (kRoom == PassRoom::kCount) {
-        pass_children<W, BLOCK, false, true>(n_pair, n_through, shift, g, dbits, has_id, ctl, nxt,
-                                             kout, cout, 0ULL, kept, st, cd);
+        pass_children<W, BLOCK, false, true>(n_pair, n_through, g, dbits, has_id, ctl, nxt,
+                                             kout, cout, 0ULL, kept, st);
         __syncthreads();
         return *kept;
     }
-    pass_children<W, BLOCK, false, false>(n_pair, n_through, shift, g, dbits, has_id, ctl, nxt,
-                                          kout, cout, 0ULL, kept, st, cd);
+    pass_children<W, BLOCK, false, false>(n_pair, n_through, g, dbits, has_id, ctl, nxt,
+                                          kout, cout, 0ULL, kept, st);
     __syncthreads();
     const uint32_t tot = *kept;
     const unsigned long long base = room(tot);
@@ -654,38 +588,34 @@ __device__ __forceinline__ uint32_t stage_pass(uint32_t n, uint32_t shift, const
     if (threadIdx.x == 0) *kept = 0u;
     __syncthreads();
     if (base != ~0ULL)
-        pass_children<W, BLOCK, true, true>(n_pair, n_through, shift, g, dbits, has_id, ctl, nxt,
-                                            kout, cout, base, kept, st, cd);
+        pass_children<W, BLOCK, true, true>(n_pair, n_through, g, dbits, has_id, ctl, nxt,
+                                            kout, cout, base, kept, st);
     else   // no room: the caller goes on with other instances, the table free
-        pass_children<W, BLOCK, false, true>(n_pair, n_through, shift, g, dbits, has_id, ctl, nxt,
-                                             kout, cout, 0ULL, kept, st, cd);
+        pass_children<W, BLOCK, false, true>(n_pair, n_through, g, dbits, has_id, ctl, nxt,
+                                             kout, cout, 0ULL, kept, st);
     __syncthreads();
     return tot;
 }
 
 // A partition above the staging capacity, in k sub-passes over the hash
 // classes of the key with the gate's sites cleared (about C/2 strings each,
-// gathered into the staging arrays).  Its children stay one segment: from
-// `pre` on when the caller holds room for 2 np children there (the same on
-// every thread), else a first round of the sub-passes only counts them,
-// room(total) gives the segment's position (~0: none, nothing is written)
-// and a second round writes them.  Every thread calls it; it returns the
-// children counted.
+// gathered into the staging arrays).  A first round of the sub-passes only
+// counts their children, room(total) gives a run's position (~0: none, nothing
+// is written) and a second round writes them.  Every thread calls it.
 template <int W, int BLOCK, class Room>
-__device__ __forceinline__ uint32_t merge_long(const PKey<W>* kp, const double* cp, uint64_t np,
+__device__ __forceinline__ void merge_long(const PKey<W>* kp, const double* cp, uint64_t np,
                                             const GateArg<W>& g, const Pending<W>& pd,
                                             double rnorm, unsigned long long dbits, bool has_id,
                                             DevCtl* ctl, int nxt, uint32_t* pass,
                                             PKey<W>* kout, double* cout, SelStats& st,
-                                            const CandRegions& cd, unsigned long long pre,
-                                            Room&& room, unsigned int* cursor_p, uint32_t* s_n) {
+                                            Room&& room, uint32_t* s_n) {
     using A = PassArgs<W>;
     constexpr uint32_t C = Stage<W>::C;
     const uint32_t k = (uint32_t)((2 * np + C - 1) / C);
     uint32_t total = 0;
-    for (int write = pre != ~0ULL ? 1 : 0; write < 2; ++write) {
-        unsigned long long base = pre;
-        if (write && pre == ~0ULL) {
+    for (int write = 0; write < 2; ++write) {
+        unsigned long long base = 0ULL;
+        if (write) {
             base = room(total);
             if (base == ~0ULL) break;
         }
@@ -713,24 +643,21 @@ __device__ __forceinline__ uint32_t merge_long(const PKey<W>* kp, const double* 
                 }
             }
             __syncthreads();
-            // every thread has read the cursor: leave it zero for the next scatter
-            if (j == 0 && cursor_p && threadIdx.x == 0) *cursor_p = 0u;
             const uint32_t n = *s_n < C ? *s_n : C;
             *pass += 1u;
             if (write) {
                 const unsigned long long at = base + done;
                 done += stage_pass<W, BLOCK, PassRoom::kAt>(
-                    n, 0u, g, pd, rnorm, dbits, has_id, ctl, nxt, *pass, kout, cout, st, cd,
+                    n, g, pd, rnorm, dbits, has_id, ctl, nxt, *pass, kout, cout, st,
                     [at](uint32_t) { return at; });
             } else {
                 done += stage_pass<W, BLOCK, PassRoom::kCount>(
-                    n, 0u, g, pd, rnorm, dbits, has_id, ctl, nxt, *pass, kout, cout, st, cd,
+                    n, g, pd, rnorm, dbits, has_id, ctl, nxt, *pass, kout, cout, st,
                     [](uint32_t) { return 0ULL; });
             }
         }
         total = done;
     }
-    return total;
 }
 
 // The partition that holds the identity (the all-zero key, in every mode of
@@ -746,8 +673,7 @@ __device__ __forceinline__ uint32_t identity_part(uint32_t P) {
 
 template <int W, int BLOCK>
 struct PartOcc {
-    // CTAs per SM the launch bound asks for: the staging and table take
-    // Stage<W>::kBytes of shared memory per CTA
+    // CTAs per SM that the launch bound of the merge in full asks for
     static constexpr int kMin = BLOCK <= 256 ? (W == 1 ? 6 : 5) : 2;
 };
 
