@@ -106,6 +106,16 @@ __device__ __forceinline__ void list_if(bool on, uint32_t* count, uint16_t* list
                  : "memory");
 }
 
+// The identity's merged child, of pattern a.  At or below the threshold the
+// trace is lost; at or below the limit predicted for the select only the
+// prediction is wrong (the thresholds of a state's first gates move by octaves),
+// and the gate is merged again in full.
+__device__ __forceinline__ void identity_kept(bool keep, unsigned long long a, DevCtl* ctl, int* over) {
+    if (keep) return;
+    if (a <= g_delta) set_status(ctl, ST_TRACE_ZERO, 1);
+    else *over = 1;
+}
+
 // A thread's strings of a pass (row r: string r * BLOCK + thread), zero past the
 // end.
 template <int W, int BLOCK>
@@ -235,7 +245,7 @@ __device__ __forceinline__ void inplace_pass(uint32_t n, const GateArg<W>& g,
         if (!kPlain && (f & kSpecial) && (f & kLive) && !dup) {
             if (has_id && key_is_zero(load_key_ca(io.keys + at))) {
                 ctl->norm[nxt] = va;
-                if (!keep) set_status(ctl, ST_TRACE_ZERO, 1);
+                identity_kept(keep, a, ctl, io.over);
                 keep = true;
             } else {
                 keep = false;
@@ -292,7 +302,7 @@ __device__ __forceinline__ void inplace_pass(uint32_t n, const GateArg<W>& g,
                 ka = above(va, thr) && (!weigh || light(X, g.maxw));
                 if (id) {
                     ctl->norm[nxt] = va;
-                    if (!ka) set_status(ctl, ST_TRACE_ZERO, 1);
+                    identity_kept(ka, abs_pattern(va), ctl, io.over);
                     ka = true;
                 }
                 __stcs(io.cout + at, ka ? va : 0.0);

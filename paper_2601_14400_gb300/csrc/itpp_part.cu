@@ -208,6 +208,7 @@ k_gate_inplace(Bufs<W> B, Homes<W> H, DevCtl* ctl, GateArg<W> g, double delta, C
         const unsigned long long dbits = (unsigned long long)__double_as_longlong(delta);
         const unsigned long long thr = ctl->sp_hi && ctl->sp_thr > dbits ? ctl->sp_thr : dbits;
         s_thr = thr;
+        g_delta = dbits;
         if (blockIdx.x == 0 && !ctl->status) {
             ctl->drop_on = thr != dbits;
             ctl->cand_regions = gridDim.x;

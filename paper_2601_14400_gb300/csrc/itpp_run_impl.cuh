@@ -327,6 +327,7 @@ __device__ bool run_instance(const RunArgs<W>& a, const RunGate<W>* gates, int n
     // start: the published state from the control block, the cursor arrays
     // zero, no chain head of an earlier use
     if (threadIdx.x < 8) s_stat[threadIdx.x] = 0ULL;
+    if (threadIdx.x == 0) g_delta = a.delta_bits;
     inplace_init<W, kBlock, 12>();
     for (uint32_t i = team.rank * kBlock + threadIdx.x; i < 3u * a.part_max; i += team.size * kBlock)
         arr.n0[(uint64_t)i * kPad] = 0u;

@@ -272,6 +272,7 @@ struct Stage {
 extern __shared__ __align__(16) unsigned char g_stage[];
 __shared__ uint32_t g_cn;        // this CTA's candidates
 __shared__ unsigned long long g_range[2];   // candidate range [lo, hi] (hi == 0: none)
+__shared__ unsigned long long g_delta;      // the threshold's own pattern
 // per pass (indexed by its parity): the work list's lengths (pairs in the low
 // half, pass-through strings in the high half) and the children kept so far
 __shared__ uint32_t g_lists[2], g_kept[2];
