@@ -220,8 +220,11 @@ __device__ __forceinline__ void inplace_pass(uint32_t n, const GateArg<W>& g,
     // child_may_pass as one sum: the high words of |c| and |m| against the
     // threshold's
     const int ht = (int)(thr >> 32);
-    const int hm = ht < 0x00100000 ? 0x40000000
-                                   : (int)(__double2hiint(g.msh) & 0x7fffffff) - 0x3ff00000 + 0x2c140 - ht;
+    // (a sum at or above zero whatever |c| is: cut off, so that |c| of 2 and
+    // more does not carry it past the largest int)
+    const int hm = ht < 0x00100000 ? 0
+                                   : min(0, (int)(__double2hiint(g.msh) & 0x7fffffff) - 0x3ff00000 +
+                                                0x2c140 - ht);
     double* op = io.cout + threadIdx.x;
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) {

@@ -141,6 +141,30 @@ def test_ties_by_key(n, M, classes, separate):
     assert max(abs(got[k] - want[k]) / want[k] for k in want) <= 3 * 2.0 ** -53
 
 
+# Coefficients far above the identity's, with no threshold: every child is kept.
+@pytest.mark.parametrize("separate", [False, True])
+@pytest.mark.parametrize("c0", [1.5, 3.0, 2.0 ** 40, 2.0 ** 300])
+@pytest.mark.parametrize("delta", [0.0, 1e-300])
+def test_large_coefficients_keep_their_children(delta, c0, separate):
+    n, M = 20, 300
+    x = np.arange(M, dtype=np.uint64)[:, None]        # X on the low sites
+    z = np.zeros((M, 1), dtype=np.uint64)
+    c = np.full(M, c0)
+    c[0] = 1.0
+    gz = np.array([[1 << 19]], dtype=np.uint64)
+    p = itpp.Propagator(n, np.zeros_like(gz), gz, np.array([0.5]), 1.0, delta, 1 << 12, 0)
+    if separate:
+        p.profile_enable(True)
+    p.set_terms(x, z, c)
+    p.apply_trotter_layer(1)
+    px, pz, pc = p.terms()
+    got = {(int(a[0]), int(b[0])): abs(v) for a, b, v in zip(px, pz, pc)}
+    t = math.sinh(0.5) / math.cosh(0.5)
+    want = {(k, q): c[k] * (t if q else 1.0) for k in range(M) for q in (0, 1 << 19)}
+    assert got.keys() == want.keys()
+    assert max(abs(got[k] - want[k]) / want[k] for k in want) <= 6 * 2.0 ** -53
+
+
 # more instances than CTAs, one instance, and a few over all of them
 @pytest.mark.parametrize("B,n,cap", [(1, 24, 9000), (3, 20, 5000), (700, 7, 300)])
 def test_batch_teams(B, n, cap):
