@@ -39,9 +39,9 @@ METRIC = "Pauli terms/s per Trotter gate"
 UNIT = "terms/s"
 # Profiling kinds of the library (itpp_profile_read) per merge path.
 KERNEL_NAMES = {
-    0: {0: "k_part_scatter (scatter by pair key)",
-        1: "k_gate_part (partition merge: branch-emit-merge-truncate)",
-        2: "top-M select chain (k_cap_*, k_cand_*, k_tie_*)",
+    0: {0: "k_part_scatter (scatter by window)",
+        1: "k_gate_inplace (partition merge in place: branch-emit-merge-truncate)",
+        2: "top-M select (k_sel_hist, k_sel_gather, k_sel_resolve)",
         3: "expectation (k_obs_*)"},
     1: {0: "(unused)",
         1: "sorted merge (expand, radix passes, segmented reduce)",
@@ -778,7 +778,7 @@ def record_traffic(args):
     with open(args.record_traffic, newline="") as f:
         lines = [ln for ln in f if ln.startswith('"')]
     for r in csv.DictReader(lines):
-        if "k_gate_part" not in r.get("Kernel Name", ""):
+        if "k_gate_inplace" not in r.get("Kernel Name", ""):
             continue
         d = rows.setdefault(r["ID"], {})
         v = float(r["Metric Value"].replace(",", ""))
@@ -789,24 +789,16 @@ def record_traffic(args):
     launches = [rows[k] for k in sorted(rows, key=int)
                 if "dram__bytes_read.sum" in rows[k] and "dram__bytes_write.sum" in rows[k]]
     if not launches:
-        print(json.dumps({"error": "no k_gate_part launch with DRAM bytes in "
+        print(json.dumps({"error": "no k_gate_inplace launch with DRAM bytes in "
                           + args.record_traffic}))
         return 1
-    # a gate launches the merge twice (the second returns at once unless the
-    # first must be redone): bytes per gate are those of a pair of launches;
-    # the recorded figure is the mean over the gates that were not redone
-    # (the mean over all of them is kept beside it)
+    # one launch of it per gate (k_gate_part, which repeats a gate in full where
+    # that must be, is not counted here: merge_retries_per_gate says how often)
     per = [d["dram__bytes_read.sum"] + d["dram__bytes_write.sum"] for d in launches]
-    pairs = [(per[i], per[i + 1] if i + 1 < len(per) else 0.0) for i in range(0, len(per), 2)]
-    tot_all = [a + b for a, b in pairs]
-    redone = [b > 1e6 for a, b in pairs]   # a second launch that returned at once moves ~0
-    tot = [a for (a, b), r in zip(pairs, redone) if not r] or tot_all
-    rec = {"kernel_class": 1, "kernel": "k_gate_part", "source_digest": source_digest(),
-           "bytes_per_launch": args.traffic_scale * sum(tot) / len(tot),
-           "measured_bytes_per_launch": sum(tot) / len(tot), "scale": args.traffic_scale,
-           "launches_measured": len(per), "gates_measured": len(tot_all),
-           "gates_redone": sum(redone),
-           "bytes_per_gate_all_measured": sum(tot_all) / len(tot_all),
+    rec = {"kernel_class": 1, "kernel": "k_gate_inplace", "source_digest": source_digest(),
+           "bytes_per_launch": args.traffic_scale * sum(per) / len(per),
+           "measured_bytes_per_launch": sum(per) / len(per), "scale": args.traffic_scale,
+           "launches_measured": len(per),
            "first_launches": [{"dram_read": int(d["dram__bytes_read.sum"]),
                                "dram_write": int(d["dram__bytes_write.sum"]),
                                "duration_ns": int(d.get("gpu__time_duration.sum", 0))}
@@ -814,7 +806,7 @@ def record_traffic(args):
            "workload": args.workload, "command": args.traffic_command}
     with open(os.path.join(ROOT, "profiles", "traffic.json"), "w") as f:
         json.dump(rec, f, indent=2)
-    print(json.dumps({"bytes_per_launch": rec["bytes_per_launch"], "gates": len(tot)}))
+    print(json.dumps({"bytes_per_launch": rec["bytes_per_launch"], "gates": len(per)}))
     return 0
 
 
@@ -1041,9 +1033,9 @@ def main():
     return 0
 
 
-# the sources of the partition merge kernel (k_gate_part): its recorded DRAM
+# the sources of the partition merge kernel (k_gate_inplace): its recorded DRAM
 # traffic stays valid while these are unchanged
-MERGE_SOURCES = ("itpp_part.cu", "itpp_stage.cuh", "itpp_common.cuh", "itpp_gate_body.cuh",
+MERGE_SOURCES = ("itpp_part.cu", "itpp_inplace.cuh", "itpp_stage.cuh", "itpp_common.cuh", "itpp_gate_body.cuh",
                  "itpp_launch.h")
 
 

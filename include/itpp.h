@@ -83,8 +83,9 @@ typedef struct {
      * 0: partitioned merge (default): the state is scattered into hash
      *    partitions of the key with a window's sites cleared (consecutive
      *    gates acting on a few sites share one scatter) or of the pair key
-     *    {K, Q.K}, and each partition is merged through an open-addressing
-     *    table in shared memory.
+     *    {K, Q.K}, and each partition is merged where it lies, partners found
+     *    through a hash of chains in shared memory.  Bounds up to 2^20 terms
+     *    run whole layers in one launch (default block_threads only).
      * 1: sort fallback: the commuting terms' children are radix-sorted on
      *    the whole key (8-bit digits, digits above bit n skipped) and runs of
      *    equal keys are summed by a segmented reduce; anticommuting terms,
@@ -94,7 +95,8 @@ typedef struct {
     int merge_path;
     /* Tuning (0 = library default or the autotuned value):
      * table_load_pct: highest load of the merge table, in percent (10..75).
-     * block_threads: threads per CTA of the gate kernels (128, 256, 512).
+     * block_threads: threads per CTA of the gate kernels (128, 256, 512;
+     * default 256, for the partitioned merge of two mask words 128).
      * items_per_thread: terms per thread per tile (1, 2, 4; the partitioned
      * merge holds at most two). */
     int table_load_pct;
@@ -114,8 +116,8 @@ typedef struct {
     int trotter_order;
     /* Partitioned merge (merge_path 0): the mean partition size the scatter
      * aims for, 64..2048 terms (0: the library default).  Larger partitions
-     * amortise the per-partition work; a partition above one CTA's staging
-     * capacity (1,024 terms at W = 1, 512 at W = 2) is merged in slower
+     * amortise the per-partition work; a partition above the capacity of a
+     * CTA's pass (1,024 terms at W = 1, 512 at W = 2) is merged in slower
      * sub-passes. */
     int partition_target;
     int reserved[2];
@@ -342,8 +344,8 @@ itpp_status itpp_set_alpha(itpp_handle h, const double* alpha);
  *   value        host or NULL: f.
  * The kept support includes the term bound: with cap_policy 1 the frozen
  * support of a step is its top-M set.  Device memory: one snapshot per
- * segment plus, for every step of the largest segment, its output before and
- * after the bound and four int32 maps, allocated for the call.  After the call the handle
+ * segment plus, for every step of the largest segment, its output after the
+ * bound and four int32 maps, allocated for the call.  After the call the handle
  * holds the forward's final state.  Synchronising. */
 itpp_status itpp_adjoint(itpp_handle h, int n_layers, int ckpt_every, const uint64_t* obs_x,
                          const uint64_t* obs_z, const double* w, int m, double* grad_alpha,
@@ -369,14 +371,13 @@ itpp_status itpp_frozen_value(itpp_handle h, int n_layers, int ckpt_every,
  * ------------------------------------------------------------------------- */
 
 /* Create B independent propagations (Algorithm 1 for each), advanced
- * together: in every Trotter layer, gate g of every instance that has one
- * runs in the same kernel launches, and the whole layer is one CUDA graph
- * launch.  Each instance's state is bit-identical to a plain run of the same
- * Hamiltonian with the same parameters.  p->merge_path 0 (default): every
- * gate scatters each instance's terms into hash partitions of its pair key
- * and merges the partitions of all instances in one launch of the
- * shared-memory merge (p->partition_target as in itpp_create); 2: one global
- * merge table per instance; 1 is not offered for batches (ITPP_ERR_ARG).
+ * together.  Each instance's state is bit-identical to a plain run of the same
+ * Hamiltonian with the same parameters.  p->merge_path 0 (default): one launch
+ * runs all layers, a team of CTAs for every instance (the partitioned merge,
+ * p->partition_target as in itpp_create); 2: one global merge table per
+ * instance, gate g of every instance that has one in the same kernel launches
+ * and a layer one CUDA graph launch; 1 is not offered for batches
+ * (ITPP_ERR_ARG).
  *   B            1..65535 instances.
  *   n[B]         sites per instance (1..128); all instances use
  *                W = ceil(max n / 64) mask words.
@@ -389,7 +390,7 @@ itpp_status itpp_frozen_value(itpp_handle h, int n_layers, int ckpt_every,
  *   cuda_stream  stream to run on; NULL makes the library create its own
  *                (graph capture needs a non-legacy stream).
  * Memory: per instance two buffers of 2*cap_M terms, a table and a control
- * block (about 0.6 MB), and for merge_path 0 a scatter buffer of about
+ * block (about 0.6 MB), and for merge_path 0 a partition buffer of about
  * 2.5*cap_M terms.  Errors: as itpp_create. */
 itpp_status itpp_batch_create(int B, const int* n, const int* n_gates, const uint64_t* gate_x,
                               const uint64_t* gate_z, const double* alpha, double dtau,
@@ -404,18 +405,18 @@ itpp_status itpp_batch_apply_trotter_layer(itpp_batch_handle h, int n_layers);
 itpp_status itpp_batch_synchronize(itpp_batch_handle h);
 
 /* The launch shape of a batch, chosen by timing (the autotuner of the
- * batched path).  Partitioned merge (merge_path 0): threads per CTA of the
- * partition merge (128, 256, 512), its CTAs per SM (2, 4, or as many as fit),
- * the scatter's CTAs per SM (4, 8, 16) and the mean partition size (350,
- * 500, 700, 1000 terms at W = 1; 150, 300, 450 at W = 2; not tried when
- * itpp_batch_create was given a partition_target).  Global table
+ * batched path).  Partitioned merge (merge_path 0): the run's CTAs per SM
+ * (fewer than fit, or as many as fit), the smallest partition that a scatter
+ * makes to give every CTA of a team one (16 insert_grid strings) and the mean
+ * partition size (not tried when itpp_batch_create was given a
+ * partition_target).  Global table
  * (merge_path 2): threads per CTA of the branch-emit kernel (128, 256, 512;
  * two terms per thread), its CTAs per SM (2, 4, 8), the table build's CTAs
  * per SM (4, 8, 16) and the merge table's highest load (25..65 %;
  * itpp_batch_create with table_load_pct 0 sizes the tables for 25 %,
  * otherwise loads below the requested one are not tried).
  * Each candidate is timed with CUDA events over probe_layers Trotter layers
- * from the identity, replayed as the layer graph; coordinate descent from
+ * from the identity; coordinate descent from
  * the default shape, one parameter at a time.  The fastest shape stays
  * installed.  Every instance is reset to the identity before each timing
  * and after the search (statistics cleared), so results never depend on the
@@ -425,11 +426,12 @@ itpp_status itpp_batch_synchronize(itpp_batch_handle h);
 typedef struct {
     int main_block;              /* threads per CTA of the merge kernel          */
     int main_grid;               /* its CTAs per SM                              */
-    int insert_grid;             /* CTAs per SM of the scatter / table build     */
+    int insert_grid;             /* partitioned: smallest partition / 16; global
+                                  * table: CTAs per SM of the table build       */
     int table_load_pct;          /* global table: highest load (%); else 0       */
     double ms_per_probe;         /* the chosen shape: probe_layers layers (ms)   */
     double ms_per_probe_default; /* the default shape (partitioned: 256 threads,
-                                  * as many CTAs as fit, 8, the default size;
+                                  * as many CTAs as fit, 128, the default size;
                                   * global table: 256, 4, 8, 50 %)              */
     int candidates;              /* shapes timed                                 */
     int partition_target;        /* partitioned: mean partition size; else 0     */

@@ -8,7 +8,7 @@
 // Every instance runs the device bodies of the single propagation
 // (itpp_gate_body.cuh), so its state is bit-identical to a plain run.  This is
 // the global-table batch (merge_path 2); the partitioned one (merge_path 0) is
-// the run kernel of itpp_run.cu with a team of CTAs for every instance.
+// the run kernel (itpp_run_impl.cuh) with a team of CTAs for every instance.
 // Instances with fewer gates per layer sit out the later steps.  A whole
 // layer (all steps) is captured once into a CUDA graph by the C ABI and
 // replayed, since every quantity that changes between layers lives on the

@@ -223,7 +223,7 @@ itpp_status launch_one_gate(itpp_ctx* h, int k) {
         h->contiguous = false;
         // a window's first gate (or any gate after the state changed
         // elsewhere) re-partitions; later gates of the window read the
-        // previous gate's segments unless a partition outgrew the limit
+        // partitions where the previous gate left them
         const int force = g.win_start || h->part_epoch != h->state_epoch ||
                           h->part_last != k - 1;
         EventPair* ev0 = prof_begin(h, 0);

@@ -5,7 +5,12 @@
 //   state buffers 0 and 1, each 2*cap_M terms:
 //     keys  PKey<W>[2*cap_M]  AoS, 16*W bytes per term: x[0..W-1], z[0..W-1]
 //     coef  double[2*cap_M]   raw (un-normalised) coefficients
+//   homes        two sets of partitions of a fixed stride (itpp_part.cu), which
+//                hold the state inside a window of gates: their keys and two
+//                coefficient arrays in one more buffer of 2.5*cap_M terms and
+//                in the state buffer the state is not in
 //   merge table  Slot<W>[2^t]  open addressing, 32 B (W=1) / 64 B (W=2) slots
+//                (global-table merge, import, gradients; scratch of the selects)
 //   DevCtl       counters, the current-buffer index, normalisers, status
 // The stored coefficient of term i is raw[i]; its value is raw[i] * rnorm[cur]
 // with rnorm = 1 / (raw identity coefficient), and exactly 1 for the identity

@@ -55,7 +55,7 @@ struct itpp_ctx {
     // changes the state bumps state_epoch
     uint64_t state_epoch = 1, part_epoch = 0;
     int part_last = -1;
-    // gates run in one launch (itpp_run.cu): bounds up to run_max terms; the
+    // gates run in one launch (itpp_run_impl.cuh): bounds up to kRunMax terms; the
     // team's shared block and the partition cursors
     bool run_ok = false;
     int run_grid = 0;

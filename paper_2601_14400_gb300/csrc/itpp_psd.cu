@@ -23,7 +23,7 @@
 // passes it goes on a queue per warp and is looked up and summed 32 at a time: a
 // warp holds the double-precision pipe for every instruction however few of its
 // lanes have a pair (448 us for 2^18 terms and 63 strings when each lane did its
-// own, 190 us this way).  Each pair {P, O_j.P} is taken once, from the member without O_j's
+// own, 185 us this way).  Each pair {P, O_j.P} is taken once, from the member without O_j's
 // lowest bit, and counts twice.
 #include "itpp_common.cuh"
 #include "itpp_gate_body.cuh"

@@ -1,5 +1,5 @@
-// itpp_run.cuh -- arguments of the run kernel (itpp_run.cu): a layer's gates
-// in one launch.
+// itpp_run.cuh -- arguments of the run kernel (itpp_run_impl.cuh): a layer's
+// gates in one launch.
 #pragma once
 
 #include <cstddef>

@@ -393,7 +393,7 @@ __device__ __forceinline__ void pass_init() {
 
 // Count (and with kWrite store) a warp's kept children: K with va, and KQ with
 // vb.  One shared atomic per warp gives the run; the order inside a
-// partition's segment is immaterial.  Every lane of the warp calls it.
+// run is immaterial.  Every lane of the warp calls it.
 template <int W, bool kWrite>
 __device__ __forceinline__ void emit_children(bool ka, bool kb, const PKey<W>& K,
                                               const GateArg<W>& g, double va, double vb,

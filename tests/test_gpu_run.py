@@ -230,3 +230,26 @@ def test_observable_table(m):
     want = np.array([at.get((int(a[0]), int(b[0])), 0.0) for a, b in zip(x, z)])
     got = g.coeffs(x, z)
     assert (got.view(np.uint64) == want.view(np.uint64)).all()
+
+
+# A layer captured on the caller's stream and replayed: one launch (0) and a
+# chain of them (128 threads).
+@pytest.mark.parametrize("block", [0, 128])
+def test_layer_under_capture(block):
+    torch = pytest.importorskip("torch")
+    H = wl.tfim_1d(24, 1.0, 1.1, periodic=True)
+    s = torch.cuda.Stream()
+    g = itpp.Propagator(H.n, H.gate_x, H.gate_z, H.alpha, 0.05, 1e-9, 3000, 1,
+                        stream=s, block_threads=block)
+    g.apply_trotter_layer(2)
+    g.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=s):
+        g.apply_trotter_layer(1)
+    with torch.cuda.stream(s):
+        graph.replay()
+        graph.replay()
+    torch.cuda.synchronize()
+    o = oracle.Oracle(H.n, H.gate_x, H.gate_z, H.alpha, 0.05, 1e-9, 3000, 1)
+    o.apply_layers(4)
+    assert_same_state(g.terms(), o.terms(), f"block {block}")
