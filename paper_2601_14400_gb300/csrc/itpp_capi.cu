@@ -572,8 +572,7 @@ itpp_status itpp_create(int n, const uint64_t* gate_x, const uint64_t* gate_z,
         if (p->cap_M <= kRunMax && (p->block_threads == 0 || p->block_threads == 256)) {
             const uint64_t parts = p->cap_M / kRunMinPart + 1;
             h->run_grid = (int)std::min<uint64_t>((uint64_t)sms * run_fit(W, false), parts);
-            h->run_part_max = (uint32_t)std::max<uint64_t>(p->cap_M / s.part_target + 2,
-                                                           (uint64_t)h->run_grid + 1);
+            h->run_part_max = (uint32_t)(p->cap_M / s.part_target + 2 + (uint64_t)h->run_grid);
             ok &= ok && cudaMalloc(&h->run_shared, run_shared_bytes()) == cudaSuccess;
             ok &= ok && cudaMalloc(reinterpret_cast<void**>(&h->run_cnt),
                                    (size_t)h->run_part_max * 3 * kRunPad * sizeof(unsigned int)) == cudaSuccess;
