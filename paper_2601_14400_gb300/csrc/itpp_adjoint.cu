@@ -660,6 +660,7 @@ itpp_status adjoint_w(itpp_ctx* h, int L, int K, const uint64_t* obs_x, const ui
     cudaStream_t st = h->stream;
     const int G = (int)h->gates.size();
     const long long S = (long long)L * G;
+    if (K > L) K = L;   // one segment holds them all
     const int n_seg = (L + K - 1) / K;
     const size_t kb = sizeof(PKey<W>);
     const int grid = s.num_sms * 8;

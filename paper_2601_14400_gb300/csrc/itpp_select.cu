@@ -76,16 +76,9 @@ struct Pick {
 };
 
 // The digit (in descending order) holding the k-th largest value, from a
-// histogram of kSelBins counts (global 64-bit counts read through L2, or
-// 32-bit shared ones); NT threads, result in *out (shared).
-template <int NT, bool kGlobal>
-__device__ __forceinline__ unsigned long long hist_at(const void* hist, int b) {
-    return kGlobal ? __ldcg(static_cast<const unsigned long long*>(hist) + b)
-                   : (unsigned long long)static_cast<const unsigned int*>(hist)[b];
-}
-
-template <int NT, bool kGlobal>
-__device__ __forceinline__ void pick_digit(const void* hist, unsigned long long k,
+// histogram of kSelBins counts; NT threads, result in *out (shared).
+template <int NT>
+__device__ __forceinline__ void pick_digit(const unsigned long long* hist, unsigned long long k,
                                            unsigned long long* s_part, Pick* out) {
     constexpr int PER = kSelBins / NT;
     const int t = threadIdx.x;
@@ -93,12 +86,12 @@ __device__ __forceinline__ void pick_digit(const void* hist, unsigned long long 
     // two passes over this thread's bins (sum, then find) instead of
     // holding PER counts in registers
     unsigned long long sum = 0;
-    for (int j = 0; j < PER; ++j) sum += hist_at<NT, kGlobal>(hist, kSelBins - 1 - PER * t - j);
+    for (int j = 0; j < PER; ++j) sum += __ldcg(hist + kSelBins - 1 - PER * t - j);
     const unsigned long long incl = scan_nt<NT>(sum, s_part);
     unsigned long long run = incl - sum;
     if (run < k && k <= incl) {
         for (int j = 0; j < PER; ++j) {
-            const unsigned long long hv = hist_at<NT, kGlobal>(hist, kSelBins - 1 - PER * t - j);
+            const unsigned long long hv = __ldcg(hist + kSelBins - 1 - PER * t - j);
             if (run < k && k <= run + hv) {
                 out->digit = kSelBins - 1 - PER * t - j;
                 out->k_in = k - run;
@@ -172,17 +165,13 @@ k_sel_hist(Bufs<W> B, Homes<W> H, DevCtl* ctl) {
     __syncthreads();
     if (!s_last) return;
     __threadfence();
-    pick_digit<256, true>(ctl->sel_hist, ctl->sel_k, s_part, &s_pick);
+    pick_digit<256>(ctl->sel_hist, ctl->sel_k, s_part, &s_pick);
     if (threadIdx.x == 0) {
         const Pick pk = s_pick;
         ctl->sel_prefix = (unsigned long long)pk.digit << sh;
         ctl->sel_mask = (unsigned long long)(kSelBins - 1) << sh;
         ctl->sel_k = pk.k_in;
         ctl->sel_top = sh;
-        if (sh == 0) {          // every bit of v fixed: the digit's terms are exact ties
-            ctl->sel_ties = pk.count;
-            ctl->sel_tie_k = pk.k_in;
-        }
         ctl->sel_done = 0u;
     }
     for (int b = threadIdx.x; b < kSelBins; b += blockDim.x) ctl->sel_hist[b] = 0ULL;
