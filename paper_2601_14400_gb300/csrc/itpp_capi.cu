@@ -178,8 +178,6 @@ itpp_status run_launch(itpp_ctx* h, int k0, int n, int n_layers, unsigned long l
     a.min_part = kRunMinPart;
     a.cap_policy = s.cap_policy;
     a.maxw = h->p.max_weight ? h->p.max_weight : (1 << 30);
-    if (!h->contiguous && launch_materialize(s, h->stream) != cudaSuccess) return cuda_fail(h);
-    h->contiguous = true;
     itpp_detail_touch(h);
     if (cudaMemsetAsync(h->run_shared, 0, run_shared_head(), h->stream) != cudaSuccess ||
         launch_run<W>(a, ch, h->run_grid, false, h->stream) != cudaSuccess)
@@ -220,7 +218,6 @@ itpp_status launch_one_gate(itpp_ctx* h, int k) {
     const HostGate& g = h->gates[(size_t)k];
     cudaError_t e = cudaSuccess;
     if (h->p.merge_path == 0) {
-        h->contiguous = false;
         // a window's first gate (or any gate after the state changed
         // elsewhere) re-partitions; later gates of the window read the
         // partitions where the previous gate left them
@@ -264,6 +261,15 @@ itpp_status launch_one_gate(itpp_ctx* h, int k) {
         h->launches += cap_launches(h->s);
     }
     return e == cudaSuccess ? ITPP_OK : cuda_fail(h);
+}
+
+// Between calls a handle with run_ok has its state in one contiguous run: the
+// run kernel starts from one, and reads rely on it.  Gates launched one by one
+// (under profiling) leave it in partitions, so such a call ends here.
+itpp_status end_separate(itpp_ctx* h) {
+    if (!h->run_ok || use_run(h)) return ITPP_OK;
+    itpp_detail_touch(h);
+    return launch_materialize(h->s, h->stream) == cudaSuccess ? ITPP_OK : cuda_fail(h);
 }
 
 itpp_status ensure_obs(itpp_ctx* h, int m, int W) {
@@ -318,7 +324,6 @@ itpp_status check_obs_args(itpp_ctx* h, const uint64_t* ox, const uint64_t* oz, 
 }  // namespace
 
 itpp_status itpp_detail_sync_ctl(itpp_ctx* h) { return sync_ctl(h); }
-itpp_status itpp_detail_launch_gate(itpp_ctx* h, int k) { return launch_one_gate(h, k); }
 
 __global__ static void k_log_count(const DevCtl* ctl, unsigned long long* log) {
     if (threadIdx.x == 0) *log = ctl->status ? ~0ULL : ctl->count[ctl->cur];
@@ -332,14 +337,17 @@ itpp_status itpp_detail_layers(itpp_ctx* h, int n_layers, unsigned long long* lo
             if (st) return st;
             if (log) k_log_count<<<1, 32, 0, h->stream>>>(h->s.ctl, log++);
         }
-    return ITPP_OK;
+    return end_separate(h);
 }
 
-// The state as one contiguous run with no select pending.
+// The state as one contiguous run with no select pending.  Whether it is that
+// already the device knows alone: a captured layer changes it whenever it is
+// replayed, and a captured read may be replayed after any gate.  Only handles
+// whose state is never anything else between calls need no look: the other
+// merge paths, and bounds that the run kernel takes (end_separate).
 cudaError_t itpp_detail_materialize(itpp_ctx* h) {
     itpp_detail_touch(h);
-    if (h->contiguous) return cudaSuccess;
-    h->contiguous = true;
+    if (h->p.merge_path != 0 || h->run_ok) return cudaSuccess;
     return launch_materialize(h->s, h->stream);
 }
 
@@ -616,7 +624,8 @@ itpp_status itpp_apply_gate(itpp_handle h, int k) {
     if (!h) return ITPP_ERR_ARG;
     if (h->sticky) return h->sticky;
     if (k < 0 || k >= (int)h->gates.size()) return ITPP_ERR_ARG;
-    return launch_one_gate(h, k);
+    const itpp_status st = launch_one_gate(h, k);
+    return st ? st : end_separate(h);
 }
 
 itpp_status itpp_apply_trotter_layer(itpp_handle h, int n_layers) {
@@ -630,7 +639,6 @@ itpp_status itpp_reset(itpp_handle h) {
     if (h->sticky == ITPP_ERR_CUDA) return h->sticky;
     h->sticky = ITPP_OK;
     itpp_detail_touch(h);
-    h->contiguous = true;
     if (clear_cursors(h) != cudaSuccess) return cuda_fail(h);
     return launch_reset_identity(h->s, h->stream) == cudaSuccess ? ITPP_OK : cuda_fail(h);
 }
@@ -790,7 +798,6 @@ itpp_status itpp_set_terms(itpp_handle h, const uint64_t* x, const uint64_t* z, 
         cudaMemcpyAsync(dc, c, (size_t)count * 8, cudaMemcpyHostToDevice, h->stream) != cudaSuccess)
         return cuda_fail(h);
     itpp_detail_touch(h);
-    h->contiguous = true;
     if (clear_cursors(h) != cudaSuccess) return cuda_fail(h);
     if (launch_import(h->s, dx, dz, dc, count, h->stream) != cudaSuccess) return cuda_fail(h);
     h->sticky = ITPP_OK;

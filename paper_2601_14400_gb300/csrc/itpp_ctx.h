@@ -62,7 +62,6 @@ struct itpp_ctx {
     uint32_t run_part_max = 0;
     void* run_shared = nullptr;
     unsigned int* run_cnt = nullptr;
-    bool contiguous = true;   // the state is one run with no select pending
     // profiling
     bool prof = false;
     std::vector<EventPair> ev[kKinds];
@@ -74,7 +73,6 @@ struct itpp_ctx {
 
 // Helpers of the C ABI used by more than one translation unit.
 itpp_status itpp_detail_sync_ctl(itpp_ctx* h);
-itpp_status itpp_detail_launch_gate(itpp_ctx* h, int k);
 // n_layers whole layers; log (device, or null) receives the term count after
 // every gate.
 itpp_status itpp_detail_layers(itpp_ctx* h, int n_layers, unsigned long long* log);
