@@ -669,7 +669,6 @@ itpp_status adjoint_w(itpp_ctx* h, int L, int K, const uint64_t* obs_x, const ui
     // ---- forward from the identity, logging counts, snapshot per segment
     DevBuf log;
     if (!log.alloc((size_t)(S + 1) * 8)) return ITPP_ERR_ALLOC;
-    itpp_detail_touch(h);
     if (!chk(launch_reset_identity(s, st))) return ITPP_ERR_CUDA;
     std::vector<DevBuf> snap((size_t)n_seg);
     std::vector<uint64_t> snap_n((size_t)n_seg);

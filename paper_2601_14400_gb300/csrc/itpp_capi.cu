@@ -178,7 +178,6 @@ itpp_status run_launch(itpp_ctx* h, int k0, int n, int n_layers, unsigned long l
     a.min_part = kRunMinPart;
     a.cap_policy = s.cap_policy;
     a.maxw = h->p.max_weight ? h->p.max_weight : (1 << 30);
-    itpp_detail_touch(h);
     if (cudaMemsetAsync(h->run_shared, 0, run_shared_head(), h->stream) != cudaSuccess ||
         launch_run<W>(a, ch, h->run_grid, false, h->stream) != cudaSuccess)
         return cuda_fail(h);
@@ -218,16 +217,9 @@ itpp_status launch_one_gate(itpp_ctx* h, int k) {
     const HostGate& g = h->gates[(size_t)k];
     cudaError_t e = cudaSuccess;
     if (h->p.merge_path == 0) {
-        // a window's first gate (or any gate after the state changed
-        // elsewhere) re-partitions; later gates of the window read the
-        // partitions where the previous gate left them
-        const int force = g.win_start || h->part_epoch != h->state_epoch ||
-                          h->part_last != k - 1;
         EventPair* ev0 = prof_begin(h, 0);
-        e = launch_part_scatter(h->s, g, force, h->stream);
+        e = launch_part_scatter(h->s, g, h->stream);
         prof_end(h, ev0);
-        h->part_epoch = h->state_epoch;
-        h->part_last = k;
         if (e == cudaSuccess) {
             EventPair* ev1 = prof_begin(h, 1);
             e = launch_part_merge(h->s, g, h->stream);
@@ -268,7 +260,6 @@ itpp_status launch_one_gate(itpp_ctx* h, int k) {
 // (under profiling) leave it in partitions, so such a call ends here.
 itpp_status end_separate(itpp_ctx* h) {
     if (!h->run_ok || use_run(h)) return ITPP_OK;
-    itpp_detail_touch(h);
     return launch_materialize(h->s, h->stream) == cudaSuccess ? ITPP_OK : cuda_fail(h);
 }
 
@@ -346,7 +337,6 @@ itpp_status itpp_detail_layers(itpp_ctx* h, int n_layers, unsigned long long* lo
 // whose state is never anything else between calls need no look: the other
 // merge paths, and bounds that the run kernel takes (end_separate).
 cudaError_t itpp_detail_materialize(itpp_ctx* h) {
-    itpp_detail_touch(h);
     if (h->p.merge_path != 0 || h->run_ok) return cudaSuccess;
     return launch_materialize(h->s, h->stream);
 }
@@ -638,7 +628,6 @@ itpp_status itpp_reset(itpp_handle h) {
     if (!h) return ITPP_ERR_ARG;
     if (h->sticky == ITPP_ERR_CUDA) return h->sticky;
     h->sticky = ITPP_OK;
-    itpp_detail_touch(h);
     if (clear_cursors(h) != cudaSuccess) return cuda_fail(h);
     return launch_reset_identity(h->s, h->stream) == cudaSuccess ? ITPP_OK : cuda_fail(h);
 }
@@ -797,7 +786,6 @@ itpp_status itpp_set_terms(itpp_handle h, const uint64_t* x, const uint64_t* z, 
         cudaMemcpyAsync(dz, z, kb, cudaMemcpyHostToDevice, h->stream) != cudaSuccess ||
         cudaMemcpyAsync(dc, c, (size_t)count * 8, cudaMemcpyHostToDevice, h->stream) != cudaSuccess)
         return cuda_fail(h);
-    itpp_detail_touch(h);
     if (clear_cursors(h) != cudaSuccess) return cuda_fail(h);
     if (launch_import(h->s, dx, dz, dc, count, h->stream) != cudaSuccess) return cuda_fail(h);
     h->sticky = ITPP_OK;

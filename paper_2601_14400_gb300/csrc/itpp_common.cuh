@@ -129,6 +129,7 @@ struct DevCtl {
     // a contiguous run.  to_*: where this gate's scatter put the state.
     int home, ha, hb, hx, hc;
     unsigned int part_P;             // partitions of the current state
+    int part_win, to_win;            // ... and the window they were made for
     unsigned long long part_R;
     int scattered, to_b, to_x, to_c;
     unsigned int to_P;

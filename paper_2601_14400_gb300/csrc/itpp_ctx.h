@@ -50,11 +50,6 @@ struct itpp_ctx {
     void* sort_mem = nullptr;
     uint64_t sort_bytes = 0;
     uint64_t launches = 0;   // kernels launched by this handle
-    // partitioned merge: the state's partitions are valid for the window of
-    // gate part_last while part_epoch == state_epoch; anything else that
-    // changes the state bumps state_epoch
-    uint64_t state_epoch = 1, part_epoch = 0;
-    int part_last = -1;
     // gates run in one launch (itpp_run_impl.cuh): bounds up to kRunMax terms; the
     // team's shared block and the partition cursors
     bool run_ok = false;
@@ -77,5 +72,3 @@ itpp_status itpp_detail_sync_ctl(itpp_ctx* h);
 // every gate.
 itpp_status itpp_detail_layers(itpp_ctx* h, int n_layers, unsigned long long* log);
 cudaError_t itpp_detail_materialize(itpp_ctx* h);
-// The state changed outside a window's merges (partitions must be rebuilt).
-inline void itpp_detail_touch(itpp_ctx* h) { ++h->state_epoch; }

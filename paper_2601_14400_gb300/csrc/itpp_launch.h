@@ -64,6 +64,7 @@ struct HostGate {
     int pair_mode = 1;       // 1: the gate alone, partitioned by its pair key
     int win_sites = 0;       // sites of the window (mask mode)
     int win_start = 1;       // first gate of its window
+    int win = 0;             // ... and that gate's index: the window's number
 };
 
 // One elementary gate: merge-table build, branch-emit-merge-truncate, post.
@@ -73,11 +74,10 @@ cudaError_t launch_gate_post(const DeviceState& s, cudaStream_t st);
 cudaError_t launch_part_post(const DeviceState& s, cudaStream_t st);
 // Partitioned merge: scatter by the window's masked key (or the pair key),
 // then one shared-memory table per partition (the default merge of a single
-// propagation).  force = 1 re-partitions unconditionally (first gate of a
-// window, or the state changed outside the window); force = 0 only when the
-// previous gate's partitions held for that gate alone (pair-key mode).
-cudaError_t launch_part_scatter(const DeviceState& s, const HostGate& g, int force,
-                                cudaStream_t st);
+// propagation).  A window's first gate re-partitions; a later one where the
+// device finds no partitions of its window (the state changed elsewhere, a
+// replayed graph among it, or the last gate's held for that gate alone).
+cudaError_t launch_part_scatter(const DeviceState& s, const HostGate& g, cudaStream_t st);
 cudaError_t launch_part_merge(const DeviceState& s, const HostGate& g, cudaStream_t st);
 uint32_t partition_max(uint64_t cap_M, int target);
 int partition_target_default(int W);

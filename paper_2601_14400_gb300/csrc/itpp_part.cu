@@ -51,9 +51,9 @@ __device__ __forceinline__ bool last_cta(DevCtl* ctl) {
 }
 
 // Scatter the current state into the partitions of a window (force), or,
-// inside a window, only when the state has no partitions or they held for the
-// previous gate alone.  The state is a contiguous run, or the partitions of
-// a home; it goes to the other home.
+// inside a window, only when the state has no partitions, or those of another
+// window, or they held for the previous gate alone.  The state is a contiguous
+// run, or the partitions of a home; it goes to the other home.
 //
 // What bounds it: the random stores and cursor claims of 32 different
 // partitions a warp, each an access of its own (2.2 ms for 2^26 terms, 1.4 TB/s
@@ -63,7 +63,7 @@ __device__ __forceinline__ bool last_cta(DevCtl* ctl) {
 // where the state sits in L2.
 template <int W>
 __global__ void __launch_bounds__(256, 4)
-k_part_scatter(Bufs<W> B, Homes<W> H, DevCtl* ctl, GateArg<W> g, PartFn<W> f, int force,
+k_part_scatter(Bufs<W> B, Homes<W> H, DevCtl* ctl, GateArg<W> g, PartFn<W> f, int force, int win,
                int n_sites, int target, int redo) {
     if (ctl->status) return;
     // the second launch of a gate's scatter runs only when the first one
@@ -72,7 +72,7 @@ k_part_scatter(Bufs<W> B, Homes<W> H, DevCtl* ctl, GateArg<W> g, PartFn<W> f, in
     if (redo && !ctl->scatter_over) return;
     if (redo) f.pair = 1;
     const int cur = ctl->cur;
-    const bool run = force || redo || ctl->need_scatter || !ctl->home;
+    const bool run = force || redo || ctl->need_scatter || !ctl->home || ctl->part_win != win;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         // the next merge's counters
         ctl->count[cur ^ 1] = 0ULL;
@@ -108,6 +108,7 @@ k_part_scatter(Bufs<W> B, Homes<W> H, DevCtl* ctl, GateArg<W> g, PartFn<W> f, in
         ctl->to_c = to_c;
         ctl->to_P = pl.P;
         ctl->to_R = pl.R;
+        ctl->to_win = win;
         if (!home) ctl->ha = cur;
         ctl->stat_scatters += 1;
         ctl->part_over = f.pair;   // such partitions hold for this gate only
@@ -408,6 +409,7 @@ k_part_post(DevCtl* ctl, CandRegions cd, uint64_t cap_M, int cap_policy, uint64_
             ctl->hc = ctl->to_c;
             ctl->part_P = ctl->to_P;
             ctl->part_R = ctl->to_R;
+            ctl->part_win = ctl->to_win;
         }
         if (ctl->retry) {
             ctl->home = 0;
@@ -502,15 +504,15 @@ static Homes<W> homes_of(const DeviceState& s) {
 }
 
 template <int W>
-static cudaError_t scatter_w(const DeviceState& s, const HostGate& h, int force, cudaStream_t st) {
+static cudaError_t scatter_w(const DeviceState& s, const HostGate& h, cudaStream_t st) {
     uint64_t gs = (s.buf_cap + 255) / 256;
     const uint64_t lim = (uint64_t)s.num_sms * 8;
     if (gs > lim) gs = lim;
     if (gs < 1) gs = 1;
     for (int redo = 0; redo < 2; ++redo) {
         k_part_scatter<W><<<(int)gs, 256, 0, st>>>(pbufs_of<W>(s), homes_of<W>(s), s.ctl,
-                                                   gate_of<W>(h), part_fn_of<W>(h), force, s.n,
-                                                   s.part_target, redo);
+                                                   gate_of<W>(h), part_fn_of<W>(h), h.win_start,
+                                                   h.win, s.n, s.part_target, redo);
     }
     return cudaGetLastError();
 }
@@ -557,9 +559,8 @@ static cudaError_t merge_w(const DeviceState& s, const HostGate& h, cudaStream_t
     }
 }
 
-cudaError_t launch_part_scatter(const DeviceState& s, const HostGate& h, int force,
-                                cudaStream_t st) {
-    return s.W == 1 ? scatter_w<1>(s, h, force, st) : scatter_w<2>(s, h, force, st);
+cudaError_t launch_part_scatter(const DeviceState& s, const HostGate& h, cudaStream_t st) {
+    return s.W == 1 ? scatter_w<1>(s, h, st) : scatter_w<2>(s, h, st);
 }
 
 cudaError_t launch_part_post(const DeviceState& s, cudaStream_t st) {
@@ -586,6 +587,7 @@ void plan_windows(int W, std::vector<HostGate>& gates) {
             HostGate& h = gates[k];
             h.pair_mode = 1;
             h.win_start = 1;
+            h.win = (int)k;
             for (int w = 0; w < 2; ++w) { h.keep_x[w] = ~0ULL; h.keep_z[w] = ~0ULL; }
             ++k;
             continue;
@@ -604,6 +606,7 @@ void plan_windows(int W, std::vector<HostGate>& gates) {
             h.pair_mode = 0;
             h.win_sites = sites(S);
             h.win_start = j == k;
+            h.win = (int)k;
             for (int w = 0; w < 2; ++w) { h.keep_x[w] = ~S[w]; h.keep_z[w] = ~S[w]; }
         }
         k = e;

@@ -87,3 +87,30 @@ def test_read_captured_before_the_gates(block):
         torch.cuda.synchronize()
         assert rel_close(float(out[m]), o.expect(O)), (block, layer)
     assert_same_state(g.terms(), o.terms(), f"block {block}")
+
+
+# Gates one by one around a replayed layer: the replay leaves the partitions
+# of the layer's last window behind.
+@pytest.mark.parametrize("block", [0, 128])
+@pytest.mark.parametrize("first", [1, 2, 3])
+def test_gates_around_a_replay(block, first):
+    torch = pytest.importorskip("torch")
+    s = torch.cuda.Stream()
+    H, g = _handle(block, s)
+    _, h = _handle(0)
+    g.apply_trotter_layer(2)
+    h.apply_trotter_layer(2)
+    g.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=s):
+        g.apply_trotter_layer(1)
+    for k in range(first):
+        g.apply_gate(k)
+        h.apply_gate(k)
+    with torch.cuda.stream(s):
+        graph.replay()
+    h.apply_trotter_layer(1)
+    for k in range(first, first + 3):
+        g.apply_gate(k)
+        h.apply_gate(k)
+    assert_same_state(g.terms(), sort_terms(*h.terms()), f"block {block} first {first}")
