@@ -207,8 +207,8 @@ itpp_status run_batch(itpp_batch_ctx* h, int n_layers) {
     a.shared_stride = run_shared_bytes();
     a.buf_cap = s.buf_cap;
     a.home_cap = std::min(s.part_cap, s.buf_cap);
-    a.cand_cap = std::min<uint64_t>(a.scratch_stride / (12 + sizeof(PKey<W>)) - 64, a.home_cap);
-    a.tie_off = (a.cand_cap * 12 + 255) / 256 * 256;
+    a.cand_cap = run_list_cap<W>(a.scratch_stride, a.home_cap);
+    a.tie_off = run_tie_off(a.cand_cap);
     a.cap_M = s.cap_M;
     a.cand_hi = std::max<uint64_t>(1024, s.cap_M / 16);
     std::memcpy(&a.delta_bits, &s.delta, sizeof a.delta_bits);

@@ -159,10 +159,8 @@ itpp_status run_launch(itpp_ctx* h, int k0, int n, int n_layers, unsigned long l
     a.log = log;
     a.buf_cap = s.buf_cap;
     a.home_cap = s.part_cap < s.buf_cap ? s.part_cap : s.buf_cap;
-    const uint64_t bytes = s.table_slots * slot_bytes(W);
-    a.cand_cap = bytes / (12 + sizeof(PKey<W>)) - 64;
-    if (a.cand_cap > a.home_cap) a.cand_cap = a.home_cap;
-    a.tie_off = (a.cand_cap * 12 + 255) / 256 * 256;
+    a.cand_cap = run_list_cap<W>(s.table_slots * slot_bytes(W), a.home_cap);
+    a.tie_off = run_tie_off(a.cand_cap);
     a.cap_M = s.cap_M;
     a.cand_hi = std::max<uint64_t>(1024, s.cap_M / 16);
     std::memcpy(&a.delta_bits, &s.delta, sizeof a.delta_bits);

@@ -90,6 +90,19 @@ struct RunArgs {
     int target, min_part, cap_policy, maxw;
 };
 
+// Entries of the candidate list, and where the ties lie behind it, in `bytes` of
+// scratch (values, then indices; the ties on a 256-byte boundary).  A select
+// without a range lists every child of one digit of |c|, and a digit may hold
+// all of them: 2 cap_M.  The table's memory has room for that at every bound
+// (64 cap_M bytes at one mask word, 128 at two, 256 slots at least): it is not
+// to be cut further.
+template <int W>
+constexpr uint64_t run_list_cap(uint64_t bytes, uint64_t home_cap) {
+    const uint64_t n = (bytes - 255) / (12 + sizeof(PKey<W>));
+    return n < home_cap ? n : home_cap;
+}
+constexpr uint64_t run_tie_off(uint64_t cand_cap) { return (cand_cap * 12 + 255) / 256 * 256; }
+
 // Bytes of one team's shared block, and of its head that a launch clears.
 size_t run_shared_bytes();
 size_t run_shared_head();
