@@ -22,7 +22,7 @@ struct itpp_batch_ctx {
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     cudaGraphExec_t layer = nullptr;
-    std::vector<int> h_status;
+    std::vector<int> h_status;          // [B] of a probed shape
     itpp_status sticky = ITPP_OK;
     void* obs_mem = nullptr;
     size_t obs_bytes = 0;
@@ -283,8 +283,9 @@ itpp_status capture_layer(itpp_batch_ctx* h) {
     return e == cudaSuccess ? ITPP_OK : ITPP_ERR_CUDA;
 }
 
-// Time probe_layers layers from the identity with the current shape.
-itpp_status time_shape(itpp_batch_ctx* h, int probe_layers, double* ms) {
+// Time probe_layers layers from the identity with the current shape; *failed
+// counts the instances that ended with an error (and may have stopped early).
+itpp_status time_shape(itpp_batch_ctx* h, int probe_layers, double* ms, int* failed) {
     if (h->layer) {
         cudaGraphExecDestroy(h->layer);
         h->layer = nullptr;
@@ -297,16 +298,23 @@ itpp_status time_shape(itpp_batch_ctx* h, int probe_layers, double* ms) {
     if (cudaEventCreate(&a) != cudaSuccess) return ITPP_ERR_CUDA;
     if (cudaEventCreate(&b) != cudaSuccess) { cudaEventDestroy(a); return ITPP_ERR_CUDA; }
     cudaEventRecord(a, h->stream);
-    if (h->s.merge_path == 0) run_layers(h, probe_layers);
-    else for (int l = 0; l < probe_layers; ++l) cudaGraphLaunch(h->layer, h->stream);
+    bool ok = true;
+    if (h->s.merge_path == 0) ok = run_layers(h, probe_layers) == ITPP_OK;
+    else for (int l = 0; l < probe_layers && ok; ++l) ok = cudaGraphLaunch(h->layer, h->stream) == cudaSuccess;
     cudaEventRecord(b, h->stream);
     float f = 0.f;
-    const bool ok = cudaEventSynchronize(b) == cudaSuccess &&
-                    cudaEventElapsedTime(&f, a, b) == cudaSuccess;
+    ok = cudaEventSynchronize(b) == cudaSuccess && cudaEventElapsedTime(&f, a, b) == cudaSuccess && ok;
     cudaEventDestroy(a);
     cudaEventDestroy(b);
     if (!ok) return ITPP_ERR_CUDA;
     *ms = f;
+    if (cudaMemcpy2DAsync(h->h_status.data(), sizeof(int), &h->s.ctls->status, sizeof(DevCtl),
+                          sizeof(int), (size_t)h->s.B, cudaMemcpyDeviceToHost, h->stream) !=
+            cudaSuccess ||
+        cudaStreamSynchronize(h->stream) != cudaSuccess)
+        return ITPP_ERR_CUDA;
+    *failed = 0;
+    for (int v : h->h_status) *failed += v != 0;
     return ITPP_OK;
 }
 
@@ -485,6 +493,7 @@ itpp_status itpp_batch_create(int B, const int* n, const int* n_gates, const uin
         return ITPP_ERR_CUDA;
     }
     h->h_ctl.resize(sizeof(DevCtl));
+    h->h_status.resize((size_t)B);
     *out = h;
     return ITPP_OK;
 }
@@ -523,35 +532,42 @@ itpp_status itpp_batch_autotune(itpp_batch_handle h, int probe_layers, itpp_tune
     // smallest mean partition in units of 16 terms, table load (global table)
     // or mean partition size (partitioned)
     struct Shape { int mb, mg, ig, load, target; };
-    auto install = [&](const Shape& c) {
+    auto install = [&](const Shape& c) -> itpp_status {
         s.main_block = c.mb;
         if (part) {
             s.team_ctas = c.mg;
             s.min_part = 16 * c.ig;
             s.part_target = c.target;
-            plan_teams(h);
-        } else {
-            s.main_grid = c.mg;
-            s.insert_grid = c.ig;
-            s.load_pct = c.load;
+            return plan_teams(h);
         }
+        s.main_grid = c.mg;
+        s.insert_grid = c.ig;
+        s.load_pct = c.load;
+        return ITPP_OK;
     };
     Shape best = part ? Shape{256, 0, 8, 0, s.part_target}
                       : Shape{256, 4, 8, 50 < h->load_floor ? h->load_floor : 50, 0};
-    install(best);
     double best_ms = 0, default_ms = 0;
-    int tried = 0;
-    itpp_status st = time_shape(h, probe_layers, &best_ms);
+    int tried = 0, best_failed = 0;
+    itpp_status st = install(best);
+    if (!st) st = time_shape(h, probe_layers, &best_ms, &best_failed);
     if (st) return h->sticky = st;
     default_ms = best_ms;
     ++tried;
+    // an instance that stops on an error is fast: a shape with more of them than
+    // the best one so far is not better, whatever its time
     auto try_shape = [&](Shape c) -> itpp_status {
-        install(c);
         double ms = 0;
-        itpp_status e = time_shape(h, probe_layers, &ms);
+        int failed = 0;
+        itpp_status e = install(c);
+        if (!e) e = time_shape(h, probe_layers, &ms, &failed);
         if (e) return e;
         ++tried;
-        if (ms < best_ms) { best_ms = ms; best = c; }
+        if (failed < best_failed || (failed == best_failed && ms < best_ms)) {
+            best_ms = ms;
+            best_failed = failed;
+            best = c;
+        }
         return ITPP_OK;
     };
     // one parameter at a time, each from the best shape so far
@@ -576,7 +592,7 @@ itpp_status itpp_batch_autotune(itpp_batch_handle h, int probe_layers, itpp_tune
         for (int v : loads)
             if (v != best.load && v >= h->load_floor) { Shape c = best; c.load = v; if ((st = try_shape(c))) return h->sticky = st; }
     }
-    install(best);
+    if ((st = install(best))) return h->sticky = st;
     if (h->layer) {
         cudaGraphExecDestroy(h->layer);
         h->layer = nullptr;

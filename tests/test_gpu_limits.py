@@ -11,6 +11,41 @@ pytestmark = pytest.mark.gpu
 itpp = pytest.importorskip("paper_2601_14400_gb300")
 
 
+def key_hash(x, z):
+    """The partition hash of one-word keys (MurmurHash3 of their 32-bit halves)."""
+    m = np.uint64(0xffffffff)
+
+    def rotl(v, r):
+        return ((v << np.uint64(r)) | (v >> np.uint64(32 - r))) & m
+
+    h = np.full(x.shape, 0x9747b28c, dtype=np.uint64)
+    for word in (x & m, x >> np.uint64(32), z & m, z >> np.uint64(32)):
+        k = rotl(word * np.uint64(0xcc9e2d51) & m, 15) * np.uint64(0x1b873593) & m
+        h = (rotl(h ^ k, 13) * np.uint64(5) + np.uint64(0xe6546b64)) & m
+    h ^= np.uint64(16)
+    h = (h ^ (h >> np.uint64(16))) * np.uint64(0x85ebca6b) & m
+    h = (h ^ (h >> np.uint64(13))) * np.uint64(0xc2b2ae35) & m
+    return h ^ (h >> np.uint64(16))
+
+
+def piled_hamiltonian(m, n=40):
+    """m wide strings whose hashes lie in the lowest sixteenth, then a wide gate
+    whose pivot none of them has: at that gate the strings themselves, which the
+    threshold keeps while it drops their products, all fall into the first
+    partition."""
+    rng = np.random.default_rng(m)
+    x = rng.integers(0, 1 << (n - 1), 64 * m, dtype=np.uint64)
+    z = rng.integers(0, 1 << n, 64 * m, dtype=np.uint64)
+    ok = key_hash(x, z) < np.uint64(1 << 28)
+    gx = np.append(x[ok][:m], np.uint64(1 << (n - 1)))[:, None]
+    gz = np.append(z[ok][:m], np.uint64((1 << (n - 1)) - 1))[:, None]
+    assert gx.shape[0] == m + 1
+    return wl.Hamiltonian(n, gx, gz, np.full(m + 1, 1.0))
+
+
+PILE_DTAU, PILE_DELTA = 0.01, 1e-3
+
+
 # Few strings and one class of magnitudes: a gate doubles the state, and the
 # select of a first gate lists every child there is.
 @pytest.mark.parametrize("M", [114, 115, 120, 127, 128, 129])
@@ -33,3 +68,18 @@ def test_list_holds_every_child(M, batch):
         p.apply_trotter_layer(2)
         got = p.terms()
     assert_same_state(got, o.terms(), f"M {M}")
+
+
+# The autotuner tries partitions of 64 strings, which the piled state overflows
+# where the default size holds it: whatever it picks runs.
+def test_autotune_picks_a_shape_that_runs():
+    cap = 192
+    H = piled_hamiltonian(cap - 4)
+    bp = itpp.BatchPropagator([H, H], PILE_DTAU, PILE_DELTA, cap, 1)
+    bp.autotune(probe_layers=2)
+    bp.apply_trotter_layer(2)
+    counts, status = bp.counts()
+    assert not status.any()
+    o = oracle.Oracle(H.n, H.gate_x, H.gate_z, H.alpha, PILE_DTAU, PILE_DELTA, cap, 1)
+    o.apply_layers(2)
+    assert_same_state(bp.terms(1), o.terms(), "after the autotuner")
