@@ -124,7 +124,7 @@ k_part_scatter(Bufs<W> B, Homes<W> H, DevCtl* ctl, GateArg<W> g, PartFn<W> f, in
         const uint64_t stride = r.cnt ? (uint64_t)blockDim.x : (uint64_t)gridDim.x * blockDim.x;
         scatter_run(r.keys + off, r.coef + off, cnt, first, stride, pd, ctl,
                     H.keys(B, a, to_b), H.coef(B, a, to_x), H.cursors(to_c), pl, g, f,
-                    &ctl->scatter_over);
+                    &ctl->scatter_over, f.pair ? 0 : 1);   // (again by the pair key)
     }
     if (redo) return;
     // when a stride was too small, the last CTA clears the cursors for the

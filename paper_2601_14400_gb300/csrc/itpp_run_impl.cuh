@@ -397,8 +397,11 @@ __device__ bool run_instance(const RunArgs<W>& a, const RunGate<W>* gates, int n
             if (want < 1) want = 1;
             if (want > most && want > wide) want = most > wide ? most : wide;
             if (want > a.part_max) want = a.part_max;
-            const int lv0 = window_level<W>(gates[k], sites, n_in, want);
-            for (int lv = lv0;; lv = -1) {
+            // a try marks that a stride ran out with its number: by the window,
+            // then by the pair key, then into half as many partitions (of twice
+            // the stride), at last into one, which holds any state
+            int lv = window_level<W>(gates[k], sites, n_in, want);
+            for (int nth = 1;; ++nth) {
                 if (threadIdx.x == 0) s_f = part_fn_of<W>(gates[k], lv);
                 __syncthreads();
                 PartFn<W> f = s_f;
@@ -420,21 +423,23 @@ __device__ bool run_instance(const RunArgs<W>& a, const RunGate<W>* gates, int n
                 const int dh = layout == 0 ? 0 : hb ^ 1, dx = layout == 0 ? 0 : cx ^ 1;
                 const int dc = next3(ci);
                 int* over = reinterpret_cast<int*>(&acc->scatter_over);
+                const int mark = plan.P > 1u ? nth : 0;
                 if (layout == 0) {
                     scatter_run<W>(arr.run_keys(run_buf), arr.run_coef(run_buf), run_n,
                                    (uint64_t)team.rank * kBlock, (uint64_t)team.size * kBlock, pd,
-                                   ctl, arr.home(dh), arr.coef(dx), arr.cnt(dc), plan, g, f, over, kPad);
+                                   ctl, arr.home(dh), arr.coef(dx), arr.cnt(dc), plan, g, f, over,
+                                   mark, kPad);
                 } else {
                     for (uint32_t p = team.rank; p < oldP; p += team.size) {
                         const uint64_t c = __ldcg(arr.cnt(ci) + (uint64_t)p * kPad);
                         scatter_run<W>(arr.home(hb) + p * oldR, arr.coef(cx) + p * oldR, c, 0,
                                        kBlock, pd, ctl, arr.home(dh), arr.coef(dx), arr.cnt(dc),
-                                       plan, g, f, over, kPad);
+                                       plan, g, f, over, mark, kPad);
                     }
                 }
                 if (!team_barrier(team, ctl)) return false;
                 if (leader && threadIdx.x == 0) s_stat[4] += 1;
-                if (lv < 0 || !__ldcg(&acc->scatter_over)) {
+                if (__ldcg(&acc->scatter_over) != (unsigned int)nth) {
                     hb = dh;
                     cx = dx;
                     ci = dc;
@@ -445,7 +450,8 @@ __device__ bool run_instance(const RunArgs<W>& a, const RunGate<W>* gates, int n
                     win_end = gi + (lv < 0 ? 1 : (lv ? gates[k].len[1] : gates[k].len[0]));
                     break;
                 }
-                // a window group passed a stride: again, by the pair key
+                if (lv < 0) want = plan.P / 2u;
+                lv = -1;
                 for (uint32_t i = team.rank * kBlock + threadIdx.x; i < a.part_max;
                      i += team.size * kBlock)
                     arr.cnt(dc)[(uint64_t)i * kPad] = 0u;

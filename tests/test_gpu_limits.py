@@ -70,6 +70,18 @@ def test_list_holds_every_child(M, batch):
     assert_same_state(got, o.terms(), f"M {M}")
 
 
+# Every string in one partition: the scatter by pair key finds no room at first.
+@pytest.mark.parametrize("B,cap", [(1, 300), (2, 300), (3, 900)])
+def test_scatter_of_a_piled_state(B, cap):
+    H = piled_hamiltonian(cap - 2)
+    bp = itpp.BatchPropagator([H] * B, PILE_DTAU, PILE_DELTA, cap, 1)
+    bp.apply_trotter_layer(2)
+    o = oracle.Oracle(H.n, H.gate_x, H.gate_z, H.alpha, PILE_DTAU, PILE_DELTA, cap, 1)
+    o.apply_layers(2)
+    for b in range(B):
+        assert_same_state(bp.terms(b), o.terms(), f"instance {b} of {B}")
+
+
 # The autotuner tries partitions of 64 strings, which the piled state overflows
 # where the default size holds it: whatever it picks runs.
 def test_autotune_picks_a_shape_that_runs():
