@@ -185,9 +185,10 @@ k_psd_pairs(Bufs<W> B, DevCtl* ctl, const Slot<W>* table, uint64_t slots, int lo
                 double cr;
                 if (table_find(table, mask, gen, key_xor(P, o), &cr, probe_limit, ctl, &probes)) {
                     const double cp = normalised(B.coef(cur)[i], rnorm, key_is_zero(P));
-                    // (doubling is exact; the identity is its own partner)
-                    const double w = __ldg(ow + j);
-                    const double v = __dmul_rn(obs_is_identity(o) ? w : w + w, __dmul_rn(cp, cr));
+                    // twice the product, not twice the weight, which may have no
+                    // double (the identity is its own partner)
+                    const double w = __dmul_rn(__ldg(ow + j), __dmul_rn(cp, cr));
+                    const double v = obs_is_identity(o) ? w : w + w;
                     kahan_add(num, cn, product_negative(P, o) ? -v : v);
                 }
             }

@@ -95,3 +95,18 @@ def test_autotune_picks_a_shape_that_runs():
     o = oracle.Oracle(H.n, H.gate_x, H.gate_z, H.alpha, PILE_DTAU, PILE_DELTA, cap, 1)
     o.apply_layers(2)
     assert_same_state(bp.terms(1), o.terms(), "after the autotuner")
+
+
+# Weights whose double is not a number of the type.
+def test_squared_state_large_weights():
+    n = 4
+    g = itpp.Propagator(n, np.zeros((0, 1), np.uint64), np.zeros((0, 1), np.uint64),
+                        np.zeros(0), 0.1, 0.0, 16, 0)
+    x = np.zeros((2, 1), dtype=np.uint64)
+    z = np.array([[0], [1]], dtype=np.uint64)
+    g.set_terms(x, z, np.array([1.0, 0.125]))
+    O = wl.Observable(n, x[1:], z[1:], np.array([1.2e308]))
+    v, num, pur = g.expect_psd(O)
+    assert pur == 1.0 + 0.125 ** 2
+    assert num == 2.0 * (1.2e308 * 0.125)             # each member of the pair once
+    assert v == num / pur
