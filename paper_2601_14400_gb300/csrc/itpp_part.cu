@@ -448,6 +448,10 @@ k_part_post(DevCtl* ctl, CandRegions cd, uint64_t cap_M, int cap_policy, uint64_
             } else {
                 ctl->stat_sel_full += 1;
             }
+        } else if (ctl->retry) {
+            // the state has fallen below its bound: with the old limit every
+            // gate from here on would be merged twice
+            ctl->sp_thr = ctl->sp_lo = ctl->sp_hi = ctl->sp_tprev = 0ULL;
         }
     }
 }

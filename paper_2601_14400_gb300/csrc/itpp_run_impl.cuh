@@ -595,6 +595,13 @@ __device__ bool run_instance(const RunArgs<W>& a, const RunGate<W>* gates, int n
                 p.lo = lo;
                 p.hi = hi;
                 p.thr = s_pub.thr;
+                if (redone && !active) {
+                    // the state has fallen below its bound: with the old limit
+                    // every gate from here on would be merged twice
+                    p.lo = p.hi = 0ULL;
+                    p.thr = a.delta_bits;
+                    s_pred.tprev = 0ULL;
+                }
                 // a state that doubled since its scatter: more partitions, before
                 // they outgrow the staging
                 p.rescatter = !redone && p.n > 2ULL * n_scat && p.n > (C / 2) * (uint64_t)P;

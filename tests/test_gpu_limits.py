@@ -4,7 +4,7 @@ import pytest
 
 import oracle
 import workloads as wl
-from tests._compare import assert_same_state
+from tests._compare import assert_same_state, sort_terms
 
 pytestmark = pytest.mark.gpu
 
@@ -110,3 +110,31 @@ def test_squared_state_large_weights():
     assert pur == 1.0 + 0.125 ** 2
     assert num == 2.0 * (1.2e308 * 0.125)             # each member of the pair once
     assert v == num / pur
+
+
+# A state that falls below its bound: the limit predicted for the select no
+# longer applies, and gates are not merged twice for it.
+@pytest.mark.parametrize("separate", [False, True])
+def test_below_the_bound(separate):
+    H = wl.tfim_1d(24, 1.0, 1.1, periodic=True)
+    g = itpp.Propagator(H.n, H.gate_x, H.gate_z, H.alpha, 0.05, 1e-9, 3000, 1)
+    if separate:
+        g.profile_enable(True)
+    g.apply_trotter_layer(3)
+    assert g.count() == 3000
+    c = np.abs(g.terms()[2])
+    g.truncate(float(np.median(c)))
+    g.set_alpha(np.zeros(H.n_gates))                  # nothing grows
+    before = g.stats()["merge_retries"]
+    want = sort_terms(*g.terms())
+    g.apply_trotter_layer(3)
+    assert_same_state(g.terms(), want, "gates of angle zero")
+    assert g.stats()["merge_retries"] - before <= 1
+    # and back at the bound, as a handle that starts from this state
+    h = itpp.Propagator(H.n, H.gate_x, H.gate_z, H.alpha, 0.05, 1e-9, 3000, 1)
+    h.set_terms(*want)
+    for p in (g, h):
+        p.set_alpha(H.alpha)
+        p.apply_trotter_layer(2)
+    assert g.count() == 3000
+    assert_same_state(g.terms(), sort_terms(*h.terms()), "back at the bound")
