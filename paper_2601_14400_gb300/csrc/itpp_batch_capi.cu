@@ -384,7 +384,7 @@ itpp_status itpp_batch_create(int B, const int* n, const int* n_gates, const uin
         // autotuner tries
         h->target_fixed = p->partition_target != 0;
         s.part_target = p->partition_target ? p->partition_target : partition_target_default(W);
-        s.min_part = kRunMinPart;
+        s.min_part = run_min_part(s.part_target);
         s.part_cap = 2 * p->cap_M + p->cap_M / 2 + 4096;
         s.part_cap += s.part_cap & 1ULL;
         const int t_min = std::min(h->target_fixed ? s.part_target : kTargetMin, s.part_target);
@@ -536,7 +536,7 @@ itpp_status itpp_batch_autotune(itpp_batch_handle h, int probe_layers, itpp_tune
         s.main_block = c.mb;
         if (part) {
             s.team_ctas = c.mg;
-            s.min_part = 16 * c.ig;
+            s.min_part = h->target_fixed ? std::min(16 * c.ig, c.target) : 16 * c.ig;
             s.part_target = c.target;
             return plan_teams(h);
         }

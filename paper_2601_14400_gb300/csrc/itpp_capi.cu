@@ -173,7 +173,7 @@ itpp_status run_launch(itpp_ctx* h, int k0, int n, int n_layers, unsigned long l
     a.gate0 = k0;
     a.n_layers = n_layers;
     a.target = s.part_target;
-    a.min_part = kRunMinPart;
+    a.min_part = run_min_part(s.part_target);
     a.cap_policy = s.cap_policy;
     a.maxw = h->p.max_weight ? h->p.max_weight : (1 << 30);
     if (cudaMemsetAsync(h->run_shared, 0, run_shared_head(), h->stream) != cudaSuccess ||
@@ -566,7 +566,7 @@ itpp_status itpp_create(int n, const uint64_t* gate_x, const uint64_t* gate_z,
         // whole layers in one launch, for the default launch shape: as many
         // CTAs as there can be partitions, at most what fits
         if (p->cap_M <= kRunMax && (p->block_threads == 0 || p->block_threads == 256)) {
-            const uint64_t parts = p->cap_M / kRunMinPart + 1;
+            const uint64_t parts = p->cap_M / run_min_part(s.part_target) + 1;
             h->run_grid = (int)std::min<uint64_t>((uint64_t)sms * run_fit(W, false), parts);
             h->run_part_max = (uint32_t)(p->cap_M / s.part_target + 2 + (uint64_t)h->run_grid);
             ok &= ok && cudaMalloc(&h->run_shared, run_shared_bytes()) == cudaSuccess;

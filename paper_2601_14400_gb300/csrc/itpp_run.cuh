@@ -55,8 +55,10 @@ void plan_run_windows(RunGate<W>* g, int n) {
 // The gates of a launch as a kernel argument: the host keeps no device copy
 // of them that a change of the coefficients or a captured launch could race.
 constexpr int kRunChunk = 256;
-// Smallest mean partition a scatter aims for to give every CTA one.
+// Smallest mean partition a scatter aims for to give every CTA one, unless the
+// caller asks for smaller ones.
 constexpr int kRunMinPart = 128;
+constexpr int run_min_part(int target) { return target < kRunMinPart ? target : kRunMinPart; }
 // Distance of two partition cursors (words).
 constexpr int kRunPad = 32;
 template <int W>

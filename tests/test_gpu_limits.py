@@ -82,6 +82,22 @@ def test_scatter_of_a_piled_state(B, cap):
         assert_same_state(bp.terms(b), o.terms(), f"instance {b} of {B}")
 
 
+# The smallest partitions a caller can ask for: more of them than by default, so
+# that the piled state finds no room where it does by default.
+def test_smallest_partition_target():
+    cap = 192
+    H = piled_hamiltonian(cap - 4)
+    scatters = []
+    for target in (0, 64):
+        bp = itpp.BatchPropagator([H], PILE_DTAU, PILE_DELTA, cap, 1, partition_target=target)
+        bp.apply_trotter_layer(1)
+        scatters.append(bp.stats(0)["repartitions"])
+        o = oracle.Oracle(H.n, H.gate_x, H.gate_z, H.alpha, PILE_DTAU, PILE_DELTA, cap, 1)
+        o.apply_layers(1)
+        assert_same_state(bp.terms(0), o.terms(), f"target {target}")
+    assert scatters[0] == H.n_gates < scatters[1]
+
+
 # The autotuner tries partitions of 64 strings, which the piled state overflows
 # where the default size holds it: whatever it picks runs.
 def test_autotune_picks_a_shape_that_runs():
