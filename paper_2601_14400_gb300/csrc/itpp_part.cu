@@ -124,7 +124,10 @@ k_part_scatter(Bufs<W> B, Homes<W> H, DevCtl* ctl, GateArg<W> g, PartFn<W> f, in
         const uint64_t stride = r.cnt ? (uint64_t)blockDim.x : (uint64_t)gridDim.x * blockDim.x;
         scatter_run(r.keys + off, r.coef + off, cnt, first, stride, pd, ctl,
                     H.keys(B, a, to_b), H.coef(B, a, to_x), H.cursors(to_c), pl, g, f,
-                    &ctl->scatter_over, f.pair ? 0 : 1);   // (again by the pair key)
+                    [&] {
+                        if (!f.pair) ctl->scatter_over = 1;   // again by the pair key
+                        else set_status(ctl, ST_CAPACITY, 40);
+                    });
     }
     if (redo) return;
     // when a stride was too small, the last CTA clears the cursors for the

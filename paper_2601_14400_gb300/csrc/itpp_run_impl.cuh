@@ -286,7 +286,7 @@ __device__ bool run_instance(const RunArgs<W>& a, const RunGate<W>* gates, int n
     __shared__ PartFn<W> s_f;
     __shared__ unsigned long long s_cv[kPushBuf];
     __shared__ uint32_t s_ci[kPushBuf];
-    __shared__ uint32_t s_cn, s_cs, s_app, s_rare, s_n;
+    __shared__ uint32_t s_cn, s_cs, s_app, s_rare, s_n, s_try;
     __shared__ int s_over;
     __shared__ unsigned long long s_at;
     __shared__ uint32_t s_red[kBlock / 32], s_kept[kBlock / 32], s_w[kBlock / 32];
@@ -371,7 +371,7 @@ __device__ bool run_instance(const RunArgs<W>& a, const RunGate<W>* gates, int n
         if (s_pub.stop) break;          // uniform over the team
         if (threadIdx.x == 0) {
             s_g = gate_arg_of<W>(gates[k], a.maxw);
-            s_cn = s_cs = s_app = s_rare = 0u;
+            s_cn = s_cs = s_app = s_rare = s_try = 0u;
             s_over = 0;
         }
         const GateArg<W>& g = s_g;
@@ -397,12 +397,14 @@ __device__ bool run_instance(const RunArgs<W>& a, const RunGate<W>* gates, int n
             if (want < 1) want = 1;
             if (want > most && want > wide) want = most > wide ? most : wide;
             if (want > a.part_max) want = a.part_max;
-            // a try marks that a stride ran out with its number: by the window,
-            // then by the pair key, then into half as many partitions (of twice
-            // the stride), at last into one, which holds any state
-            int lv = window_level<W>(gates[k], sites, n_in, want);
-            for (int nth = 1;; ++nth) {
-                if (threadIdx.x == 0) s_f = part_fn_of<W>(gates[k], lv);
+            // by the window, then by the pair key, then into half as many
+            // partitions (of twice the stride), at last into one, which holds any
+            // state; a try whose stride ran out leaves its number behind
+            for (int lv = window_level<W>(gates[k], sites, n_in, want);; lv = -1) {
+                if (threadIdx.x == 0) {
+                    s_f = part_fn_of<W>(gates[k], lv);
+                    s_try += 1u;
+                }
                 __syncthreads();
                 PartFn<W> f = s_f;
                 uint64_t np = want;
@@ -422,24 +424,24 @@ __device__ bool run_instance(const RunArgs<W>& a, const RunGate<W>* gates, int n
                 pd.tk = tk;
                 const int dh = layout == 0 ? 0 : hb ^ 1, dx = layout == 0 ? 0 : cx ^ 1;
                 const int dc = next3(ci);
-                int* over = reinterpret_cast<int*>(&acc->scatter_over);
-                const int mark = plan.P > 1u ? nth : 0;
+                auto over = [&] { *(volatile unsigned int*)&acc->scatter_over = s_try; };
                 if (layout == 0) {
                     scatter_run<W>(arr.run_keys(run_buf), arr.run_coef(run_buf), run_n,
                                    (uint64_t)team.rank * kBlock, (uint64_t)team.size * kBlock, pd,
-                                   ctl, arr.home(dh), arr.coef(dx), arr.cnt(dc), plan, g, f, over,
-                                   mark, kPad);
+                                   ctl, arr.home(dh), arr.coef(dx), arr.cnt(dc), plan, g, f, over, kPad);
                 } else {
                     for (uint32_t p = team.rank; p < oldP; p += team.size) {
                         const uint64_t c = __ldcg(arr.cnt(ci) + (uint64_t)p * kPad);
                         scatter_run<W>(arr.home(hb) + p * oldR, arr.coef(cx) + p * oldR, c, 0,
                                        kBlock, pd, ctl, arr.home(dh), arr.coef(dx), arr.cnt(dc),
-                                       plan, g, f, over, mark, kPad);
+                                       plan, g, f, over, kPad);
                     }
                 }
                 if (!team_barrier(team, ctl)) return false;
                 if (leader && threadIdx.x == 0) s_stat[4] += 1;
-                if (__ldcg(&acc->scatter_over) != (unsigned int)nth) {
+                const bool full = __ldcg(&acc->scatter_over) == s_try;
+                if (full && plan.P == 1u && threadIdx.x == 0) set_status(ctl, ST_CAPACITY, 40);
+                if (!full || plan.P == 1u) {
                     hb = dh;
                     cx = dx;
                     ci = dc;
@@ -451,7 +453,6 @@ __device__ bool run_instance(const RunArgs<W>& a, const RunGate<W>* gates, int n
                     break;
                 }
                 if (lv < 0) want = plan.P / 2u;
-                lv = -1;
                 for (uint32_t i = team.rank * kBlock + threadIdx.x; i < a.part_max;
                      i += team.size * kBlock)
                     arr.cnt(dc)[(uint64_t)i * kPad] = 0u;

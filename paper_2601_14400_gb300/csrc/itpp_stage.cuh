@@ -113,16 +113,16 @@ __device__ __forceinline__ Pending<W> pending_of(const DevCtl* ctl) {
 
 // Scatter terms [0, n) of a run (this CTA's part of it: from `first` on, every
 // `stride`) into the partitions of a plan: the kept set of a pending select,
-// one cursor claim per distinct partition of a warp.  A stride that runs out sets
-// *over to mark, and the caller scatters again; without a mark it is an error.
-template <int W>
+// one cursor claim per distinct partition of a warp.  over() is called where a
+// stride has run out.
+template <int W, class Over>
 __device__ __forceinline__ void scatter_run(const PKey<W>* __restrict__ kin,
                                             const double* __restrict__ cin, uint64_t n,
                                             uint64_t first, uint64_t stride, const Pending<W>& pd,
                                             DevCtl* ctl, PKey<W>* pk, double* pc,
                                             unsigned int* cursor, const PartPlan& pl,
                                             const GateArg<W>& g, const PartFn<W>& f,
-                                            int* over, int mark, uint32_t pad = 1u) {
+                                            Over&& over, uint32_t pad = 1u) {
     // whole warps iterate together (the cursor claim below is warp-wide);
     // U items per thread per round, their loads issued before any claim
     constexpr int U = 4;
@@ -173,10 +173,8 @@ __device__ __forceinline__ void scatter_run(const PKey<W>* __restrict__ kin,
                 const uint64_t d = (uint64_t)part[u] * pl.R + pos;
                 store_key(pk + d, K[u]);
                 pc[d] = c[u];
-            } else if (mark) {
-                *over = mark;
             } else {
-                set_status(ctl, ST_CAPACITY, 40);
+                over();
             }
         }
     }
