@@ -524,6 +524,11 @@ __device__ __forceinline__ uint32_t stage_pass(uint32_t n, const GateArg<W>& g,
     double* vals = A::vals();
     const uint32_t lane = threadIdx.x & 31u, par = pass & 1u;
     const unsigned int lt = (1u << lane) - 1u;
+    // the identity as the gate: every string is its own partner
+    uint64_t qbits = 0;
+#pragma unroll
+    for (int w = 0; w < W; ++w) qbits |= g.qx[w] | g.qz[w];
+    const bool self = qbits == 0;
     for (uint32_t i0 = threadIdx.x & ~31u; i0 < n; i0 += BLOCK) {   // whole warps
         const uint32_t i = i0 + lane;
         uint32_t slot = 0;
@@ -540,9 +545,13 @@ __device__ __forceinline__ uint32_t stage_pass(uint32_t n, const GateArg<W>& g,
                 c = 1.0;   // the identity's normalised value is exactly 1
                 if (!live) set_status(ctl, ST_TRACE_ZERO, 43);
             }
-            vals[i] = c;
             bool neg;
-            const bool comm = commute_sign(K, g, &neg);
+            bool comm = commute_sign(K, g, &neg);
+            if (self) {
+                c = __dadd_rn(__dmul_rn(c, g.ch), __dmul_rn(c, g.msh));
+                comm = false;   // done: the rest is that of a string that passes through
+            }
+            vals[i] = c;
             through = live && !comm;
             if (live && comm) owner = pair_enter(K, g, i, neg, A::keys(), A::tab(), ctl, &slot);
         }

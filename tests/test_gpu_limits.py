@@ -154,3 +154,21 @@ def test_below_the_bound(separate):
         p.apply_trotter_layer(2)
     assert g.count() == 3000
     assert_same_state(g.terms(), sort_terms(*h.terms()), "back at the bound")
+
+
+# The identity among the gates where gates are merged in full: every string is
+# its own partner.
+@pytest.mark.parametrize("separate", [False, True])
+@pytest.mark.parametrize("n,cap", [(1, 1), (9, 300), (40, 129), (40, 3000), (80, 300)])
+def test_identity_gates_merged_in_full(n, cap, separate):
+    H = wl.random_pauli_hamiltonian(n, 24, 5, max_weight=min(n, 3))
+    H.gate_x[::3] = 0
+    H.gate_z[::3] = 0
+    g = itpp.Propagator(H.n, H.gate_x, H.gate_z, H.alpha, 0.3, 1e-9, cap, 1)
+    if separate:
+        g.profile_enable(True)
+    o = oracle.Oracle(H.n, H.gate_x, H.gate_z, H.alpha, 0.3, 1e-9, cap, 1)
+    for layer in range(4):
+        g.apply_trotter_layer(1)
+        o.apply_layers(1)
+        assert_same_state(g.terms(), o.terms(), f"n {n} layer {layer}")
