@@ -14,8 +14,8 @@
 // strings are appended to the partition's stride, so keys are written only
 // where they are new and no scatter runs between the gates of a window.  A
 // group holds at most 4^|S| terms; a partition above a pass's capacity is
-// merged in sub-passes, each taking the pairs of one hash class of the key with
-// the gate's sites cleared, so no partition size forces a re-partition.  A gate
+// merged in sub-passes, each taking the pairs of one hash class of the pair
+// key, so no partition size forces a re-partition.  A gate
 // acting on more sites than a window allows is a window of its own,
 // partitioned by its pair key (the member of {K, QK} with the gate's lowest bit
 // clear).

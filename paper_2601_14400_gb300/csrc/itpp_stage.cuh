@@ -196,19 +196,27 @@ __device__ __forceinline__ uint32_t smem_addr(const void* p) {
     return (uint32_t)__cvta_generic_to_shared(p);
 }
 
-// Sub-pass of a long partition's commuting string: a hash of the key with
-// the gate's sites cleared, which K and Q.K share (they differ exactly on
-// Q's bits), so a string and its partner always fall into the same one.  The
-// hash is seeded apart from the partition hash: for a string with both of
-// the gate's bits clear the masked key is the pair key the partition was
-// chosen by, and the same hash would put all such strings of a partition in
-// one class.
+// Sub-pass of a long partition's commuting string: a hash of its pair key (the
+// member of {K, Q.K} without the gate's lowest bit), so a string and its partner
+// always fall into the same one.  (With the gate's sites cleared instead, a gate
+// on every site of a small system leaves a few keys for all strings, and one
+// sub-pass gets more than it holds.)  The hash is seeded apart from the
+// partition hash, which would put all strings of a partition in one class.
 template <int W>
 __device__ __forceinline__ uint32_t sub_pass(const PKey<W>& K, const GateArg<W>& g, uint32_t k) {
+    uint64_t bit = 0, seen = 0;   // the lowest bit in K; bits of the gate so far
+#pragma unroll
+    for (int w = 0; w < 2 * W; ++w) {
+        const uint64_t q = w < W ? g.qx[w] : g.qz[w - W];
+        const uint64_t v = w < W ? K.x[w] : K.z[w - W];
+        if (!seen) bit = v & q & (~q + 1ULL);
+        seen |= q;
+    }
+    const uint64_t flip = bit ? ~0ULL : 0ULL;
     uint32_t h = 0x3c6ef372u;
 #pragma unroll
     for (int w = 0; w < W; ++w) {
-        const uint64_t mx = K.x[w] & ~g.qx[w], mz = K.z[w] & ~g.qz[w];
+        const uint64_t mx = K.x[w] ^ (g.qx[w] & flip), mz = K.z[w] ^ (g.qz[w] & flip);
         h = murmur_mix(h, (uint32_t)mx);
         h = murmur_mix(h, (uint32_t)(mx >> 32));
         h = murmur_mix(h, (uint32_t)mz);
@@ -607,7 +615,7 @@ __device__ __forceinline__ uint32_t stage_pass(uint32_t n, const GateArg<W>& g,
 }
 
 // A partition above the staging capacity, in k sub-passes over the hash
-// classes of the key with the gate's sites cleared (about C/2 strings each,
+// classes of the pair key (about C/2 strings each,
 // gathered into the staging arrays).  A first round of the sub-passes only
 // counts their children, room(total) gives a run's position (~0: none, nothing
 // is written) and a second round writes them.  Every thread calls it.

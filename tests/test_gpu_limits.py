@@ -172,3 +172,25 @@ def test_identity_gates_merged_in_full(n, cap, separate):
         g.apply_trotter_layer(1)
         o.apply_layers(1)
         assert_same_state(g.terms(), o.terms(), f"n {n} layer {layer}")
+
+
+# A gate on every site, Y on most: few bits of a key lie outside it, and long
+# partitions are merged in classes of strings all the same.
+@pytest.mark.parametrize("separate", [False, True])
+@pytest.mark.parametrize("n,layers", [(8, 6), (9, 5)])
+def test_long_partitions_of_a_wide_gate(n, layers, separate):
+    H = wl.tfim_1d(n, 1.0, 0.9, periodic=True)
+    all_sites = np.uint64((1 << n) - 1)
+    gx = np.concatenate([H.gate_x, [[all_sites]], [[all_sites >> np.uint64(1)]]])
+    gz = np.concatenate([H.gate_z, [[all_sites]], [[all_sites]]])
+    alpha = np.concatenate([H.alpha, [0.7, -0.4]])
+    cap = 20000
+    g = itpp.Propagator(n, gx, gz, alpha, 0.1, 1e-9, cap, 1, partition_target=2048)
+    if separate:
+        g.profile_enable(True)
+    o = oracle.Oracle(n, gx, gz, alpha, 0.1, 1e-9, cap, 1)
+    for layer in range(layers):
+        g.apply_trotter_layer(1)
+        o.apply_layers(1)
+        assert_same_state(g.terms(), o.terms(), f"n {n} layer {layer}")
+    assert g.count() > 4096
