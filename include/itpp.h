@@ -196,7 +196,12 @@ itpp_status itpp_destroy(itpp_handle h);
  * (Algorithm 1, "Accumulate"), terms with |c| <= delta are dropped, the cap
  * policy is applied, and every coefficient is divided by the identity's
  * ("Truncate and normalize", Sec. II.C per-step trace normalisation).
- * Asynchronous.  n_layers >= 0. */
+ * Asynchronous.  n_layers >= 0.
+ * Bounds up to 2^20 terms (and batches): whole layers are one cooperative
+ * launch of up to 4,096 gates that fills the GPU, so work on other streams
+ * waits for its end, up to tenths of a second; apply fewer layers per call
+ * where that matters.  A layer may be captured into a CUDA graph; its replays
+ * and eager calls on the same stream may follow one another in any order. */
 itpp_status itpp_apply_trotter_layer(itpp_handle h, int n_layers);
 
 /* Apply the single gate k (0 <= k < n_gates) of the Trotter order; the same
@@ -418,7 +423,8 @@ itpp_status itpp_batch_synchronize(itpp_batch_handle h);
  * Each candidate is timed with CUDA events over probe_layers Trotter layers
  * from the identity; coordinate descent from
  * the default shape, one parameter at a time.  The fastest shape stays
- * installed.  Every instance is reset to the identity before each timing
+ * installed (among those on which the fewest instances ended with an error).
+ * Every instance is reset to the identity before each timing
  * and after the search (statistics cleared), so results never depend on the
  * tuning: every shape gives bit-identical states.  Synchronising.
  *   probe_layers  >= 1.
