@@ -109,8 +109,8 @@ constexpr uint64_t run_tie_off(uint64_t cand_cap) { return (cand_cap * 12 + 255)
 size_t run_shared_bytes();
 size_t run_shared_head();
 // The kernel with few CTAs per SM (3; 2 with two mask words), or the wide one
-// with one more.  The register file is shared out: the first spills less (904
-// bytes of stores against 1,176, with two words 132 against 1,048), the second
+// with one more.  The register file is shared out: the first spills less (844
+// bytes of stores against 1,184, with two words 132 against 1,004), the second
 // hides more latency.  For
 // one propagation of 2^16 or 2^18 terms a layer takes 3.21 and 3.14 ms with the
 // first, 3.55 and 3.45 with the second; at 2^20 both 9.3.  Batches of 4 x 2^16

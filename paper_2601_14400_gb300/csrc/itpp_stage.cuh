@@ -365,6 +365,15 @@ __device__ __forceinline__ bool pair_enter(const PKey<W>& K, const GateArg<W>& g
     return false;
 }
 
+// The identity as the gate: every string is its own partner.
+template <int W>
+__device__ __forceinline__ bool gate_is_identity(const GateArg<W>& g) {
+    uint64_t q = 0;
+#pragma unroll
+    for (int w = 0; w < W; ++w) q |= g.qx[w] | g.qz[w];
+    return q == 0;
+}
+
 // Of the kept children: the largest pattern.
 struct SelStats {
     unsigned long long out_max;
@@ -483,10 +492,11 @@ __device__ __forceinline__ void pass_children(uint32_t n_pair, uint32_t n_throug
             }
         } else {
             const uint32_t j = j0 - pair_end + lane;
-            if (j < n_through) {   // {P,Q} = 0: unchanged
+            if (j < n_through) {   // {P,Q} = 0: unchanged (or Q = I)
                 const uint32_t i = A::list()[Stage<W>::C - 1 - j];
                 K = A::keys()[i];
                 va = vals[i];
+                if (gate_is_identity(g)) va = __dadd_rn(__dmul_rn(va, g.ch), __dmul_rn(va, g.msh));
                 ka = above(va, dbits) && light(K, g.maxw);
                 if (has_id && key_is_zero(K)) {
                     if (kWrite) ctl->norm[nxt] = va;
@@ -532,11 +542,6 @@ __device__ __forceinline__ uint32_t stage_pass(uint32_t n, const GateArg<W>& g,
     double* vals = A::vals();
     const uint32_t lane = threadIdx.x & 31u, par = pass & 1u;
     const unsigned int lt = (1u << lane) - 1u;
-    // the identity as the gate: every string is its own partner
-    uint64_t qbits = 0;
-#pragma unroll
-    for (int w = 0; w < W; ++w) qbits |= g.qx[w] | g.qz[w];
-    const bool self = qbits == 0;
     for (uint32_t i0 = threadIdx.x & ~31u; i0 < n; i0 += BLOCK) {   // whole warps
         const uint32_t i = i0 + lane;
         uint32_t slot = 0;
@@ -553,13 +558,9 @@ __device__ __forceinline__ uint32_t stage_pass(uint32_t n, const GateArg<W>& g,
                 c = 1.0;   // the identity's normalised value is exactly 1
                 if (!live) set_status(ctl, ST_TRACE_ZERO, 43);
             }
-            bool neg;
-            bool comm = commute_sign(K, g, &neg);
-            if (self) {
-                c = __dadd_rn(__dmul_rn(c, g.ch), __dmul_rn(c, g.msh));
-                comm = false;   // done: the rest is that of a string that passes through
-            }
             vals[i] = c;
+            bool neg;
+            const bool comm = commute_sign(K, g, &neg) && !gate_is_identity(g);
             through = live && !comm;
             if (live && comm) owner = pair_enter(K, g, i, neg, A::keys(), A::tab(), ctl, &slot);
         }

@@ -12,8 +12,8 @@ from tests.test_kernel_resources import _find, _report
 # kernel -> CTA size, CTAs per SM, bytes of spill stores and loads it was
 # measured with
 KERNELS = {
-    "itpp_run.cu": {"k_run<1, false>": (256, 3, 904, 1680), "k_run<2, false>": (256, 2, 132, 276)},
-    "itpp_run_wide.cu": {"k_run<1, true>": (256, 4, 1176, 2252), "k_run<2, true>": (256, 3, 1048, 1908)},
+    "itpp_run.cu": {"k_run<1, false>": (256, 3, 844, 1692), "k_run<2, false>": (256, 2, 132, 268)},
+    "itpp_run_wide.cu": {"k_run<1, true>": (256, 4, 1184, 2208), "k_run<2, true>": (256, 3, 1004, 1788)},
     "itpp_part.cu": {"k_gate_inplace<1, 256>": (256, 4, 0, 0), "k_gate_inplace<2, 128>": (128, 6, 276, 96)},
     "itpp_select.cu": {"k_sel_resolve<1>": (256, 2, 0, 0), "k_sel_resolve<2>": (256, 2, 0, 0)},
     "itpp_adjoint.cu": {"k_adj_recompute<1>": (256, 4, 0, 0), "k_adj_recompute<2>": (256, 4, 44, 36),
