@@ -219,6 +219,7 @@ __global__ void k_import_begin(DevCtl* ctl, uint64_t count) {
         ctl->home = 0;
         ctl->need_scatter = ctl->part_over = ctl->scattered = ctl->over = 0;
         ctl->ticket = 0;
+        ctl->alloc = 0;
         ctl->sp_lo = ctl->sp_hi = ctl->sp_thr = 0;
         ctl->sp_shift = 0;
         ctl->sp_tprev = 0;
@@ -358,6 +359,7 @@ __global__ void k_reset_identity(BufsA<W> B, DevCtl* ctl) {
         ctl->home = 0;
         ctl->need_scatter = ctl->part_over = ctl->scattered = ctl->over = 0;
         ctl->ticket = 0;
+        ctl->alloc = 0;
         ctl->sp_lo = ctl->sp_hi = ctl->sp_thr = 0;
         ctl->sp_shift = 0;
         ctl->sp_tprev = 0;

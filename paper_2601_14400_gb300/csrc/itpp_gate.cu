@@ -240,21 +240,23 @@ __device__ __forceinline__ PKey<W> pend_tie_key(const DevCtl* ctl) {
 // Materialise the state of the partitioned merge for a reader that wants a
 // contiguous run: the stored terms that the pending select keeps (a zero is no
 // term), gathered from the partitions into the buffer they leave free, or
-// compacted into the other buffer.
+// compacted into the other buffer.  One launch, as every read of a large state
+// makes it and most find nothing to do (2.3 us of a read of 94 us, three launches
+// 14): the last CTA switches the state over, once no other has anything left to
+// read of where it was.  ctl->alloc is zero between the kernels that count with it.
 __device__ __forceinline__ bool mat_needed(const DevCtl* ctl) { return ctl->pend || ctl->home; }
 __device__ __forceinline__ int mat_buf(const DevCtl* ctl) { return ctl->home ? ctl->ha : ctl->cur ^ 1; }
-
-__global__ void k_mat_begin(DevCtl* ctl) {
-    if (threadIdx.x != 0 || !mat_needed(ctl) || ctl->status) return;
-    ctl->alloc = 0ULL;
-}
 
 template <int W, int BLOCK>
 __global__ void __launch_bounds__(BLOCK)
 k_materialize(Bufs<W> B, Homes<W> H, DevCtl* ctl) {
-    if (!mat_needed(ctl) || ctl->status) return;
     __shared__ uint32_t s_scan[BLOCK / 32];
     __shared__ unsigned long long s_base;
+    __shared__ int s_run;
+    // one look for the whole CTA (another may set the status meanwhile)
+    if (threadIdx.x == 0) s_run = mat_needed(ctl) && !ctl->status;
+    __syncthreads();
+    if (!s_run) return;
     const bool pend = ctl->pend != 0;
     const unsigned long long T = pend ? ctl->pend_T : 0ULL;
     const bool all_ties = !pend || ctl->pend_all_ties;
@@ -291,18 +293,17 @@ k_materialize(Bufs<W> B, Homes<W> H, DevCtl* ctl) {
             }
         }
     }
-}
-
-__global__ void k_mat_end(DevCtl* ctl) {
-    if (threadIdx.x != 0 || !mat_needed(ctl)) return;
-    if (!ctl->status) {
+    __syncthreads();
+    if (threadIdx.x != 0 || !last_cta(ctl)) return;
+    if (!*(volatile int*)&ctl->status) {
         const int cur = ctl->cur, d = mat_buf(ctl);
         const double norm = ctl->norm[cur], rnorm = ctl->rnorm[cur];
         ctl->norm[d] = norm;
         ctl->rnorm[d] = rnorm;
-        ctl->count[d] = ctl->alloc;
+        ctl->count[d] = __ldcg(&ctl->alloc);
         ctl->cur = d;
     }
+    ctl->alloc = 0ULL;
     ctl->pend = 0;
     ctl->home = 0;
 }
@@ -407,10 +408,8 @@ int cap_launches(const DeviceState& s) {
 
 template <int W>
 static cudaError_t materialize_w(const DeviceState& s, cudaStream_t st) {
-    k_mat_begin<<<1, 32, 0, st>>>(s.ctl);
     k_materialize<W, 256><<<stream_grid(s, 256, 8), 256, 0, st>>>(bufs_of<W>(s), homes_of<W>(s),
                                                                   s.ctl);
-    k_mat_end<<<1, 32, 0, st>>>(s.ctl);
     return cudaGetLastError();
 }
 

@@ -91,6 +91,18 @@ __device__ __forceinline__ StateRuns<W> state_runs(const DevCtl* ctl, const Bufs
     return r;
 }
 
+// Is this the last CTA of the launch to get here?  (One thread; what the CTA
+// wrote before the barrier ahead of it is then seen by the last one.)
+__device__ __forceinline__ bool last_cta(DevCtl* ctl) {
+    __threadfence();
+    const bool last = atomicAdd(&ctl->ticket, 1u) == gridDim.x - 1u;
+    if (last) {
+        ctl->ticket = 0u;
+        __threadfence();
+    }
+    return last;
+}
+
 // ---------------------------------------------------------------------------
 // Merge-table probe
 // ---------------------------------------------------------------------------

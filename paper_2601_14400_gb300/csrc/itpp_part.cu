@@ -38,18 +38,6 @@
 
 namespace itpp {
 
-// Is this the last CTA of the launch to get here?  (One thread; what the CTA
-// wrote before the barrier ahead of it is then seen by the last one.)
-__device__ __forceinline__ bool last_cta(DevCtl* ctl) {
-    __threadfence();
-    const bool last = atomicAdd(&ctl->ticket, 1u) == gridDim.x - 1u;
-    if (last) {
-        ctl->ticket = 0u;
-        __threadfence();
-    }
-    return last;
-}
-
 // Scatter the current state into the partitions of a window (force), or,
 // inside a window, only when the state has no partitions, or those of another
 // window, or they held for the previous gate alone.  The state is a contiguous
@@ -417,6 +405,7 @@ k_part_post(DevCtl* ctl, CandRegions cd, uint64_t cap_M, int cap_policy, uint64_
         if (ctl->retry) {
             ctl->home = 0;
             ctl->count[ctl->cur ^ 1] = ctl->alloc;
+            ctl->alloc = 0ULL;
         } else {
             ctl->hx ^= 1;
             ctl->hc = next3(ctl->hc);
